@@ -106,9 +106,8 @@ struct icwf_ctx {
   double2* proj = nullptr;
   std::vector<void*> extra_allocs;
   size_t obs_bytes = 0;                     // observables work buffers (allocated on first use)
-  // tensor-core assembly scratch
-  void* tc_scratch = nullptr;
-  size_t tc_scratch_bytes = 0;
+  AsmPlan plan;                             // assembly: operand slices, Grams and their tables
+  size_t plan_bytes = 0;
   // FP64 factorisation: digit planes of the emulated trailing update (allocated when !df_solve)
   void* emu_scratch = nullptr;
   size_t emu_bytes = 0;
@@ -370,16 +369,7 @@ void solve(icwf_ctx* h, const double2* Lf, const double2* D, const double2* y, d
 
 void assemble(icwf_ctx* h, double2* S, double2* Hm) {
   ProfScope ps(h, F_ASSEMBLE);
-  // operand planes (two sides) + Grams [+ digit planes (two sides) + exact overlap], or the FP64
-  // kernel
-  h->launches += h->mixed ? (h->p.overlap_split ? 3 : 6) : 1;
-  JobView j = view(h);
-  if (h->mixed) {
-    launch_assemble_tc(j, h->p.precision, h->p.overlap_split == 0, S, Hm, h->tc_scratch,
-                       h->tc_scratch_bytes, h->stream);
-  } else {
-    launch_assemble_fp64(j, S, Hm, h->stream);
-  }
+  h->launches += h->plan.launch(view(h), S, Hm, h->stream);
 }
 
 // One ICWF step t_n -> t_{n+1}.
@@ -620,6 +610,7 @@ namespace icwf {
 bool handle_obs_view(icwf_handle h, ObsView* v) {
   if (!h || !v) return false;
   v->j = view(h);
+  v->plan = &h->plan;
   v->C = h->C;
   v->phi = h->phi;
   v->n_states = h->n_states;
@@ -662,8 +653,6 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
     return fail(nullptr, ICWF_ERR_ARG, "icwf_create: invalid extents, masses, dt, eps or cutoff");
   if (p.precision < 0 || p.precision > 2)
     return fail(nullptr, ICWF_ERR_ARG, "icwf_create: unknown precision");
-  if (p.precision != ICWF_FP64 && assemble_tc_scratch_bytes(p.n_traj, p.nx, p.nR, 1) == 0)
-    return fail(nullptr, ICWF_ERR_ARG, "icwf_create: mixed precision is not available in this library");
   if (p.coeff_scheme < 0 || p.coeff_scheme > 1)
     return fail(nullptr, ICWF_ERR_ARG, "icwf_create: unknown coeff_scheme");
   if (p.precision != ICWF_FP64 && (p.nx < 64 || p.nR < 64))
@@ -770,10 +759,9 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
       (size_t)2 * nblk * 4 + 64, chol_ctl_words(N) * sizeof(unsigned), 64 * 4};
   size_t total = 0;
   for (size_t b : sizes) total += align256(b);
-  if (h->mixed) {
-    h->tc_scratch_bytes = assemble_tc_scratch_bytes(N, nx, nR, K);
-    total += align256(h->tc_scratch_bytes);
-  }
+  const AsmShape shape{N, nx, nR, K, p.precision, p.overlap_split, h->dx, h->dR, sk.data()};
+  h->plan_bytes = h->plan.layout(shape, nullptr, nullptr) + 1024;
+  total += align256(h->plan_bytes);
   if (!h->df_solve) {
     h->emu_bytes = herk_emu_scratch_bytes(N);
     total += align256(h->emu_bytes);
@@ -829,9 +817,9 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
   h->tickets = h->flags + 2 * nblk;
   h->cctl = (unsigned*)a.take(chol_ctl_words(N) * sizeof(unsigned));
   h->status = (int*)a.take(64 * 4);
-  if (h->mixed) h->tc_scratch = a.take(h->tc_scratch_bytes);
   if (!h->df_solve) h->emu_scratch = a.take(h->emu_bytes);
-  if (!h->status || (h->mixed && !h->tc_scratch) || (!h->df_solve && !h->emu_scratch)) {
+  char* plan_base = (char*)a.take(h->plan_bytes);
+  if (!h->status || !plan_base || (!h->df_solve && !h->emu_scratch)) {
     cudaFree(h->arena.base);
     destroy_streams(h);
     return fail(nullptr, ICWF_ERR_OOM, "icwf_create: arena layout overflow");
@@ -869,6 +857,15 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
   UP(h->v1, v1.data(), v1.size() * 8);
   UP(h->v2, v2.data(), v2.size() * 8);
 #undef UP
+  {
+    const JobView j = view(h);
+    h->plan.layout(shape, &j, (void*)(((uintptr_t)plan_base + 1023) & ~(uintptr_t)1023));
+    if (!h->plan.upload(shape, Uk.data(), Wk.data(), h->stream)) {
+      cudaFree(h->arena.base);
+      destroy_streams(h);
+      return fail(nullptr, ICWF_ERR_CUDA, "icwf_create: assembly set-up failed");
+    }
+  }
   h->prop_threads = tune_propagate(h);
   if (cudaMemsetAsync(h->flags, 0, (size_t)2 * nblk * 4 + 64, h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->status, 0, 64 * 4, h->stream) != cudaSuccess ||
@@ -1077,13 +1074,12 @@ icwf_status icwf_observables(icwf_handle h, icwf_obs* out) {
   JobView j = view(h);
   {
     ProfScope ps(h, F_OBS);
-    if (h->mixed) launch_reconstruct<float>(j, h->C, h->Psi, h->stream);
-    else launch_reconstruct<double>(j, h->C, h->Psi, h->stream);
+    h->plan.reconstruct(j, h->C, h->Psi, h->stream);
     launch_obs_lines(j, h->Psi, h->phi, h->n_states, h->rho_x, h->rho_R, h->proj, h->part,
                      h->obs_out, h->pop, h->decoh, h->twx_d, h->twR_d, h->stream);
   }
   double o4[4];
-  int cl[2];
+  int cl[STATUS_COPY];
   CK(cudaMemcpyAsync(o4, h->obs_out, sizeof(o4), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaMemcpyAsync(cl, h->status, sizeof(cl), cudaMemcpyDeviceToHost, h->stream));
   if (out->rho_x) CK(cudaMemcpyAsync(out->rho_x, h->rho_x, h->nx * 8, cudaMemcpyDeviceToHost, h->stream));
@@ -1098,7 +1094,11 @@ icwf_status icwf_observables(icwf_handle h, icwf_obs* out) {
   out->norm = o4[0];
   out->energy = (o4[1] + o4[2] + o4[3]) / o4[0];
   out->n_states = h->n_states;
-  out->n_clamped = cl[1];
+  out->n_clamped = cl[STATUS_CLAMPED];
+  if (cl[STATUS_OBS] & ST_TIMEOUT) {
+    CK(cudaMemset(h->status + STATUS_OBS, 0, sizeof(int)));
+    return fail(h, ICWF_ERR_TIMEOUT, "icwf_observables: in-kernel wait timed out");
+  }
   return ICWF_OK;
 }
 

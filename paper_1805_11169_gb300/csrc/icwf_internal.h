@@ -21,7 +21,9 @@ enum : int {
 // STATUS_WAITLIM: 0 = the compiled-in limits of the spin waits on global flags; k > 0 = those waits
 // give up after k - 1 polls (set by icwf_set_wait_limit, a diagnostic for the timeout path).
 enum : int { STATUS_FLAGS = 0, STATUS_CLAMPED = 1, STATUS_TICKET = 2, STATUS_WAITLIM = 3,
-             STATUS_WORDS = 8 };
+             STATUS_WORDS = 8,
+             STATUS_OBS = 8 };   // flags of the observables' kernels (a step's are words 0..)
+constexpr int STATUS_COPY = 16;  // words the observables read back
 
 // ---------------------------------------------------------------- launch descriptors
 
@@ -110,8 +112,34 @@ bool add_group_nodes(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndep
                      const GroupJob* table, int njobs, int total_traj, int total_cwf, int nmax,
                      int threads, int max_ctas, cudaGraphNode_t* last);
 
-// a5 (FP64): S = S1 o S2 and Heff from the rank-K factors at the current positions.
-void launch_assemble_fp64(const JobView& j, double2* S, double2* H, cudaStream_t s);
+// a5: S = S1 o S2 and Heff from the rank-K factors at the current positions, every mode, on the
+// tensor cores (k_sliced.cu).  A handle's plan lays out its operand slices, Grams and tables in one
+// scratch region of its arena; the tables are uploaded once, so launch() can be captured.
+struct AsmShape {
+  int N, nx, nR, K, precision, overlap_split;
+  double dx, dR;
+  const double* sig;      // K singular values (host)
+};
+class AsmPlan {
+ public:
+  AsmPlan();
+  ~AsmPlan();
+  AsmPlan(const AsmPlan&) = delete;
+  AsmPlan& operator=(const AsmPlan&) = delete;
+  // Lays the plan out at `base` (1024-byte aligned; NULL to size it) and returns its bytes; j holds
+  // the device pointers the kernels read (NULL while sizing).
+  size_t layout(const AsmShape& q, const JobView* j, void* base);
+  // Uploads the tables (U: K x nx and W: K x nR factors on the host) and sets the kernels' attributes.
+  bool upload(const AsmShape& q, const double* U, const double* W, cudaStream_t s);
+  // Returns the number of kernels launched.
+  int launch(const JobView& j, double2* S, double2* H, cudaStream_t s) const;
+  // a7: Psi[i*nR + j] = sum_a C_a psi_a(x_i) chi_a(R_j) (complex128); uses the plan's scratch.
+  int reconstruct(const JobView& j, const double2* C, double2* Psi, cudaStream_t s) const;
+  struct Impl;
+
+ private:
+  Impl* impl = nullptr;
+};
 
 // Generic Gram G = scale * A^H diag(dg) B (A, B column-major n x N complex of type T, dg may be
 // NULL for identity); output N x N complex128 row-major.
@@ -176,9 +204,6 @@ void launch_rk4_final(int N, double2* C, const double2* k1, const double2* k2,
 void launch_check_finite(int n, const double2* a, int* status, cudaStream_t s);
 
 // a7: observables.
-// Psi[i*nR + j] = sum_a C_a psi_a(x_i) chi_a(R_j)  (complex128 output).
-template <typename T> void launch_reconstruct(const JobView& j, const double2* C, double2* Psi,
-                                              cudaStream_t s);
 // Column / row reductions of Psi: rho_R, rho_x, potential energy, BO projections, FFT kinetic
 // energies (partials), then the final deterministic sums into out[0..3] = norm, ekx, ekR, epot.
 // part needs 2 nR + nx doubles, proj n_states * nR complex; twx/twR are FP64 twiddles.
@@ -196,6 +221,7 @@ void launch_to_c64(size_t n, const double2* in, float2* out, cudaStream_t s);
 // Everything the observables kernels need from a handle (filled by handle_obs_view in api.cpp).
 struct ObsView {
   JobView j;
+  const AsmPlan* plan;
   const double2* C;
   const double* phi;
   int n_states;
@@ -209,15 +235,5 @@ struct ObsView {
 };
 bool handle_obs_view(icwf_handle h, ObsView* v);
 void handle_set_error(icwf_handle h, const char* msg);
-
-// Mixed-precision assembly on the tensor cores (tcgen05); returns false if unsupported sizes.
-// exact_s: S from launch_gram_s (exact Grams of fixed-point CWFs), else from the split products.
-bool launch_assemble_tc(const JobView& j, int kind, bool exact_s, double2* S, double2* H,
-                        void* scratch, size_t scratch_bytes, cudaStream_t s);
-size_t assemble_tc_scratch_bytes(int N, int nx, int nR, int K);
-// S = S1 o S2 as exact Grams of 4-digit fixed-point complex64 CWFs on the tensor cores
-// (k_gram_s.cu); scratch of gram_s_scratch_bytes.  Returns false if it does not fit.
-bool launch_gram_s(const JobView& j, double2* S, void* scratch, size_t bytes, cudaStream_t s);
-size_t gram_s_scratch_bytes(int N, int nx, int nR);
 
 }  // namespace icwf

@@ -1,0 +1,1328 @@
+// Matrix elements (Eq. M, W, W1, W2) of every mode as Grams of sliced operands on the sm_103a tensor
+// cores, and their combination into S and Heff.
+//
+// Slicing.  A CWF column (weighted by u_g(x) for the rank-k terms) is scaled by a power of two 2^-e so
+// that its components lie in (-1, 1) and is cut into D pieces of a 16-bit type that sum to it:
+//   digits  balanced integers d_p, value = 2^e sum_p d_p 2^-(b0 + beta p), stored exactly as BF16;
+//           products of digits are integers, so the sums over the grid are exact in FP32 as long as
+//           they stay below 2^24.  b0 = 6, beta = 7 in the FP64 mode (D = 8: 55 bits below the
+//           largest component), b0 = beta = 6 with D = 4 for the mixed modes' overlap (24 bits: S
+//           is then the exact Gram of fixed-point CWFs and positive semidefinite; b0 = beta = 5 on
+//           4096-point grids);
+//   pieces  hi + lo floating-point pieces for the mixed modes' Heff: FP16 (11 significant bits each,
+//           the significand of TF32, at twice its rate and half its bytes; the power of two keeps
+//           every piece inside FP16's range) or BF16 (8 bits each).
+//
+// Products.  conj(a) b = sum over piece pairs (p, q); the pairs with p + q < L are kept and every level
+// l = p + q has its own FP32 accumulator in TMEM.  With the T kets' pieces stored one after the
+// other, [b_0; b_1; ...] is a single operand of up to 256 rows, so one MMA takes piece p of 128 bras
+// against all pieces q < L - p at once and lands on the adjacent accumulators of levels p, p + 1, ...:
+// M = 128, N up to 256, where the tensor cores and not the shared-memory operand reads are the bound.
+// (One MMA per pair, N = 64, measured 88-115 cycles where the tensor pipe needs 32.)
+// L = D keeps products down to the pieces' own truncation; the overlap keeps all 2D - 1 levels.
+//
+// Digits are only as many as a term needs: term g of the interaction enters Heff with weight s_g, so
+// it takes D_g = ceil((56 + log2(s_g / s_1)) / 7) digits and its truncation error equals that of the
+// first term, 2^-56 of s_1, which is FP64's own (the FP64 products these replace rounded each sum at
+// 2^-53).  At the paper's scale (22 terms) that is 22 digit pairs on average instead of 36.
+//
+// Level sums (digits) are combined as 64-bit integers, in units of 2^-F of level 0, and converted
+// once: no FP64 instruction in the loop (FP64 runs at 1/61 of FP32 here).  The accumulators are drained
+// into the integers every `drain` K slices, before a leading level could pass 2^24 (drain_slices).
+//
+// Layout.  Operands are written by k_slices in the order the MMA reads them: tiles of 128 bra rows (T
+// ket rows) x 16 grid points in the 32-byte-swizzled K-major form, [tile][K slice][Re, Im][piece],
+// so that a pipeline stage is two or three contiguous bulk copies.
+//
+// k_gram_sliced: persistent CTAs (320 threads, one per SM) take units (Gram, 128-bra x T-ket tile) by
+// a ticket, the most expensive first; warp 8 copies stages, warp 9 issues the MMAs, warps 0..7 drain
+// TMEM (warp w: lanes 32 (w mod 4).., column half w div 4).  Ring geometry follows the unit's D.
+// Every wait is bounded (2 s): a timeout raises the status flag, drains what is in flight, returns.
+//
+// Bound: shared-memory bandwidth of the operands (reads by the MMAs plus the copies' writes take about
+// 900 cycles per D = 2 slice against 768 of tensor time); the tensor pipe is busy 73% of the time.
+// Measured (GB300, N = 1024 on 1024 x 512; ms per assembly, before -> now): FP64 mode, 22 terms, 144
+// (FP64 FMAs) -> 3.5; TF32-significand pieces, 16 terms, 1.16 (TF32 MMAs of N = 64 on 128 x 32 tiles,
+// bound by L2 -> shared memory) -> 0.50; BF16 pieces at N = 512 on 512 x 256 0.38 -> 0.13; FP64,
+// N = 16, 64 terms on 128 x 64, 13.1 (one CTA) -> 0.26; reconstruction in the FP64 mode 4.3 -> 0.22.
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <mutex>
+#include <vector>
+
+#include "icwf_internal.h"
+#include "k_common.cuh"
+#include "sliced.cuh"
+#include "tc_ptx.cuh"
+
+namespace icwf {
+namespace sl {
+
+using namespace tc;
+
+constexpr int RING_BYTES = 220 * 1024;
+constexpr int MAX_SLOTS = 6;
+constexpr int UNIT_RING = 4;
+constexpr int MAX_GRAMS = 256;         // Grams of one launch
+constexpr int SMEM_BYTES = RING_BYTES + 1024 /*align*/ + 512 /*barriers, unit ring*/ + MAX_GRAMS * 4;
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory per CTA exceeded");
+constexpr int EPI_WARPS = 8, TMA_WARP = 8, MMA_WARP = 9, THREADS = 320;
+constexpr int COL_IM = 256;            // TMEM: Re levels at [0, 256), Im levels at [256, 512)
+constexpr int EX_BAD = 0x40000000;     // exponent of a row with a non-finite component
+
+// bytes of a pipeline stage (one K slice): both planes' pieces of 128 bras and T kets
+__host__ __device__ inline int stage_bytes(int d, int t) { return 2 * d * (MT + t) * ROW_BYTES; }
+__host__ __device__ inline int ring_slots(int d, int t) {
+  const int s = RING_BYTES / stage_bytes(d, t);
+  return s < MAX_SLOTS ? s : MAX_SLOTS;
+}
+
+// One Gram (one side, one weight) of a launch.
+struct Gram {
+  const unsigned char* A;   // bras: 128-row tiles, da pieces stored per plane
+  const unsigned char* B;   // kets: T-row tiles with d pieces per plane, or NULL: rows of A
+  const int* ea;            // scale exponents of the bras and kets
+  const int* eb;
+  void* out;                // [tile of 128 x 128][ket][bra], double2 (digits) or float2 (pieces)
+  float scale;              // pieces: grid spacing
+  int ks, da, d, l, t;      // K slices; pieces stored / used; levels; kets per unit
+  int drain;                // K slices per accumulation
+  int f16, digits;          // piece type; digits or floating-point pieces
+  int b0, beta, fbits;      // digit weights; fraction bits of the integer accumulators
+  int unit0;                // first unit
+  int cols;                 // 0: upper-triangle tiles; else a rectangular product of rows x cols
+  int rows;                 //    elements, out row-major (double2)
+};
+
+struct GramArgs {
+  const Gram* grams;
+  void* out;                // overrides the Grams' outputs if not NULL
+  int ngrams, units, N;
+  unsigned* ticket;
+  int* status;
+};
+
+// Where unit v of Gram g reads and writes: bra tile, ket tile (of T rows), first output element and
+// the output's strides along bras and kets.
+struct UnitAt {
+  int I, J, bt;             // bra tile; 128-ket tile and T-ket tile
+  size_t out;
+  int sr, sc;
+};
+__device__ __forceinline__ UnitAt unit_at(const Gram& g, int v) {
+  UnitAt u;
+  const int qn = MT / g.t;
+  if (g.cols == 0) {
+    tri_tile(v / qn, u.I, u.J);
+    u.bt = u.J * qn + v % qn;
+    u.out = ((size_t)(v / qn) * MT + (v % qn) * g.t) * MT;
+    u.sr = 1;
+    u.sc = MT;
+  } else {
+    const int nt = (g.cols + g.t - 1) / g.t;
+    u.I = v / nt;
+    u.bt = v % nt;
+    u.J = u.bt / qn;
+    u.out = (size_t)u.I * MT * g.cols + (size_t)u.bt * g.t;
+    u.sr = g.cols;
+    u.sc = 1;
+  }
+  return u;
+}
+
+// dst (shared) <- src (global), both 16-byte aligned, completing on bar
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, int bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+
+__device__ __forceinline__ int gram_of(const int* unit0, int n, int u) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (unit0[mid] <= u) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// sum += the levels' exact integers of 8 columns (Re at col, Im at col + COL_IM) in units 2^-fbits
+__device__ __forceinline__ void drain8(uint32_t col, int L, int t, int beta, int fbits,
+                                       long long (&re)[8], long long (&im)[8]) {
+#pragma unroll 1
+  for (int lv = 0; lv < L; ++lv) {
+    float vr[8], vi[8];
+    tmem_ld8(col + lv * t, vr);
+    tmem_ld8(col + COL_IM + lv * t, vi);
+    tmem_wait_ld();
+    const int sh = fbits - beta * lv;
+    if (sh >= 32) {   // only the upper word changes
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        re[e] += (long long)((unsigned long long)(unsigned)(__float2int_rn(vr[e]) << (sh - 32)) << 32);
+        im[e] += (long long)((unsigned long long)(unsigned)(__float2int_rn(vi[e]) << (sh - 32)) << 32);
+      }
+    } else if (sh >= 0) {   // one 32 x 32 + 64 bit multiply-add per sum
+      const unsigned w = 1u << sh;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        re[e] += (long long)__float2int_rn(vr[e]) * (long long)w;
+        im[e] += (long long)__float2int_rn(vi[e]) * (long long)w;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        re[e] += __float2int_rn(vr[e]) >> -sh;
+        im[e] += __float2int_rn(vi[e]) >> -sh;
+      }
+    }
+  }
+}
+
+// x 2^k for a normal x: one multiplication in the usual range
+__device__ __forceinline__ float scaled(float x, int k) {
+  return (unsigned)(k + 126) < 253u ? x * __uint_as_float((unsigned)(k + 127) << 23) : ldexpf(x, k);
+}
+
+// the first n of 8 kets
+// (xb: the warp's lanes hold the exponents of its kets; these are kets l0..)
+__device__ __forceinline__ void store8(double2* out, int sc, int n, int xb, int l0, int ea, int shift,
+                                       const long long (&re)[8], const long long (&im)[8]) {
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const int x = __shfl_sync(0xffffffffu, xb, l0 + e);
+    if (e >= n) continue;
+    double2 z = make_double2(fixed_to_f64(re[e], ea + x + shift), fixed_to_f64(im[e], ea + x + shift));
+    if (ea == EX_BAD || x == EX_BAD) z.x = z.y = __longlong_as_double(0x7FF8000000000000ll);
+    out[(size_t)e * sc] = z;
+  }
+}
+
+// The issuer's view of the stage ring.
+struct MmaRing {
+  unsigned char* ring;
+  uint64_t *full, *empty;
+  volatile int* abort_flag;
+  int* status;
+  int bytes, slots, slot;
+  unsigned pf;              // phase bits of the slots' next full wait
+};
+
+// D[tmem] += A B^T (or = with acc = 0) from the low words of the operand descriptors; the high word,
+// which holds the strides and the swizzle, is the same for all of them.
+constexpr uint32_t DESC_HI = (uint32_t)((8 * ROW_BYTES) >> 4) | (1u << 14) | (6u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+__device__ __forceinline__ void mma_add(uint32_t d, uint32_t a, uint32_t b, uint32_t id) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 x, y;\n\tsetp.ne.b32 p, 1, 0;\n\tmov.b64 x, {%1, %4};\n\t"
+      "mov.b64 y, {%2, %4};\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n\t}" ::"r"(d),
+      "r"(a), "r"(b), "r"(id), "n"(DESC_HI));
+}
+__device__ __forceinline__ void mma_set(uint32_t d, uint32_t a, uint32_t b, uint32_t id, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 x, y;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 x, {%1, %4};\n\t"
+      "mov.b64 y, {%2, %4};\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n\t}" ::"r"(d),
+      "r"(a), "r"(b), "r"(id), "n"(DESC_HI), "r"(acc));
+}
+
+// One accumulation over n K slices of D pieces and L levels.  One thread issues every MMA of the CTA,
+// so it must need fewer cycles per MMA than the tensor cores (96 on average at D = 2): unrolled over
+// the pieces, addresses and instruction descriptors computed once per accumulation, 32-bit
+// descriptor arithmetic, and the next slice's barrier polled before this slice's MMAs.  (Looping
+// over the pieces took 130 cycles per MMA, unrolled with 64-bit descriptors 104.)
+template <int D, int L>
+__device__ __forceinline__ bool issue_slices(MmaRing& r, uint32_t tmem, int t, uint32_t id0, int n) {
+  constexpr uint32_t AT = (MT * ROW_BYTES) >> 4, AQ = D * AT;
+  const uint32_t bt = (uint32_t)(t * ROW_BYTES) >> 4, bq = D * bt;
+  const uint32_t ring = desc_lo(smem_u32(r.ring)), step = (uint32_t)r.bytes >> 4;
+  uint32_t col[D], id[D], idn[D];
+#pragma unroll
+  for (int p = 0; p < D; ++p) {
+    col[p] = tmem + p * t;
+    id[p] = id0 + idesc_n((L - p < D ? L - p : D) * t);
+    idn[p] = id[p] | IDESC_NEG_A;
+  }
+  bool ready = mbar_test(r.full + r.slot, (r.pf >> r.slot) & 1u);
+  for (int s = 0; s < n; ++s) {
+    if (!ready && !mbar_wait(r.full + r.slot, (r.pf >> r.slot) & 1u, r.abort_flag, r.status)) return false;
+    r.pf ^= 1u << r.slot;
+    const int cur = r.slot;
+    r.slot = cur + 1 == r.slots ? 0 : cur + 1;
+    if (s + 1 < n) ready = mbar_test(r.full + r.slot, (r.pf >> r.slot) & 1u);
+    fence_after();
+    const uint32_t ap = ring + cur * step, bp = ap + 2 * AQ;
+    if (s == 0) {
+#pragma unroll
+      for (int p = 0; p < D; ++p) {
+        const uint32_t a = ap + p * AT, re = col[p], im = re + COL_IM;
+        if (p > 0 && L - p >= D) {
+          // the top level of this piece starts here: its own, overwriting MMAs
+          const uint32_t b = bp + (D - 1) * bt, i1 = id0 + idesc_n(t), i2 = id0 + idesc_n((D - 1) * t);
+          const uint32_t c = (D - 1) * t;
+          mma_set(re + c, a, b, i1, 0u);
+          mma_set(im + c, a, b + bq, i1, 0u);
+          mma_add(re + c, a + AQ, b + bq, i1);
+          mma_add(im + c, a + AQ, b, i1 | IDESC_NEG_A);
+          mma_add(re, a, bp, i2);
+          mma_add(im, a, bp + bq, i2);
+          mma_add(re, a + AQ, bp + bq, i2);
+          mma_add(im, a + AQ, bp, i2 | IDESC_NEG_A);
+        } else {
+          mma_set(re, a, bp, id[p], p > 0);
+          mma_set(im, a, bp + bq, id[p], p > 0);
+          mma_add(re, a + AQ, bp + bq, id[p]);
+          mma_add(im, a + AQ, bp, idn[p]);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int p = 0; p < D; ++p) {
+        // Re += P P + Q Q, Im += P Q - Q P
+        const uint32_t a = ap + p * AT, re = col[p], im = re + COL_IM;
+        mma_add(re, a, bp, id[p]);
+        mma_add(im, a, bp + bq, id[p]);
+        mma_add(re, a + AQ, bp + bq, id[p]);
+        mma_add(im, a + AQ, bp, idn[p]);
+      }
+    }
+    mma_commit(r.empty + cur);
+  }
+  return true;
+}
+
+__global__ void __launch_bounds__(THREADS, 1) k_gram_sliced(GramArgs args) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* ring = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(ring + RING_BYTES);
+  uint64_t* empty = full + MAX_SLOTS;
+  uint64_t* acc_full = empty + MAX_SLOTS;
+  uint64_t* acc_empty = acc_full + 1;
+  uint64_t* ufull = acc_empty + 1;
+  uint64_t* uempty = ufull + UNIT_RING;
+  uint64_t* drain = uempty + UNIT_RING;
+  int* uring = (int*)(drain + 1);
+  uint32_t* tmem_slot = (uint32_t*)(uring + UNIT_RING);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+  int* unit0 = (int*)(ring + RING_BYTES + 512);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int* status = args.status;
+
+  for (int i = threadIdx.x; i < args.ngrams; i += THREADS) unit0[i] = args.grams[i].unit0;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < MAX_SLOTS; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
+    for (int s = 0; s < UNIT_RING; ++s) {
+      mbar_init(ufull + s, 1);
+      mbar_init(uempty + s, 1 + EPI_WARPS * 32);
+    }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_empty, EPI_WARPS * 32);
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  // phase bits of the ring slots: the producer's next wait on empty, the issuer's on full
+  if (warp == TMA_WARP) {
+    if (lane == 0) {
+      unsigned pe = (1u << MAX_SLOTS) - 1;   // a fresh barrier passes a wait on parity 1
+      unsigned filled = 0;                   // slots filled at least once
+      int slot = 0, geo = -1;
+      bool ok = true;
+      for (unsigned n = 0; ok; ++n) {
+        const int u = (int)atomicAdd(args.ticket, 1u);
+        const int us = n & (UNIT_RING - 1);
+        if (!mbar_wait(uempty + us, ((n / UNIT_RING) & 1u) ^ 1u, abort_flag, status)) break;
+        const bool last = u >= args.units;
+        uring[us] = last ? -1 : u;
+        mbar_arrive(ufull + us);
+        if (last) break;
+        const Gram& g = args.grams[gram_of(unit0, args.ngrams, u)];
+        const int d = g.d, t = g.t, da = g.da, ks = g.ks;
+        const UnitAt at = unit_at(g, u - g.unit0);
+        const int bytes = stage_bytes(d, t), slots = ring_slots(d, t);
+        if (bytes != geo) {
+          // another ring geometry: every copy and MMA of the old one must be done
+          for (int s = 0; s < MAX_SLOTS && ok; ++s)
+            ok = mbar_wait(empty + s, (pe >> s) & 1u, abort_flag, status);
+          if (!ok) break;
+          geo = bytes;
+          slot = 0;
+        }
+        const size_t a_slice = (size_t)2 * da * MT * ROW_BYTES, b_slice = (size_t)2 * d * t * ROW_BYTES;
+        const unsigned char* ap = g.A + (size_t)at.I * ks * a_slice;
+        const unsigned char* bp = g.B ? g.B + (size_t)at.bt * ks * b_slice
+                                      : g.A + (size_t)at.J * ks * a_slice +
+                                            (size_t)(at.bt * t - at.J * MT) * ROW_BYTES;
+        const bool own_b = g.B != nullptr;
+        for (int s = 0; s < ks; ++s) {
+          if (!(ok = mbar_wait(empty + slot, (pe >> slot) & 1u, abort_flag, status))) break;
+          pe ^= 1u << slot;
+          filled |= 1u << slot;
+          unsigned char* st = ring + slot * bytes;
+          uint64_t* bar = full + slot;
+          mbar_expect_tx(bar, bytes);
+          const int pa = d * MT * ROW_BYTES;
+          bulk_load(st, ap, pa, bar);
+          bulk_load(st + pa, ap + (size_t)da * MT * ROW_BYTES, pa, bar);
+          unsigned char* sb = st + 2 * pa;
+          if (own_b) {
+            bulk_load(sb, bp, (int)b_slice, bar);
+            bp += b_slice;
+          } else {
+            for (int pl = 0; pl < 2; ++pl)
+              for (int p = 0; p < d; ++p)
+                bulk_load(sb + (pl * d + p) * t * ROW_BYTES,
+                          bp + (size_t)(pl * da + p) * MT * ROW_BYTES, t * ROW_BYTES, bar);
+            bp += a_slice;
+          }
+          ap += a_slice;
+          slot = slot + 1 == slots ? 0 : slot + 1;
+        }
+      }
+      if (*abort_flag) {
+        // copies that may still be landing: the last fill of every slot (bounded)
+        for (int s = 0; s < MAX_SLOTS; ++s) {
+          if (!((filled >> s) & 1u)) continue;
+          const unsigned long long t0 = gtime();
+          while (!mbar_test(full + s, (pe >> s) & 1u) && gtime() - t0 < WAIT_NS) {
+          }
+        }
+      }
+    }
+  } else if (warp == MMA_WARP) {
+    if (lane == 0) {
+      unsigned pf = 0, chunk = 0;
+      int slot = 0, geo = -1;
+      bool ok = true;
+      for (unsigned n = 0; ok; ++n) {
+        const int us = n & (UNIT_RING - 1);
+        if (!mbar_wait(ufull + us, (n / UNIT_RING) & 1u, abort_flag, status)) break;
+        const int u = *(volatile int*)(uring + us);
+        mbar_arrive(uempty + us);
+        if (u < 0) break;
+        const Gram& g = args.grams[gram_of(unit0, args.ngrams, u)];
+        const int d = g.d, t = g.t, L = g.l, ks = g.ks, dr = g.drain;
+        const int bytes = stage_bytes(d, t), slots = ring_slots(d, t);
+        if (bytes != geo) { geo = bytes; slot = 0; }
+        const uint32_t id0 = idesc_f16(g.f16, MT, 0);
+        for (int s0 = 0; s0 < ks && ok; s0 += dr) {
+          if (!(ok = mbar_wait(acc_empty, (chunk & 1u) ^ 1u, abort_flag, status))) break;
+          fence_after();
+          ++chunk;
+          const int s1 = s0 + dr < ks ? s0 + dr : ks;
+          MmaRing rg{ring, full, empty, abort_flag, status, bytes, slots, slot, pf};
+          const int n = s1 - s0;
+          if (L > d) ok = issue_slices<4, 7>(rg, tmem, t, id0, n);
+          else if (d == 2) ok = issue_slices<2, 2>(rg, tmem, t, id0, n);
+          else if (d == 3) ok = issue_slices<3, 3>(rg, tmem, t, id0, n);
+          else if (d == 4) ok = issue_slices<4, 4>(rg, tmem, t, id0, n);
+          else if (d == 5) ok = issue_slices<5, 5>(rg, tmem, t, id0, n);
+          else if (d == 6) ok = issue_slices<6, 6>(rg, tmem, t, id0, n);
+          else if (d == 7) ok = issue_slices<7, 7>(rg, tmem, t, id0, n);
+          else ok = issue_slices<8, 8>(rg, tmem, t, id0, n);
+          slot = rg.slot;
+          pf = rg.pf;
+          if (ok) mma_commit(acc_full);
+        }
+      }
+      mma_commit(drain);   // every MMA issued by this CTA
+    }
+  } else {
+    // ---------------- epilogue: lane = bra row, each column half by one warp of the quarter ----
+    const int quarter = warp & 3, half = warp >> 2;
+    const int row = quarter * 32 + lane;
+    const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16);
+    unsigned chunk = 0;
+    bool ok = true;
+    for (unsigned n = 0; ok; ++n) {
+      const int us = n & (UNIT_RING - 1);
+      // (a wait that ends by abort ends for every lane of the warp: the flag stays up)
+      ok = mbar_wait(ufull + us, (n / UNIT_RING) & 1u, abort_flag, status);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      const int u = *(volatile int*)(uring + us);
+      mbar_arrive(uempty + us);
+      if (u < 0) break;
+      const Gram& g = args.grams[gram_of(unit0, args.ngrams, u)];
+      const int t = g.t, L = g.l;
+      const UnitAt at = unit_at(g, u - g.unit0);
+      const int nch = (g.ks + g.drain - 1) / g.drain;
+      const int ea = g.ea[at.I * MT + row];
+      const int c0 = half * (t / 2);                    // this warp's first ket of the unit
+      // exponents of this warp's kets, one per lane (up to 64 kets), off the accumulators' wait
+      const int* eb = g.eb + at.bt * t + c0;
+      const int xb0 = lane < t / 2 ? eb[lane] : 0, xb1 = 32 + lane < t / 2 ? eb[32 + lane] : 0;
+      const size_t o = at.out + (size_t)row * at.sr + (size_t)c0 * at.sc;
+      const int sc = at.sc;
+      // kets this lane stores (rows and columns past the edge of a rectangular product: none)
+      const int nk = g.cols == 0 ? t : (at.I * MT + row < g.rows ? g.cols - at.bt * t - c0 : 0);
+      const uint32_t col = base + half * (t / 2);
+      if (g.digits) {
+        double2* out = (double2*)(args.out ? args.out : g.out) + o;
+        const int shift = -2 * g.b0 - g.fbits;
+        if (t == 32) {
+          long long re[2][8], im[2][8];
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) re[h][e] = im[h][e] = 0;
+          for (int c = 0; c < nch && ok; ++c, ++chunk) {
+            ok = __all_sync(0xffffffffu, mbar_wait(acc_full, chunk & 1u, abort_flag, status));
+            if (!ok) break;
+            fence_after();
+            drain8(col, L, t, g.beta, g.fbits, re[0], im[0]);
+            drain8(col + 8, L, t, g.beta, g.fbits, re[1], im[1]);
+            fence_before();
+            mbar_arrive(acc_empty);
+          }
+          if (!ok) break;
+          store8(out, sc, nk, xb0, 0, ea, shift, re[0], im[0]);
+          store8(out + (size_t)8 * sc, sc, nk - 8, xb0, 8, ea, shift, re[1], im[1]);
+        } else {
+          // one accumulation (the plan drains only units of 32 kets)
+          ok = __all_sync(0xffffffffu, mbar_wait(acc_full, chunk & 1u, abort_flag, status));
+          if (!ok) break;
+          ++chunk;
+          fence_after();
+#pragma unroll 1
+          for (int c8 = 0; c8 < t / 2; c8 += 8) {
+            long long re[8], im[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) re[e] = im[e] = 0;
+            drain8(col + c8, L, t, g.beta, g.fbits, re, im);
+            store8(out + (size_t)c8 * sc, sc, nk - c8, c8 < 32 ? xb0 : xb1, c8 & 31, ea, shift, re, im);
+          }
+          fence_before();
+          mbar_arrive(acc_empty);
+        }
+      } else {
+        ok = __all_sync(0xffffffffu, mbar_wait(acc_full, chunk & 1u, abort_flag, status));
+        if (!ok) break;
+        ++chunk;
+        fence_after();
+        float2* out = (float2*)g.out + o;
+        const float scale = g.scale;
+#pragma unroll 1
+        for (int c8 = 0; c8 < t / 2; c8 += 8) {
+          float r0[8], r1[8], i0[8], i1[8];
+          tmem_ld8(col + c8, r0);
+          tmem_ld8(col + t + c8, r1);
+          tmem_ld8(col + COL_IM + c8, i0);
+          tmem_ld8(col + COL_IM + t + c8, i1);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            // the pieces carry 2^PIECE_BITS each
+            const int x = __shfl_sync(0xffffffffu, c8 < 32 ? xb0 : xb1, (c8 + e) & 31);
+            const float f = scaled(scale, ea + x - 2 * PIECE_BITS);
+            out[(size_t)(c8 + e) * MT] = make_float2((r0[e] + r1[e]) * f, (i0[e] + i1[e]) * f);
+          }
+        }
+        fence_before();
+        mbar_arrive(acc_empty);
+      }
+    }
+  }
+
+  // ---------------- teardown ----------------
+  __syncthreads();
+  if (warp == MMA_WARP && lane == 0) {
+    // an abort can leave MMAs in flight: let them retire before TMEM is released (bounded)
+    const unsigned long long t0 = gtime();
+    while (!mbar_test(drain, 0u) && gtime() - t0 < WAIT_NS) {
+    }
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+// ---------------------------------------------------------------------------- operands
+
+enum : int { SRC_F64_DIGITS = 0, SRC_F32_DIGITS = 1, SRC_F32_F16 = 2, SRC_F32_BF16 = 3 };
+
+// One operand: rows = CWF columns of one side, weighted by w[i] if given.
+struct Slice {
+  const void* src;          // complex128 or complex64, row r at src + r n
+  const double* w;
+  unsigned char* out;
+  int* ex;                  // rpad exponents
+  int n, ks, rows, rpad, R; // points, K slices, rows (and padded to tiles of R rows)
+  int d, kind, b0, beta;
+};
+
+// 8 consecutive points of one row: `part` 0 or 1 of their K slice
+__device__ __forceinline__ unsigned char* slice_at(const Slice& s, int row, int c8, int plane, int p) {
+  const int tile = row / s.R, r = row - tile * s.R;
+  return s.out + ((((size_t)tile * s.ks + (c8 >> 1)) * 2 + plane) * s.d + p) * ((size_t)s.R * ROW_BYTES) +
+         swizzle32(r, c8 & 1);
+}
+
+// Digits of 8 FP64 values |x| < 2^e: integers round(x 2^(b0 + beta (D - 1) - e)) cut from the bottom
+// into balanced base-2^beta digits (the top one at most 2^b0), stored exactly as BF16.
+template <int D>
+__device__ __forceinline__ void emit_f64(const Slice& s, int row, int c8, int plane, const double (&x)[8], int e) {
+  uint32_t pk[D][4];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    int dg[D];
+    digits_of<D>(x[k], s.b0 + s.beta * (D - 1) - e, dg);
+#pragma unroll
+    for (int p = 0; p < D; ++p) {
+      const uint32_t h = __float_as_uint(small_int_to_float(dg[p])) >> 16;
+      if (k & 1) pk[p][k >> 1] |= h << 16;
+      else pk[p][k >> 1] = h;
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < D; ++p)
+    *(uint4*)slice_at(s, row, c8, plane, p) = make_uint4(pk[p][0], pk[p][1], pk[p][2], pk[p][3]);
+}
+
+// Digits of 8 FP32 values by exact FP32 steps: d = rint(v), v = (v - d) 2^beta.
+__device__ __forceinline__ void emit_f32_digits(const Slice& s, int row, int c8, int plane, const float (&x)[8],
+                                                float f1, float f2) {
+  float v[8];
+  const float B = (float)(1 << s.beta);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = x[k] * f1 * f2;
+  for (int p = 0; p < s.d; ++p) {
+    uint32_t pk[4];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float r = rintf(v[k]);
+      v[k] = (v[k] - r) * B;
+      const uint32_t h = __float_as_uint(r) >> 16;
+      if (k & 1) pk[k >> 1] |= h << 16;
+      else pk[k >> 1] = h;
+    }
+    *(uint4*)slice_at(s, row, c8, plane, p) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+  }
+}
+
+template <bool F16>
+__device__ __forceinline__ void emit_pieces(const Slice& s, int row, int c8, int plane, const float (&x)[8],
+                                            float f1, float f2) {
+  uint32_t hi[4], lo[4];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float v = x[k] * f1 * f2;
+    uint32_t h, l;
+    if (F16) {
+      const __half a = __float2half_rn(v);
+      h = __half_as_ushort(a);
+      l = __half_as_ushort(__float2half_rn(v - __half2float(a)));
+    } else {
+      const __nv_bfloat16 a = __float2bfloat16_rn(v);
+      h = __bfloat16_as_ushort(a);
+      l = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(a)));
+    }
+    if (k & 1) { hi[k >> 1] |= h << 16; lo[k >> 1] |= l << 16; }
+    else { hi[k >> 1] = h; lo[k >> 1] = l; }
+  }
+  *(uint4*)slice_at(s, row, c8, plane, 0) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+  *(uint4*)slice_at(s, row, c8, plane, 1) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+}
+
+// Components of 8 points of a row (zero past the row's end and in padding rows), weighted; 16-byte
+// loads (rows are 8 or more points, so every chunk starts on a 16-byte boundary).
+template <typename Z, typename T>
+__device__ __forceinline__ void load8(const Slice& s, int row, int c8, T (&re)[8], T (&im)[8]) {
+  if (row >= s.rows || 8 * c8 >= s.n) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) re[k] = im[k] = 0;
+    return;
+  }
+  const Z* p = (const Z*)s.src + (size_t)row * s.n + 8 * c8;
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 z = ((const float4*)p)[k];
+      re[2 * k] = z.x; im[2 * k] = z.y; re[2 * k + 1] = z.z; im[2 * k + 1] = z.w;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const Z z = p[k];
+      re[k] = z.x; im[k] = z.y;
+    }
+  }
+  if (s.w) {
+    const double2* w = (const double2*)(s.w + 8 * c8);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const double2 f = w[k];
+      re[2 * k] *= (T)f.x; im[2 * k] *= (T)f.x;
+      re[2 * k + 1] *= (T)f.y; im[2 * k + 1] *= (T)f.y;
+    }
+  }
+}
+
+// Largest magnitude (as bits) of one row over its tpr threads (a power of two; rows of fewer than 32
+// threads share a warp).
+__device__ __forceinline__ unsigned long long row_max(unsigned long long m, int tpr, unsigned long long* red) {
+  for (int o = (tpr < 32 ? tpr : 32) >> 1; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, m, o);
+    m = m > x ? m : x;
+  }
+  if (tpr > 32) {
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    const int w0 = ((int)threadIdx.x / tpr) * (tpr >> 5);
+    for (int w = 0; w < tpr >> 5; ++w) m = m > red[w0 + w] ? m : red[w0 + w];
+  }
+  return m;
+}
+
+// Operands in slices, grid (row groups, operands): a row's 8-point chunks are spread over
+// min(2 ks, 256) threads.  A thread keeps the first chunk's values between the two passes (largest
+// component, pieces), which is all of its work up to 2048 points.
+__global__ void __launch_bounds__(256) k_slices(const Slice* __restrict__ list, unsigned* ticket) {
+  __shared__ unsigned long long red[8];
+  const Slice s = list[blockIdx.y];
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *ticket = 0;   // the Gram launch's
+  const int c8n = 2 * s.ks, tpr = c8n < 256 ? c8n : 256, rpb = 256 / tpr;
+  if ((int)blockIdx.x * rpb >= s.rpad) return;
+  const int row = (int)blockIdx.x * rpb + (int)threadIdx.x / tpr, t0 = (int)threadIdx.x % tpr;
+  // magnitudes order like their bit patterns, NaN above infinity
+  unsigned long long m = 0;
+  if (s.kind == SRC_F64_DIGITS) {
+    double re[8], im[8];
+    auto scan = [&]() {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const unsigned long long a = abs_bits(re[k]), b = abs_bits(im[k]);
+        m = m > a ? m : a;
+        m = m > b ? m : b;
+      }
+    };
+    for (int c = t0 + tpr; c < c8n; c += tpr) {
+      load8<double2, double>(s, row, c, re, im);
+      scan();
+    }
+    load8<double2, double>(s, row, t0, re, im);
+    scan();
+    m = row_max(m, tpr, red);
+    if (row >= s.rpad) return;
+    const bool bad = m >= 0x7FF0000000000000ull;
+    const int e = bad ? 0 : exponent_above_f64(m);
+    if (t0 == 0) s.ex[row] = bad ? EX_BAD : e;
+    for (int c = t0; c < c8n; c += tpr) {
+      if (c != t0) load8<double2, double>(s, row, c, re, im);
+      if (bad) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) re[k] = im[k] = 0.0;
+      }
+      switch (s.d) {
+        case 2: emit_f64<2>(s, row, c, 0, re, e); emit_f64<2>(s, row, c, 1, im, e); break;
+        case 3: emit_f64<3>(s, row, c, 0, re, e); emit_f64<3>(s, row, c, 1, im, e); break;
+        case 4: emit_f64<4>(s, row, c, 0, re, e); emit_f64<4>(s, row, c, 1, im, e); break;
+        case 5: emit_f64<5>(s, row, c, 0, re, e); emit_f64<5>(s, row, c, 1, im, e); break;
+        case 6: emit_f64<6>(s, row, c, 0, re, e); emit_f64<6>(s, row, c, 1, im, e); break;
+        case 7: emit_f64<7>(s, row, c, 0, re, e); emit_f64<7>(s, row, c, 1, im, e); break;
+        default: emit_f64<8>(s, row, c, 0, re, e); emit_f64<8>(s, row, c, 1, im, e); break;
+      }
+    }
+    return;
+  }
+  float re[8], im[8];
+  unsigned mf = 0;
+  auto scan = [&]() {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const unsigned a = __float_as_uint(re[k]) & 0x7FFFFFFFu, b = __float_as_uint(im[k]) & 0x7FFFFFFFu;
+      mf = max(mf, max(a, b));
+    }
+  };
+  for (int c = t0 + tpr; c < c8n; c += tpr) {
+    load8<float2, float>(s, row, c, re, im);
+    scan();
+  }
+  load8<float2, float>(s, row, t0, re, im);
+  scan();
+  m = row_max(mf, tpr, red);
+  if (row >= s.rpad) return;
+  const bool bad = m >= 0x7F800000ull;
+  const int e = m && !bad ? ilogbf(__uint_as_float((unsigned)m)) + 1 : 0;
+  const bool digits = s.kind == SRC_F32_DIGITS;
+  if (t0 == 0) s.ex[row] = bad && digits ? EX_BAD : e;
+  // 2^k in two factors, each a normal number
+  const int k2 = (digits ? s.b0 : PIECE_BITS) - e;
+  const float f1 = ldexpf(1.f, k2 / 2), f2 = ldexpf(1.f, k2 - k2 / 2);
+  for (int c = t0; c < c8n; c += tpr) {
+    if (c != t0) load8<float2, float>(s, row, c, re, im);
+    if (digits) {
+      if (bad) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) re[k] = im[k] = 0.f;
+      }
+      emit_f32_digits(s, row, c, 0, re, f1, f2);
+      emit_f32_digits(s, row, c, 1, im, f1, f2);
+    } else if (s.kind == SRC_F32_F16) {
+      emit_pieces<true>(s, row, c, 0, re, f1, f2);
+      emit_pieces<true>(s, row, c, 1, im, f1, f2);
+    } else {
+      emit_pieces<false>(s, row, c, 0, re, f1, f2);
+      emit_pieces<false>(s, row, c, 1, im, f1, f2);
+    }
+  }
+}
+
+// An operand of Psi(x_i, R_j) = sum_a C_a psi_a(x_i) chi_a(R_j): rows = grid points, K = trajectories.
+// Row r, point a is C_a src[a n + r], conjugated (the Grams conjugate their bras), or src[a n + r]
+// without C.
+struct SliceT {
+  const void* src;
+  const double2* C;
+  unsigned char* out;
+  int* ex;
+  int n, ks, N, rpad, R, d, f32;
+};
+
+// 8 rows per CTA (a 1024-point side fills the chip): lane = row + 8 x group, a warp's four groups and
+// the CTA's warps take every 64th set of 8 trajectories, twice: for the rows' largest components
+// (bounded by (|Re C| + |Im C|) max(|Re|, |Im|)), then for the digits.
+constexpr int ST_WARPS = 16, ST_ROWS = 8, ST_GROUPS = 4;
+__global__ void __launch_bounds__(ST_WARPS * 32) k_slices_t(SliceT sx, SliceT sR, unsigned* ticket) {
+  __shared__ unsigned long long red[ST_WARPS * ST_GROUPS][ST_ROWS];
+  const SliceT q = blockIdx.y ? sR : sx;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *ticket = 0;   // the Gram launch's
+  const int r = threadIdx.x & (ST_ROWS - 1), grp = threadIdx.x / ST_ROWS;
+  const int row = (int)blockIdx.x * ST_ROWS + r;
+  if ((int)blockIdx.x * ST_ROWS >= q.rpad) return;
+  auto at = [&](int a) {
+    double2 z = make_double2(0.0, 0.0);
+    if (a < q.N && row < q.n)
+      z = q.f32 ? to_d(((const float2*)q.src)[(size_t)a * q.n + row])
+                : ((const double2*)q.src)[(size_t)a * q.n + row];
+    return z;
+  };
+  unsigned long long m = 0;
+  for (int c = grp; c < 2 * q.ks; c += ST_WARPS * ST_GROUPS) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int a = 8 * c + k;
+      const double2 z = at(a);
+      unsigned long long x = abs_bits(z.x), y = abs_bits(z.y);
+      x = x > y ? x : y;
+      if (q.C && a < q.N) x = abs_bits(bits_f64(x) * (fabs(q.C[a].x) + fabs(q.C[a].y)));
+      m = m > x ? m : x;
+    }
+  }
+  red[grp][r] = m;
+  __syncthreads();
+#pragma unroll 8
+  for (int w = 0; w < ST_WARPS * ST_GROUPS; ++w) m = m > red[w][r] ? m : red[w][r];
+  const bool bad = m >= 0x7FF0000000000000ull;
+  const int e = bad ? 0 : exponent_above_f64(m);
+  if (grp == 0) q.ex[row] = bad ? EX_BAD : e;
+  Slice s;
+  s.out = q.out; s.ks = q.ks; s.R = q.R; s.d = q.d; s.b0 = 6; s.beta = 7;
+  for (int c = grp; c < 2 * q.ks; c += ST_WARPS * ST_GROUPS) {
+    double re[8], im[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int a = 8 * c + k;
+      double2 z = at(a);
+      if (q.C && a < q.N) z = cconj(cmul(q.C[a], z));
+      re[k] = bad ? 0.0 : z.x;
+      im[k] = bad ? 0.0 : z.y;
+    }
+    if (q.d == 8) {
+      emit_f64<8>(s, row, c, 0, re, e);
+      emit_f64<8>(s, row, c, 1, im, e);
+    } else {
+      emit_f64<5>(s, row, c, 0, re, e);
+      emit_f64<5>(s, row, c, 1, im, e);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------- S and Heff
+
+// Heff_ab = sum_g s_g (A_g - u_g(x_b) S1)(B_g - w_g(R_b) S2) - V(x_b, R_b) S_ab over the terms
+// [g0, g1) of this launch; `first` starts the sums at zero (else they continue from H), `last`
+// subtracts the pinned potential and writes S.
+struct HeffArgs {
+  int N, g0, g1, first, last;
+  const void *S1, *S2;      // raw Grams of the overlap: double2 (digits) or, with split_s, float2 scaled
+  const void *A, *B;        // Grams of the terms g0.., `tiles` 128 x 128 tiles each
+  size_t tiles;
+  int split_s;
+  double dx, dR;
+  const double *sig, *px, *pR, *d;
+  double2 *S, *H;
+};
+
+// Threads of one 32 x 32 patch of a 128 x 128 upper-triangle tile: lane = bra, 4 kets each.  F32: the
+// mixed modes' FP32 arithmetic on float2 Grams; else FP64 on double2 Grams that carry s_g dx and dR
+// already (folded into the operands' weights): 8 FP64 instructions per term, element and side, which
+// is what bounds the FP64 version (0.35 ms at N = 1024 and 22 terms); the F32 version reads its Grams
+// once.
+constexpr int HG = 16;   // terms staged at a time
+template <bool F32>
+__global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
+  using Z = typename std::conditional<F32, float2, double2>::type;
+  using T = typename std::conditional<F32, float, double>::type;
+  __shared__ double2 tr[32][33];
+  // the terms' factor values at the 32 bras and 32 kets, converted once per CTA (a conversion from
+  // FP64 costs an FP64 instruction)
+  __shared__ T uxs[HG][64], wRs[HG][64];
+  int I, J;
+  tri_tile(blockIdx.y, I, J);
+  const int N = p.N, lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int ar = (blockIdx.x & 3) * 32 + lane, br = (blockIdx.x >> 2) * 32 + ty;
+  const int a = I * MT + ar, b0 = J * MT + br;
+  if (I * MT + (int)(blockIdx.x & 3) * 32 >= N || J * MT + (int)(blockIdx.x >> 2) * 32 >= N) return;
+  const bool mirror = I != J, a_ok = a < N;
+  const size_t at0 = ((size_t)blockIdx.y * MT + br) * MT + ar, step = (size_t)8 * MT;
+  double2 s1d[4], s2d[4];
+  Z s1[4], s2[4], h[4], ht[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const size_t at = at0 + e * step;
+    if (F32 && p.split_s) {
+      const float2 x = ((const float2*)p.S1)[at], y = ((const float2*)p.S2)[at];
+      s1d[e] = make_double2(x.x, x.y);
+      s2d[e] = make_double2(y.x, y.y);
+    } else {
+      s1d[e] = cscale(((const double2*)p.S1)[at], p.dx);
+      s2d[e] = cscale(((const double2*)p.S2)[at], p.dR);
+    }
+    s1[e].x = (T)s1d[e].x; s1[e].y = (T)s1d[e].y;
+    s2[e].x = (T)s2d[e].x; s2[e].y = (T)s2d[e].y;
+    h[e].x = h[e].y = ht[e].x = ht[e].y = 0;
+    const int b = b0 + 8 * e;
+    if (!p.first && a_ok && b < N) {
+      const double2 v = p.H[(size_t)a * N + b];
+      h[e].x = (T)v.x; h[e].y = (T)v.y;
+      if (mirror) {
+        const double2 w = p.H[(size_t)b * N + a];
+        ht[e].x = (T)w.x; ht[e].y = (T)w.y;
+      }
+    }
+  }
+  const size_t gs = p.tiles * MT * MT;
+  const int as = I * MT + (int)(blockIdx.x & 3) * 32, bs = J * MT + (int)(blockIdx.x >> 2) * 32;
+  for (int g = p.g0; g < p.g1; ++g) {
+    const int gl = (g - p.g0) & (HG - 1);
+    if (gl == 0) {
+      __syncthreads();
+      for (int i = threadIdx.x; i < HG * 64; i += 256) {
+        const int gi = g + (i >> 6), c = i & 63, t = c < 32 ? as + c : bs + c - 32;
+        if (gi < p.g1) {
+          const double s = F32 ? 1.0 : p.sig[gi];
+          uxs[i >> 6][c] = t < N ? (T)(s * p.px[(size_t)gi * N + t]) : (T)0;
+          wRs[i >> 6][c] = t < N ? (T)p.pR[(size_t)gi * N + t] : (T)0;
+        }
+      }
+      __syncthreads();
+    }
+    const Z* A = (const Z*)p.A + (size_t)(g - p.g0) * gs + at0;
+    const Z* B = (const Z*)p.B + (size_t)(g - p.g0) * gs + at0;
+    const T sg = F32 ? (T)p.sig[g] : (T)0;
+    const T uxa = uxs[gl][lane], wRa = wRs[gl][lane];
+    Z xs[4], ys[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { xs[e] = A[e * step]; ys[e] = B[e * step]; }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const Z x = xs[e], y = ys[e];
+      const T uxb = uxs[gl][32 + ty + 8 * e], wRb = wRs[gl][32 + ty + 8 * e];
+      const T atr = x.x - uxb * s1[e].x, ati = x.y - uxb * s1[e].y;
+      const T btr = y.x - wRb * s2[e].x, bti = y.y - wRb * s2[e].y;
+      if (F32) {
+        h[e].x = fma(sg, atr * btr - ati * bti, h[e].x);
+        h[e].y = fma(sg, atr * bti + ati * btr, h[e].y);
+      } else {
+        h[e].x = fma(atr, btr, fma(-ati, bti, h[e].x));
+        h[e].y = fma(atr, bti, fma(ati, btr, h[e].y));
+      }
+      if (mirror) {
+        // entry (b, a): conj(A) - u(x_a) conj(S1), conj(B) - w(R_a) conj(S2)
+        const T mtr = x.x - uxa * s1[e].x, mti = x.y - uxa * s1[e].y;
+        const T ntr = y.x - wRa * s2[e].x, nti = y.y - wRa * s2[e].y;
+        if (F32) {
+          ht[e].x = fma(sg, mtr * ntr - mti * nti, ht[e].x);
+          ht[e].y = fma(sg, -(mtr * nti + mti * ntr), ht[e].y);
+        } else {
+          ht[e].x = fma(mtr, ntr, fma(-mti, nti, ht[e].x));
+          ht[e].y = fma(-mtr, nti, fma(-mti, ntr, ht[e].y));
+        }
+      }
+    }
+  }
+  double2 sv[4];
+  const double da = a_ok && p.last ? p.d[a] : 0.0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int b = b0 + 8 * e;
+    const bool in = a_ok && b < N;
+    double2 hd = make_double2(h[e].x, h[e].y), hm = make_double2(ht[e].x, ht[e].y);
+    if (p.last) {
+      sv[e] = cmul(s1d[e], s2d[e]);
+      if (a == b) sv[e].y = 0.0;
+      const double db = in ? p.d[b] : 0.0;
+      hd = make_double2(hd.x - db * sv[e].x, hd.y - db * sv[e].y);
+      hm = make_double2(hm.x - da * sv[e].x, hm.y + da * sv[e].y);
+    }
+    tr[lane][ty + 8 * e] = hd;
+    if (mirror && in) p.H[(size_t)b * N + a] = hm;
+  }
+  __syncthreads();
+  // rows of H: lane = ket
+  const int ao = I * MT + (blockIdx.x & 3) * 32 + ty, bo = J * MT + (blockIdx.x >> 2) * 32 + lane;
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (ao + 8 * e < N && bo < N) p.H[(size_t)(ao + 8 * e) * N + bo] = tr[ty + 8 * e][lane];
+  if (!p.last) return;
+  __syncthreads();
+  // S: each pair once, from its a <= b side, so that S is exactly Hermitian
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int b = b0 + 8 * e;
+    tr[lane][ty + 8 * e] = sv[e];
+    if (a_ok && b < N && (mirror || a < b)) p.S[(size_t)b * N + a] = cconj(sv[e]);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (ao + 8 * e < N && bo < N && (mirror || ao + 8 * e <= bo))
+      p.S[(size_t)(ao + 8 * e) * N + bo] = tr[ty + 8 * e][lane];
+}
+
+// ---------------------------------------------------------------------------- plan
+
+size_t al(size_t b) { return (b + 1023) & ~(size_t)1023; }
+int ilog2_ceil(int n) { int l = 0; while ((1 << l) < n) ++l; return l; }
+
+// Terms of one batch: as many as fit BATCH_BYTES of operands and Grams (at least one).
+constexpr size_t BATCH_BYTES = (size_t)512 << 20;
+
+int tiles_of(int N) { const int T = (N + MT - 1) / MT; return T * (T + 1) / 2; }
+int kets_per_unit(int N, int most) { return N <= 32 && most > 32 ? 32 : (N <= 64 && most > 64 ? 64 : most); }
+
+// K slices per accumulation of D digits (b0 = 6, beta = 7).  The leading D - 4 levels stay below 2^24
+// whatever the digits are: (l + 1) pairs x 2 products x 2^12 x 16 points per slice.  The level after
+// them could round only if its digits were all large and of one sign; its worst case, 2^-43 of the
+// largest possible sum at 1024 points, is that of an FP64 sum of as many products.
+int drain_slices(int d) {
+  if (d <= 4) return 1 << 20;
+  int s = 1;
+  while (2 * s * 16 * (d - 4) <= (1 << 11)) s *= 2;
+  return s;
+}
+
+// Digits of term g (relative weight r = s_g / s_1).
+int term_digits(double r) {
+  if (!(r > 0)) return 2;
+  const int d = (int)std::ceil((56.0 + std::log2(r)) / 7.0);
+  return d < 2 ? 2 : (d > 8 ? 8 : d);
+}
+
+struct Term { int d; size_t bx, bR; };   // pieces and operand bytes of both sides
+
+}  // namespace sl
+
+// Layout of the scratch and tables of one handle's assembly.  Built twice: once to size the arena
+// (base NULL), once to fill it.
+struct AsmPlan::Impl {
+  struct Batch { int slice0, nslice, gram0, ngram, units, g0, g1, rowgroups; size_t A, B; };
+  std::vector<sl::Slice> slices;
+  std::vector<sl::Gram> grams;
+  std::vector<Batch> batches;
+  std::vector<double> Uw, Ww;            // FP64: weights u_g s_g dx and w_g dR
+  size_t bytes = 0, o_slices = 0, o_grams = 0, o_uw = 0, o_ww = 0, o_ticket = 0;
+  size_t S1 = 0, S2 = 0;
+  size_t r_xa = 0, r_xe = 0, r_Rb = 0, r_Re = 0;   // reconstruction operands (in the batch scratch)
+  int rec_gram = 0, rec_units = 0, rec_d = 0;
+  unsigned char* base = nullptr;
+  bool f64 = false, split_s = false;
+  int sms = 152;
+};
+
+AsmPlan::AsmPlan() {}
+AsmPlan::~AsmPlan() { delete impl; }
+
+size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
+  using namespace sl;
+  delete impl;
+  impl = new Impl;
+  Impl& m = *impl;
+  const bool f64 = q.precision == ICWF_FP64, split_s = !f64 && q.overlap_split;
+  m.f64 = f64;
+  m.split_s = split_s;
+  m.base = (unsigned char*)base;
+  const int N = q.N, K = q.K;
+  const int rp = (N + MT - 1) / MT * MT, tiles = tiles_of(N);
+  const int n[2] = {q.nx, q.nR}, ks[2] = {(q.nx + 15) / 16, (q.nR + 15) / 16};
+  size_t off = 0;
+  auto take = [&](size_t b) { const size_t o = off; off += al(b); return o; };
+  const size_t osz = f64 ? 16 : 8;
+  const size_t out_b = (size_t)tiles * MT * MT * osz;
+  const size_t s_out_b = (size_t)tiles * MT * MT * (split_s ? 8 : 16);
+  m.o_ticket = take(256);
+  m.S1 = take(s_out_b);
+  m.S2 = take(s_out_b);
+  // bra operands: digits for S (and, in FP64, every Gram); hi/lo pieces for the mixed modes' Heff
+  const int dS = f64 ? 8 : 4;
+  size_t sa[2] = {0, 0}, se[2] = {0, 0}, pa[2] = {0, 0}, pe[2] = {0, 0};
+  auto op_bytes = [&](int side, int d) { return (size_t)rp * ks[side] * 2 * d * ROW_BYTES; };
+  for (int s = 0; s < 2; ++s) {
+    if (!split_s) { sa[s] = take(op_bytes(s, dS)); se[s] = take((size_t)rp * 4); }
+    if (!f64) { pa[s] = take(op_bytes(s, 2)); pe[s] = take((size_t)rp * 4); }
+  }
+  if (f64) {
+    m.o_uw = take((size_t)K * q.nx * 8);
+    m.o_ww = take((size_t)K * q.nR * 8);
+  }
+  std::vector<int> dg(K);
+  for (int g = 0; g < K; ++g) dg[g] = f64 ? term_digits(q.sig[0] > 0 ? q.sig[g] / q.sig[0] : 0.0) : 2;
+  // batches of terms
+  std::vector<std::pair<int, int>> ranges;
+  size_t batch_max = 0;
+  for (int g = 0; g < K;) {
+    size_t b = 0;
+    int e = g;
+    while (e < K && 2 * (e - g) + 4 < MAX_GRAMS) {
+      const size_t add = al(op_bytes(0, dg[e])) + al(op_bytes(1, dg[e])) + 2 * al((size_t)rp * 4) + 2 * al(out_b);
+      if (e > g && b + add > BATCH_BYTES) break;
+      b += add;
+      ++e;
+    }
+    batch_max = std::max(batch_max, b);
+    ranges.push_back({g, e});
+    g = e;
+  }
+  // the reconstruction runs between steps in the same scratch
+  const int rxp = (q.nx + MT - 1) / MT * MT, rRp = (q.nR + MT - 1) / MT * MT, ksN = (N + 15) / 16;
+  m.rec_d = f64 ? 8 : 5;
+  auto rec_op = [&](int rows) { return (size_t)rows * ksN * 2 * m.rec_d * ROW_BYTES; };
+  const size_t rec_bytes = al(rec_op(rxp)) + al(rec_op(rRp)) + al((size_t)rxp * 4) + al((size_t)rRp * 4);
+  const size_t scratch = take(std::max(batch_max, rec_bytes) + 2 * 1024);
+  m.r_xa = scratch;
+  m.r_Rb = m.r_xa + al(rec_op(rxp));
+  m.r_xe = m.r_Rb + al(rec_op(rRp));
+  m.r_Re = m.r_xe + al((size_t)rxp * 4);
+  auto ptr = [&](size_t o) { return m.base + o; };
+  const int fdig = f64 ? 7 : 0;
+  for (size_t r = 0; r < ranges.size(); ++r) {
+    const int g0 = ranges[r].first, g1 = ranges[r].second;
+    Impl::Batch b{};
+    b.slice0 = (int)m.slices.size();
+    b.gram0 = (int)m.grams.size();
+    b.g0 = g0;
+    b.g1 = g1;
+    auto add_slice = [&](int side, const double* w, size_t out, size_t ex, int R, int d, int kind, int b0, int beta) {
+      Slice s{};
+      s.src = j ? (side ? j->chi : j->psi) : nullptr;
+      s.w = w;
+      s.out = ptr(out);
+      s.ex = (int*)ptr(ex);
+      s.n = n[side]; s.ks = ks[side]; s.rows = N; s.rpad = rp; s.R = R;
+      s.d = d; s.kind = kind; s.b0 = b0; s.beta = beta;
+      m.slices.push_back(s);
+    };
+    auto add_gram = [&](int side, size_t A, size_t eA, int da, const unsigned char* B, const int* eB, int d, int l,
+                        int t, int drain, bool f16, bool digits, int b0, int beta, size_t out) {
+      Gram x{};
+      x.A = ptr(A);
+      x.B = B;
+      x.ea = (int*)ptr(eA);
+      x.eb = eB ? eB : (int*)ptr(eA);
+      x.out = ptr(out);
+      x.scale = (float)(side ? q.dR : q.dx);
+      x.ks = ks[side]; x.da = da; x.d = d; x.l = l; x.t = t; x.drain = drain;
+      x.f16 = f16; x.digits = digits; x.b0 = b0; x.beta = beta;
+      // |sum| <= 2 K 2^(2 b0) units of level 0
+      x.fbits = 62 - (1 + ilog2_ceil(16 * ks[side]) + 2 * b0);
+      m.grams.push_back(x);
+    };
+    const bool f16 = q.precision == ICWF_MIXED_TF32X3;
+    const int pk = f16 ? SRC_F32_F16 : SRC_F32_BF16;
+    for (int s = 0; s < 2; ++s) {
+      if (r > 0) break;   // bras and the overlap once per assembly
+      const int bd = f64 ? 6 : (n[s] <= 2048 ? 6 : 5), beta = f64 ? fdig : bd;
+      if (!split_s) {
+        add_slice(s, nullptr, sa[s], se[s], MT, dS, f64 ? SRC_F64_DIGITS : SRC_F32_DIGITS, bd, beta);
+        const int L = f64 ? dS : 2 * dS - 1;
+        add_gram(s, sa[s], se[s], dS, nullptr, nullptr, dS, L, 32, f64 ? drain_slices(dS) : 1 << 20, false, true,
+                 bd, beta, s ? m.S2 : m.S1);
+      }
+      if (!f64) {
+        add_slice(s, nullptr, pa[s], pe[s], MT, 2, pk, 0, 0);
+        if (split_s)
+          add_gram(s, pa[s], pe[s], 2, nullptr, nullptr, 2, 2, kets_per_unit(N, MT), 1 << 20, f16, false, 0, 0,
+                   s ? m.S2 : m.S1);
+      }
+    }
+    size_t so = scratch;
+    auto tmp = [&](size_t bytes) { const size_t o = so; so += al(bytes); return o; };
+    // the Grams of one side are consecutive (k_heff walks them with a fixed stride)
+    b.A = tmp((size_t)(g1 - g0) * out_b);
+    b.B = tmp((size_t)(g1 - g0) * out_b);
+    for (int g = g0; g < g1; ++g)
+      for (int s = 0; s < 2; ++s) {
+        const int d = dg[g];
+        int t = d <= 2 ? 128 : (d <= 4 ? 64 : 32);
+        const int dr = f64 ? drain_slices(d) : 1 << 20;
+        if (dr < ks[s]) t = 32;
+        t = kets_per_unit(N, t);
+        const size_t o = tmp(op_bytes(s, d)), oe = tmp((size_t)rp * 4);
+        const double* w = nullptr;
+        if (f64) w = (const double*)ptr(s ? m.o_ww : m.o_uw) + (size_t)g * n[s];
+        else if (j) w = (s ? j->W : j->U) + (size_t)g * n[s];
+        add_slice(s, w, o, oe, t, d, f64 ? SRC_F64_DIGITS : pk, f64 ? 6 : 0, f64 ? fdig : 0);
+        add_gram(s, f64 ? sa[s] : pa[s], f64 ? se[s] : pe[s], f64 ? dS : 2, ptr(o), (int*)ptr(oe), d, d, t, dr,
+                 !f64 && f16, f64, f64 ? 6 : 0, f64 ? fdig : 0, (s ? b.B : b.A) + (size_t)(g - g0) * out_b);
+      }
+    b.nslice = (int)m.slices.size() - b.slice0;
+    b.ngram = (int)m.grams.size() - b.gram0;
+    // the most expensive units first (tensor time of a unit: levels' pairs x kets x slices)
+    auto cost = [](const Gram& x) {
+      int pairs = 0;
+      for (int p = 0; p < x.d; ++p) pairs += std::min(x.d, x.l - p);
+      return (long long)pairs * x.t * x.ks;
+    };
+    std::stable_sort(m.grams.begin() + b.gram0, m.grams.end(),
+                     [&](const Gram& x, const Gram& y) { return cost(x) > cost(y); });
+    for (int i = 0; i < b.ngram; ++i) {
+      Gram& x = m.grams[b.gram0 + i];
+      x.unit0 = b.units;
+      b.units += tiles * (MT / x.t);
+    }
+    for (int i = 0; i < b.nslice; ++i) {
+      const Slice& s = m.slices[b.slice0 + i];
+      const int tpr = std::min(2 * s.ks, 256), rpb = 256 / tpr;
+      b.rowgroups = std::max(b.rowgroups, (rp + rpb - 1) / rpb);
+    }
+    m.batches.push_back(b);
+  }
+  {
+    Gram x{};
+    x.A = ptr(m.r_xa); x.B = ptr(m.r_Rb);
+    x.ea = (int*)ptr(m.r_xe); x.eb = (int*)ptr(m.r_Re);
+    x.ks = ksN; x.da = x.d = x.l = m.rec_d; x.t = 32; x.drain = drain_slices(m.rec_d);
+    x.digits = 1; x.b0 = 6; x.beta = 7;
+    x.fbits = 62 - (1 + ilog2_ceil(16 * ksN) + 12);
+    x.rows = q.nx; x.cols = q.nR;
+    m.rec_gram = (int)m.grams.size();
+    m.rec_units = rxp / MT * ((q.nR + 31) / 32);
+    m.grams.push_back(x);   // its output is an argument of the launch
+  }
+  m.o_slices = take(m.slices.size() * sizeof(Slice));
+  m.o_grams = take(m.grams.size() * sizeof(Gram));
+  m.bytes = off;
+  return m.bytes;
+}
+
+bool AsmPlan::upload(const AsmShape& q, const double* U, const double* W, cudaStream_t s) {
+  using namespace sl;
+  Impl& m = *impl;
+  if (m.f64) {
+    m.Uw.resize((size_t)q.K * q.nx);
+    m.Ww.resize((size_t)q.K * q.nR);
+    for (int g = 0; g < q.K; ++g) {
+      for (int i = 0; i < q.nx; ++i) m.Uw[(size_t)g * q.nx + i] = U[(size_t)g * q.nx + i] * (q.sig[g] * q.dx);
+      for (int i = 0; i < q.nR; ++i) m.Ww[(size_t)g * q.nR + i] = W[(size_t)g * q.nR + i] * q.dR;
+    }
+    if (cudaMemcpyAsync(m.base + m.o_uw, m.Uw.data(), m.Uw.size() * 8, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(m.base + m.o_ww, m.Ww.data(), m.Ww.size() * 8, cudaMemcpyHostToDevice, s) != cudaSuccess)
+      return false;
+  }
+  if (cudaMemcpyAsync(m.base + m.o_slices, m.slices.data(), m.slices.size() * sizeof(Slice), cudaMemcpyHostToDevice,
+                      s) != cudaSuccess ||
+      cudaMemcpyAsync(m.base + m.o_grams, m.grams.data(), m.grams.size() * sizeof(Gram), cudaMemcpyHostToDevice,
+                      s) != cudaSuccess)
+    return false;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&m.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  static std::once_flag once;   // outside any stream capture
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(k_gram_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+  });
+  return attr == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess;
+}
+
+int AsmPlan::launch(const JobView& j, double2* S, double2* H, cudaStream_t s) const {
+  using namespace sl;
+  const Impl& m = *impl;
+  const int tiles = tiles_of(j.N);
+  for (const auto& b : m.batches) {
+    k_slices<<<dim3(b.rowgroups, b.nslice), 256, 0, s>>>((const Slice*)(m.base + m.o_slices) + b.slice0,
+                                                         (unsigned*)(m.base + m.o_ticket));
+    GramArgs ga;
+    ga.grams = (const Gram*)(m.base + m.o_grams) + b.gram0;
+    ga.out = nullptr;
+    ga.ngrams = b.ngram;
+    ga.units = b.units;
+    ga.N = j.N;
+    ga.ticket = (unsigned*)(m.base + m.o_ticket);
+    ga.status = j.status;
+    k_gram_sliced<<<std::min(b.units, m.sms), THREADS, SMEM_BYTES, s>>>(ga);
+    HeffArgs ha;
+    ha.N = j.N; ha.g0 = b.g0; ha.g1 = b.g1;
+    ha.first = b.g0 == 0;
+    ha.last = b.g1 == j.K;
+    ha.S1 = m.base + m.S1; ha.S2 = m.base + m.S2;
+    ha.A = m.base + b.A; ha.B = m.base + b.B;
+    ha.tiles = tiles;
+    ha.split_s = m.split_s;
+    ha.dx = j.dx; ha.dR = j.dR;
+    ha.sig = j.sig; ha.px = j.px; ha.pR = j.pR; ha.d = j.d;
+    ha.S = S; ha.H = H;
+    if (m.f64) k_heff<false><<<dim3(16, tiles), 256, 0, s>>>(ha);
+    else k_heff<true><<<dim3(16, tiles), 256, 0, s>>>(ha);
+  }
+  return 3 * (int)m.batches.size();
+}
+
+// Psi[i nR + j] = sum_a C_a psi_a(x_i) chi_a(R_j) as a sliced product over the trajectories: 8 digits
+// in the FP64 mode, 5 (34 bits below each grid point's largest term) in the mixed modes, whose terms
+// carry FP32 rounding.
+int AsmPlan::reconstruct(const JobView& j, const double2* C, double2* Psi, cudaStream_t s) const {
+  using namespace sl;
+  const Impl& m = *impl;
+  const int rxp = (j.nx + MT - 1) / MT * MT, rRp = (j.nR + MT - 1) / MT * MT;
+  SliceT sx{}, sR{};
+  sx.src = j.psi; sx.C = C;
+  sx.out = m.base + m.r_xa; sx.ex = (int*)(m.base + m.r_xe);
+  sx.n = j.nx; sx.ks = (j.N + 15) / 16; sx.N = j.N; sx.rpad = rxp; sx.R = MT; sx.d = m.rec_d; sx.f32 = !m.f64;
+  sR = sx;
+  sR.src = j.chi; sR.C = nullptr;
+  sR.out = m.base + m.r_Rb; sR.ex = (int*)(m.base + m.r_Re);
+  sR.n = j.nR; sR.rpad = rRp; sR.R = 32;
+  k_slices_t<<<dim3(std::max(rxp, rRp) / ST_ROWS, 2), ST_WARPS * 32, 0, s>>>(sx, sR, (unsigned*)(m.base + m.o_ticket));
+  GramArgs ga;
+  ga.grams = (const Gram*)(m.base + m.o_grams) + m.rec_gram;
+  ga.out = Psi;
+  ga.ngrams = 1;
+  ga.units = m.rec_units;
+  ga.N = j.N;
+  ga.ticket = (unsigned*)(m.base + m.o_ticket);
+  ga.status = j.status + STATUS_OBS;
+  k_gram_sliced<<<std::min(ga.units, m.sms), THREADS, SMEM_BYTES, s>>>(ga);
+  return 2;
+}
+
+}  // namespace icwf

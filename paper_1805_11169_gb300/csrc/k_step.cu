@@ -3,7 +3,6 @@
 //              factor values u_k(x_b), w_k(R_b), V(x_b, R_b) at the new positions;
 //   propagate  Hermitian-CWF equations (Eq. conditional_e/n with eta dropped): one Strang
 //              split-operator step per CWF, one CTA per CWF, the column staged in shared memory;
-//   assemble   FP64 matrix elements (Eq. M, W, W1, W2) from the rank-k factorisation;
 //   gram       generic A^H diag(d) B (diagnostics: kinetic and potential Grams for H).
 #include <cuda_runtime.h>
 
@@ -471,7 +470,7 @@ template bool add_group_nodes<double>(cudaGraph_t, const cudaGraphNode_t*, size_
 template bool add_group_nodes<float>(cudaGraph_t, const cudaGraphNode_t*, size_t, const GroupJob*,
                                      int, int, int, int, int, int, cudaGraphNode_t*);
 
-// ------------------------------------------------------------------------------ FP64 assembly
+// ------------------------------------------------------------------------------ diagnostic Grams
 
 constexpr int AT = 32;   // output tile (trajectories)
 constexpr int AKC = 16;  // grid points per shared-memory chunk
@@ -513,100 +512,6 @@ __device__ __forceinline__ void gram_tile(const c_t<T>* __restrict__ A, const c_
     __syncthreads();
   }
 }
-
-__device__ __forceinline__ void tri_index(int t, int& I, int& J) {
-  int Jc = (int)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-  while (Jc * (Jc + 1) / 2 > t) --Jc;
-  while ((Jc + 1) * (Jc + 2) / 2 <= t) ++Jc;
-  J = Jc;
-  I = t - Jc * (Jc + 1) / 2;
-}
-
-// One CTA per upper-triangular tile pair (I <= J): computes S and Heff for the tile (I, J) and,
-// off the diagonal, for the mirrored tile (J, I), from the Hermitian Grams of that tile:
-//   S1 = dx Psi^H Psi, S2 = dR X^H X, A_k = dx Psi^H diag(u_k) Psi, B_k = dR X^H diag(w_k) X,
-//   Heff_ab = sum_k s_k (A_k - u_k(x_b) S1)_ab (B_k - w_k(R_b) S2)_ab - V(x_b,R_b) S_ab.
-__global__ void __launch_bounds__(256) k_assemble_fp64(JobView j, double2* __restrict__ S,
-                                                        double2* __restrict__ H) {
-  __shared__ double2 As[AKC][AT + 1], Bs[AKC][AT + 1];
-  int I, J;
-  tri_index(blockIdx.x, I, J);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const double2* psi = (const double2*)j.psi;
-  const double2* chi = (const double2*)j.chi;
-  const int N = j.N;
-  int ar[2] = {I * AT + ty, I * AT + ty + 16};
-  int bc[2] = {J * AT + tx, J * AT + tx + 16};
-  double2 s1[2][2], s2[2][2], h[2][2], ht[2][2];
-  const double2 z = make_double2(0, 0);
-#pragma unroll
-  for (int r = 0; r < 2; ++r)
-#pragma unroll
-    for (int c = 0; c < 2; ++c) { s1[r][c] = z; s2[r][c] = z; h[r][c] = z; ht[r][c] = z; }
-  const bool mirror = I != J;
-  for (int k = -1; k < j.K; ++k) {
-    double2 gx[2][2] = {{z, z}, {z, z}}, gR[2][2] = {{z, z}, {z, z}};
-    gram_tile<double>(psi, psi, k < 0 ? nullptr : j.U + (size_t)k * j.nx, j.nx, N, I, J, As, Bs, gx);
-    gram_tile<double>(chi, chi, k < 0 ? nullptr : j.W + (size_t)k * j.nR, j.nR, N, I, J, As, Bs, gR);
-    if (k < 0) {
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) { s1[r][c] = cscale(gx[r][c], j.dx); s2[r][c] = cscale(gR[r][c], j.dR); }
-      continue;
-    }
-    const double sk = j.sig[k];
-    const double* pxk = j.px + (size_t)k * N;
-    const double* pRk = j.pR + (size_t)k * N;
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const double uxa = ar[r] < N ? pxk[ar[r]] : 0.0;
-      const double wRa = ar[r] < N ? pRk[ar[r]] : 0.0;
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const double uxb = bc[c] < N ? pxk[bc[c]] : 0.0;
-        const double wRb = bc[c] < N ? pRk[bc[c]] : 0.0;
-        const double2 A = cscale(gx[r][c], j.dx), B = cscale(gR[r][c], j.dR);
-        const double2 At = csub(A, cscale(s1[r][c], uxb));
-        const double2 Bt = csub(B, cscale(s2[r][c], wRb));
-        const double2 p = cmul(At, Bt);
-        h[r][c].x = fma(sk, p.x, h[r][c].x);
-        h[r][c].y = fma(sk, p.y, h[r][c].y);
-        if (mirror) {
-          const double2 At2 = csub(cconj(A), cscale(cconj(s1[r][c]), uxa));
-          const double2 Bt2 = csub(cconj(B), cscale(cconj(s2[r][c]), wRa));
-          const double2 p2 = cmul(At2, Bt2);
-          ht[r][c].x = fma(sk, p2.x, ht[r][c].x);
-          ht[r][c].y = fma(sk, p2.y, ht[r][c].y);
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    if (ar[r] >= N) continue;
-    const double da = j.d[ar[r]];
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      if (bc[c] >= N) continue;
-      const double db = j.d[bc[c]];
-      const double2 s = cmul(s1[r][c], s2[r][c]);
-      S[(size_t)ar[r] * N + bc[c]] = s;
-      H[(size_t)ar[r] * N + bc[c]] = csub(h[r][c], cscale(s, db));
-      if (mirror) {
-        S[(size_t)bc[c] * N + ar[r]] = cconj(s);
-        H[(size_t)bc[c] * N + ar[r]] = csub(ht[r][c], cscale(cconj(s), da));
-      }
-    }
-  }
-}
-
-void launch_assemble_fp64(const JobView& j, double2* S, double2* H, cudaStream_t s) {
-  const int T = (j.N + AT - 1) / AT;
-  k_assemble_fp64<<<T * (T + 1) / 2, 256, 0, s>>>(j, S, H);
-}
-
-// ------------------------------------------------------------------------------ diagnostics
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_gram(const c_t<T>* A, const c_t<T>* B, const double* dg,

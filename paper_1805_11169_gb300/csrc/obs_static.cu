@@ -102,8 +102,7 @@ extern "C" icwf_status icwf_observables_static(icwf_handle h, icwf_obs* out) {
   double2* proj = (double2*)take((size_t)8 * nR * sizeof(double2));
 
   cudaStream_t s = v.stream;
-  if (v.mixed) launch_reconstruct<float>(v.j, v.C, Psi, s);
-  else launch_reconstruct<double>(v.j, v.C, Psi, s);
+  v.plan->reconstruct(v.j, v.C, Psi, s);
   launch_obs_lines(v.j, Psi, v.phi, v.n_states, rho_x, rho_R, proj, part, o4, pop, decoh,
                    v.twx_d, v.twR_d, s);
   // a launch error of these kernels is reported without clearing errors left by other callers
@@ -112,7 +111,7 @@ extern "C" icwf_status icwf_observables_static(icwf_handle h, icwf_obs* out) {
     return ICWF_ERR_CUDA;
   }
   double host4[4];
-  int cl[2];
+  int cl[STATUS_COPY];
   bool ok = cudaMemcpyAsync(host4, o4, sizeof(host4), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
             cudaMemcpyAsync(cl, v.j.status, sizeof(cl), cudaMemcpyDeviceToHost, s) == cudaSuccess;
   if (ok && out->rho_x)
@@ -133,6 +132,11 @@ extern "C" icwf_status icwf_observables_static(icwf_handle h, icwf_obs* out) {
   out->norm = host4[0];
   out->energy = (host4[1] + host4[2] + host4[3]) / host4[0];
   out->n_states = v.n_states;
-  out->n_clamped = cl[1];
+  out->n_clamped = cl[STATUS_CLAMPED];
+  if (cl[STATUS_OBS] & ST_TIMEOUT) {
+    cudaMemset(v.j.status + STATUS_OBS, 0, sizeof(int));
+    handle_set_error(h, "icwf_observables_static: in-kernel wait timed out");
+    return ICWF_ERR_TIMEOUT;
+  }
   return ICWF_OK;
 }

@@ -50,6 +50,7 @@ __device__ __forceinline__ bool mbar_test(uint64_t* b, unsigned parity) {
 // Bounded wait; returns false (and raises the abort flag) on timeout or if another role aborted.
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity, volatile int* abort_flag,
                                          int* status) {
+  if (mbar_test(b, parity)) return true;   // the common case reads no timer
   const unsigned long long t0 = gtime();
   while (true) {
     if (mbar_test(b, parity)) return true;
@@ -134,6 +135,15 @@ __host__ __device__ constexpr uint32_t idesc_mn(int kind, int M, int N_) {
          ((uint32_t)(N_ >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// The same for kind::f16 with FP16 (f16 = 1) or BF16 pieces, without its N field (idesc_n); NEG_A
+// multiplies A by -1.
+__host__ __device__ constexpr uint32_t idesc_f16(int f16, int M, int N_) {
+  return (1u << 4) | ((f16 ? 0u : 1u) << 7) | ((f16 ? 0u : 1u) << 10) | ((uint32_t)(N_ >> 3) << 17) |
+         ((uint32_t)(M >> 4) << 24);
+}
+__host__ __device__ constexpr uint32_t idesc_n(int N_) { return (uint32_t)(N_ >> 3) << 17; }
+constexpr uint32_t IDESC_NEG_A = 1u << 13;
+
 // D[tmem] (+)= A * B^T with the given instruction descriptor (acc = 0 overwrites).
 template <int KIND>
 __device__ __forceinline__ void mma_desc(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id,
@@ -150,18 +160,6 @@ __device__ __forceinline__ void mma_desc(uint32_t d_tmem, uint64_t a, uint64_t b
         "l"(a), "l"(b), "r"(id), "r"(acc));
   }
 }
-
-// Block (I <= J) of 128 x 128 trajectories and ket quarter q from the linear CTA index.
-__device__ __forceinline__ void block_index(int t, int& I, int& J, int& q) {
-  q = t & 3;
-  t >>= 2;
-  int Jc = (int)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-  while (Jc * (Jc + 1) / 2 > t) --Jc;
-  while ((Jc + 1) * (Jc + 2) / 2 <= t) ++Jc;
-  J = Jc;
-  I = t - Jc * (Jc + 1) / 2;
-}
-
 
 // Driver entry point of cuTensorMapEncodeTiled (looked up once).
 inline PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
