@@ -558,13 +558,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_gram_sliced(GramArgs args) {
 
 enum : int { SRC_F64_DIGITS = 0, SRC_F32_DIGITS = 1, SRC_F32_F16 = 2, SRC_F32_BF16 = 3 };
 
-// One operand: rows = CWF columns of one side, weighted by w[i] if given.
+// Operands of up to SLICE_GROUP terms in the same format: rows = CWF columns of one side, weighted by
+// w[i] of each term if given (FP64 weights for complex128 CWFs, FP32 for complex64).
+constexpr int SLICE_GROUP = 4;
 struct Slice {
   const void* src;          // complex128 or complex64, row r at src + r n
-  const double* w;
-  unsigned char* out;
+  const void* w;            // ng weights of n points each
+  unsigned char* out;       // term q at out + q ostride, its exponents at ex + q estride
   int* ex;                  // rpad exponents
-  int n, ks, rows, rpad, R; // points, K slices, rows (and padded to tiles of R rows)
+  size_t ostride, estride;
+  int ng, n, ks, rows, rpad, R;   // terms, points, K slices, rows (and padded to tiles of R rows)
   int d, kind, b0, beta;
 };
 
@@ -641,38 +644,61 @@ __device__ __forceinline__ void emit_pieces(const Slice& s, int row, int c8, int
   *(uint4*)slice_at(s, row, c8, plane, 1) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
 }
 
-// Components of 8 points of a row (zero past the row's end and in padding rows), weighted; 16-byte
-// loads (rows are 8 or more points, so every chunk starts on a 16-byte boundary).
-template <typename Z, typename T>
-__device__ __forceinline__ void load8(const Slice& s, int row, int c8, T (&re)[8], T (&im)[8]) {
-  if (row >= s.rows || 8 * c8 >= s.n) {
+// Components of 8 points of a row (zero past the row's end and in padding rows); 16-byte loads (rows
+// are 8 or more points, so every chunk starts on a 16-byte boundary).
+__device__ __forceinline__ void load8(const Slice& s, int row, int c8, float (&re)[8], float (&im)[8]) {
+  const float4* p = (const float4*)((const float2*)s.src + (size_t)row * s.n + 8 * c8);
+  const bool in = row < s.rows && 8 * c8 < s.n;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) re[k] = im[k] = 0;
-    return;
+  for (int k = 0; k < 4; ++k) {
+    const float4 z = in ? p[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+    re[2 * k] = z.x; im[2 * k] = z.y; re[2 * k + 1] = z.z; im[2 * k + 1] = z.w;
   }
-  const Z* p = (const Z*)s.src + (size_t)row * s.n + 8 * c8;
-  if constexpr (sizeof(T) == 4) {
+}
+__device__ __forceinline__ void load8(const Slice& s, int row, int c8, double (&re)[8], double (&im)[8]) {
+  const double2* p = (const double2*)s.src + (size_t)row * s.n + 8 * c8;
+  const bool in = row < s.rows && 8 * c8 < s.n;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float4 z = ((const float4*)p)[k];
-      re[2 * k] = z.x; im[2 * k] = z.y; re[2 * k + 1] = z.z; im[2 * k + 1] = z.w;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const Z z = p[k];
-      re[k] = z.x; im[k] = z.y;
-    }
+  for (int k = 0; k < 8; ++k) {
+    const double2 z = in ? p[k] : make_double2(0.0, 0.0);
+    re[k] = z.x; im[k] = z.y;
   }
-  if (s.w) {
-    const double2* w = (const double2*)(s.w + 8 * c8);
+}
+__device__ __forceinline__ void weight8(const Slice& s, int q, int c8, float (&re)[8], float (&im)[8]) {
+  if (!s.w || 8 * c8 >= s.n) return;
+  const float4* w = (const float4*)((const float*)s.w + (size_t)q * s.n + 8 * c8);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const double2 f = w[k];
-      re[2 * k] *= (T)f.x; im[2 * k] *= (T)f.x;
-      re[2 * k + 1] *= (T)f.y; im[2 * k + 1] *= (T)f.y;
-    }
+  for (int k = 0; k < 2; ++k) {
+    const float4 f = w[k];
+    re[4 * k] *= f.x; re[4 * k + 1] *= f.y; re[4 * k + 2] *= f.z; re[4 * k + 3] *= f.w;
+    im[4 * k] *= f.x; im[4 * k + 1] *= f.y; im[4 * k + 2] *= f.z; im[4 * k + 3] *= f.w;
   }
+}
+__device__ __forceinline__ void weight8(const Slice& s, int q, int c8, double (&re)[8], double (&im)[8]) {
+  if (!s.w || 8 * c8 >= s.n) return;
+  const double2* w = (const double2*)((const double*)s.w + (size_t)q * s.n + 8 * c8);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double2 f = w[k];
+    re[2 * k] *= f.x; im[2 * k] *= f.x;
+    re[2 * k + 1] *= f.y; im[2 * k + 1] *= f.y;
+  }
+}
+__device__ __forceinline__ unsigned long long max8(unsigned long long m, const double (&re)[8], const double (&im)[8]) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const unsigned long long a = abs_bits(re[k]), b = abs_bits(im[k]);
+    m = m > a ? m : a;
+    m = m > b ? m : b;
+  }
+  return m;
+}
+__device__ __forceinline__ unsigned long long max8(unsigned long long m, const float (&re)[8], const float (&im)[8]) {
+  unsigned x = (unsigned)m;
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    x = max(x, max(__float_as_uint(re[k]) & 0x7FFFFFFFu, __float_as_uint(im[k]) & 0x7FFFFFFFu));
+  return x;
 }
 
 // Largest magnitude (as bits) of one row over its tpr threads (a power of two; rows of fewer than 32
@@ -691,98 +717,96 @@ __device__ __forceinline__ unsigned long long row_max(unsigned long long m, int 
   return m;
 }
 
-// Operands in slices, grid (row groups, operands): a row's 8-point chunks are spread over
-// min(2 ks, 256) threads.  A thread keeps the first chunk's values between the two passes (largest
-// component, pieces), which is all of its work up to 2048 points.
-__global__ void __launch_bounds__(256) k_slices(const Slice* __restrict__ list, unsigned* ticket) {
-  __shared__ unsigned long long red[8];
-  const Slice s = list[blockIdx.y];
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *ticket = 0;   // the Gram launch's
+// pieces or digits of 8 points of row `row`, term q
+__device__ __forceinline__ void emit8(const Slice& s, int row, int c, int e, const double (&re)[8],
+                                      const double (&im)[8]) {
+  switch (s.d) {
+    case 2: emit_f64<2>(s, row, c, 0, re, e); emit_f64<2>(s, row, c, 1, im, e); break;
+    case 3: emit_f64<3>(s, row, c, 0, re, e); emit_f64<3>(s, row, c, 1, im, e); break;
+    case 4: emit_f64<4>(s, row, c, 0, re, e); emit_f64<4>(s, row, c, 1, im, e); break;
+    case 5: emit_f64<5>(s, row, c, 0, re, e); emit_f64<5>(s, row, c, 1, im, e); break;
+    case 6: emit_f64<6>(s, row, c, 0, re, e); emit_f64<6>(s, row, c, 1, im, e); break;
+    case 7: emit_f64<7>(s, row, c, 0, re, e); emit_f64<7>(s, row, c, 1, im, e); break;
+    default: emit_f64<8>(s, row, c, 0, re, e); emit_f64<8>(s, row, c, 1, im, e); break;
+  }
+}
+__device__ __forceinline__ void emit8(const Slice& s, int row, int c, int e, const float (&re)[8],
+                                      const float (&im)[8]) {
+  // 2^k in two factors, each a normal number
+  const int k2 = (s.kind == SRC_F32_DIGITS ? s.b0 : PIECE_BITS) - e;
+  const float f1 = scaled(1.f, k2 / 2), f2 = scaled(1.f, k2 - k2 / 2);
+  if (s.kind == SRC_F32_DIGITS) {
+    emit_f32_digits(s, row, c, 0, re, f1, f2);
+    emit_f32_digits(s, row, c, 1, im, f1, f2);
+  } else if (s.kind == SRC_F32_F16) {
+    emit_pieces<true>(s, row, c, 0, re, f1, f2);
+    emit_pieces<true>(s, row, c, 1, im, f1, f2);
+  } else {
+    emit_pieces<false>(s, row, c, 0, re, f1, f2);
+    emit_pieces<false>(s, row, c, 1, im, f1, f2);
+  }
+}
+
+// Operands in slices, grid (row groups, operand groups): a row's 8-point chunks are spread over
+// min(2 ks, 256) threads, and a thread keeps its chunk (all of its work up to 2048 points) for every
+// term of the group: what bounds this kernel is the load/store unit's passes over scattered 32-byte
+// rows.  (N = 1024, 16 terms on 1024 x 512: 153 us with one term per thread and FP64 weights converted
+// here, 76 us with four terms and FP32 weights; 226 MB written, 33 us at the copy rate.)
+template <typename T>
+__device__ __forceinline__ void slice_rows(Slice s, unsigned long long (&red)[2][8]) {
+  constexpr bool F64 = sizeof(T) == 8;
   const int c8n = 2 * s.ks, tpr = c8n < 256 ? c8n : 256, rpb = 256 / tpr;
   if ((int)blockIdx.x * rpb >= s.rpad) return;
   const int row = (int)blockIdx.x * rpb + (int)threadIdx.x / tpr, t0 = (int)threadIdx.x % tpr;
-  // magnitudes order like their bit patterns, NaN above infinity
-  unsigned long long m = 0;
-  if (s.kind == SRC_F64_DIGITS) {
-    double re[8], im[8];
-    auto scan = [&]() {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const unsigned long long a = abs_bits(re[k]), b = abs_bits(im[k]);
-        m = m > a ? m : a;
-        m = m > b ? m : b;
-      }
-    };
+  T zr[8], zi[8];
+  load8(s, row, t0, zr, zi);
+  for (int q = 0; q < s.ng; ++q) {
+    T re[8], im[8];
+    unsigned long long m = 0;
     for (int c = t0 + tpr; c < c8n; c += tpr) {
-      load8<double2, double>(s, row, c, re, im);
-      scan();
+      load8(s, row, c, re, im);
+      weight8(s, q, c, re, im);
+      m = max8(m, re, im);
     }
-    load8<double2, double>(s, row, t0, re, im);
-    scan();
-    m = row_max(m, tpr, red);
-    if (row >= s.rpad) return;
-    const bool bad = m >= 0x7FF0000000000000ull;
-    const int e = bad ? 0 : exponent_above_f64(m);
-    if (t0 == 0) s.ex[row] = bad ? EX_BAD : e;
-    for (int c = t0; c < c8n; c += tpr) {
-      if (c != t0) load8<double2, double>(s, row, c, re, im);
-      if (bad) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) re[k] = im[k] = 0.0;
-      }
-      switch (s.d) {
-        case 2: emit_f64<2>(s, row, c, 0, re, e); emit_f64<2>(s, row, c, 1, im, e); break;
-        case 3: emit_f64<3>(s, row, c, 0, re, e); emit_f64<3>(s, row, c, 1, im, e); break;
-        case 4: emit_f64<4>(s, row, c, 0, re, e); emit_f64<4>(s, row, c, 1, im, e); break;
-        case 5: emit_f64<5>(s, row, c, 0, re, e); emit_f64<5>(s, row, c, 1, im, e); break;
-        case 6: emit_f64<6>(s, row, c, 0, re, e); emit_f64<6>(s, row, c, 1, im, e); break;
-        case 7: emit_f64<7>(s, row, c, 0, re, e); emit_f64<7>(s, row, c, 1, im, e); break;
-        default: emit_f64<8>(s, row, c, 0, re, e); emit_f64<8>(s, row, c, 1, im, e); break;
-      }
+    for (int k = 0; k < 8; ++k) { re[k] = zr[k]; im[k] = zi[k]; }
+    weight8(s, q, t0, re, im);
+    m = max8(m, re, im);
+    // magnitudes order like their bit patterns, NaN above infinity
+    m = row_max(m, tpr, red[q & 1]);
+    const bool bad = m >= (F64 ? 0x7FF0000000000000ull : 0x7F800000ull);
+    int e = 0;
+    if (!bad) {
+      if constexpr (F64) e = exponent_above_f64(m);
+      else e = m ? ilogbf(__uint_as_float((unsigned)m)) + 1 : 0;
     }
-    return;
-  }
-  float re[8], im[8];
-  unsigned mf = 0;
-  auto scan = [&]() {
+    const bool digits = F64 || s.kind == SRC_F32_DIGITS;
+    if (row < s.rpad) {
+      if (t0 == 0) s.ex[row] = bad && digits ? EX_BAD : e;
+      for (int c = t0; c < c8n; c += tpr) {
+        if (c != t0) {
+          load8(s, row, c, re, im);
+          weight8(s, q, c, re, im);
+        }
+        if (bad && digits) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const unsigned a = __float_as_uint(re[k]) & 0x7FFFFFFFu, b = __float_as_uint(im[k]) & 0x7FFFFFFFu;
-      mf = max(mf, max(a, b));
-    }
-  };
-  for (int c = t0 + tpr; c < c8n; c += tpr) {
-    load8<float2, float>(s, row, c, re, im);
-    scan();
-  }
-  load8<float2, float>(s, row, t0, re, im);
-  scan();
-  m = row_max(mf, tpr, red);
-  if (row >= s.rpad) return;
-  const bool bad = m >= 0x7F800000ull;
-  const int e = m && !bad ? ilogbf(__uint_as_float((unsigned)m)) + 1 : 0;
-  const bool digits = s.kind == SRC_F32_DIGITS;
-  if (t0 == 0) s.ex[row] = bad && digits ? EX_BAD : e;
-  // 2^k in two factors, each a normal number
-  const int k2 = (digits ? s.b0 : PIECE_BITS) - e;
-  const float f1 = ldexpf(1.f, k2 / 2), f2 = ldexpf(1.f, k2 - k2 / 2);
-  for (int c = t0; c < c8n; c += tpr) {
-    if (c != t0) load8<float2, float>(s, row, c, re, im);
-    if (digits) {
-      if (bad) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) re[k] = im[k] = 0.f;
+          for (int k = 0; k < 8; ++k) re[k] = im[k] = 0;
+        }
+        emit8(s, row, c, e, re, im);
       }
-      emit_f32_digits(s, row, c, 0, re, f1, f2);
-      emit_f32_digits(s, row, c, 1, im, f1, f2);
-    } else if (s.kind == SRC_F32_F16) {
-      emit_pieces<true>(s, row, c, 0, re, f1, f2);
-      emit_pieces<true>(s, row, c, 1, im, f1, f2);
-    } else {
-      emit_pieces<false>(s, row, c, 0, re, f1, f2);
-      emit_pieces<false>(s, row, c, 1, im, f1, f2);
     }
+    s.out += s.ostride;
+    s.ex += s.estride;
   }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_slices(const Slice* __restrict__ list,
+                                                                        unsigned* ticket) {
+  __shared__ unsigned long long red[2][8];
+  const Slice s = list[blockIdx.y];
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *ticket = 0;   // the Gram launch's
+  slice_rows<T>(s, red);
 }
 
 // An operand of Psi(x_i, R_j) = sum_a C_a psi_a(x_i) chi_a(R_j): rows = grid points, K = trajectories.
@@ -869,13 +893,18 @@ struct HeffArgs {
   double dx, dR;
   const double *sig, *px, *pR, *d;
   double2 *S, *H;
+  int split;                // term groups (blockIdx.z); > 1: partial sums meet in `part`
+  void* part;               // [group][tile][direct, mirrored][128 x 128] of Z
+  unsigned* done;           // [tile][patch]: groups finished (zero between launches)
 };
 
 // Threads of one 32 x 32 patch of a 128 x 128 upper-triangle tile: lane = bra, 4 kets each.  F32: the
 // mixed modes' FP32 arithmetic on float2 Grams; else FP64 on double2 Grams that carry s_g dx and dR
 // already (folded into the operands' weights): 8 FP64 instructions per term, element and side, which
-// is what bounds the FP64 version (0.35 ms at N = 1024 and 22 terms); the F32 version reads its Grams
-// once.
+// is what bounds the FP64 version (0.39 ms at N = 1024 and 22 terms); the F32 version reads its Grams
+// once (60 us at N = 1024, 16 terms; 136 us with the factors' conversions in the loop).  With fewer
+// patches than SMs the terms are split over CTAs as well (16 trajectories, 64 terms, FP64: 202 us
+// without, 50 us with).
 constexpr int HG = 16;   // terms staged at a time
 template <bool F32>
 __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
@@ -885,6 +914,7 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
   // the terms' factor values at the 32 bras and 32 kets, converted once per CTA (a conversion from
   // FP64 costs an FP64 instruction)
   __shared__ T uxs[HG][64], wRs[HG][64];
+  __shared__ int s_last;
   int I, J;
   tri_tile(blockIdx.y, I, J);
   const int N = p.N, lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -910,7 +940,7 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
     s2[e].x = (T)s2d[e].x; s2[e].y = (T)s2d[e].y;
     h[e].x = h[e].y = ht[e].x = ht[e].y = 0;
     const int b = b0 + 8 * e;
-    if (!p.first && a_ok && b < N) {
+    if (!p.first && blockIdx.z == 0 && a_ok && b < N) {
       const double2 v = p.H[(size_t)a * N + b];
       h[e].x = (T)v.x; h[e].y = (T)v.y;
       if (mirror) {
@@ -921,13 +951,15 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
   }
   const size_t gs = p.tiles * MT * MT;
   const int as = I * MT + (int)(blockIdx.x & 3) * 32, bs = J * MT + (int)(blockIdx.x >> 2) * 32;
-  for (int g = p.g0; g < p.g1; ++g) {
-    const int gl = (g - p.g0) & (HG - 1);
+  const int z0 = p.g0 + (int)((long long)(p.g1 - p.g0) * blockIdx.z / p.split);
+  const int z1 = p.g0 + (int)((long long)(p.g1 - p.g0) * (blockIdx.z + 1) / p.split);
+  for (int g = z0; g < z1; ++g) {
+    const int gl = (g - z0) & (HG - 1);
     if (gl == 0) {
       __syncthreads();
       for (int i = threadIdx.x; i < HG * 64; i += 256) {
         const int gi = g + (i >> 6), c = i & 63, t = c < 32 ? as + c : bs + c - 32;
-        if (gi < p.g1) {
+        if (gi < z1) {
           const double s = F32 ? 1.0 : p.sig[gi];
           uxs[i >> 6][c] = t < N ? (T)(s * p.px[(size_t)gi * N + t]) : (T)0;
           wRs[i >> 6][c] = t < N ? (T)p.pR[(size_t)gi * N + t] : (T)0;
@@ -965,6 +997,39 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
         } else {
           ht[e].x = fma(mtr, ntr, fma(-mti, nti, ht[e].x));
           ht[e].y = fma(-mtr, nti, fma(-mti, ntr, ht[e].y));
+        }
+      }
+    }
+  }
+  if (p.split > 1) {
+    // few tiles: the terms are spread over CTAs; the last one to finish a patch adds the groups' sums
+    // in their order (so the result does not depend on timing) and goes on
+    const size_t dir = (size_t)MT * MT, grp = p.tiles * 2 * dir;
+    Z* mine = (Z*)p.part + blockIdx.z * grp + (size_t)blockIdx.y * 2 * dir + (size_t)br * MT + ar;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      mine[e * step] = h[e];
+      if (mirror) mine[dir + e * step] = ht[e];
+    }
+    __threadfence();
+    __syncthreads();
+    unsigned* cnt = p.done + blockIdx.y * 16 + blockIdx.x;
+    if (threadIdx.x == 0) s_last = atomicAdd(cnt, 1u) == (unsigned)p.split - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) *cnt = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) h[e].x = h[e].y = ht[e].x = ht[e].y = 0;
+    for (int z = 0; z < p.split; ++z) {
+      const Z* q = (const Z*)p.part + z * grp + (size_t)blockIdx.y * 2 * dir + (size_t)br * MT + ar;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const Z v = __ldcg(q + e * step);
+        h[e].x += v.x; h[e].y += v.y;
+        if (mirror) {
+          const Z w = __ldcg(q + dir + e * step);
+          ht[e].x += w.x; ht[e].y += w.y;
         }
       }
     }
@@ -1049,6 +1114,9 @@ struct AsmPlan::Impl {
   std::vector<sl::Gram> grams;
   std::vector<Batch> batches;
   std::vector<double> Uw, Ww;            // FP64: weights u_g s_g dx and w_g dR
+  std::vector<float> Uf, Wf;             // mixed modes: u_g and w_g
+  size_t part = 0, o_done = 0;           // split term sums of k_heff
+  int split = 1;
   size_t bytes = 0, o_slices = 0, o_grams = 0, o_uw = 0, o_ww = 0, o_ticket = 0;
   size_t S1 = 0, S2 = 0;
   size_t r_xa = 0, r_xe = 0, r_Rb = 0, r_Re = 0;   // reconstruction operands (in the batch scratch)
@@ -1089,10 +1157,13 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     if (!split_s) { sa[s] = take(op_bytes(s, dS)); se[s] = take((size_t)rp * 4); }
     if (!f64) { pa[s] = take(op_bytes(s, 2)); pe[s] = take((size_t)rp * 4); }
   }
-  if (f64) {
-    m.o_uw = take((size_t)K * q.nx * 8);
-    m.o_ww = take((size_t)K * q.nR * 8);
-  }
+  m.o_uw = take((size_t)K * q.nx * (f64 ? 8 : 4));
+  m.o_ww = take((size_t)K * q.nR * (f64 ? 8 : 4));
+  // few tiles leave SMs idle in k_heff: spread the terms over up to 16 groups of 4 or more
+  const int patches = tiles_of(N) == 1 ? ((N + 31) / 32) * ((N + 31) / 32) : tiles * 16;
+  m.split = std::max(1, std::min({16, 304 / patches, K / 4}));
+  m.o_done = take((size_t)tiles * 16 * 4);
+  if (m.split > 1) m.part = take((size_t)m.split * tiles * 2 * MT * MT * osz);
   std::vector<int> dg(K);
   for (int g = 0; g < K; ++g) dg[g] = f64 ? term_digits(q.sig[0] > 0 ? q.sig[g] / q.sig[0] : 0.0) : 2;
   // batches of terms
@@ -1130,10 +1201,11 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     b.gram0 = (int)m.grams.size();
     b.g0 = g0;
     b.g1 = g1;
-    auto add_slice = [&](int side, const double* w, size_t out, size_t ex, int R, int d, int kind, int b0, int beta) {
+    auto add_slice = [&](int side, const void* w, size_t out, size_t ex, int R, int d, int kind, int b0, int beta) {
       Slice s{};
       s.src = j ? (side ? j->chi : j->psi) : nullptr;
       s.w = w;
+      s.ng = 1;
       s.out = ptr(out);
       s.ex = (int*)ptr(ex);
       s.n = n[side]; s.ks = ks[side]; s.rows = N; s.rpad = rp; s.R = R;
@@ -1178,6 +1250,7 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     // the Grams of one side are consecutive (k_heff walks them with a fixed stride)
     b.A = tmp((size_t)(g1 - g0) * out_b);
     b.B = tmp((size_t)(g1 - g0) * out_b);
+    int grp[2] = {-1, -1};
     for (int g = g0; g < g1; ++g)
       for (int s = 0; s < 2; ++s) {
         const int d = dg[g];
@@ -1186,10 +1259,22 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
         if (dr < ks[s]) t = 32;
         t = kets_per_unit(N, t);
         const size_t o = tmp(op_bytes(s, d)), oe = tmp((size_t)rp * 4);
-        const double* w = nullptr;
-        if (f64) w = (const double*)ptr(s ? m.o_ww : m.o_uw) + (size_t)g * n[s];
-        else if (j) w = (s ? j->W : j->U) + (size_t)g * n[s];
-        add_slice(s, w, o, oe, t, d, f64 ? SRC_F64_DIGITS : pk, f64 ? 6 : 0, f64 ? fdig : 0);
+        const void* w = f64 ? (const void*)((const double*)ptr(s ? m.o_ww : m.o_uw) + (size_t)g * n[s])
+                            : (const void*)((const float*)ptr(s ? m.o_ww : m.o_uw) + (size_t)g * n[s]);
+        // consecutive terms in the same format share a group (their operands are evenly spaced)
+        Slice* last = grp[s] >= 0 ? &m.slices[grp[s]] : nullptr;
+        if (last && last->ng < SLICE_GROUP && last->d == d && last->R == t) {
+          const size_t os = (size_t)(ptr(o) - last->out), es = (size_t)((int*)ptr(oe) - last->ex);
+          if (last->ng == 1) { last->ostride = os; last->estride = es; }
+          if (os == last->ng * last->ostride && es == last->ng * last->estride) ++last->ng;
+          else last = nullptr;
+        } else {
+          last = nullptr;
+        }
+        if (!last) {
+          grp[s] = (int)m.slices.size();
+          add_slice(s, w, o, oe, t, d, f64 ? SRC_F64_DIGITS : pk, f64 ? 6 : 0, f64 ? fdig : 0);
+        }
         add_gram(s, f64 ? sa[s] : pa[s], f64 ? se[s] : pe[s], f64 ? dS : 2, ptr(o), (int*)ptr(oe), d, d, t, dr,
                  !f64 && f16, f64, f64 ? 6 : 0, f64 ? fdig : 0, (s ? b.B : b.A) + (size_t)(g - g0) * out_b);
       }
@@ -1236,17 +1321,28 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
 bool AsmPlan::upload(const AsmShape& q, const double* U, const double* W, cudaStream_t s) {
   using namespace sl;
   Impl& m = *impl;
+  const size_t nu = (size_t)q.K * q.nx, nw = (size_t)q.K * q.nR;
+  const void *hu, *hw;
   if (m.f64) {
-    m.Uw.resize((size_t)q.K * q.nx);
-    m.Ww.resize((size_t)q.K * q.nR);
+    m.Uw.resize(nu);
+    m.Ww.resize(nw);
     for (int g = 0; g < q.K; ++g) {
       for (int i = 0; i < q.nx; ++i) m.Uw[(size_t)g * q.nx + i] = U[(size_t)g * q.nx + i] * (q.sig[g] * q.dx);
       for (int i = 0; i < q.nR; ++i) m.Ww[(size_t)g * q.nR + i] = W[(size_t)g * q.nR + i] * q.dR;
     }
-    if (cudaMemcpyAsync(m.base + m.o_uw, m.Uw.data(), m.Uw.size() * 8, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(m.base + m.o_ww, m.Ww.data(), m.Ww.size() * 8, cudaMemcpyHostToDevice, s) != cudaSuccess)
-      return false;
+    hu = m.Uw.data();
+    hw = m.Ww.data();
+  } else {
+    m.Uf.assign(U, U + nu);
+    m.Wf.assign(W, W + nw);
+    hu = m.Uf.data();
+    hw = m.Wf.data();
   }
+  const size_t ws = m.f64 ? 8 : 4;
+  if (cudaMemcpyAsync(m.base + m.o_uw, hu, nu * ws, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+      cudaMemcpyAsync(m.base + m.o_ww, hw, nw * ws, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+      cudaMemsetAsync(m.base + m.o_done, 0, (size_t)tiles_of(q.N) * 16 * 4, s) != cudaSuccess)
+    return false;
   if (cudaMemcpyAsync(m.base + m.o_slices, m.slices.data(), m.slices.size() * sizeof(Slice), cudaMemcpyHostToDevice,
                       s) != cudaSuccess ||
       cudaMemcpyAsync(m.base + m.o_grams, m.grams.data(), m.grams.size() * sizeof(Gram), cudaMemcpyHostToDevice,
@@ -1269,8 +1365,10 @@ int AsmPlan::launch(const JobView& j, double2* S, double2* H, cudaStream_t s) co
   const Impl& m = *impl;
   const int tiles = tiles_of(j.N);
   for (const auto& b : m.batches) {
-    k_slices<<<dim3(b.rowgroups, b.nslice), 256, 0, s>>>((const Slice*)(m.base + m.o_slices) + b.slice0,
-                                                         (unsigned*)(m.base + m.o_ticket));
+    const Slice* sl0 = (const Slice*)(m.base + m.o_slices) + b.slice0;
+    unsigned* ticket = (unsigned*)(m.base + m.o_ticket);
+    if (m.f64) k_slices<double><<<dim3(b.rowgroups, b.nslice), 256, 0, s>>>(sl0, ticket);
+    else k_slices<float><<<dim3(b.rowgroups, b.nslice), 256, 0, s>>>(sl0, ticket);
     GramArgs ga;
     ga.grams = (const Gram*)(m.base + m.o_grams) + b.gram0;
     ga.out = nullptr;
@@ -1291,8 +1389,11 @@ int AsmPlan::launch(const JobView& j, double2* S, double2* H, cudaStream_t s) co
     ha.dx = j.dx; ha.dR = j.dR;
     ha.sig = j.sig; ha.px = j.px; ha.pR = j.pR; ha.d = j.d;
     ha.S = S; ha.H = H;
-    if (m.f64) k_heff<false><<<dim3(16, tiles), 256, 0, s>>>(ha);
-    else k_heff<true><<<dim3(16, tiles), 256, 0, s>>>(ha);
+    ha.split = std::max(1, std::min(m.split, (b.g1 - b.g0) / 4));
+    ha.part = m.base + m.part;
+    ha.done = (unsigned*)(m.base + m.o_done);
+    if (m.f64) k_heff<false><<<dim3(16, tiles, ha.split), 256, 0, s>>>(ha);
+    else k_heff<true><<<dim3(16, tiles, ha.split), 256, 0, s>>>(ha);
   }
   return 3 * (int)m.batches.size();
 }
