@@ -9,13 +9,16 @@
 // style of Ogita, Rump and Oishi's Dot2 (TwoProduct + TwoSum, errors summed separately), which
 // returns them as accurately as if evaluated in twice the FP32 precision.
 //
-// Kernels: k_shift_mix_df (S -> S + eps I, converted); k_chol_step_df (the blocked Cholesky, one
-// launch per block column with look-ahead: quadrant updates, diagonal factor, panel slabs,
+// Kernels: k_shift_mix_df (S -> S + eps I, converted); k_chol_df (the blocked Cholesky, one
+// persistent launch with look-ahead: diagonal updates, diagonal factors, panel slabs,
 // trailing tiles and the inverses of the diagonal blocks as ticket-ordered tasks; the panel tasks
 // also write L^H into the upper triangle); k_chol_solve_cluster (both triangular solves in one
 // 8-CTA cluster, N <= 2048) and k_trsv_lower_df / k_trsv_upper_df (per-block kernels with global
 // flags, larger N).
 #include <cuda_runtime.h>
+
+#include <algorithm>
+#include <mutex>
 
 #include "df64.cuh"
 #include "icwf_internal.h"
@@ -142,25 +145,43 @@ __device__ __forceinline__ void tri_index(int t, int& I, int& J) {
 
 // ---------------------------------------------------------------------------- blocked factorisation
 //
-// Right-looking blocked Cholesky with one launch per block column and a look-ahead: launch li
-// applies panel li - 1 to the trailing matrix and, in the same launch, factors diagonal block li
-// and solves panel li.  Its CTAs take tickets in dependency order
-//   [3 quadrant updates of diagonal block li] [diagonal factor li] [trailing tiles right of
-//   block column li] [panel-li slabs of 8 rows],
-// and wait (bounded) only for tasks with smaller tickets, which are already running: the diagonal
-// factor waits for its three quadrants, the panel slabs for the diagonal factor.  So the chain
-// quadrants -> factor -> slabs overlaps the bulk of the trailing update, and the factor of block
-// li + 1 starts as soon as launch li + 1 does.  All arithmetic is double-float with compensated
-// (Dot2) accumulation; complex products in the updates use three real products (Karatsuba).
+// Right-looking blocked Cholesky of up to two matrices in one persistent launch.  Every CTA is two
+// groups of 256 threads with their own barriers and shared memory.  The first nbatch CTAs to arrive
+// become the matrices' chain CTAs: chain m factors the diagonal blocks 0, 1, 2, ... of matrix m, alone
+// on its SM.  All other groups take tickets for the remaining tasks, which are numbered block column
+// by block column li (jb = li - 1 is the panel being applied):
+//   [10 updates of diagonal block li] [some trailing tiles] [panel-li slabs of 8 rows] [the other
+//   trailing tiles] [inverse of diagonal block li - 1].
+// A task waits (bounded) on control words for exactly the data it reads, which come from smaller
+// tickets or from a diagonal factor; a diagonal factor waits for updates whose tickets precede
+// everything that waits for it.  So whatever is running can finish: progress needs only that the
+// chains and one more CTA are resident.  The trailing tiles ahead of the slabs are as many as run
+// while the diagonal factor does, so neither the slabs wait behind the whole trailing update nor the
+// groups behind the factor.
+// Why one launch: a launch per block column started every diagonal factor with a cold instruction
+// cache (15-25 us each instead of 11) and kept the slabs behind all trailing tiles of their launch.
+// All arithmetic is double-float with compensated (Dot2) accumulation; complex products in the
+// updates use three real products (Karatsuba).
 
 constexpr int CS_THREADS = 256;
+constexpr int DIAG_TASKS = 10;                // 8 x 8 blocks of a diagonal block's lower triangle
 constexpr int TS_ROWS = 8;                    // panel rows per slab task
 constexpr unsigned CS_WAIT_LIMIT = 1u << 24;
 constexpr int CS_SMEM = 6 * NB * NB * 8;      // largest task: trailing tile, 6 double-float planes
-// shared memory requested per CTA: more than the tasks use, so that at most two CTAs share an SM
-// and the dependency chain (diagonal factor, panel slabs) is not starved by trailing tiles
-constexpr int CS_SMEM_LAUNCH = 100 * 1024;
-static_assert(CS_SMEM <= CS_SMEM_LAUNCH, "tasks need more shared memory than the launch asks for");
+constexpr int CTA_THREADS = 2 * CS_THREADS;   // two groups
+// shared memory requested per CTA: more than half an SM's, so that a chain CTA shares its SM with no
+// other CTA of the launch
+constexpr int CS_SMEM_LAUNCH = 116 * 1024;
+static_assert(2 * CS_SMEM <= CS_SMEM_LAUNCH, "tasks need more shared memory than the launch asks for");
+constexpr int AHEAD_TILES = 300;              // trailing tiles ahead of the slabs: one per group
+
+// One group of CS_THREADS threads of a CTA.
+struct Grp {
+  int tid, bar;
+  __device__ __forceinline__ void sync() const {
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(CS_THREADS) : "memory");
+  }
+};
 
 __device__ __forceinline__ cdf ldcg4(const float4* p) { return ld4(__ldcg(p)); }
 __device__ __forceinline__ cdf cdf_sub_sloppy(cdf a, cdf b) {
@@ -177,33 +198,58 @@ __device__ __forceinline__ cdf kara_val(acc2 p1, acc2 p2, acc2 p3) {
   return cdf_make(acc_val(acc_merge(p1, p2)), acc_val(acc_merge(acc_merge(p3, acc_neg(p1)), p2)));
 }
 
+// until *f >= target, or with kBits until all bits of target are set
+template <bool kBits = false>
 __device__ __forceinline__ bool cs_wait(const unsigned* f, unsigned target, int* status) {
   const unsigned lim = wait_budget(status, CS_WAIT_LIMIT);
   for (unsigned it = 0; it < lim; ++it) {
-    if (ld_acquire(f) >= target) return true;
+    const unsigned v = ld_acquire(f);
+    if (kBits ? (v & target) == target : v >= target) return true;
     if (it > 256) __nanosleep(128);
   }
   set_flag(status, ST_TIMEOUT);
   return false;
 }
-// all of this CTA's global writes, then a release increment of *f
-__device__ __forceinline__ void cs_signal(unsigned* f) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
+// all of this group's global writes, then a release increment of *f
+__device__ __forceinline__ void cs_signal(const Grp& g, unsigned* f) {
+  g.sync();
+  if (g.tid == 0) {
     __threadfence();
     atomicAdd(f, 1u);
   }
+}
+
+// a -= x conj(y) with each part of a as an unevaluated sum whose low word is not renormalised: the two
+// leading products of a part are added error-free, everything of second order goes to the low word.
+// 24 FP32 operations per part, 16 of them on the longest chain.
+__device__ __forceinline__ df df_sub2(df a, df x1, df y1, df x2, df y2) {   // a - x1 y1 - x2 y2
+  const float p1 = DF_MUL(-x1.h, y1.h), p2 = DF_MUL(-x2.h, y2.h);
+  const float e1 = DF_FMA(-x1.h, y1.h, -p1), e2 = DF_FMA(-x2.h, y2.h, -p2);
+  float c = DF_FMA(-x1.h, y1.l, e1);
+  c = DF_FMA(-x1.l, y1.h, c);
+  float d = DF_FMA(-x2.h, y2.l, e2);
+  d = DF_FMA(-x2.l, y2.h, d);
+  const df t1 = two_sum(a.h, p1);
+  const df t2 = two_sum(t1.h, p2);
+  return df_make(t2.h, DF_ADD(DF_ADD(DF_ADD(a.l, t1.l), DF_ADD(c, d)), t2.l));
+}
+__device__ __forceinline__ void sub_mulc(cdf& a, cdf x, cdf y) {
+  a.re = df_sub2(a.re, x.re, y.re, x.im, y.im);
+  a.im = df_sub2(a.im, x.im, y.re, df_neg(x.re), y.im);
+}
+__device__ __forceinline__ cdf renorm(cdf a) {
+  return cdf_make(fast_two_sum(a.re.h, a.re.l), fast_two_sum(a.im.h, a.im.l));
 }
 
 // One output per thread of an R x C block (R C = 256): returns A[orow][ocol] - sum_k X[r][k] conj(Y[c][k])
 // with X = rows xrow0.., Y = rows yrow0.. of A over columns k0..k0+31.
 template <int R, int C>
 __device__ __forceinline__ cdf upd_one(const float4* A, int N, int xrow0, int yrow0, int k0,
-                                       int orow, int ocol, bool ok, unsigned char* smem) {
+                                       int orow, int ocol, bool ok, unsigned char* smem, const Grp& g) {
   df(*Xp)[R][NB] = (df(*)[R][NB])smem;                        // [3][R][32]
   df(*Yp)[NB][C] = (df(*)[NB][C])(smem + 3 * R * NB * 8);     // [3][32][C]
   const cdf a = ok ? ldcg4(A + (size_t)orow * N + ocol) : czero();   // issued first, used last
-  for (int e = threadIdx.x; e < R * NB; e += CS_THREADS) {
+  for (int e = g.tid; e < R * NB; e += CS_THREADS) {
     const int r = e / NB, k = e % NB;
     cdf x = czero();
     if (xrow0 + r < N && k0 + k < N) x = ldcg4(A + (size_t)(xrow0 + r) * N + k0 + k);
@@ -211,7 +257,7 @@ __device__ __forceinline__ cdf upd_one(const float4* A, int N, int xrow0, int yr
     Xp[1][r][k] = x.im;
     Xp[2][r][k] = df_add_sloppy(x.re, x.im);
   }
-  for (int e = threadIdx.x; e < C * NB; e += CS_THREADS) {
+  for (int e = g.tid; e < C * NB; e += CS_THREADS) {
     const int k = e / C, c = e % C;
     cdf y = czero();
     if (yrow0 + c < N && k0 + k < N) y = ldcg4(A + (size_t)(yrow0 + c) * N + k0 + k);
@@ -219,8 +265,8 @@ __device__ __forceinline__ cdf upd_one(const float4* A, int N, int xrow0, int yr
     Yp[1][k][c] = y.im;
     Yp[2][k][c] = df_add_sloppy(y.re, df_neg(y.im));
   }
-  __syncthreads();
-  const int r = threadIdx.x / C, c = threadIdx.x % C;
+  g.sync();
+  const int r = g.tid / C, c = g.tid % C;
   acc2 p1 = acc_zero(), p2 = acc_zero(), p3 = acc_zero();
 #pragma unroll 8
   for (int k = 0; k < NB; ++k) {
@@ -228,17 +274,50 @@ __device__ __forceinline__ cdf upd_one(const float4* A, int N, int xrow0, int yr
     acc_prod_df(p2, Xp[1][r][k], Yp[1][k][c]);
     acc_prod_df(p3, Xp[2][r][k], Yp[2][k][c]);
   }
-  __syncthreads();
+  g.sync();
   return cdf_sub(a, kara_val(p1, p2, p3));
+}
+
+// 8 x 8 block (rb, cb), cb <= rb < 4, of diagonal block jp: A -= L_jp,jb L_jp,jb^H.  Each output's 32
+// products are split over four lanes (8 each), whose sums meet by shuffles: the update sits on the
+// factorisation's dependency chain, and ten such tasks take 2.5 us where three 16 x 16 ones took 4.
+__device__ __forceinline__ void diag_update8(float4* A, int N, int jp, int jb, int rb, int cb, unsigned char* smem, const Grp& g) {
+  cdf(*X)[NB + 1] = (cdf(*)[NB + 1])smem;                          // [8][33]
+  cdf(*Y)[NB + 1] = (cdf(*)[NB + 1])(smem + 8 * (NB + 1) * 16);    // [8][33]
+  const int r0 = jp * NB + rb * 8, c0 = jp * NB + cb * 8;
+  {
+    const int r = g.tid >> 5, k = g.tid & 31;
+    X[r][k] = r0 + r < N ? ldcg4(A + (size_t)(r0 + r) * N + jb * NB + k) : czero();
+    Y[r][k] = c0 + r < N ? ldcg4(A + (size_t)(c0 + r) * N + jb * NB + k) : czero();
+  }
+  const int o = g.tid >> 2, q = g.tid & 3, r = o >> 3, c = o & 7;
+  const int gr = r0 + r, gc = c0 + c;
+  const bool ok = gr < N && gc < N && gc <= gr;
+  const cdf a = ok && q == 0 ? ldcg4(A + (size_t)gr * N + gc) : czero();
+  g.sync();
+  cdf s = a;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) sub_mulc(s, X[r][q + 4 * k], Y[c][q + 4 * k]);
+  s = renorm(s);
+#pragma unroll
+  for (int off = 1; off < 4; off <<= 1) {
+    cdf t;
+    t.re.h = __shfl_xor_sync(0xffffffffu, s.re.h, off);
+    t.re.l = __shfl_xor_sync(0xffffffffu, s.re.l, off);
+    t.im.h = __shfl_xor_sync(0xffffffffu, s.im.h, off);
+    t.im.l = __shfl_xor_sync(0xffffffffu, s.im.l, off);
+    s = cdf_make(df_add_sloppy(s.re, t.re), df_add_sloppy(s.im, t.im));
+  }
+  if (ok && q == 0) A[(size_t)gr * N + gc] = st4(s);
 }
 
 // Trailing tile (rb, cb), cb <= rb: A_rc -= L_r,jb L_c,jb^H, 2 x 2 outputs per thread.
 __device__ __forceinline__ void herk_tile(float4* A, int N, int jb, int rb, int cb,
-                                          unsigned char* smem) {
+                                          unsigned char* smem, const Grp& g) {
   df(*Rp)[NB][NB] = (df(*)[NB][NB])smem;                      // [plane][row][k]
   df(*Cp)[NB][NB] = (df(*)[NB][NB])(smem + 3 * NB * NB * 8);  // [plane][k][col]
   const int k0 = jb * NB;
-  for (int e = threadIdx.x; e < NB * NB; e += CS_THREADS) {
+  for (int e = g.tid; e < NB * NB; e += CS_THREADS) {
     const int r = e / NB, m = e % NB;
     cdf a = czero();
     if (rb * NB + r < N && k0 + m < N) a = ldcg4(A + (size_t)(rb * NB + r) * N + k0 + m);
@@ -253,8 +332,8 @@ __device__ __forceinline__ void herk_tile(float4* A, int N, int jb, int rb, int 
     Cp[1][m2][r2] = b.im;
     Cp[2][m2][r2] = df_add_sloppy(b.re, df_neg(b.im));
   }
-  __syncthreads();
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  g.sync();
+  const int tx = g.tid & 15, ty = g.tid >> 4;
   acc2 acc[3][2][2];
 #pragma unroll
   for (int p = 0; p < 3; ++p)
@@ -287,124 +366,120 @@ __device__ __forceinline__ void herk_tile(float4* A, int N, int jb, int rb, int 
 }
 
 // Factor diagonal block jp in place: L L^H = A_jp,jp (lower triangle), reciprocal pivots to inv.
-// Warp 7 runs the pivot chain: at step s it takes column s+1 as left by step s-1 (all columns up to
-// s-1 applied), applies column s itself, forms the pivot d = a_{s+1,s+1}, y = 1/sqrt(d) (one
-// refinement step) and publishes l_{.,s+1} = a_{.,s+1} y.  Warps 0..6 own the entries of columns
-// >= 2 in column-descending order, so the entries that step s must update (columns >= s+2) are a
-// prefix of that order and idle warps skip the step; each entry keeps A and a compensated
-// accumulator of sum_k l_rk conj(l_qk) in registers, and the entries of column s+2 hand their
-// value to the pivot warp through a double-buffered shared-memory row.  One barrier per column.
-constexpr int PW_BULK = 7 * 32;
-constexpr int PW_PAIRS = (NB - 2) * (NB - 1) / 2;                  // entries of columns 2..31
-constexpr int PW_SLOTS = (PW_PAIRS + PW_BULK - 1) / PW_BULK;
+// Warp w owns columns 4w .. 4w + 3 in registers, lane = row, and the columns flow through shared
+// memory without a barrier: a warp subtracts column k's products as soon as flag k is up, then factors
+// its own four columns (pivot by shuffle, y = 1/sqrt(d) with one refinement step, scaling, the next
+// columns updated by shuffles), raises their flags, writes them out and sets its bit of *done, so that
+// the slabs below follow the factor column by column.
+// What bounds it is the pivots' dependency chain (shuffle, reciprocal square root, scaling, hand-over,
+// update; about 300 cycles each).  With a barrier and a hand-over per pivot, and a column's updates
+// spread over all warps, the block took 14 us; with a panel of 8 columns in one warp 14.6 (its 230
+// instructions per pivot, not their latency).
+constexpr int PB = 4;                       // columns per warp
+__device__ __forceinline__ void flag_wait(const volatile int* f, int* status) {
+  int it = 0;
+  while (!*f && ++it < (1 << 20)) {
+  }
+  if (it == (1 << 20)) set_flag(status, ST_TIMEOUT);
+  __threadfence_block();
+}
 
-__device__ __forceinline__ void potrf_task(int N, float4* A, float2* inv, int jp, int* status,
-                                           unsigned char* smem) {
-  cdf* col = (cdf*)smem;                   // col[c * 32 + r] = l_rc, r >= c
-  cdf* pend = col + NB * NB;               // [2][32]: column handed to the pivot warp
-  df* yv = (df*)(pend + 2 * NB);           // 1 / sqrt(d_c)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = jp * NB;
+// columns c0 + J .. c0 + 3 (lane = row); L[c * 32 + r] and flag[c] receive the finished ones
+template <int J>
+__device__ __forceinline__ void panel_steps(cdf (&a)[PB], df (&y)[PB], int c0, cdf* L, volatile int* flag, bool& bad) {
+  const int lane = threadIdx.x & 31, c = c0 + J;
+  const cdf v = renorm(a[J]);
+  df d;
+  d.h = __shfl_sync(0xffffffffu, v.re.h, c);
+  d.l = __shfl_sync(0xffffffffu, v.re.l, c);
+  const bool ok = d.h > 0.f;
+  bad = bad || !ok;
+  d = ok ? d : df_make(1.f, 0.f);
+  y[J] = df_rsqrt1(d);
+  cdf l = cdf_scale(v, y[J]);
+  l = lane == c ? cdf_make(df_mul(d, y[J]), df_make(0.f, 0.f)) : l;
+  l = lane < c ? czero() : l;
+  L[c * NB + lane] = l;
+  __syncwarp();
+  if (lane == 0) {
+    __threadfence_block();
+    flag[c] = 1;
+  }
+  a[J] = l;
+  if constexpr (J + 1 < PB) {
+#pragma unroll
+    for (int q = J + 1; q < PB; ++q) sub_mulc(a[q], l, shfl_cdf(l, c0 + q));
+    panel_steps<J + 1>(a, y, c0, L, flag, bad);
+  }
+}
+
+__device__ __forceinline__ void potrf_task(int N, float4* A, float2* inv, int jp, int* status, unsigned* done,
+                                           unsigned char* smem, const Grp& g) {
+  cdf* L = (cdf*)smem;                       // L[c * 32 + r]
+  volatile int* flag = (volatile int*)(L + NB * NB);
+  const int warp = g.tid >> 5, lane = g.tid & 31;
+  const int r0 = jp * NB, c0 = warp * PB;
   const df zero = df_make(0.f, 0.f), one = df_make(1.f, 0.f);
-  auto load = [&](int r, int q) -> cdf {
-    if (r0 + r < N) return ldcg4(A + (size_t)(r0 + r) * N + r0 + q);
-    return cdf_make(r == q ? one : zero, zero);
-  };
-  if (warp == 7) {
-    // pivot warp: columns 0 and 1 straight from A
-    const cdf a0 = load(lane, 0);
-    cdf a1 = lane >= 1 ? load(lane, 1) : czero();
-    df d;
-    d.h = __shfl_sync(0xffffffffu, a0.re.h, 0);
-    d.l = __shfl_sync(0xffffffffu, a0.re.l, 0);
-    if (!(d.h > 0.f)) {
-      if (lane == 0) set_flag(status, ST_CHOL);
-      d = one;
-    }
-    const df y = df_rsqrt1(d);
-    col[lane] = lane == 0 ? cdf_make(df_mul(d, y), zero) : cdf_scale(a0, y);
-    if (lane == 0) yv[0] = y;
-    pend[NB + lane] = a1;                  // column 1, nothing applied yet (parity 1)
-  }
-  // bulk entries: column-descending order over columns 31..2, column q holds rows q..31
-  int er[PW_SLOTS], eq[PW_SLOTS];
-  cdf av[PW_SLOTS];
-  cacc acc[PW_SLOTS];
+  cdf a[PB];
 #pragma unroll
-  for (int i = 0; i < PW_SLOTS; ++i) {
-    int e = threadIdx.x + i * PW_BULK, q = NB - 1;
-    while (q > 2 && e >= NB - q) { e -= NB - q; --q; }
-    const bool on = warp < 7 && threadIdx.x + i * PW_BULK < PW_PAIRS;
-    er[i] = on ? q + e : -1;
-    eq[i] = q;
-    av[i] = on ? load(q + e, q) : czero();
-    acc[i] = cacc_zero();
+  for (int j = 0; j < PB; ++j) {
+    a[j] = cdf_make(lane == c0 + j ? one : zero, zero);   // rows past the matrix: identity
+    if (lane >= c0 + j && r0 + lane < N) a[j] = ldcg4(A + (size_t)(r0 + lane) * N + r0 + c0 + j);
   }
-  __syncthreads();
-  for (int s = 0; s < NB - 1; ++s) {
-    if (warp == 7) {
-      // column s+1: v = (value through column s-1) - l_{r,s} conj(l_{s+1,s}), then its pivot
-      const int c = s + 1;
-      const cdf w = pend[(c & 1) * NB + lane];
-      const cdf lr = col[s * NB + lane];
-      const cdf lq = col[s * NB + c];
-      const cdf v = cdf_sub_sloppy(w, cdf_mul_conj(lr, lq));
-      df d;
-      d.h = __shfl_sync(0xffffffffu, v.re.h, c);
-      d.l = __shfl_sync(0xffffffffu, v.re.l, c);
-      if (!(d.h > 0.f)) {
-        if (lane == 0) set_flag(status, ST_CHOL);
-        d = one;
-      }
-      const df y = df_rsqrt1(d);
-      if (lane > c) col[c * NB + lane] = cdf_scale(v, y);
-      else if (lane == c) col[c * NB + c] = cdf_make(df_mul(d, y), zero);
-      if (lane == 0) yv[c] = y;
-    } else if (warp * 32 < (NB - 2 - s) * (NB - 1 - s) / 2) {
-      // entries of columns >= s+2 (the first (30-s)(31-s)/2 of the order) take column s
-      const int nact = (NB - 2 - s) * (NB - 1 - s) / 2;
-      const cdf* cs = col + s * NB;
+  g.sync();                                  // the previous block's columns have been read
+  if (g.tid < NB) flag[g.tid] = 0;
+  g.sync();
+  // all but the last earlier column; that one joins the warp's own (its products for the first own
+  // column are the ones on the chain, the others fill the pivot's latency)
+#pragma unroll 1
+  for (int k = 0; k + 1 < c0; ++k) {
+    flag_wait(flag + k, status);
+    const cdf lr = L[k * NB + lane];
 #pragma unroll
-      for (int i = 0; i < PW_SLOTS; ++i) {
-        if (threadIdx.x + i * PW_BULK < nact) {
-          const int r = er[i], q = eq[i];
-          cacc_mulc(acc[i], cs[r], cs[q]);
-          if (q == s + 2) pend[(q & 1) * NB + r] = cdf_sub_sloppy(av[i], cacc_val(acc[i]));
-        }
-      }
-    }
-    __syncthreads();
+    for (int j = 0; j < PB; ++j) sub_mulc(a[j], lr, L[k * NB + c0 + j]);
   }
-  for (int e = threadIdx.x; e < NB * NB; e += CS_THREADS) {
-    const int q = e / NB, r = e % NB;
-    if (r >= q && r0 + r < N) A[(size_t)(r0 + r) * N + r0 + q] = st4(col[q * NB + r]);
+  if (c0 > 0) {
+    flag_wait(flag + c0 - 1, status);
+    const cdf lr = L[(c0 - 1) * NB + lane];
+#pragma unroll
+    for (int j = 0; j < PB; ++j) sub_mulc(a[j], lr, L[(c0 - 1) * NB + c0 + j]);
   }
-  if (threadIdx.x < NB && r0 + threadIdx.x < N)
-    inv[r0 + threadIdx.x] = make_float2(yv[threadIdx.x].h, yv[threadIdx.x].l);
+  df y[PB];
+  bool bad = false;
+  panel_steps<0>(a, y, c0, L, flag, bad);
+#pragma unroll
+  for (int j = 0; j < PB; ++j) {
+    if (lane >= c0 + j && r0 + lane < N) A[(size_t)(r0 + lane) * N + r0 + c0 + j] = st4(a[j]);
+    if (lane == 0 && r0 + c0 + j < N) inv[r0 + c0 + j] = make_float2(y[j].h, y[j].l);
+  }
+  if (bad && lane == 0) set_flag(status, ST_CHOL);
+  __threadfence();
+  __syncwarp();
+  if (lane == 0) atomicOr(done, 1u << warp);
 }
 
 // D = L^{-1} of diagonal block jp (final), by 2 x 2 blocks of 16:
 //   D11 = L11^{-1}, D22 = L22^{-1} (forward substitution of the unit vectors, one column per
 //   half-warp, compensated accumulation), then D21 = -D22 (L21 D11) as two 16 x 16 products.
 __device__ __forceinline__ void trtri_task(int N, const float4* A, const float2* inv, float4* D,
-                                           int jp, unsigned char* smem) {
+                                           int jp, unsigned char* smem, const Grp& g) {
   constexpr int H = NB / 2;
   cdf(*Ls)[NB + 1] = (cdf(*)[NB + 1])smem;                                  // [32][33]
   cdf(*Ds)[NB + 1] = (cdf(*)[NB + 1])(smem + NB * (NB + 1) * 16);           // [32][33]
   cdf(*Ts)[H + 1] = (cdf(*)[H + 1])(smem + 2 * NB * (NB + 1) * 16);         // [16][17]
   df* ys = (df*)(smem + 2 * NB * (NB + 1) * 16 + H * (H + 1) * 16);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = g.tid >> 5, lane = g.tid & 31;
   const int r0 = jp * NB;
   const df zero = df_make(0.f, 0.f), one = df_make(1.f, 0.f);
-  for (int e = threadIdx.x; e < NB * NB; e += CS_THREADS) {
+  for (int e = g.tid; e < NB * NB; e += CS_THREADS) {
     const int r = e / NB, c = e % NB;
     Ls[r][c] = (c < r && r0 + r < N) ? ldcg4(A + (size_t)(r0 + r) * N + r0 + c) : czero();
   }
-  if (threadIdx.x < NB) {
-    const float2 v = r0 + threadIdx.x < N ? __ldcg(inv + r0 + threadIdx.x) : make_float2(1.f, 0.f);
-    ys[threadIdx.x] = df_make(v.x, v.y);
+  if (g.tid < NB) {
+    const float2 v = r0 + g.tid < N ? __ldcg(inv + r0 + g.tid) : make_float2(1.f, 0.f);
+    ys[g.tid] = df_make(v.x, v.y);
   }
-  __syncthreads();
+  g.sync();
   // the 32 unit-vector solves (block b, column j) in two passes of 16 half-warps; rows above j
   // come out as zero by themselves (right-hand side and accumulator are zero there)
   const int hl = lane & (H - 1);
@@ -427,204 +502,231 @@ __device__ __forceinline__ void trtri_task(int N, const float4* A, const float2*
     Ds[o + hl][o + j] = dv;
     Ds[o + hl][H - o + j] = czero();      // the other 16 columns of these rows: D12 = 0 / D21 later
   }
-  __syncthreads();
+  g.sync();
   // T = L21 D11, then D21 = -D22 T
-  const int r = threadIdx.x / H, c = threadIdx.x % H;
+  const int r = g.tid / H, c = g.tid % H;
   cacc t = cacc_zero();
 #pragma unroll 4
   for (int m = 0; m < H; ++m) cacc_mul(t, Ls[H + r][m], Ds[m][c]);
   Ts[r][c] = cacc_val(t);
-  __syncthreads();
+  g.sync();
   cacc u = cacc_zero();
 #pragma unroll 4
   for (int m = 0; m < H; ++m) cacc_mul(u, Ds[H + r][H + m], Ts[m][c]);
   const cdf d21 = cacc_val(u);
   Ds[H + r][c] = cdf_make(df_neg(d21.re), df_neg(d21.im));
-  __syncthreads();
-  for (int e = threadIdx.x; e < NB * NB; e += CS_THREADS) {
+  g.sync();
+  for (int e = g.tid; e < NB * NB; e += CS_THREADS) {
     const int rr = e / NB, cc = e % NB;
     if (r0 + rr < N) D[((size_t)jp * NB + rr) * NB + cc] = st4(Ds[rr][cc]);
   }
 }
 
-// Control words of one factorisation call (zeroed before its first launch), per matrix m:
-//   ctl[li]                          ticket counter of launch li
-//   diag  [li][m]  at (T+2) + 2 li   finished quadrant updates of diagonal block li
-//   pdone [li][m]  at 3(T+2) + 2 li  diagonal factor of block li published
-//   slabdone[m][l][b]                finished 8-row panel slabs of launch l in row block b
+// Control words of one factorisation (zeroed before its launch), per matrix m:
+//   ticket, role                     counters of the worker tasks and of the CTAs
+//   diag  [li][m]                    finished 8 x 8 updates of diagonal block li
+//   pdone [li][m]                    bit w: columns 4w.. of diagonal factor li published
+//   slabdone[m][l][b]                finished 8-row panel slabs of block column l in row block b
 //   tilecnt [m][r][c]                trailing updates applied to tile (r, c)
-// Tasks wait (bounded) on these rather than on the end of the previous launch, so the chain of
-// block column li + 1 (quadrants -> diagonal factor -> panel) overlaps the trailing updates of
-// launch li.
 struct CholCtl {
-  unsigned *slabdone, *tilecnt;
+  unsigned* w;
   int T, N;
-  __device__ unsigned* sd(int m, int l, int b) const { return slabdone + ((size_t)m * (T + 1) + l) * T + b; }
-  __device__ unsigned* tc(int m, int r, int c) const { return tilecnt + ((size_t)m * T + r) * T + c; }
+  __device__ CholCtl(unsigned* ctl, int n) : w(ctl), T((n + NB - 1) / NB), N(n) {}
+  __device__ unsigned* ticket() const { return w; }
+  __device__ unsigned* role() const { return w + 1; }
+  __device__ unsigned* diag(int li, int m) const { return w + (T + 2) + 2 * li + m; }
+  __device__ unsigned* pdone(int li, int m) const { return w + 3 * (T + 2) + 2 * li + m; }
+  __device__ unsigned* sd(int m, int l, int b) const { return w + 5 * (T + 2) + ((size_t)m * (T + 1) + l) * T + b; }
+  __device__ unsigned* tc(int m, int r, int c) const {
+    return w + 5 * (T + 2) + 2 * (size_t)(T + 1) * T + ((size_t)m * T + r) * T + c;
+  }
   __device__ unsigned slabs_in(int b) const {
     const int rows = N - b * NB < NB ? N - b * NB : NB;
     return (unsigned)((rows + TS_ROWS - 1) / TS_ROWS);
   }
 };
 
-// thread 0 waits (bounded) until *f >= target, then fences; the caller synchronises the CTA
-__device__ __forceinline__ void wait_count(const unsigned* f, unsigned target, int* status) {
-  if (threadIdx.x == 0 && target > 0) {
+// column c is one of the eight from k0
+constexpr int SB = 8;   // columns a slab takes at a time
+__device__ __forceinline__ bool lane_of(int c, int k0) { return (c & ~(SB - 1)) == k0; }
+
+// threads 0..2 wait (bounded) for one control word each, then fence; the caller synchronises the group
+__device__ __forceinline__ void wait_counts(const Grp& g, const unsigned* f0, unsigned t0, const unsigned* f1,
+                                            unsigned t1, const unsigned* f2, unsigned t2, int* status) {
+  if (g.tid < 3) {
+    const unsigned* f = g.tid == 0 ? f0 : (g.tid == 1 ? f1 : f2);
+    const unsigned t = g.tid == 0 ? t0 : (g.tid == 1 ? t1 : t2);
+    if (t > 0) {
+      cs_wait(f, t, status);
+      __threadfence();
+    }
+  }
+}
+// thread 0 waits (bounded) until *f >= target, then fences; the caller synchronises the group
+__device__ __forceinline__ void wait_count(const Grp& g, const unsigned* f, unsigned target, int* status) {
+  if (g.tid == 0 && target > 0) {
     cs_wait(f, target, status);
     __threadfence();
   }
 }
 
-__device__ __forceinline__ void chol_task(int N, Batch mb, int nb, int li, unsigned* ctl,
-                                          int* status) {
-  extern __shared__ __align__(16) unsigned char sm[];
-  __shared__ unsigned s_t;
-  const int T = (N + NB - 1) / NB;
+// Tasks of block column li besides its diagonal factor, per matrix.
+struct StepTasks {
+  int diag, herk, slab, inv;
+  __host__ __device__ StepTasks(int N, int li) {
+    const int T = (N + NB - 1) / NB, rt = T - li - 1, rows = N - (li + 1) * NB;
+    diag = (li > 0 && li < T) ? DIAG_TASKS : 0;
+    herk = (li > 0 && rt > 0) ? rt * (rt + 1) / 2 : 0;
+    slab = (li < T && rows > 0) ? (rows + TS_ROWS - 1) / TS_ROWS : 0;
+    inv = li > 0 ? 1 : 0;
+  }
+  __host__ __device__ int count() const { return diag + herk + slab + inv; }
+};
+
+// Task t of block column li (all matrices).
+__device__ __forceinline__ void chol_task(const Grp& g, int N, const Batch& mb, int nb, int li, int t, const StepTasks& st,
+                                          const CholCtl& cc, int* status, unsigned char* sm) {
   const int jp = li, jb = li - 1;
-  unsigned* diag = ctl + (T + 2) + 2 * li;     // [li][matrix]: finished quadrants
-  unsigned* pdone = ctl + 3 * (T + 2) + 2 * li;  // [li][matrix]: diagonal factor published
-  CholCtl cc;
-  cc.slabdone = ctl + 5 * (T + 2);
-  cc.tilecnt = cc.slabdone + 2 * (size_t)(T + 1) * T;
-  cc.T = T;
-  cc.N = N;
-  if (threadIdx.x == 0) s_t = atomicAdd(ctl + li, 1u);
-  __syncthreads();
-  int t = (int)s_t;
-  const int ndiag = (jb >= 0 && jp < T) ? 3 : 0;
-  const int rt = T - jb - 2;
-  const int nherk = (jb >= 0 && rt > 0) ? rt * (rt + 1) / 2 : 0;
-  const int rows = N - (jp + 1) * NB;
-  const int nslab = (jp < T && rows > 0) ? (rows + TS_ROWS - 1) / TS_ROWS : 0;
-  if (t < nb * ndiag) {
-    // quadrant (rh, ch) of diagonal block jp: A -= L_jp,jb L_jp,jb^H; needs panel jb on the rows
+  if (t < nb * st.diag) {
+    // 8 x 8 block (rb, cb) of diagonal block jp: A -= L_jp,jb L_jp,jb^H; needs panel jb on the rows
     // of block jp and the jb earlier trailing updates of the diagonal tile
-    const int m = t % nb, qd = t / nb;
-    const int rh = qd > 0 ? 1 : 0, ch = qd > 1 ? 1 : 0;
-    wait_count(cc.sd(m, jb, jp), cc.slabs_in(jp), status);
-    wait_count(cc.tc(m, jp, jp), (unsigned)jb, status);
-    __syncthreads();
-    float4* A = pick2(mb.m, m);
-    const int r = threadIdx.x / 16, c = threadIdx.x % 16;
-    const int orow = jp * NB + rh * 16 + r, ocol = jp * NB + ch * 16 + c;
-    const bool ok = orow < N && ocol < N && (rh != ch || c <= r);
-    const cdf v = upd_one<16, 16>(A, N, jp * NB + rh * 16, jp * NB + ch * 16, jb * NB, orow, ocol,
-                                  ok, sm);
-    if (ok) A[(size_t)orow * N + ocol] = st4(v);
-    cs_signal(diag + m);
-    return;
-  }
-  t -= nb * ndiag;
-  const int npotrf = jp < T ? 1 : 0;
-  if (t < nb * npotrf) {
-    const int m = t;
-    if (ndiag > 0) {
-      if (threadIdx.x == 0) {
-        cs_wait(diag + m, 3u, status);
-        __threadfence();
-      }
-      __syncthreads();
-    }
-    potrf_task(N, pick2(mb.m, m), pick2(mb.inv, m), jp, status, sm);
-    cs_signal(pdone + m);
-    return;
-  }
-  t -= nb * npotrf;
-  const int ntrtri = jp >= 1 ? 1 : 0;
-  if (t < nb * ntrtri) {
-    // inverse of the previous diagonal block (final once its factor is published), for the solves
-    const int m = t;
-    wait_count(ctl + 3 * (T + 2) + 2 * (li - 1) + m, 1u, status);
-    __syncthreads();
-    trtri_task(N, pick2(mb.m, m), pick2(mb.inv, m), pick2(mb.D, m), jp - 1, sm);
-    return;
-  }
-  t -= nb * ntrtri;
-  if (t < nb * nherk) {
     const int m = t % nb;
-    int I, J;
-    tri_index(t / nb, I, J);
-    const int rb = jb + 2 + J, cb = jb + 2 + I;
-    // panel jb on both row blocks, and the tile's jb - 1 earlier updates
-    wait_count(cc.sd(m, jb, rb), cc.slabs_in(rb), status);
-    wait_count(cc.sd(m, jb, cb), cc.slabs_in(cb), status);
-    wait_count(cc.tc(m, rb, cb), (unsigned)(jb > 0 ? jb : 0), status);
-    __syncthreads();
-    herk_tile(pick2(mb.m, m), N, jb, rb, cb, sm);
-    cs_signal(cc.tc(m, rb, cb));
+    int cb, rb;
+    tri_index(t / nb, cb, rb);
+    wait_counts(g, cc.sd(m, jb, jp), cc.slabs_in(jp), cc.tc(m, jp, jp), (unsigned)jb, nullptr, 0, status);
+    g.sync();
+    diag_update8(pick2(mb.m, m), N, jp, jb, rb, cb, sm, g);
+    cs_signal(g, cc.diag(li, m));
     return;
   }
-  t -= nb * nherk;
-  if (t < nb * nslab) {
+  t -= nb * st.diag;
+  // trailing tiles, the slabs after the first AHEAD_TILES of them
+  const int ahead = nb * st.herk < AHEAD_TILES ? nb * st.herk : AHEAD_TILES;
+  const bool slab = t >= ahead && t < ahead + nb * st.slab;
+  if (t < nb * (st.herk + st.slab) && !slab) {
+    if (t >= ahead) t -= nb * st.slab;
+    const int m = t % nb;
+    // block columns from the left (the next steps need them first), rows from the diagonal
+    int I, J;
+    tri_index(st.herk - 1 - t / nb, I, J);
+    const int rb = cc.T - 1 - I, cb = cc.T - 1 - J;
+    // panel jb on both row blocks, and the tile's jb - 1 earlier updates
+    wait_counts(g, cc.sd(m, jb, rb), cc.slabs_in(rb), cc.sd(m, jb, cb), cc.slabs_in(cb), cc.tc(m, rb, cb),
+                (unsigned)(jb > 0 ? jb : 0), status);
+    g.sync();
+    herk_tile(pick2(mb.m, m), N, jb, rb, cb, sm, g);
+    cs_signal(g, cc.tc(m, rb, cb));
+    return;
+  }
+  if (slab) {
     // panel slab: rows i0..i0+7 of block column jp.  a = A - L_i,jb L_jp,jb^H, then x L^H = a by
     // substitution along the row (warp = row, lane = column): x_m = (a_m - sum_k<m x_k conj(L_mk)) / L_mm
+    t -= ahead;
     const int m = t % nb, sl = t / nb;
     float4* A = pick2(mb.m, m);
     const float2* inv = pick2(mb.inv, m);
     const int i0 = (jp + 1) * NB + sl * TS_ROWS;
-    const int r = threadIdx.x / NB, c = threadIdx.x % NB;
+    const int r = g.tid / NB, c = g.tid % NB;
     const bool ok = i0 + r < N;
     const int bi = i0 / NB;
     if (jb >= 0) {
       // panel jb on these rows and on the rows of block jp, and the tile's jb earlier updates
-      wait_count(cc.sd(m, jb, bi), cc.slabs_in(bi), status);
-      wait_count(cc.sd(m, jb, jp), cc.slabs_in(jp), status);
-      wait_count(cc.tc(m, bi, jp), (unsigned)jb, status);
-      __syncthreads();
+      wait_counts(g, cc.sd(m, jb, bi), cc.slabs_in(bi), cc.sd(m, jb, jp), cc.slabs_in(jp), cc.tc(m, bi, jp),
+                  (unsigned)jb, status);
+      g.sync();
     }
     cdf a;
-    if (jb >= 0) a = upd_one<TS_ROWS, NB>(A, N, i0, jp * NB, jb * NB, i0 + r, jp * NB + c, ok, sm);
+    if (jb >= 0) a = upd_one<TS_ROWS, NB>(A, N, i0, jp * NB, jb * NB, i0 + r, jp * NB + c, ok, sm, g);
     else a = ok ? ldcg4(A + (size_t)(i0 + r) * N + jp * NB + c) : czero();
-    if (threadIdx.x == 0) {
-      cs_wait(pdone + m, 1u, status);
-      __threadfence();
-    }
-    __syncthreads();
-    // with L' = L diag(y) (y_k = 1 / L_kk) and x = z diag(y): z_k = a_k - sum_j<k z_j conj(L'_kj),
-    // so the chain carries no scaling; L' is formed while staging the block
-    cdf(*Ls)[NB + 1] = (cdf(*)[NB + 1])sm;                      // [32][33]
-    df* ys = (df*)(sm + NB * (NB + 1) * 16);
-    if (threadIdx.x < NB) {
-      const float2 v = __ldcg(inv + jp * NB + threadIdx.x);
-      ys[threadIdx.x] = df_make(v.x, v.y);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < NB * NB; e += CS_THREADS) {
-      const int rr = e / NB, cc = e % NB;
-      Ls[rr][cc] = cc < rr ? cdf_scale(ldcg4(A + (size_t)(jp * NB + rr) * N + jp * NB + cc), ys[cc])
-                           : czero();
-    }
-    __syncthreads();
-    cacc s = cacc_zero();
+    // with L' = L diag(y) (y_k = 1 / L_kk) and x = z diag(y): z_k = a_k - sum_j<k z_j conj(L'_kj), so
+    // the chain carries no scaling.  Eight columns at a time, as the diagonal factor publishes them:
+    // only the last eight are left when it finishes.
     cdf z = czero();
-    cdf lnext = Ls[c][0];
-#pragma unroll 4
-    for (int k = 0; k < NB; ++k) {
-      const cdf lk = lnext;
-      if (k + 1 < NB) lnext = Ls[c][k + 1];   // next step's operand, off the chain
-      const cdf zk = shfl_cdf(cdf_sub_sloppy(a, cacc_val(s)), k);
-      if (c == k) z = zk;
-      if (c > k) cacc_mulc(s, zk, lk);
+    df yc = df_make(0.f, 0.f);
+#pragma unroll 1
+    for (int k0 = 0; k0 < NB; k0 += SB) {
+      if (g.tid == 0) {
+        cs_wait<true>(cc.pdone(li, m), (1u << ((k0 + SB) / PB)) - 1u, status);
+        __threadfence();
+      }
+      g.sync();
+      cdf lk[SB];
+      const float4* lp = A + (size_t)(jp * NB + c) * N + jp * NB + k0;
+      const float2 yv = lane_of(c, k0) ? __ldcg(inv + jp * NB + c) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < SB; ++k) lk[k] = k0 + k < c ? ldcg4(lp + k) : czero();
+      if (lane_of(c, k0)) yc = df_make(yv.x, yv.y);
+#pragma unroll
+      for (int k = 0; k < SB; ++k) {
+        df y;
+        y.h = __shfl_sync(0xffffffffu, yv.x, k0 + k);
+        y.l = __shfl_sync(0xffffffffu, yv.y, k0 + k);
+        lk[k] = cdf_scale(lk[k], y);
+      }
+#pragma unroll
+      for (int k = 0; k < SB; ++k) {
+        a = renorm(a);
+        const cdf zk = shfl_cdf(a, k0 + k);
+        if (c == k0 + k) z = zk;
+        sub_mulc(a, zk, lk[k]);   // lk = 0 for c <= k
+      }
     }
     if (ok) {
-      const cdf x = cdf_scale(z, ys[c]);
+      const cdf x = cdf_scale(z, yc);
       A[(size_t)(i0 + r) * N + jp * NB + c] = st4(x);
       // L^H in the (otherwise unused) upper triangle: the backward solve reads it by rows
       A[(size_t)(jp * NB + c) * N + i0 + r] = st4(cdf_make(x.re, df_neg(x.im)));
     }
-    cs_signal(cc.sd(m, li, bi));
+    cs_signal(g, cc.sd(m, li, bi));
+    return;
+  }
+  t -= nb * (st.herk + st.slab);
+  {
+    // inverse of the previous diagonal block (final once its factor is published), for the solves
+    const int m = t;
+    if (g.tid == 0) {
+      cs_wait<true>(cc.pdone(li - 1, m), (1u << (NB / PB)) - 1u, status);
+      __threadfence();
+    }
+    g.sync();
+    trtri_task(N, pick2(mb.m, m), pick2(mb.inv, m), pick2(mb.D, m), jp - 1, sm, g);
   }
 }
 
-__global__ void __launch_bounds__(CS_THREADS, 3) k_chol_step_df(int N, Batch mb, int nb, int li,
-                                                            unsigned* ctl, int* status) {
-  // programmatic dependent launch: the next block column's launch may become resident at once;
-  // its tasks wait on the control words for exactly the data they read
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  chol_task(N, mb, nb, li, ctl, status);
-  // the grid completes only after its predecessor has, so later work in the stream sees the whole
-  // factorisation
-  if (threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+__global__ void __launch_bounds__(CTA_THREADS, 1) k_chol_df(int N, Batch mb, int nb, unsigned* ctl, int* status) {
+  extern __shared__ __align__(16) unsigned char smem_all[];
+  __shared__ unsigned s_role, s_t[2];
+  const CholCtl cc(ctl, N);
+  if (threadIdx.x == 0) s_role = atomicAdd(cc.role(), 1u);
+  __syncthreads();
+  const int half = threadIdx.x / CS_THREADS;
+  const Grp g{(int)threadIdx.x % CS_THREADS, 1 + half};
+  unsigned char* sm = smem_all + half * CS_SMEM;
+  if ((int)s_role < nb) {
+    if (half) return;
+    const int m = (int)s_role;
+    for (int li = 0; li < cc.T; ++li) {
+      if (li > 0) wait_count(g, cc.diag(li, m), (unsigned)DIAG_TASKS, status);
+      g.sync();
+      potrf_task(N, pick2(mb.m, m), pick2(mb.inv, m), li, status, cc.pdone(li, m), sm, g);
+    }
+    return;
+  }
+  int li = 0;
+  unsigned base = 0;
+  StepTasks st(N, 0);
+  while (true) {
+    if (g.tid == 0) s_t[half] = atomicAdd(cc.ticket(), 1u);
+    g.sync();
+    const unsigned t = s_t[half];
+    g.sync();   // shared memory of the previous task and s_t are free after this
+    while (li <= cc.T && t - base >= (unsigned)(nb * st.count())) {
+      base += nb * st.count();
+      st = StepTasks(N, ++li);
+    }
+    if (li > cc.T) return;
+    chol_task(g, N, mb, nb, li, (int)(t - base), st, cc, status, sm);
+  }
 }
 
 // ---------------------------------------------------------------------------- triangular solves
@@ -1162,35 +1264,21 @@ int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, 
     mb.D[q] = (float4*)D[k];
   }
   const int T = (N + NB - 1) / NB;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_chol_step_df, cudaFuncAttributeMaxDynamicSharedMemorySize, CS_SMEM_LAUNCH);
-    attr = true;
-  }
+  static std::once_flag once;
+  static int sms = 0;
+  std::call_once(once, [] {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaFuncSetAttribute(k_chol_df, cudaFuncAttributeMaxDynamicSharedMemorySize, CS_SMEM_LAUNCH);
+  });
   cudaMemsetAsync(ctl, 0, chol_ctl_words(N) * sizeof(unsigned), s);
-  // launches 1.. are programmatic dependents of the previous one (the kernel waits on
-  // griddepcontrol before touching data), so a launch's CTAs are resident when its predecessor
-  // ends instead of paying the launch latency on the factorisation's critical path
-  cudaLaunchAttribute pdl[1];
-  pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  pdl[0].val.programmaticStreamSerializationAllowed = 1;
-  for (int li = 0; li <= T; ++li) {
-    const int jb = li - 1;
-    const int rt = T - jb - 2;
-    const int nherk = (jb >= 0 && rt > 0) ? rt * (rt + 1) / 2 : 0;
-    const int rows = N - (li + 1) * NB;
-    const int nslab = (li < T && rows > 0) ? (rows + TS_ROWS - 1) / TS_ROWS : 0;
-    const int per = (jb >= 0 && li < T ? 3 : 0) + (li < T ? 1 : 0) + (li >= 1 ? 1 : 0) + nherk + nslab;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nbatch * per);
-    cfg.blockDim = dim3(CS_THREADS);
-    cfg.dynamicSmemBytes = CS_SMEM_LAUNCH;
-    cfg.stream = s;
-    cfg.attrs = pdl;
-    cfg.numAttrs = li > 0 ? 1 : 0;   // the first launch follows the memset in stream order
-    cudaLaunchKernelEx(&cfg, k_chol_step_df, N, mb, nbatch, li, ctl, status);
-  }
-  return T + 2;
+  // chain CTAs and two groups per worker CTA, no more workers than the widest step has tasks
+  int widest = 1;
+  for (int li = 0; li <= T; ++li) widest = std::max(widest, nbatch * StepTasks(N, li).count());
+  const int grid = std::min(std::max(sms, nbatch + 1), nbatch + (widest + 1) / 2);
+  k_chol_df<<<grid, CTA_THREADS, CS_SMEM_LAUNCH, s>>>(N, mb, nbatch, ctl, status);
+  return 1;
 }
 
 size_t chol_ctl_words(int N) {
