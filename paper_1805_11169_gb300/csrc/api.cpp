@@ -744,6 +744,7 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
   const size_t cw = h->cwf_elem, rw = h->mixed ? sizeof(float) : sizeof(double);
   const size_t NN = (size_t)N * N;
   const int nblk = (N + 31) / 32;
+  const size_t dl = h->df_solve ? diag_inv_bytes(N) : (size_t)N * 512;
   std::vector<size_t> sizes = {
       nV * sizeof(double), nV * rw, (size_t)K * nx * 8, (size_t)K * nR * 8, (size_t)K * 8,
       (size_t)nx * 8, (size_t)nR * 8,
@@ -755,7 +756,7 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
       (size_t)N * 8,       // C in FP32
       NN * 16 * 7,         // S[2], H[2], L[2], Lh
       (size_t)N * 8, (size_t)N * 8, (size_t)N * 8,   // reciprocal pivots of L[2], Lh
-      (size_t)N * 512, (size_t)N * 512, (size_t)N * 512,   // inverted diagonal blocks
+      dl, dl, dl,                                    // inverted diagonal blocks
       (size_t)2 * nblk * 4 + 64, chol_ctl_words(N) * sizeof(unsigned), 64 * 4};
   size_t total = 0;
   for (size_t b : sizes) total += align256(b);
@@ -810,9 +811,9 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
   h->invL[0] = (double*)a.take((size_t)N * 8);
   h->invL[1] = (double*)a.take((size_t)N * 8);
   h->invLh = (double*)a.take((size_t)N * 8);
-  h->DL[0] = (double2*)a.take((size_t)N * 512);
-  h->DL[1] = (double2*)a.take((size_t)N * 512);
-  h->DLh = (double2*)a.take((size_t)N * 512);
+  h->DL[0] = (double2*)a.take(dl);
+  h->DL[1] = (double2*)a.take(dl);
+  h->DLh = (double2*)a.take(dl);
   h->flags = (unsigned*)a.take((size_t)2 * nblk * 4 + 64);
   h->tickets = h->flags + 2 * nblk;
   h->cctl = (unsigned*)a.take(chol_ctl_words(N) * sizeof(unsigned));
@@ -1264,6 +1265,12 @@ icwf_status icwf_load_state(icwf_handle h, const void* buf, size_t bytes) {
   for (auto& r : state_regions(h)) {
     CK(cudaMemcpy(r.first, p, r.second, cudaMemcpyHostToDevice));
     p += r.second;
+  }
+  if (h->df_solve) {   // what the solves need beside the saved factor
+    CK(cudaStreamSynchronize(0));   // a copy from pageable memory may still be on its way
+    void *l = h->L[h->cur], *d = h->DL[h->cur];
+    launch_near_products(h->N, &l, &d, 1, h->stream);
+    CK(cudaGetLastError());
   }
   const int flags0 = 0;
   CK(cudaMemcpy(h->status + STATUS_FLAGS, &flags0, sizeof(int), cudaMemcpyHostToDevice));

@@ -194,6 +194,11 @@ void launch_shift_mix_df(int N, const double2* S0, const double2* S1, double eps
 int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, int nbatch,
                        unsigned* ctl, int* status, cudaStream_t s);
 size_t chol_ctl_words(int N);
+// Bytes of the D buffer of one matrix (double-float solver): the N x 32 inverted diagonal blocks, then
+// their products with the neighbouring blocks, which launch_cholesky_df and launch_near_products
+// (after a restored factor) compute.
+size_t diag_inv_bytes(int N);
+int launch_near_products(int N, void* const* L, void* const* D, int nbatch, cudaStream_t s);
 void launch_chol_solve_df(int N, const void* L, const void* D, const double2* y, void* work,
                           double2* out, bool minus_i, unsigned* flags, unsigned* tickets,
                           unsigned epoch, int* status, cudaStream_t s);
