@@ -229,13 +229,14 @@ icwf_status icwf_set_emulated_update(icwf_handle h, int32_t on);
 icwf_status icwf_set_step_graphs(icwf_handle h, int32_t on);
 
 /* Diagnostic: poll budget of the in-kernel spin waits on global flags (the look-ahead tickets of
- * the blocked Cholesky factorisation and the block flags of the triangular solves).  polls >= 0:
+ * the blocked Cholesky factorisation and the block flags of the triangular solves above N = 2048).  polls >= 0:
  * such a wait gives up after that many polls, sets the timeout flag and the kernel continues
  * without its input (results are then meaningless and the call returns ICWF_ERR_TIMEOUT);
  * polls < 0 restores the compiled-in limits (well under a second of polling).  Waits on
  * shared-memory barriers that guard asynchronous copies (the tensor-core assembly, the cluster
  * triangular solve) always keep their 2-second limit, so that no copy can land after its kernel
- * has released its memory.  icwf_init_* reset the budget to the defaults. */
+ * has released its memory; in the triangular solve a block that is not there after polls >= 0
+ * polls raises the timeout flag all the same.  icwf_init_* reset the budget to the defaults. */
 icwf_status icwf_set_wait_limit(icwf_handle h, int64_t polls);
 
 /* The handle's CUDA stream (a cudaStream_t) for callers that record events on it. */

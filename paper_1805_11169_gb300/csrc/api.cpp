@@ -359,12 +359,11 @@ void solve(icwf_ctx* h, const double2* Lf, const double2* D, const double2* y, d
   ProfScope ps(h, F_SOLVE, s);
   h->epoch = 1;   // the launchers zero the block flags before every solve
   if (h->df_solve)
-    launch_chol_solve_df(h->N, Lf, D, y, h->work, out, minus_i, h->flags, h->tickets, h->epoch,
-                         h->status, s);
+    h->launches += launch_chol_solve_df(h->N, Lf, D, y, h->work, out, minus_i, h->flags, h->tickets, h->epoch,
+                                        h->status, s);
   else
-    launch_chol_solve(h->N, Lf, D, y, h->work, out, minus_i, h->flags, h->tickets, h->epoch,
-                      h->status, s);
-  h->launches += 2;
+    h->launches += launch_chol_solve(h->N, Lf, D, y, h->work, out, minus_i, h->flags, h->tickets, h->epoch,
+                                     h->status, s);
 }
 
 void assemble(icwf_ctx* h, double2* S, double2* Hm) {
@@ -744,7 +743,7 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
   const size_t cw = h->cwf_elem, rw = h->mixed ? sizeof(float) : sizeof(double);
   const size_t NN = (size_t)N * N;
   const int nblk = (N + 31) / 32;
-  const size_t dl = h->df_solve ? diag_inv_bytes(N) : (size_t)N * 512;
+  const size_t dl = diag_inv_bytes(N);
   std::vector<size_t> sizes = {
       nV * sizeof(double), nV * rw, (size_t)K * nx * 8, (size_t)K * nR * 8, (size_t)K * 8,
       (size_t)nx * 8, (size_t)nR * 8,
@@ -1266,12 +1265,11 @@ icwf_status icwf_load_state(icwf_handle h, const void* buf, size_t bytes) {
     CK(cudaMemcpy(r.first, p, r.second, cudaMemcpyHostToDevice));
     p += r.second;
   }
-  if (h->df_solve) {   // what the solves need beside the saved factor
-    CK(cudaStreamSynchronize(0));   // a copy from pageable memory may still be on its way
-    void *l = h->L[h->cur], *d = h->DL[h->cur];
-    launch_near_products(h->N, &l, &d, 1, h->stream);
-    CK(cudaGetLastError());
-  }
+  // what the solves need beside the saved factor
+  CK(cudaStreamSynchronize(0));   // a copy from pageable memory may still be on its way
+  void *lp = h->L[h->cur], *dp = h->DL[h->cur];
+  launch_near_products(h->N, &lp, &dp, 1, h->df_solve, h->stream);
+  CK(cudaGetLastError());
   const int flags0 = 0;
   CK(cudaMemcpy(h->status + STATUS_FLAGS, &flags0, sizeof(int), cudaMemcpyHostToDevice));
   h->steps = hd.steps;

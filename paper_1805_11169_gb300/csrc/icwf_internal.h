@@ -181,7 +181,7 @@ void launch_matvec(int N, const double2* H0, const double2* H1, double theta, co
 // minus_i, else 1.  work needs 2N complex; flags holds 2*ceil(N/32) block flags followed by the
 // 2 tickets (the launcher zeroes all of them first, so any fixed epoch > 0 works and a captured
 // sequence can be replayed); `tickets` is unused.
-void launch_chol_solve(int N, const double2* L, const double2* D, const double2* y, double2* work,
+int launch_chol_solve(int N, const double2* L, const double2* D, const double2* y, double2* work,
                        double2* out, bool minus_i, unsigned* flags, unsigned* tickets,
                        unsigned epoch, int* status, cudaStream_t s);
 // Mixed modes: the same factorisation and solves in double-float arithmetic (k_linalg_df.cu).
@@ -194,12 +194,15 @@ void launch_shift_mix_df(int N, const double2* S0, const double2* S1, double eps
 int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, int nbatch,
                        unsigned* ctl, int* status, cudaStream_t s);
 size_t chol_ctl_words(int N);
-// Bytes of the D buffer of one matrix (double-float solver): the N x 32 inverted diagonal blocks, then
-// their products with the neighbouring blocks, which launch_cholesky_df and launch_near_products
-// (after a restored factor) compute.
+// Bytes of the D buffer of one matrix (either solver): the N x 32 inverted diagonal blocks, then their
+// products with the neighbouring blocks, which the factorisations and launch_near_products (after a
+// restored factor) compute and the cluster solve reads (k_solve.cu; df: double-float storage).
 size_t diag_inv_bytes(int N);
-int launch_near_products(int N, void* const* L, void* const* D, int nbatch, cudaStream_t s);
-void launch_chol_solve_df(int N, const void* L, const void* D, const double2* y, void* work,
+int launch_near_products(int N, void* const* L, void* const* D, int nbatch, bool df, cudaStream_t s);
+// Both triangular solves in one launch; false, with nothing launched, above its largest size.
+bool launch_cluster_solve(int N, const void* L, const void* D, const double2* y, double2* out, bool minus_i,
+                          bool df, int* status, cudaStream_t s);
+int launch_chol_solve_df(int N, const void* L, const void* D, const double2* y, void* work,
                           double2* out, bool minus_i, unsigned* flags, unsigned* tickets,
                           unsigned epoch, int* status, cudaStream_t s);
 // C += dt/6 (k1 + 2 k2 + 2 k3 + k4); flags non-finite values.

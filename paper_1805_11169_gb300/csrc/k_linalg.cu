@@ -329,7 +329,9 @@ int launch_cholesky(int N, double2* const* A, double* const* inv, double2* const
     }
   }
   k_trtri_diag<<<dim3(T, nbatch), 128, 0, s>>>(N, mb);
-  return launches + 1;
+  void* a[2] = {A[0], mb.m[1]};
+  void* d[2] = {D[0], mb.D[1]};
+  return launches + 1 + launch_near_products(N, a, d, nbatch, false, s);
 }
 
 // ------------------------------------------------------------------------------ matvec
@@ -642,9 +644,10 @@ __global__ void __launch_bounds__(TW * 32) k_trsv_upper(int N, const double2* __
   }
 }
 
-void launch_chol_solve(int N, const double2* L, const double2* D, const double2* y, double2* work,
+int launch_chol_solve(int N, const double2* L, const double2* D, const double2* y, double2* work,
                        double2* out, bool minus_i, unsigned* flags, unsigned* tickets,
                        unsigned epoch, int* status, cudaStream_t s) {
+  if (launch_cluster_solve(N, L, D, y, out, minus_i, false, status, s)) return 1;
   const int nblk = (N + NB - 1) / NB;
   // the block flags start from zero in every solve (one memset with the tickets, which follow
   // them), so a captured launch sequence can be replayed with the same epoch
@@ -654,6 +657,7 @@ void launch_chol_solve(int N, const double2* L, const double2* D, const double2*
   // work[0, N) holds z; work[N, 2N) holds w for the backward pass's consumers
   k_trsv_upper<<<nblk, TW * 32, 0, s>>>(N, L, D, work, out, minus_i, work + N, flags + nblk,
                                         flags + 2 * nblk + 1, epoch, status);
+  return 2;
 }
 
 // ------------------------------------------------------------------------------ RK4 combination

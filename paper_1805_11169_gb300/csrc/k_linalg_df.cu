@@ -12,15 +12,14 @@
 // Kernels: k_shift_mix_df (S -> S + eps I, converted); k_chol_df (the blocked Cholesky, one
 // persistent launch with look-ahead: diagonal updates, diagonal factors, panel slabs,
 // trailing tiles and the inverses of the diagonal blocks as ticket-ordered tasks; the panel tasks
-// also write L^H into the upper triangle); k_chol_solve_cluster (both triangular solves in one
-// 16-CTA cluster, N <= 2048) and k_trsv_lower_df / k_trsv_upper_df (per-block kernels with global
-// flags, larger N).
+// also write L^H into the upper triangle); k_trsv_lower_df / k_trsv_upper_df (triangular solves above
+// N = 2048, per-block kernels with global flags; k_solve.cu has the others).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <mutex>
 
-#include "df64.cuh"
+#include "cdf.cuh"
 #include "icwf_internal.h"
 #include "k_common.cuh"
 
@@ -29,76 +28,6 @@ namespace dfs {
 
 constexpr int NB = 32;
 constexpr unsigned WAIT_LIMIT = 1u << 22;
-
-__device__ __forceinline__ cdf ld4(const float4 v) {
-  return cdf_make(df_make(v.x, v.y), df_make(v.z, v.w));
-}
-__device__ __forceinline__ float4 st4(cdf z) { return make_float4(z.re.h, z.re.l, z.im.h, z.im.l); }
-__device__ __forceinline__ cdf czero() { return cdf_make(df_make(0.f, 0.f), df_make(0.f, 0.f)); }
-
-// Compensated accumulator: value = s + c.
-struct acc2 {
-  float s, c;
-};
-__device__ __forceinline__ void acc_prod(acc2& a, float x, float y) {
-  const float p = DF_MUL(x, y);
-  const float e = DF_FMA(x, y, -p);
-  const df t = two_sum(a.s, p);
-  a.s = t.h;
-  a.c = DF_ADD(a.c, DF_ADD(t.l, e));
-}
-__device__ __forceinline__ void acc_small(acc2& a, float x) { a.c = DF_ADD(a.c, x); }
-__device__ __forceinline__ df acc_val(acc2 a) { return two_sum(a.s, a.c); }
-__device__ __forceinline__ acc2 acc_zero() { acc2 a; a.s = 0.f; a.c = 0.f; return a; }
-__device__ __forceinline__ acc2 acc_merge(acc2 a, acc2 b) {
-  const df t = two_sum(a.s, b.s);
-  acc2 r;
-  r.s = t.h;
-  r.c = DF_ADD(DF_ADD(a.c, b.c), t.l);
-  return r;
-}
-
-struct cacc {
-  acc2 re, im;
-};
-__device__ __forceinline__ cacc cacc_zero() { cacc z; z.re = acc_zero(); z.im = acc_zero(); return z; }
-__device__ __forceinline__ cacc cacc_merge(cacc a, cacc b) {
-  cacc r; r.re = acc_merge(a.re, b.re); r.im = acc_merge(a.im, b.im); return r;
-}
-__device__ __forceinline__ cdf cacc_val(cacc a) { return cdf_make(acc_val(a.re), acc_val(a.im)); }
-// a += x * y
-__device__ __forceinline__ void cacc_mul(cacc& a, cdf x, cdf y) {
-  acc_prod(a.re, x.re.h, y.re.h);
-  acc_prod(a.re, -x.im.h, y.im.h);
-  acc_small(a.re, DF_FMA(x.re.h, y.re.l, DF_MUL(x.re.l, y.re.h)));
-  acc_small(a.re, -DF_FMA(x.im.h, y.im.l, DF_MUL(x.im.l, y.im.h)));
-  acc_prod(a.im, x.re.h, y.im.h);
-  acc_prod(a.im, x.im.h, y.re.h);
-  acc_small(a.im, DF_FMA(x.re.h, y.im.l, DF_MUL(x.re.l, y.im.h)));
-  acc_small(a.im, DF_FMA(x.im.h, y.re.l, DF_MUL(x.im.l, y.re.h)));
-}
-// a += x * conj(y)
-__device__ __forceinline__ void cacc_mulc(cacc& a, cdf x, cdf y) {
-  acc_prod(a.re, x.re.h, y.re.h);
-  acc_prod(a.re, x.im.h, y.im.h);
-  acc_small(a.re, DF_FMA(x.re.h, y.re.l, DF_MUL(x.re.l, y.re.h)));
-  acc_small(a.re, DF_FMA(x.im.h, y.im.l, DF_MUL(x.im.l, y.im.h)));
-  acc_prod(a.im, x.im.h, y.re.h);
-  acc_prod(a.im, -x.re.h, y.im.h);
-  acc_small(a.im, DF_FMA(x.im.h, y.re.l, DF_MUL(x.im.l, y.re.h)));
-  acc_small(a.im, -DF_FMA(x.re.h, y.im.l, DF_MUL(x.re.l, y.im.h)));
-}
-// a += conj(x) * y
-__device__ __forceinline__ void cacc_cmul(cacc& a, cdf x, cdf y) {
-  acc_prod(a.re, x.re.h, y.re.h);
-  acc_prod(a.re, x.im.h, y.im.h);
-  acc_small(a.re, DF_FMA(x.re.h, y.re.l, DF_MUL(x.re.l, y.re.h)));
-  acc_small(a.re, DF_FMA(x.im.h, y.im.l, DF_MUL(x.im.l, y.im.h)));
-  acc_prod(a.im, x.re.h, y.im.h);
-  acc_prod(a.im, -x.im.h, y.re.h);
-  acc_small(a.im, DF_FMA(x.re.h, y.im.l, DF_MUL(x.re.l, y.im.h)));
-  acc_small(a.im, -DF_FMA(x.im.h, y.re.l, DF_MUL(x.im.l, y.re.h)));
-}
 
 struct Batch {
   float4* m[2];
@@ -918,393 +847,6 @@ __global__ void __launch_bounds__(TW * 32) k_trsv_upper_df(int N, const float4* 
   }
 }
 
-// ---------------------------------------------------------------------------- cluster solve
-
-// Products of the inverted diagonal blocks with the two blocks next to them, per block row m:
-//   P[0] = D_m L[m, m-1], P[1] = D_m L[m, m-2] (forward), P[2] = D_m^H L^H[m, m+1],
-//   P[3] = D_m^H L^H[m, m+2] (backward), each stored as rows of 32 like D.
-// grid (4 x block rows, 4, matrices): 8 rows per CTA, warp = row, lane = column, so that two warps share
-// a scheduler and the 32 terms of an entry run at latency, not at issue rate (32 rows per CTA: 9 us for
-// two matrices at N = 64).  The triangular factor's zeros are skipped.  With the products a solve's
-// chain has one 32 x 32 product per block instead of two.
-constexpr int NPR = 8;
-__global__ void __launch_bounds__(NPR * 32) k_near_products(int N, const float4* __restrict__ L0, const float4* __restrict__ L1,
-                                                            const float4* __restrict__ D0, const float4* __restrict__ D1,
-                                                            float4* __restrict__ P0, float4* __restrict__ P1) {
-  __shared__ cdf Ds[NPR][NB + 1], Bs[NB][NB];
-  const int per = NB / NPR, T = gridDim.x / per, m = blockIdx.x / per, which = blockIdx.y;
-  const float4* L = blockIdx.z ? L1 : L0;
-  const float4* D = blockIdx.z ? D1 : D0;
-  float4* P = (blockIdx.z ? P1 : P0) + (size_t)which * T * NB * NB;
-  const bool fwd = which < 2;
-  const int j = fwd ? m - 1 - which : m + 1 + (which - 2);
-  if (j < 0 || j >= T) return;
-  const int w = threadIdx.x >> 5, c = threadIdx.x & 31, r0 = (blockIdx.x % per) * NPR, r = r0 + w;
-  if (fwd) {
-    const int row = m * NB + r;
-    Ds[w][c] = row < N ? ld4(D[(size_t)row * NB + c]) : czero();
-  } else {   // D^H's rows r0.. are D's columns
-    const int k = threadIdx.x / NPR, q = threadIdx.x % NPR;
-    Ds[q][k] = m * NB + k < N ? ld4(D[(size_t)(m * NB + k) * NB + r0 + q]) : czero();
-  }
-#pragma unroll
-  for (int i = 0; i < NB / NPR; ++i) {
-    const int k = w + NPR * i, row = m * NB + k, col = j * NB + c;
-    Bs[k][c] = row < N && col < N ? ld4(L[(size_t)row * N + col]) : czero();
-  }
-  __syncthreads();
-  cacc s = cacc_zero();
-  if (fwd) {
-    for (int k = 0; k <= r; ++k) cacc_mul(s, Ds[w][k], Bs[k][c]);
-  } else {
-    for (int k = r; k < NB; ++k) cacc_cmul(s, Ds[w][k], Bs[k][c]);
-  }
-  P[(size_t)(m * NB + r) * NB + c] = st4(cacc_val(s));
-}
-
-// Both triangular solves of one RK4 stage in a single launch of one 16-CTA thread-block cluster.
-// Every CTA keeps the whole forward solution z and backward solution w in its shared memory.
-// CTA rank r owns block rows jb = r, r + 16, ...; when it finishes a block, the 32 values go from
-// registers into all the CTAs' shared memory by st.async, completing the transaction count of
-// the receiver's per-block mbarrier, so consumers wait on a local barrier instead of polling
-// global memory.  Forward (backward alike, from the last block, with L^H, D^H and the other P):
-//   z_m = u_m - P1_m z_{m-1} - P2_m z_{m-2},   u_m = D_m (y_m - sum_{j <= m-3} L_mj z_j),
-// so that on the arrival of block m
-//   row m + 1's owner adds P1 z_m to what it holds and sends z_{m+1}: the chain, one product;
-//   row m + 2's owner subtracts P2 z_m from u_{m+2};
-//   row m + 3's owner adds its last product L z_m and multiplies by D;
-// (three different CTAs) and every CTA adds block m's products to its later rows.  Products use
-// compensated double-float dot products; a block is spread as 8 warps x 4 rows, 8 lanes per row
-// with 4 columns each, so the sums over a row are 3 shuffle steps.
-// Bound: the chain's latency per block (product, row sum, exchange through distributed shared
-// memory; ~2000 cycles).  With both the product by L[m+1, m] and the one by D on it and 8 CTAs, a step's
-// four solves took 84 / 182 / 256 / 662 / 2330 us at N = 100 / 333 / 512 / 1024 / 2048; now 65 / 147 /
-// 204 / 455 / 1361.  The neighbour products cost 5-15 us a step.  At 32 rows a CTA's dot products are
-// issue-bound (256 threads: 635 cycles for 4 complex terms, 400 at one warp per scheduler).
-constexpr int CL = 16;         // CTAs per cluster
-constexpr int CRPC = 4;        // maximum block rows per CTA (N <= CL * CRPC * 32 = 2048)
-constexpr int CTH = 256;       // threads per CTA
-constexpr unsigned long long CWAIT_NS = 2000000000ull;
-
-__device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned long long gtime_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t map_rank(uint32_t local, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void mbar_init_c(uint64_t* b, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s_u32(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_c(uint64_t* b, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_test_c(uint64_t* b, unsigned parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(s_u32(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded wait for phase 0 of a local block barrier (the timer and the abort flag are looked at every
-// 64th poll: they would lengthen the usual short wait)
-__device__ __forceinline__ bool block_wait(uint64_t* b, volatile int* abort_flag, int* status) {
-  unsigned long long t0 = 0;
-  for (unsigned it = 1; !mbar_test_c(b, 0u); ++it) {
-    if (it & 63u) continue;
-    if (*abort_flag) return false;
-    const unsigned long long t = gtime_ns();
-    if (t0 == 0) t0 = t;
-    if (t - t0 > CWAIT_NS) {
-      *abort_flag = 1;
-      set_flag(status, ST_TIMEOUT);
-      return false;
-    }
-  }
-  return true;
-}
-// store 16 bytes into CTA `rank`'s shared memory (the address is this CTA's twin of it) and
-// complete 16 bytes of the transaction count of that CTA's barrier `bar`
-__device__ __forceinline__ void st_async16(float4 v, const void* dst_local, uint64_t* bar_local,
-                                           uint32_t rank) {
-  const uint32_t dst = map_rank(s_u32(dst_local), rank);
-  const uint32_t bar = map_rank(s_u32(bar_local), rank);
-  asm volatile(
-      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
-      ::"r"(dst), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
-      : "memory");
-}
-
-// Shared-memory layout of the cluster solve (per CTA).
-struct CLayout {
-  float4* zs;        // nblk*32 forward solution
-  float4* ws;        // nblk*32 backward solution
-  float4* yown;      // CRPC*32 right-hand side of the own rows (double-floats)
-  cdf* vsh;          // 32: right-hand side minus products, for the diagonal-block product
-  cacc* acc;         // [CRPC][CTH]: each thread's partial sums of the own block rows
-  uint64_t* barF;    // nblk
-  uint64_t* barB;    // nblk
-  int* abort_flag;
-};
-__host__ __device__ inline size_t clayout_bytes(int nblk) {
-  return (size_t)(2 * nblk + CRPC + 1) * NB * 16 + (size_t)CRPC * CTH * sizeof(cacc) +
-         (size_t)2 * nblk * 8 + 16;
-}
-__device__ __forceinline__ CLayout clayout(unsigned char* base, int nblk) {
-  CLayout c;
-  c.zs = (float4*)base;
-  c.ws = c.zs + nblk * NB;
-  c.yown = c.ws + nblk * NB;
-  c.vsh = (cdf*)(c.yown + CRPC * NB);
-  c.acc = (cacc*)(c.vsh + NB);
-  c.barF = (uint64_t*)(c.acc + CRPC * CTH);
-  c.barB = c.barF + nblk;
-  c.abort_flag = (int*)(c.barB + nblk);
-  return c;
-}
-
-// Sum over the 8 lanes of a row group (lane bits 0..2): every lane gets the same value, since the
-// compensated merge is symmetric in its operands.
-__device__ __forceinline__ cacc group_sum(cacc a) {
-#pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-    cacc b;
-    b.re.s = __shfl_xor_sync(0xffffffffu, a.re.s, o);
-    b.re.c = __shfl_xor_sync(0xffffffffu, a.re.c, o);
-    b.im.s = __shfl_xor_sync(0xffffffffu, a.im.s, o);
-    b.im.c = __shfl_xor_sync(0xffffffffu, a.im.c, o);
-    a = cacc_merge(a, b);
-  }
-  return a;
-}
-
-__device__ __forceinline__ void pf_l1(const void* p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
-// Waits for block m on a local barrier; the outcome is made uniform over the CTA.
-__device__ __forceinline__ bool cta_wait_block(const CLayout& c, uint64_t* bar, int* status) {
-  const bool ok = block_wait(bar, (volatile int*)c.abort_flag, status);
-  return !__syncthreads_or(!ok);
-}
-
-// p += sum_q m[q] z[q] (H: conj(m[q])).  Unrolled with z in registers: a rolled loop over shared memory
-// (tried against instruction-cache misses) made a solve at N = 1024 17% slower.
-template <bool H = false>
-__device__ __forceinline__ void dot4(cacc& p, const cdf (&m)[4], const float4* z) {
-  cdf zc[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) zc[q] = ld4(z[q]);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (H) cacc_cmul(p, m[q], zc[q]);
-    else cacc_mul(p, m[q], zc[q]);
-  }
-}
-
-// a block row's 32 values into every CTA (st.async, completing on their barriers for that block): each
-// of the 8 lanes of a row serves its share of the CTAs
-__device__ __forceinline__ void send_block(const CLayout& c, float4* dst, uint64_t* bar, cdf v) {
-  const float4 f = st4(v);
-  if (!*(volatile int*)c.abort_flag) {
-#pragma unroll
-    for (uint32_t r = 0; r < CL / 8; ++r) st_async16(f, dst, bar, (threadIdx.x & 7) + 8 * r);
-  }
-}
-
-// u = D_b (rhs - sum) for this lane's row of block b (every lane of a row group gets it); all threads
-template <bool FWD>
-__device__ __forceinline__ cdf diag_product(const CLayout& c, int N, int b, const cacc& sum, const cdf (&dk)[4]) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rb = warp * 4 + (lane >> 3), c0 = (lane & 7) * 4;
-  const int row = b * NB + rb;
-  const cdf s = cacc_val(group_sum(sum));
-  const cdf rhs = FWD ? ld4(c.yown[(b / CL) * NB + rb]) : ld4(c.zs[row < N ? row : 0]);
-  __syncthreads();   // vsh of an earlier block has been read
-  if ((lane & 7) == 0) c.vsh[rb] = row < N ? cdf_sub(rhs, s) : czero();
-  __syncthreads();
-  cacc o = cacc_zero();
-  dot4<!FWD>(o, dk, (const float4*)c.vsh + c0);
-  return cacc_val(group_sum(o));
-}
-
-// One pass.  Step t handles block blk(t) = t forward, nblk - 1 - t backward.
-template <bool FWD>
-__device__ __forceinline__ bool solve_pass(const CLayout& c, int N, int nblk, int rank, const float4* __restrict__ L,
-                                           const float4* __restrict__ D, const float4* __restrict__ P,
-                                           double2* __restrict__ out, bool minus_i, int* status) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rb = warp * 4 + (lane >> 3);     // this lane's row within a block
-  const int c0 = (lane & 7) * 4;             // and its 4 columns
-  float4* sol = FWD ? c.zs : c.ws;
-  uint64_t* bars = FWD ? c.barF : c.barB;
-  const size_t PB_ = (size_t)nblk * NB * NB;
-  const float4* P1 = P + (FWD ? 0 : 2) * PB_;
-  const float4* P2 = P1 + PB_;
-  cacc* acc = c.acc + threadIdx.x;           // acc[i * CTH]: partial sums of own block rows
-  for (int i = 0; i < CRPC; ++i) acc[i * CTH] = cacc_zero();
-  auto blk = [&](int t) { return FWD ? t : nblk - 1 - t; };
-  auto load_mat = [&](int b, int mb, cdf (&k)[4]) {      // (L or L^H)[b, mb]
-    const int row = b * NB + rb;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int col = mb * NB + c0 + q;
-      k[q] = row < N && col < N ? ld4(__ldg(L + (size_t)row * N + col)) : czero();
-    }
-  };
-  auto load_p = [&](const float4* p, int b, cdf (&k)[4]) {
-    const float4* q0 = p + (size_t)(b * NB + rb) * NB + c0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) k[q] = ld4(__ldg(q0 + q));
-  };
-  auto load_d = [&](int b, cdf (&k)[4]) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int rd = b * NB + (FWD ? rb : c0 + q);
-      k[q] = rd < N ? ld4(__ldg(D + (size_t)rd * NB + (FWD ? c0 + q : rb))) : czero();
-    }
-  };
-  auto emit = [&](int b, cdf v) {
-    const int row = b * NB + rb;
-    {
-      const cdf vv = row < N ? v : czero();
-      send_block(c, sol + row, bars + b, vv);
-      if (!FWD && row < N && (lane & 7) == 0) {
-        const double re = df_to(vv.re), im = df_to(vv.im);
-        out[row] = minus_i ? make_double2(im, -re) : make_double2(re, im);
-      }
-    }
-  };
-  // operands of a row's next parts into L1 (an L2 access is longer than the wait before its use)
-  auto pf_p = [&](int b) {
-    const size_t o = (size_t)(b * NB + rb) * NB + c0;
-    pf_l1(P2 + o);
-    pf_l1(P1 + o);
-  };
-  auto pf_d = [&](int b) {
-    if (FWD) {
-      if (b * NB + rb < N) pf_l1(D + (size_t)(b * NB + rb) * NB + c0);
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (b * NB + c0 + q < N) pf_l1(D + (size_t)(b * NB + c0 + q) * NB + rb);
-    }
-  };
-  cdf held = czero();                        // u of a row two steps ahead, then u - P2 z of the next
-  // the first three rows have nothing to subtract before their D products
-  for (int t = 0; t < 3 && t < nblk; ++t)
-    if (blk(t) % CL == rank) {
-      cdf dk[4];
-      if (t > 0) pf_p(blk(t));
-      load_d(blk(t), dk);
-      held = diag_product<FWD>(c, N, blk(t), cacc_zero(), dk);
-      if (t == 0) emit(blk(0), held);
-    }
-  for (int t = 0; t + 1 < nblk; ++t) {
-    const int b = blk(t);
-    // this CTA's part on the arrival of block b: 1 sends row t + 1, 2 and 3 prepare the ones after
-    int role = 0;
-    for (int k = 1; k <= 3; ++k)
-      if (t + k < nblk && blk(t + k) % CL == rank) role = k;
-    cdf mk[4], dk[4];
-    if (role == 1) load_p(P1, blk(t + 1), mk);
-    else if (role == 2) load_p(P2, blk(t + 2), mk);
-    else if (role == 3) { load_mat(blk(t + 3), b, mk); load_d(blk(t + 3), dk); }
-    if (!cta_wait_block(c, bars + b, status)) return false;
-    const float4* zc = sol + b * NB + c0;
-    if (role == 1 || role == 2) {
-      cacc p = cacc_zero();
-      dot4(p, mk, zc);
-      held = cdf_sub(held, cacc_val(group_sum(p)));
-      if (role == 1) emit(blk(t + 1), held);
-    } else if (role == 3) {
-      const int nb3 = blk(t + 3);
-      cacc p = acc[(nb3 / CL) * CTH];
-      dot4(p, mk, zc);
-      pf_p(nb3);
-      held = diag_product<FWD>(c, N, nb3, p, dk);
-    }
-    // the later own rows
-#pragma unroll 1
-    for (int i = 0; i < CRPC; ++i) {
-      const int jb = rank + CL * i;
-      if (jb >= nblk) break;
-      const int tj = FWD ? jb : nblk - 1 - jb;
-      if (tj < t + 4) continue;
-      const int row = jb * NB + rb;
-      cacc a = acc[i * CTH];
-      cdf k[4];
-      load_mat(jb, b, k);
-      dot4(a, k, zc);
-      acc[i * CTH] = a;
-      // the next block's operands of this row, into L1 while the CTA waits for that block
-      if (row < N) pf_l1(L + (size_t)row * N + blk(t + 1) * NB + c0);
-      if (tj == t + 4) pf_d(jb);
-    }
-  }
-  // every block is in place before the next pass reads it
-  return cta_wait_block(c, bars + blk(nblk - 1), status);
-}
-
-__global__ void __launch_bounds__(CTH, 1)
-k_chol_solve_cluster(int N, const float4* __restrict__ L, const float4* __restrict__ D, const float4* __restrict__ P,
-                     const double2* __restrict__ y, double2* __restrict__ out, bool minus_i,
-                     int* status) {
-  extern __shared__ __align__(128) unsigned char csm[];
-  const int nblk = (N + NB - 1) / NB;
-  const CLayout c = clayout(csm, nblk);
-  const int rank = (int)cluster_rank();
-
-  if (threadIdx.x == 0) {
-    for (int m = 0; m < nblk; ++m) {
-      mbar_init_c(c.barF + m, 1);
-      mbar_init_c(c.barB + m, 1);
-    }
-    *c.abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    for (int m = 0; m < nblk; ++m) {
-      mbar_expect_c(c.barF + m, 512u);
-      mbar_expect_c(c.barB + m, 512u);
-    }
-  }
-  // right-hand side of the own rows, converted to double-floats once
-  for (int e = threadIdx.x; e < CRPC * NB; e += CTH) {
-    const int row = (rank + CL * (e / NB)) * NB + e % NB;
-    const double2 yv = row < N ? y[row] : make_double2(0.0, 0.0);
-    c.yown[e] = st4(cdf_make(df_from(yv.x), df_from(yv.y)));
-  }
-  __syncthreads();
-  cluster_sync();
-  if (solve_pass<true>(c, N, nblk, rank, L, D, P, out, minus_i, status))
-    solve_pass<false>(c, N, nblk, rank, L, D, P, out, minus_i, status);
-  __syncthreads();
-  cluster_sync();
-  if (*(volatile int*)c.abort_flag) {
-    // a wait gave up: stores from other CTAs may still be landing in this CTA's shared memory,
-    // which outlives none of them only after they complete; they take microseconds, so linger
-    const unsigned long long t0 = gtime_ns();
-    while (gtime_ns() - t0 < 200000ull) {
-    }
-  }
-}
-
-size_t cluster_solve_smem(int N) { return clayout_bytes((N + NB - 1) / NB); }
-
 }  // namespace dfs
 
 // ---------------------------------------------------------------------------- launchers
@@ -1314,7 +856,6 @@ void launch_shift_mix_df(int N, const double2* S0, const double2* S1, double eps
   dfs::k_shift_mix_df<<<N, 256, 0, s>>>(N, S0, S1, eps, theta, (float4*)A);
 }
 
-static size_t near_offset(int N);
 int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, int nbatch,
                        unsigned* ctl, int* status, cudaStream_t s) {
   using namespace dfs;
@@ -1340,21 +881,7 @@ int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, 
   for (int li = 0; li <= T; ++li) widest = std::max(widest, nbatch * StepTasks(N, li).count());
   const int grid = std::min(std::max(sms, nbatch + 1), nbatch + (widest + 1) / 2);
   k_chol_df<<<grid, CTA_THREADS, CS_SMEM_LAUNCH, s>>>(N, mb, nbatch, ctl, status);
-  return 1 + launch_near_products(N, A, D, nbatch, s);
-}
-
-// The products next to the inverted diagonal blocks follow them in the D buffer, whole blocks each
-// (diag_inv_bytes); the solves above CL * CRPC block rows do not use them.
-static size_t near_offset(int N) { return (size_t)((N + dfs::NB - 1) / dfs::NB) * dfs::NB * dfs::NB; }
-size_t diag_inv_bytes(int N) { return 5 * near_offset(N) * sizeof(float4); }
-int launch_near_products(int N, void* const* L, void* const* D, int nbatch, cudaStream_t s) {
-  using namespace dfs;
-  const int T = (N + NB - 1) / NB, k = nbatch > 1 ? 1 : 0;
-  if (T > CL * CRPC || T < 2) return 0;
-  float4 *d0 = (float4*)D[0], *d1 = (float4*)D[k];
-  k_near_products<<<dim3(T * (NB / NPR), 4, nbatch), NPR * 32, 0, s>>>(N, (const float4*)L[0], (const float4*)L[k], d0, d1,
-                                                      d0 + near_offset(N), d1 + near_offset(N));
-  return 1;
+  return 1 + launch_near_products(N, A, D, nbatch, true, s);
 }
 
 size_t chol_ctl_words(int N) {
@@ -1362,35 +889,12 @@ size_t chol_ctl_words(int N) {
   return 5 * (T + 2) + 2 * (T + 1) * T + 2 * T * T;
 }
 
-void launch_chol_solve_df(int N, const void* L, const void* D, const double2* y, void* work,
+int launch_chol_solve_df(int N, const void* L, const void* D, const double2* y, void* work,
                           double2* out, bool minus_i, unsigned* flags, unsigned* tickets,
                           unsigned epoch, int* status, cudaStream_t s) {
   using namespace dfs;
+  if (launch_cluster_solve(N, L, D, y, out, minus_i, true, status, s)) return 1;
   const int nblk = (N + NB - 1) / NB;
-  if (nblk <= CL * CRPC) {
-    // one 16-CTA cluster, both passes in one launch
-    const size_t sm = cluster_solve_smem(N);
-    static std::once_flag once;
-    std::call_once(once, [] {
-      cudaFuncSetAttribute(k_chol_solve_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)cluster_solve_smem(CL * CRPC * NB));
-      cudaFuncSetAttribute(k_chol_solve_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    });
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(CL);
-    cfg.blockDim = dim3(CTH);
-    cfg.dynamicSmemBytes = sm;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_chol_solve_cluster, N, (const float4*)L, (const float4*)D,
-                       (const float4*)D + near_offset(N), y, out, minus_i, status);
-    return;
-  }
   // block flags and tickets (which follow them) start from zero in every solve, so a captured
   // launch sequence can be replayed with the same epoch
   cudaMemsetAsync(flags, 0, (2 * (size_t)nblk + 2) * sizeof(unsigned), s);
@@ -1400,6 +904,7 @@ void launch_chol_solve_df(int N, const void* L, const void* D, const double2* y,
                                             flags + 2 * nblk, epoch, status);
   k_trsv_upper_df<<<nblk, TW * 32, 0, s>>>(N, (const float4*)L, (const float4*)D, zb, out, minus_i,
                                             zb + N, flags + nblk, flags + 2 * nblk + 1, epoch, status);
+  return 2;
 }
 
 }  // namespace icwf
