@@ -93,6 +93,7 @@ struct icwf_ctx {
   double *invL[2] = {nullptr, nullptr}, *invLh = nullptr;   // reciprocal Cholesky pivots
   double2 *DL[2] = {nullptr, nullptr}, *DLh = nullptr;       // inverted 32 x 32 diagonal blocks
   unsigned *flags = nullptr, *tickets = nullptr;
+  void* herk_scratch = nullptr;                              // two-level double-float factorisation
   unsigned* cctl = nullptr;                                  // blocked-factorisation tickets/flags
   int* status = nullptr;
   int cur = 0;
@@ -346,7 +347,7 @@ void factor(icwf_ctx* h, int n, const double2* const* S0, const double2* const* 
     void* a[2] = {dst[0], n > 1 ? dst[1] : dst[0]};
     void* iv[2] = {inv[0], n > 1 ? inv[1] : inv[0]};
     void* dd[2] = {D[0], n > 1 ? D[1] : D[0]};
-    h->launches += launch_cholesky_df(h->N, a, iv, dd, n, h->cctl, h->status, h->stream);
+    h->launches += launch_cholesky_df(h->N, a, iv, dd, n, h->cctl, h->herk_scratch, h->status, h->stream);
   } else {
     h->launches += launch_cholesky(h->N, dst, inv, D, n, h->status, h->stream,
                                    h->emu_update ? h->emu_scratch : nullptr, h->emu_bytes);
@@ -767,6 +768,8 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
     total += align256(h->emu_bytes);
     herk_emu_attributes();
   }
+  const size_t herk_bytes = h->df_solve ? herk_df_bytes(N) : 0;
+  total += align256(herk_bytes);
   total += 4096;
   if (cudaMalloc(&h->arena.base, total) != cudaSuccess) {
     destroy_streams(h);
@@ -818,8 +821,9 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
   h->cctl = (unsigned*)a.take(chol_ctl_words(N) * sizeof(unsigned));
   h->status = (int*)a.take(64 * 4);
   if (!h->df_solve) h->emu_scratch = a.take(h->emu_bytes);
+  if (herk_bytes) h->herk_scratch = a.take(herk_bytes);
   char* plan_base = (char*)a.take(h->plan_bytes);
-  if (!h->status || !plan_base || (!h->df_solve && !h->emu_scratch)) {
+  if (!h->status || !plan_base || (!h->df_solve && !h->emu_scratch) || (herk_bytes && !h->herk_scratch)) {
     cudaFree(h->arena.base);
     destroy_streams(h);
     return fail(nullptr, ICWF_ERR_OOM, "icwf_create: arena layout overflow");

@@ -192,8 +192,15 @@ void launch_shift_mix_df(int N, const double2* S0, const double2* S1, double eps
 // One launch per block column with look-ahead; ctl holds chol_ctl_words(N) words of ticket and
 // flag state (the launcher zeroes it).
 int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, int nbatch,
-                       unsigned* ctl, int* status, cudaStream_t s);
+                       unsigned* ctl, void* herk_scratch, int* status, cudaStream_t s);
 size_t chol_ctl_words(int N);
+// Block columns per launch of the two-level form, 0 at sizes where the factorisation is one launch.
+int chol_panel(int N);
+// Trailing update of the two-level form, A[r, c] -= L[r, k] L[c, k]^H for c <= r from row R0 on and the
+// 128 columns from k0, on the tensor cores (k_sliced.cu).  herk_df_bytes: scratch for two matrices, 0
+// at sizes where the factorisation runs as one launch.
+size_t herk_df_bytes(int N);
+int launch_herk_df(int N, int k0, int R0, void* const* A, int nb, void* scratch, int* status, cudaStream_t s);
 // Bytes of the D buffer of one matrix (either solver): the N x 32 inverted diagonal blocks, then their
 // products with the neighbouring blocks, which the factorisations and launch_near_products (after a
 // restored factor) compute and the cluster solve reads (k_solve.cu; df: double-float storage).

@@ -10,7 +10,8 @@
 // returns them as accurately as if evaluated in twice the FP32 precision.
 //
 // Kernels: k_shift_mix_df (S -> S + eps I, converted); k_chol_df (the blocked Cholesky, one
-// persistent launch with look-ahead: diagonal updates, diagonal factors, panel slabs,
+// persistent launch with look-ahead, above 26 block columns several with the trailing updates between
+// them on the tensor cores: diagonal updates, diagonal factors, panel slabs,
 // trailing tiles and the inverses of the diagonal blocks as ticket-ordered tasks; the panel tasks
 // also write L^H into the upper triangle); k_trsv_lower_df / k_trsv_upper_df (triangular solves above
 // N = 2048, per-block kernels with global flags; k_solve.cu has the others).
@@ -102,6 +103,15 @@ constexpr int CTA_THREADS = 2 * CS_THREADS;   // two groups
 // other CTA of the launch
 constexpr int CS_SMEM_LAUNCH = 116 * 1024;
 static_assert(2 * CS_SMEM <= CS_SMEM_LAUNCH, "tasks need more shared memory than the launch asks for");
+// Two-level form: while more than ONE_LAUNCH block columns are left, a launch factors PANEL of them and the
+// trailing update from those runs on the tensor cores (launch_herk_df); the rest is one launch.  The
+// FP32 tiles of a single launch bound its early steps (a 32 x 32 tile takes a group 12 us); the two
+// launches of an update and a cold start of the diagonal factor cost about 30 us per panel.  All in
+// panels / one launch, two matrices, us: 597 / 473 at N = 640, 788 / 652 at 769, 949 / 872 at 900, 1027 /
+// 1076 at 1024, 1744 / 2667 at 1500, 2815 / 6059 at 2048; four columns cost 161 in panels and 219 in one
+// launch from 29 blocks on, 178 and 162 from 25.
+constexpr int PANEL = 4;
+constexpr int ONE_LAUNCH = 26;
 constexpr int AHEAD_TILES = 300;              // trailing tiles ahead of the slabs: one per group
 
 // One group of CS_THREADS threads of a CTA.
@@ -452,7 +462,7 @@ __device__ __forceinline__ void trtri_task(int N, const float4* A, const float2*
 }
 
 // Control words of one factorisation (zeroed before its launch), per matrix m:
-//   ticket, role                     counters of the worker tasks and of the CTAs
+//   ticket[p], role[p]               counters of the worker tasks and of the CTAs of launch p
 //   diag  [li][m]                    finished 8 x 8 updates of diagonal block li
 //   pdone [li][m]                    bit w: columns 4w.. of diagonal factor li published
 //   slabdone[m][l][b]                finished 8-row panel slabs of block column l in row block b
@@ -461,8 +471,9 @@ struct CholCtl {
   unsigned* w;
   int T, N;
   __device__ CholCtl(unsigned* ctl, int n) : w(ctl), T((n + NB - 1) / NB), N(n) {}
-  __device__ unsigned* ticket() const { return w; }
-  __device__ unsigned* role() const { return w + 1; }
+  // launches start PANEL block columns apart
+  __device__ unsigned* ticket(int lo) const { return w + 2 * (lo / PANEL); }
+  __device__ unsigned* role(int lo) const { return w + 2 * (lo / PANEL) + 1; }
   __device__ unsigned* diag(int li, int m) const { return w + (T + 2) + 2 * li + m; }
   __device__ unsigned* pdone(int li, int m) const { return w + 3 * (T + 2) + 2 * li + m; }
   __device__ unsigned* sd(int m, int l, int b) const { return w + 5 * (T + 2) + ((size_t)m * (T + 1) + l) * T + b; }
@@ -499,30 +510,33 @@ __device__ __forceinline__ void wait_count(const Grp& g, const unsigned* f, unsi
   }
 }
 
-// Tasks of block column li besides its diagonal factor, per matrix.
+// Tasks of block column li besides its diagonal factor, per matrix, in a launch over the block columns
+// [lo, hi): the updates from its own columns to the columns up to hi.
 struct StepTasks {
-  int diag, herk, slab, inv;
-  __host__ __device__ StepTasks(int N, int li) {
-    const int T = (N + NB - 1) / NB, rt = T - li - 1, rows = N - (li + 1) * NB;
-    diag = (li > 0 && li < T) ? DIAG_TASKS : 0;
-    herk = (li > 0 && rt > 0) ? rt * (rt + 1) / 2 : 0;
-    slab = (li < T && rows > 0) ? (rows + TS_ROWS - 1) / TS_ROWS : 0;
-    inv = li > 0 ? 1 : 0;
+  int diag, herk, slab, inv, tiles;   // tiles: of the whole trailing triangle
+  __host__ __device__ StepTasks(int N, int lo, int hi, int li) {
+    const int T = (N + NB - 1) / NB, rt = T - li - 1, rows = N - (li + 1) * NB, w = hi - 1 - li;
+    diag = (li > lo && li < hi) ? DIAG_TASKS : 0;
+    tiles = rt * (rt + 1) / 2;
+    herk = (li > lo && w > 0) ? w * rt - w * (w - 1) / 2 : 0;
+    slab = (li < hi && rows > 0) ? (rows + TS_ROWS - 1) / TS_ROWS : 0;
+    inv = li > lo ? 1 : 0;
   }
   __host__ __device__ int count() const { return diag + herk + slab + inv; }
 };
 
 // Task t of block column li (all matrices).
-__device__ __forceinline__ void chol_task(const Grp& g, int N, const Batch& mb, int nb, int li, int t, const StepTasks& st,
+__device__ __forceinline__ void chol_task(const Grp& g, int N, const Batch& mb, int nb, int lo, int li, int t, const StepTasks& st,
                                           const CholCtl& cc, int* status, unsigned char* sm) {
   const int jp = li, jb = li - 1;
+  const unsigned before = (unsigned)(li > lo ? jb - lo : 0);   // earlier updates of a tile in this launch
   if (t < nb * st.diag) {
     // 8 x 8 block (rb, cb) of diagonal block jp: A -= L_jp,jb L_jp,jb^H; needs panel jb on the rows
-    // of block jp and the jb earlier trailing updates of the diagonal tile
+    // of block jp and the earlier trailing updates of the diagonal tile
     const int m = t % nb;
     int cb, rb;
     tri_index(t / nb, cb, rb);
-    wait_counts(g, cc.sd(m, jb, jp), cc.slabs_in(jp), cc.tc(m, jp, jp), (unsigned)jb, nullptr, 0, status);
+    wait_counts(g, cc.sd(m, jb, jp), cc.slabs_in(jp), cc.tc(m, jp, jp), before, nullptr, 0, status);
     g.sync();
     diag_update8(pick2(mb.m, m), N, jp, jb, rb, cb, sm, g);
     cs_signal(g, cc.diag(li, m));
@@ -537,11 +551,11 @@ __device__ __forceinline__ void chol_task(const Grp& g, int N, const Batch& mb, 
     const int m = t % nb;
     // block columns from the left (the next steps need them first), rows from the diagonal
     int I, J;
-    tri_index(st.herk - 1 - t / nb, I, J);
+    tri_index(st.tiles - 1 - t / nb, I, J);
     const int rb = cc.T - 1 - I, cb = cc.T - 1 - J;
-    // panel jb on both row blocks, and the tile's jb - 1 earlier updates
+    // panel jb on both row blocks, and the tile's earlier updates
     wait_counts(g, cc.sd(m, jb, rb), cc.slabs_in(rb), cc.sd(m, jb, cb), cc.slabs_in(cb), cc.tc(m, rb, cb),
-                (unsigned)(jb > 0 ? jb : 0), status);
+                before, status);
     g.sync();
     herk_tile(pick2(mb.m, m), N, jb, rb, cb, sm, g);
     cs_signal(g, cc.tc(m, rb, cb));
@@ -558,14 +572,14 @@ __device__ __forceinline__ void chol_task(const Grp& g, int N, const Batch& mb, 
     const int r = g.tid / NB, c = g.tid % NB;
     const bool ok = i0 + r < N;
     const int bi = i0 / NB;
-    if (jb >= 0) {
-      // panel jb on these rows and on the rows of block jp, and the tile's jb earlier updates
+    if (li > lo) {
+      // panel jb on these rows and on the rows of block jp, and the tile's earlier updates
       wait_counts(g, cc.sd(m, jb, bi), cc.slabs_in(bi), cc.sd(m, jb, jp), cc.slabs_in(jp), cc.tc(m, bi, jp),
-                  (unsigned)jb, status);
+                  before, status);
       g.sync();
     }
     cdf a;
-    if (jb >= 0) a = upd_one<TS_ROWS, NB>(A, N, i0, jp * NB, jb * NB, i0 + r, jp * NB + c, ok, sm, g);
+    if (li > lo) a = upd_one<TS_ROWS, NB>(A, N, i0, jp * NB, jb * NB, i0 + r, jp * NB + c, ok, sm, g);
     else a = ok ? ldcg4(A + (size_t)(i0 + r) * N + jp * NB + c) : czero();
     // with L' = L diag(y) (y_k = 1 / L_kk) and x = z diag(y): z_k = a_k - sum_j<k z_j conj(L'_kj), so
     // the chain carries no scaling.  Eight columns at a time, as the diagonal factor publishes them:
@@ -622,11 +636,11 @@ __device__ __forceinline__ void chol_task(const Grp& g, int N, const Batch& mb, 
   }
 }
 
-__global__ void __launch_bounds__(CTA_THREADS, 1) k_chol_df(int N, Batch mb, int nb, unsigned* ctl, int* status) {
+__global__ void __launch_bounds__(CTA_THREADS, 1) k_chol_df(int N, Batch mb, int nb, int lo, int hi, unsigned* ctl, int* status) {
   extern __shared__ __align__(16) unsigned char smem_all[];
   __shared__ unsigned s_role, s_t[2];
   const CholCtl cc(ctl, N);
-  if (threadIdx.x == 0) s_role = atomicAdd(cc.role(), 1u);
+  if (threadIdx.x == 0) s_role = atomicAdd(cc.role(lo), 1u);
   __syncthreads();
   const int half = threadIdx.x / CS_THREADS;
   const Grp g{(int)threadIdx.x % CS_THREADS, 1 + half};
@@ -634,27 +648,27 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) k_chol_df(int N, Batch mb, int
   if ((int)s_role < nb) {
     if (half) return;
     const int m = (int)s_role;
-    for (int li = 0; li < cc.T; ++li) {
-      if (li > 0) wait_count(g, cc.diag(li, m), (unsigned)DIAG_TASKS, status);
+    for (int li = lo; li < hi; ++li) {
+      if (li > lo) wait_count(g, cc.diag(li, m), (unsigned)DIAG_TASKS, status);
       g.sync();
       potrf_task(N, pick2(mb.m, m), pick2(mb.inv, m), li, status, cc.pdone(li, m), sm, g);
     }
     return;
   }
-  int li = 0;
+  int li = lo;
   unsigned base = 0;
-  StepTasks st(N, 0);
+  StepTasks st(N, lo, hi, lo);
   while (true) {
-    if (g.tid == 0) s_t[half] = atomicAdd(cc.ticket(), 1u);
+    if (g.tid == 0) s_t[half] = atomicAdd(cc.ticket(lo), 1u);
     g.sync();
     const unsigned t = s_t[half];
     g.sync();   // shared memory of the previous task and s_t are free after this
-    while (li <= cc.T && t - base >= (unsigned)(nb * st.count())) {
+    while (li <= hi && t - base >= (unsigned)(nb * st.count())) {
       base += nb * st.count();
-      st = StepTasks(N, ++li);
+      st = StepTasks(N, lo, hi, ++li);
     }
-    if (li > cc.T) return;
-    chol_task(g, N, mb, nb, li, (int)(t - base), st, cc, status, sm);
+    if (li > hi) return;
+    chol_task(g, N, mb, nb, lo, li, (int)(t - base), st, cc, status, sm);
   }
 }
 
@@ -857,7 +871,7 @@ void launch_shift_mix_df(int N, const double2* S0, const double2* S1, double eps
 }
 
 int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, int nbatch,
-                       unsigned* ctl, int* status, cudaStream_t s) {
+                       unsigned* ctl, void* herk_scratch, int* status, cudaStream_t s) {
   using namespace dfs;
   Batch mb;
   for (int q = 0; q < 2; ++q) {
@@ -876,14 +890,21 @@ int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, 
     cudaFuncSetAttribute(k_chol_df, cudaFuncAttributeMaxDynamicSharedMemorySize, CS_SMEM_LAUNCH);
   });
   cudaMemsetAsync(ctl, 0, chol_ctl_words(N) * sizeof(unsigned), s);
-  // chain CTAs and two groups per worker CTA, no more workers than the widest step has tasks
-  int widest = 1;
-  for (int li = 0; li <= T; ++li) widest = std::max(widest, nbatch * StepTasks(N, li).count());
-  const int grid = std::min(std::max(sms, nbatch + 1), nbatch + (widest + 1) / 2);
-  k_chol_df<<<grid, CTA_THREADS, CS_SMEM_LAUNCH, s>>>(N, mb, nbatch, ctl, status);
-  return 1 + launch_near_products(N, A, D, nbatch, true, s);
+  int launches = 0;
+  for (int lo = 0, hi; lo < T; lo = hi) {
+    hi = herk_scratch && T - lo > ONE_LAUNCH ? lo + PANEL : T;
+    // chain CTAs and two groups per worker CTA, no more workers than the widest step has tasks
+    int widest = 1;
+    for (int li = lo; li <= hi; ++li) widest = std::max(widest, nbatch * StepTasks(N, lo, hi, li).count());
+    const int grid = std::min(std::max(sms, nbatch + 1), nbatch + (widest + 1) / 2);
+    k_chol_df<<<grid, CTA_THREADS, CS_SMEM_LAUNCH, s>>>(N, mb, nbatch, lo, hi, ctl, status);
+    ++launches;
+    if (hi < T) launches += launch_herk_df(N, lo * NB, hi * NB, A, nbatch, herk_scratch, status, s);
+  }
+  return launches + launch_near_products(N, A, D, nbatch, true, s);
 }
 
+int chol_panel(int N) { return (N + dfs::NB - 1) / dfs::NB > dfs::ONE_LAUNCH ? dfs::PANEL : 0; }
 size_t chol_ctl_words(int N) {
   const size_t T = (N + dfs::NB - 1) / dfs::NB;
   return 5 * (T + 2) + 2 * (T + 1) * T + 2 * T * T;

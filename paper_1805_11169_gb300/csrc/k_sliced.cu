@@ -54,6 +54,7 @@
 #include <mutex>
 #include <vector>
 
+#include "df64.cuh"
 #include "icwf_internal.h"
 #include "k_common.cuh"
 #include "sliced.cuh"
@@ -73,6 +74,9 @@ static_assert(SMEM_BYTES <= 227 * 1024, "shared memory per CTA exceeded");
 constexpr int EPI_WARPS = 8, TMA_WARP = 8, MMA_WARP = 9, THREADS = 320;
 constexpr int COL_IM = 256;            // TMEM: Re levels at [0, 256), Im levels at [256, 512)
 constexpr int EX_BAD = 0x40000000;     // exponent of a row with a non-finite component
+
+// the double-float trailing update's panel and digits (see k_herk_slices)
+constexpr int HERK_COLS = 128, HERK_KS = HERK_COLS / 16, HERK_D = 7, HERK_B0 = 6, HERK_BETA = 7;
 
 // bytes of a pipeline stage (one K slice): both planes' pieces of 128 bras and T kets
 __host__ __device__ inline int stage_bytes(int d, int t) { return 2 * d * (MT + t) * ROW_BYTES; }
@@ -102,6 +106,8 @@ struct GramArgs {
   const Gram* grams;
   void* out;                // overrides the Grams' outputs if not NULL
   int ngrams, units, N;
+  float4* herk[2];          // if set: Gram i's conj(bra) ket is subtracted from the double-floats
+  int R0;                   //    herk[i][(R0 + ket) N + R0 + bra], bra <= ket, R0 + ket < N
   unsigned* ticket;
   int* status;
 };
@@ -201,6 +207,47 @@ __device__ __forceinline__ void store8(double2* out, int sc, int n, int xb, int 
     double2 z = make_double2(fixed_to_f64(re[e], ea + x + shift), fixed_to_f64(im[e], ea + x + shift));
     if (ea == EX_BAD || x == EX_BAD) z.x = z.y = __longlong_as_double(0x7FF8000000000000ll);
     out[(size_t)e * sc] = z;
+  }
+}
+
+// Subtraction of 8 kets' sums from the rows r..r + 7 of A, lane = bra (column c of A), a: the old values.
+// The levels (exact integers) are added from the smallest up in double-float arithmetic.
+__device__ __forceinline__ void herk_load8(const float4* __restrict__ A, int N, int r, int c, float4 (&a)[8]) {
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+    a[e] = r + e < N && c <= r + e ? A[(size_t)(r + e) * N + c] : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+template <int L, int BETA>
+__device__ __forceinline__ void herk_levels8(uint32_t col, int t, df (&re)[8], df (&im)[8]) {
+#pragma unroll
+  for (int lv = L - 1; lv >= 0; --lv) {
+    float vr[8], vi[8];
+    tmem_ld8(col + lv * t, vr);
+    tmem_ld8(col + COL_IM + lv * t, vi);
+    tmem_wait_ld();
+    const float w = __int_as_float((127 - BETA * lv) << 23);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if (lv == L - 1) {
+        re[e] = df_make(vr[e] * w, 0.f);
+        im[e] = df_make(vi[e] * w, 0.f);
+      } else {
+        re[e] = df_add_f(re[e], vr[e] * w);
+        im[e] = df_add_f(im[e], vi[e] * w);
+      }
+    }
+  }
+}
+__device__ __forceinline__ void herk_store8(float4* __restrict__ A, int N, int r, int c, int xb, int l0, int ea,
+                                            int shift, const float4 (&a)[8], const df (&re)[8], const df (&im)[8]) {
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const int x = __shfl_sync(0xffffffffu, xb, l0 + e), k = ea + x + shift;
+    df vr = df_make(scaled(re[e].h, k), scaled(re[e].l, k)), vi = df_make(scaled(im[e].h, k), scaled(im[e].l, k));
+    if (ea == EX_BAD || x == EX_BAD) vr.h = vi.h = __int_as_float(0x7FC00000);
+    vr = df_sub(df_make(a[e].x, a[e].y), vr);
+    vi = df_sub(df_make(a[e].z, a[e].w), vi);
+    if (r + e < N && c <= r + e) A[(size_t)(r + e) * N + c] = make_float4(vr.h, vr.l, vi.h, vi.l);
   }
 }
 
@@ -472,7 +519,28 @@ __global__ void __launch_bounds__(THREADS, 1) k_gram_sliced(GramArgs args) {
       // kets this lane stores (rows and columns past the edge of a rectangular product: none)
       const int nk = g.cols == 0 ? t : (at.I * MT + row < g.rows ? g.cols - at.bt * t - c0 : 0);
       const uint32_t col = base + half * (t / 2);
-      if (g.digits) {
+      if (args.herk[0]) {
+        float4* A = args.ngrams > 1 && u >= unit0[1] ? args.herk[1] : args.herk[0];
+        const int r = args.R0 + at.bt * t + c0, c = args.R0 + at.I * MT + row;
+#pragma unroll 1
+        for (int h = 0; h < 2 && ok; ++h) {
+          float4 a[8];   // on their way while the MMAs run and the levels are read
+          herk_load8(A, args.N, r + 8 * h, c, a);
+          if (h == 0) {
+            ok = __all_sync(0xffffffffu, mbar_wait(acc_full, chunk & 1u, abort_flag, status));
+            if (!ok) break;
+            ++chunk;
+            fence_after();
+          }
+          df re[8], im[8];
+          herk_levels8<HERK_D, HERK_BETA>(col + 8 * h, t, re, im);
+          if (h == 1) {
+            fence_before();
+            mbar_arrive(acc_empty);
+          }
+          herk_store8(A, args.N, r + 8 * h, c, xb0, 8 * h, ea, -2 * HERK_B0, a, re, im);
+        }
+      } else if (g.digits) {
         double2* out = (double2*)(args.out ? args.out : g.out) + o;
         const int shift = -2 * g.b0 - g.fbits;
         if (t == 32) {
@@ -1104,7 +1172,138 @@ int term_digits(double r) {
 
 struct Term { int d; size_t bx, bR; };   // pieces and operand bytes of both sides
 
+// ---------------------------------------------------------------------------- trailing update
+//
+// The double-float Cholesky's trailing update over a panel of HERK_COLS columns as one Gram of the
+// panel's rows: HERK_D digits (48 bits below a row's largest component, the precision of a double-float)
+// and the pairs up to 2^-48 of the leading one; the epilogue subtracts in double-float.
+// Bound: the tensor pipe, 8 slices of 2000 cycles per unit (128 x 32 elements; 2330 measured), and at few
+// units the serial rest: 7300 cycles to the first MMA, 11000 from the last one to the stores.  (With the
+// 64-bit integer sums of the other Grams and A read after them that was 24000.)
+struct HerkSlices {
+  const float4* A[2];
+  unsigned char* out[2];
+  int* ex[2];
+  int N, k0, R0, rpad;
+  Gram* grams;
+  Gram g[2];
+  int ng;
+  unsigned* ticket;
+};
+
+// round(x 2^q), |x| 2^q < 2^62, half away from zero
+__device__ __forceinline__ long long fixed_of_f32(float x, int q) {
+  const uint32_t u = __float_as_uint(x), E = (u >> 23) & 0xFFu;
+  const unsigned long long mant = (u & 0x7FFFFFu) | (E ? 0x800000u : 0u);
+  const int s = (E ? (int)E - 150 : -149) + q;
+  unsigned long long r;
+  if (s >= 0) r = mant << s;
+  else if (s <= -25) r = 0;
+  else r = (mant + (1ull << (-s - 1))) >> (-s);
+  return u >> 31 ? -(long long)r : (long long)r;
+}
+
+// Digits of the panel's rows from R0 on, 16 threads per row with 8 columns each; rows past N: zeros.
+// Also resets the Gram launch's ticket and writes its table.
+__global__ void __launch_bounds__(256) k_herk_slices(HerkSlices p) {
+  const int m = blockIdx.y, row = blockIdx.x * 16 + (threadIdx.x >> 4), c8 = threadIdx.x & 15;
+  if (blockIdx.x == 0 && m == 0 && threadIdx.x == 0) {
+    *p.ticket = 0;
+    for (int i = 0; i < p.ng; ++i) p.grams[i] = i ? p.g[1] : p.g[0];
+  }
+  const float4* A = m ? p.A[1] : p.A[0];
+  unsigned char* out = m ? p.out[1] : p.out[0];
+  const int r = p.R0 + row;
+  float4 v[8];
+  unsigned mx = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    v[k] = r < p.N ? A[(size_t)r * p.N + p.k0 + 8 * c8 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
+    mx = max(mx, max(__float_as_uint(v[k].x) & 0x7FFFFFFFu, __float_as_uint(v[k].z) & 0x7FFFFFFFu));
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const bool bad = mx >= 0x7F800000u;
+  const int e = mx == 0 || bad ? 0 : max((int)(mx >> 23), 1) - 126;
+  if (c8 == 0) (m ? p.ex[1] : p.ex[0])[row] = bad ? EX_BAD : e;
+  const int q = HERK_B0 + HERK_BETA * (HERK_D - 1) - e;
+#pragma unroll
+  for (int plane = 0; plane < 2; ++plane) {
+    uint32_t pk[HERK_D][4];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float h = plane ? v[k].z : v[k].x, l = plane ? v[k].w : v[k].y;
+      long long X = bad ? 0 : fixed_of_f32(h, q) + fixed_of_f32(l, q);
+#pragma unroll
+      for (int d = HERK_D - 1; d >= 0; --d) {
+        const int dg = d > 0 ? (int)((X + 64) & 127) - 64 : (int)X;
+        X = (X - dg) >> 7;
+        const uint32_t b = __float_as_uint(small_int_to_float(dg)) >> 16;
+        if (k & 1) pk[d][k >> 1] |= b << 16;
+        else pk[d][k >> 1] = b;
+      }
+    }
+    const int tile = row / MT, rr = row - tile * MT;
+#pragma unroll
+    for (int d = 0; d < HERK_D; ++d)
+      *(uint4*)(out + ((((size_t)tile * HERK_KS + (c8 >> 1)) * 2 + plane) * HERK_D + d) * (MT * ROW_BYTES) +
+                swizzle32(rr, c8 & 1)) = make_uint4(pk[d][0], pk[d][1], pk[d][2], pk[d][3]);
+  }
+}
+
+size_t herk_rows(int N) { return (size_t)(N + MT - 1) / MT * MT; }
+size_t herk_operand(int N) { return herk_rows(N) * HERK_COLS * 2 * HERK_D * 2; }
+
 }  // namespace sl
+
+size_t herk_df_bytes(int N) {
+  using namespace sl;
+  return chol_panel(N) == 0 ? 0 : 1024 + 2 * (herk_rows(N) * sizeof(int) + herk_operand(N));
+}
+
+int launch_herk_df(int N, int k0, int R0, void* const* A, int nb, void* scratch, int* status, cudaStream_t s) {
+  using namespace sl;
+  static_assert(2 * sizeof(Gram) <= 768, "table");
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  unsigned char* b = (unsigned char*)scratch;
+  HerkSlices p{};
+  p.N = N; p.k0 = k0; p.R0 = R0; p.ng = nb;
+  p.rpad = (N - R0 + MT - 1) / MT * MT;
+  p.ticket = (unsigned*)b;
+  p.grams = (Gram*)(b + 256);
+  const int tiles = p.rpad / MT, units = tiles * (tiles + 1) / 2 * (MT / 32);
+  GramArgs ga{};
+  for (int m = 0; m < 2; ++m) {
+    const int k = m < nb ? m : 0;
+    p.A[m] = (const float4*)A[k];
+    p.ex[m] = (int*)(b + 1024) + k * herk_rows(N);
+    p.out[m] = b + 1024 + 2 * herk_rows(N) * sizeof(int) + k * herk_operand(N);
+    Gram& g = p.g[m];
+    g.A = p.out[m];
+    g.ea = g.eb = p.ex[m];
+    g.ks = g.drain = HERK_KS;
+    g.da = g.d = g.l = HERK_D;
+    g.t = 32;
+    g.digits = 1;
+    g.b0 = HERK_B0;
+    g.beta = HERK_BETA;
+    g.fbits = 62 - (1 + 7 + 2 * HERK_B0);   // sums of 128 x 2 products below 2^(2 b0)
+    g.unit0 = m * units;
+    ga.herk[m] = (float4*)A[k];
+  }
+  k_herk_slices<<<dim3(p.rpad / 16, nb), 256, 0, s>>>(p);
+  ga.grams = p.grams;
+  ga.ngrams = nb;
+  ga.units = nb * units;
+  ga.N = N;
+  ga.R0 = R0;
+  ga.ticket = p.ticket;
+  ga.status = status;
+  k_gram_sliced<<<std::min(ga.units, sms), THREADS, SMEM_BYTES, s>>>(ga);
+  return 2;
+}
 
 // Layout of the scratch and tables of one handle's assembly.  Built twice: once to size the arena
 // (base NULL), once to fill it.
@@ -1369,7 +1568,7 @@ int AsmPlan::launch(const JobView& j, double2* S, double2* H, cudaStream_t s) co
     unsigned* ticket = (unsigned*)(m.base + m.o_ticket);
     if (m.f64) k_slices<double><<<dim3(b.rowgroups, b.nslice), 256, 0, s>>>(sl0, ticket);
     else k_slices<float><<<dim3(b.rowgroups, b.nslice), 256, 0, s>>>(sl0, ticket);
-    GramArgs ga;
+    GramArgs ga{};
     ga.grams = (const Gram*)(m.base + m.o_grams) + b.gram0;
     ga.out = nullptr;
     ga.ngrams = b.ngram;
@@ -1414,7 +1613,7 @@ int AsmPlan::reconstruct(const JobView& j, const double2* C, double2* Psi, cudaS
   sR.out = m.base + m.r_Rb; sR.ex = (int*)(m.base + m.r_Re);
   sR.n = j.nR; sR.rpad = rRp; sR.R = 32;
   k_slices_t<<<dim3(std::max(rxp, rRp) / ST_ROWS, 2), ST_WARPS * 32, 0, s>>>(sx, sR, (unsigned*)(m.base + m.o_ticket));
-  GramArgs ga;
+  GramArgs ga{};
   ga.grams = (const Gram*)(m.base + m.o_grams) + m.rec_gram;
   ga.out = Psi;
   ga.ngrams = 1;

@@ -1,7 +1,9 @@
 """The cluster's triangular solves, double-float and FP64, at the edges of their 32-row blocks and of the
 16 warps: one block (no neighbour products), two and three (every block among the first three rows), a
 ragged last block, 16 / 17 and 32 / 33 blocks (a warp's second and third block), 64 (the largest), and a
-restored state, whose neighbour products are recomputed from the saved factor.
+restored state, whose neighbour products are recomputed from the saved factor.  From 27 blocks on the
+double-float factorisation behind them has tensor-core trailing updates (832: the last single launch,
+833 and 959: ragged trailing matrices after the first panel, 2048: ten panels).
 
 Bounds of the residual, fixed beforehand.  Double-float: 2^-44 per operation, N <= 545 terms per entry and
 the explicit inverses of 32 x 32 diagonal blocks with condition numbers up to 1 / eps = 1e4 give 545 *
@@ -21,7 +23,7 @@ EPS = 1e-4
 
 
 @pytest.mark.parametrize("fp64", [0, 1])
-@pytest.mark.parametrize("N", [1, 2, 31, 32, 33, 64, 65, 96, 97, 129, 511, 512, 513, 545, 1024, 1025, 2048])
+@pytest.mark.parametrize("N", [1, 2, 31, 32, 33, 64, 65, 96, 97, 129, 511, 512, 513, 545, 832, 833, 959, 1024, 1025, 2048])
 def test_residual_and_restored_state(N, fp64):
     w = shin_metiu(n_traj=N, svd_rel_cutoff=1e-8, s_reg_eps=EPS if N <= 1024 else 1e-3)
     eps = w.s_reg_eps
