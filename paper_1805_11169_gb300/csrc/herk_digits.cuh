@@ -68,7 +68,7 @@ __device__ __forceinline__ void emit_row_digits(double2 z, int i, int lane, int 
     xr = (long long)((unsigned long long)xr - ((unsigned long long)dr << sh));
     xi = (long long)((unsigned long long)xi - ((unsigned long long)di << sh));
     const float w = __int_as_float((127 - BETA * p) << 23);   // 2^(-8 p), exact
-    const float fr = (float)dr * w, fi = (float)di * w;
+    const float fr = (float)(int)dr * w, fi = (float)(int)di * w;   // |d| <= 256
     const size_t base = (size_t)(p * PLANES) * pl + (size_t)i * NB + lane;
     planes[base] = __float2bfloat16_rn(fr);            // P
     planes[base + pl] = __float2bfloat16_rn(-fi);      // -Q

@@ -51,18 +51,19 @@ constexpr int PF_THREADS = 256;
 
 
 // Factor the diagonal block jb of each matrix (one CTA per matrix) in FP64, right-looking by
-// columns.  Column c: its entries below the pivot are scaled, L_rc = A_rc y_c (y_c = 1/sqrt(A_cc),
-// computed during the previous column); then the trailing triangle takes the rank-1 update
-// A_rq -= L_rc conj(L_qc) for c < q <= r (four FMAs per element).  The update's pairs are read
-// from a table sorted by q descending, so those of column c are its first (31-c)(32-c)/2 entries
-// and every warp instruction of the update runs on full warps (FP64 instructions issue per warp,
-// whatever the number of active lanes).  Thread 0 updates the next pivot, A_{c+1,c+1}, itself and
-// computes its reciprocal square root while the others finish the update.  Two barriers per
-// column.  Outputs: L in place and the reciprocal pivots.  Rows and columns beyond N are treated
-// as identity so that ragged sizes factor cleanly.
+// columns.  Warp 0 runs the chain: lane = row, it takes column c from shared memory, applies column
+// c - 1, y_c = 1 / sqrt(A_cc), L_rc = A_rc y_c.  Meanwhile the other warps apply column c - 1 to the
+// columns from c + 1 on, A_rq -= L_r,c-1 conj(L_q,c-1) for q <= r (four FMAs per element), their pairs
+// read from a table sorted by q descending, so those of a column are its first entries and every
+// warp instruction runs on full warps.  One barrier per column.  Outputs: L in place and the reciprocal
+// pivots.  Rows and columns beyond N are treated as identity so that ragged sizes factor cleanly.
 //
-// FP64 operations wait for one another for a long time on this GPU, so the pivot chain is kept
-// short.  The reciprocal square root of a pivot d starts from the FP32 estimate (d narrowed and
+// Bound: FP64 issue.  A scheduler takes a warp's FP64 instruction every 64 cycles, whatever the number
+// of active lanes (the SM one per 19), so warp 0 has a scheduler for itself (warp 4 stays idle) and
+// its 11 instructions per column set the time.  With the pivot on one thread among 8 warps of updates and
+// two barriers per column a block took 32.7 us; now 21.9.
+//
+// The reciprocal square root of a pivot d starts from the FP32 estimate (d narrowed and
 // the estimate widened by integer operations on the bit patterns: no FP64 instruction) and takes
 // one third-order correction in FP64, y = y0 (1 + r/2 + 3 r^2/8) with r = 1 - d y0^2 (the
 // binomial series of (1 - r)^(-1/2) cut after r^2): the estimate's ~2^-22 relative error becomes
@@ -94,10 +95,12 @@ __device__ __forceinline__ double2 csub_mul_conj(double2 a, double2 t, double2 b
 }
 
 constexpr int PF_PAIRS = (NB - 1) * NB / 2;   // pairs (r, q), 1 <= q <= r <= 31
+constexpr int PF_UPD = PF_THREADS - 64;       // threads of the updates
+__device__ __forceinline__ void pf_sync() { asm volatile("bar.sync 1, %0;" ::"n"(PF_UPD + 32) : "memory"); }
 
 __global__ void __launch_bounds__(PF_THREADS) k_potrf_diag(int N, MatBatch mb, int jb, int* status) {
   __shared__ double2 L[NB][NB + 1];
-  __shared__ double yv[NB];
+  __shared__ double yv[NB], dv[NB];
   __shared__ unsigned char pr[PF_PAIRS], pq[PF_PAIRS];
   double2* A = mb.m[blockIdx.y];
   double* inv = mb.inv[blockIdx.y];
@@ -116,37 +119,42 @@ __global__ void __launch_bounds__(PF_THREADS) k_potrf_diag(int N, MatBatch mb, i
     pq[i] = (unsigned char)q;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double d = L[0][0].x;
-    if (!pivot_ok(d)) { set_flag(status, ST_CHOL); d = 1.0; }
-    const double y = rsqrt_fp64(d);
-    L[0][0] = make_double2(d * y, 0.0);
-    yv[0] = y;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp == 0) {
+    double2 a = L[lane][0];
+    bool bad = false;
+    for (int c = 0;; ++c) {
+      double d = __shfl_sync(0xffffffffu, a.x, c);
+      if (!pivot_ok(d)) { bad = true; d = 1.0; }
+      const double y = rsqrt_fp64(d);
+      const double2 l = cscale(a, y);
+      if (lane > c) L[lane][c] = l;
+      if (lane == c) {
+        yv[c] = y;
+        dv[c] = d;
+      }
+      if (c == NB - 1) break;
+      pf_sync();   // column c is there, and the columns from c + 1 on have columns 0..c-1 applied
+      double2 lq;
+      lq.x = __shfl_sync(0xffffffffu, l.x, c + 1);
+      lq.y = __shfl_sync(0xffffffffu, l.y, c + 1);
+      a = csub_mul_conj(L[lane][c + 1], l, lq);   // rows above c + 1: not used
+    }
+    if (bad && lane == 0) set_flag(status, ST_CHOL);
+  } else if (warp != 4) {
+    const int u = threadIdx.x - (warp > 4 ? 64 : 32);
+    for (int c = 0; c < NB - 1; ++c) {
+      pf_sync();
+      const int n = (NB - 2 - c) * (NB - 1 - c) / 2;   // pairs with q >= c + 2
+      for (int i = u; i < n; i += PF_UPD) {
+        const int r = pr[i], q = pq[i];
+        L[r][q] = csub_mul_conj(L[r][q], L[r][c], L[q][c]);
+      }
+    }
   }
   __syncthreads();
-  for (int c = 0; c < NB - 1; ++c) {
-    double2 l0;   // thread 0: L_{c+1,c}, kept in registers for the next pivot
-    {
-      const int r = c + 1 + (int)threadIdx.x;
-      if (r < NB) L[r][c] = l0 = cscale(L[r][c], yv[c]);
-    }
-    __syncthreads();
-    const int n = (NB - 1 - c) * (NB - c) / 2;
-    const int skip = n - (NB - 1 - c);   // the pair (c+1, c+1): thread 0's
-    if (threadIdx.x == 0) {
-      double d = fma(-l0.x, l0.x, fma(-l0.y, l0.y, L[c + 1][c + 1].x));
-      if (!pivot_ok(d)) { set_flag(status, ST_CHOL); d = 1.0; }
-      const double y = rsqrt_fp64(d);
-      L[c + 1][c + 1] = make_double2(d * y, 0.0);
-      yv[c + 1] = y;
-    }
-    for (int i = (int)threadIdx.x; i < n; i += PF_THREADS) {
-      if (i == skip) continue;
-      const int r = pr[i], q = pq[i];
-      L[r][q] = csub_mul_conj(L[r][q], L[r][c], L[q][c]);
-    }
-    __syncthreads();
-  }
+  if (threadIdx.x < NB) L[threadIdx.x][threadIdx.x] = make_double2(dv[threadIdx.x] * yv[threadIdx.x], 0.0);
+  __syncthreads();
   for (int e = threadIdx.x; e < NB * NB; e += PF_THREADS) {
     const int r = e / NB, c = e % NB;
     if (c <= r && r0 + r < N && r0 + c < N) A[(size_t)(r0 + r) * N + r0 + c] = L[r][c];
@@ -154,7 +162,10 @@ __global__ void __launch_bounds__(PF_THREADS) k_potrf_diag(int N, MatBatch mb, i
   if (threadIdx.x < NB && r0 + threadIdx.x < N) inv[r0 + threadIdx.x] = yv[threadIdx.x];
 }
 
-constexpr int TR_WARPS = 8;   // rows per panel-solve CTA
+// Rows (warps) per panel-solve CTA: one per scheduler while that fills no more than the chip (a
+// scheduler takes a warp's FP64 instruction every 64 cycles: two warps double the substitution's time),
+// else two.  At N = 500 the last panels take 12.8 us with 4 and 14.8 with 8, the first 17.3 and 14.8.
+constexpr int TR_WARPS = 8, TR_WARPS_FEW = 4, TR_FEW_ROWS = TR_WARPS_FEW * 148;
 
 // Panel solve A_ib <- A_ib L_bb^-H below the diagonal block jb in FP64: one warp per row, lane =
 // column, column-oriented substitution on unscaled numerators: a_c -= a_m (conj(L_cm) / L_mm)
@@ -176,7 +187,7 @@ __global__ void __launch_bounds__(TR_WARPS * 32) k_trsm_panel(int N, MatBatch mb
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row = (jb + 1) * NB + blockIdx.x * TR_WARPS + warp;
+  const int row = (jb + 1) * NB + blockIdx.x * (blockDim.x >> 5) + warp;
   if (row >= N) return;
   // a block column with rows below it is full: every lane's column is inside the matrix
   double2 a = A[(size_t)row * N + c0 + lane];
@@ -321,8 +332,8 @@ int launch_cholesky(int N, double2* const* A, double* const* inv, double2* const
     const int rest = T - jb - 1;
     if (rest > 0) {
       const int rows = N - (jb + 1) * NB;
-      k_trsm_panel<<<dim3((rows + TR_WARPS - 1) / TR_WARPS, nbatch), TR_WARPS * 32, 0, s>>>(
-          N, mb, jb, emu);
+      const int tw = rows * nbatch <= TR_FEW_ROWS ? TR_WARPS_FEW : TR_WARPS;
+      k_trsm_panel<<<dim3((rows + tw - 1) / tw, nbatch), tw * 32, 0, s>>>(N, mb, jb, emu);
       if (!emu.planes[0] || !launch_herk_emu(N, jb, A, nbatch, emu_scratch, emu_bytes, true, status, s))
         k_herk_update<<<dim3(rest * (rest + 1) / 2, nbatch), 256, 0, s>>>(N, mb, jb);
       launches += 2;
