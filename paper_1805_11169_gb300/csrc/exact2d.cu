@@ -4,64 +4,37 @@
 // This is the reference the paper's figures compare the ICWF densities, populations and
 // decoherence indicators with.  FP64; Psi row-major nx x nR (x slow).
 //
-// One step is three kernels:
-//   k_rows (forward): per x row, multiply by e^{-i V dt/2}, radix-2 FFT along R (bit-reversed out);
-//   k_cols: per group of CB adjacent R columns (coalesced CB-wide loads), FFT along x, multiply by
-//           the kinetic phase of (kx, kR) (both tables bit-reversed, 1/n folded in), inverse FFT
-//           along x;
-//   k_rows (inverse): per x row, inverse FFT along R (natural order out), multiply by the half
-//           potential phase.
+// A step is two kernels, with one more at the end of a run of steps:
+//   k_rows: per x row, inverse FFT along R of the step before (not at the start), the potential phase
+//           (half of it at the start and the end, the whole between two steps), FFT along R;
+//   k_cols: per group of CB adjacent R columns, FFT along x, the kinetic phase of (kx, kR) (both tables
+//           bit-reversed, 1/n folded in), inverse FFT along x.
+// Both turn around in registers: the last stages of one transform, the phase and the first stages of
+// the other are one pass (fft_reg.cuh).
+// Bound: FP64 instructions, 112 per point and step at 1024 x 512 (172 with radix-2 passes of eight
+// instructions per butterfly, three kernels and both half phases).  50 steps and the observables there:
+// 11.2 ms before, 7.45 now.
 // Observables use per-row / per-CTA partial sums finished on the host in a fixed order.
 #include <cuda_runtime.h>
 
 #include <cmath>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/icwf_exact2d.h"
 #include "icwf_internal.h"
 #include "k_common.cuh"
+#include "fft_reg.cuh"
 
 namespace icwf {
 namespace e2d {
 
 constexpr int TPB = 256;
 constexpr int MAX_STATES = 8;
-
-// nb transforms of length n = 2^logn stored back to back in shared memory; all threads take part.
-__device__ __forceinline__ void fft_dif_b(double2* buf, const double2* __restrict__ tw, int n,
-                                          int logn, int nb) {
-  const int half = n >> 1;
-  for (int s = logn - 1; s >= 0; --s) {
-    const int h = 1 << s, tstride = n >> (s + 1);
-    for (int idx = threadIdx.x; idx < nb * half; idx += blockDim.x) {
-      const int b = idx >> (logn - 1), id = idx & (half - 1);
-      const int j = id & (h - 1);
-      const int i1 = b * n + ((id >> s) << (s + 1)) + j, i2 = i1 + h;
-      const double2 u = buf[i1], v = buf[i2];
-      buf[i1] = cadd(u, v);
-      buf[i2] = cmul(csub(u, v), tw[j * tstride]);
-    }
-    __syncthreads();
-  }
-}
-__device__ __forceinline__ void ifft_dit_b(double2* buf, const double2* __restrict__ tw, int n,
-                                           int logn, int nb) {
-  const int half = n >> 1;
-  for (int s = 0; s < logn; ++s) {
-    const int h = 1 << s, tstride = n >> (s + 1);
-    for (int idx = threadIdx.x; idx < nb * half; idx += blockDim.x) {
-      const int b = idx >> (logn - 1), id = idx & (half - 1);
-      const int j = id & (h - 1);
-      const int i1 = b * n + ((id >> s) << (s + 1)) + j, i2 = i1 + h;
-      const double2 u = buf[i1];
-      const double2 t = cmul(buf[i2], cconj(tw[j * tstride]));
-      buf[i1] = cadd(u, t);
-      buf[i2] = csub(u, t);
-    }
-    __syncthreads();
-  }
-}
+// R columns per CTA of k_cols: a 32-byte sector; several CTAs per SM up to nx = 2048
+constexpr int CB = 2;
+using fftr::Tw;
 
 __device__ __forceinline__ double block_sum(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -75,68 +48,129 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;   // valid in thread 0
 }
 
-// One x row per CTA.  inverse = 0: out = FFT_R(half * in) (half may be null); inverse = 1:
-// out = half * IFFT_R(in).  in and out may alias.
-__global__ void __launch_bounds__(TPB) k_rows(const double2* in, double2* out,
-                                              const double2* __restrict__ half,
-                                              const double2* __restrict__ tw, int nR, int logR,
-                                              int inverse) {
+// One x row per CTA: inverse FFT (INV), times ph (may be null), FFT (FWD).  in and out may alias.
+template <int L, bool INV, bool FWD>
+__global__ void __launch_bounds__(TPB) k_rows(const double2* in, double2* out, const double2* __restrict__ ph,
+                                              const Tw* __restrict__ tf, const Tw* __restrict__ ti) {
   extern __shared__ __align__(16) double2 buf[];
-  const size_t base = (size_t)blockIdx.x * nR;
-  for (int j = threadIdx.x; j < nR; j += blockDim.x) {
+  constexpr int n = 1 << L;
+  const size_t base = (size_t)blockIdx.x * n;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
     double2 z = in[base + j];
-    if (!inverse && half) z = cmul(half[base + j], z);
-    buf[j] = z;
+    if (!INV && ph) z = cmul(ph[base + j], z);
+    buf[fftr::pad(j)] = z;
   }
   __syncthreads();
-  if (inverse) ifft_dit_b(buf, tw, nR, logR, 1);
-  else fft_dif_b(buf, tw, nR, logR, 1);
-  for (int j = threadIdx.x; j < nR; j += blockDim.x) {
-    double2 z = buf[j];
-    if (inverse && half) z = cmul(half[base + j], z);
+  if (INV && FWD) {
+    if (fftr::passes(L)) fftr::inv_pass<L, 3, 0>(buf, ti, 1);
+    fftr::inv_passes<L, fftr::passes(L) - 1, 1>(buf, ti, 1);
+    fftr::turn_space<L>(buf, tf, ti, [&](int j, double2 z) { return cmul(ph[base + j], z); });
+    fftr::fwd_passes<L, 1, fftr::passes(L)>(buf, tf, 1);
+    if (fftr::passes(L)) fftr::fwd_pass<L, 3, L - 3>(buf, tf, 1);
+  } else if (INV) {
+    fftr::inv_all<L>(buf, ti, 1);
+  } else {
+    fftr::fwd_all<L>(buf, tf, 1);
+  }
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    double2 z = buf[fftr::pad(j)];
+    if (INV && !FWD) z = cmul(ph[base + j], z);
     out[base + j] = z;
   }
 }
 
-// CB adjacent R columns per CTA (bit-reversed R frequencies after k_rows).  mode 0: FFT along x,
-// multiply by kinx[m] kinR[col], inverse FFT along x, store.  mode 1: FFT along x and
+// CB adjacent R columns per CTA (bit-reversed R frequencies after k_rows).  ENERGY false: FFT along x,
+// multiply by kinx[m] kinR[col], inverse FFT along x, store.  ENERGY true: FFT along x and
 // part[blockIdx.x] = sum |F|^2 (Tx[m] + TR[col]) (kinetic energy, not stored).
+template <int L, bool ENERGY>
 __global__ void __launch_bounds__(TPB) k_cols(double2* a, const double2* __restrict__ kinx,
-                                              const double2* __restrict__ kinR,
-                                              const double2* __restrict__ tw, int nx, int logx,
-                                              int nR, int CB, int mode,
-                                              const double* __restrict__ Tx,
+                                              const double2* __restrict__ kinR, const Tw* __restrict__ tf,
+                                              const Tw* __restrict__ ti, int nR, const double* __restrict__ Tx,
                                               const double* __restrict__ TR, double* part) {
-  extern __shared__ __align__(16) double2 buf[];   // [CB][nx]
+  extern __shared__ __align__(16) double2 buf[];   // [CB][padded n]
   __shared__ double red[TPB / 32];
+  constexpr int n = 1 << L;
   const int j0 = blockIdx.x * CB;
-  for (int e = threadIdx.x; e < nx * CB; e += blockDim.x) {
-    const int i = e / CB, c = e - i * CB;
-    buf[c * nx + i] = a[(size_t)i * nR + j0 + c];
+  for (int e = threadIdx.x; e < n * CB; e += blockDim.x) {
+    const int i = e / CB, c = e % CB;
+    buf[c * fftr::padded(n) + fftr::pad(i)] = a[(size_t)i * nR + j0 + c];
   }
   __syncthreads();
-  fft_dif_b(buf, tw, nx, logx, CB);
-  if (mode == 0) {
-    for (int e = threadIdx.x; e < nx * CB; e += blockDim.x) {
-      const int c = e / nx, m = e - c * nx;
-      buf[e] = cmul(buf[e], cmul(kinx[m], kinR[j0 + c]));
-    }
-    __syncthreads();
-    ifft_dit_b(buf, tw, nx, logx, CB);
-    for (int e = threadIdx.x; e < nx * CB; e += blockDim.x) {
-      const int i = e / CB, c = e - i * CB;
-      a[(size_t)i * nR + j0 + c] = buf[c * nx + i];
+  fftr::fwd_passes<L, 0, fftr::passes(L)>(buf, tf, CB);
+  if (!ENERGY) {
+    double2 kr[CB];
+#pragma unroll
+    for (int c = 0; c < CB; ++c) kr[c] = kinR[j0 + c];
+    fftr::turn_freq<L>(buf, tf, ti, CB, [&](int c, int m, double2 z) {
+      double2 k = kr[0];
+#pragma unroll
+      for (int q = 1; q < CB; ++q) if (c == q) k = kr[q];
+      return cmul(z, cmul(kinx[m], k));
+    });
+    fftr::inv_passes<L, fftr::passes(L) - 1, 0>(buf, ti, CB);
+    for (int e = threadIdx.x; e < n * CB; e += blockDim.x) {
+      const int i = e / CB, c = e % CB;
+      a[(size_t)i * nR + j0 + c] = buf[c * fftr::padded(n) + fftr::pad(i)];
     }
   } else {
+    fftr::fwd_pass<L, 3, L - 3>(buf, tf, CB);
     double s = 0.0;
-    for (int e = threadIdx.x; e < nx * CB; e += blockDim.x) {
-      const int c = e / nx, m = e - c * nx;
-      const double2 z = buf[e];
+    for (int e = threadIdx.x; e < n * CB; e += blockDim.x) {
+      const int c = e >> L, m = e & (n - 1);
+      const double2 z = buf[c * fftr::padded(n) + fftr::pad(m)];
       s += (z.x * z.x + z.y * z.y) * (Tx[m] + TR[j0 + c]);
     }
     s = block_sum(s, red);
     if (threadIdx.x == 0) part[blockIdx.x] = s;
   }
+}
+
+int smem_rows(int n) { return fftr::padded(n) * (int)sizeof(double2); }
+int smem_cols(int n) { return CB * smem_rows(n); }
+// a thread per group of eight points, up to TPB
+int threads(int points) { return points / 8 < 32 ? 32 : (points / 8 > TPB ? TPB : points / 8); }
+
+// f(std::integral_constant<int, L>) for L = log2 of a grid of 8 .. 4096 points
+template <typename F>
+void by_size(int L, const F& f) {
+  switch (L) {
+    case 3: f(std::integral_constant<int, 3>()); break;
+    case 4: f(std::integral_constant<int, 4>()); break;
+    case 5: f(std::integral_constant<int, 5>()); break;
+    case 6: f(std::integral_constant<int, 6>()); break;
+    case 7: f(std::integral_constant<int, 7>()); break;
+    case 8: f(std::integral_constant<int, 8>()); break;
+    case 9: f(std::integral_constant<int, 9>()); break;
+    case 10: f(std::integral_constant<int, 10>()); break;
+    case 11: f(std::integral_constant<int, 11>()); break;
+    case 12: f(std::integral_constant<int, 12>()); break;
+  }
+}
+template <bool INV, bool FWD>
+void rows(int nx, int nR, int logR, const double2* in, double2* out, const double2* ph, const Tw* tf, const Tw* ti,
+          cudaStream_t s) {
+  by_size(logR, [&](auto L) {
+    k_rows<L(), INV, FWD><<<nx, threads(nR), smem_rows(nR), s>>>(in, out, ph, tf, ti);
+  });
+}
+template <bool ENERGY>
+void cols(int nx, int nR, int logx, double2* a, const double2* kinx, const double2* kinR, const Tw* tf, const Tw* ti,
+          const double* Tx, const double* TR, double* part, cudaStream_t s) {
+  by_size(logx, [&](auto L) {
+    k_cols<L(), ENERGY><<<nR / CB, threads(CB * nx), smem_cols(nx), s>>>(a, kinx, kinR, tf, ti, nR, Tx, TR, part);
+  });
+}
+// the largest dynamic shared memory any handle uses, so that handles of different sizes can coexist
+void attributes() {
+  for (int l = 3; l <= 12; ++l)
+    by_size(l, [&](auto L) {
+      const int r = smem_rows(1 << L()), c = smem_cols(1 << L());
+      cudaFuncSetAttribute(k_rows<L(), false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, r);
+      cudaFuncSetAttribute(k_rows<L(), true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, r);
+      cudaFuncSetAttribute(k_rows<L(), true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, r);
+      cudaFuncSetAttribute(k_cols<L(), false>, cudaFuncAttributeMaxDynamicSharedMemorySize, c);
+      cudaFuncSetAttribute(k_cols<L(), true>, cudaFuncAttributeMaxDynamicSharedMemorySize, c);
+    });
 }
 
 // Per x row: dens[i] = sum_j |Psi|^2, pot[i] = sum_j |Psi|^2 V.
@@ -198,14 +232,16 @@ int ilog2i(int n) {
   return l;
 }
 
-// kin[mp] = e^{-i k^2 dt / 2m} / n and T[mp] = k^2 / 2m at bit-reversed position mp; tw = e^{-2 pi i k / n}.
-void tables(int n, double d, double mass, double dt, std::vector<double2>& kin,
-            std::vector<double>& T, std::vector<double2>& tw) {
+// kin[mp] = e^{-i k^2 dt / 2m} / n and T[mp] = k^2 / 2m at bit-reversed position mp; tf, ti: forward
+// twiddles by block, inverse ones by position.
+void tables(int n, double d, double mass, double dt, std::vector<double2>& kin, std::vector<double>& T,
+            std::vector<Tw>& tf, std::vector<Tw>& ti) {
   const int logn = ilog2i(n);
   const double PI = 3.14159265358979323846;
   kin.resize(n);
   T.resize(n);
-  tw.resize(n / 2);
+  tf.resize(n / 2);
+  ti.resize(n / 2);
   for (int mp = 0; mp < n; ++mp) {
     int m = 0;
     for (int b = 0; b < logn; ++b)
@@ -216,9 +252,17 @@ void tables(int n, double d, double mass, double dt, std::vector<double2>& kin,
     T[mp] = e;
     kin[mp] = make_double2(std::cos(-e * dt) / n, std::sin(-e * dt) / n);
   }
+  // w = m (1 + i r), or -i m (1 + i r) i = m (1 + i r) with cos, sin of the angle minus 90 degrees
+  auto entry = [](double angle, int form) {
+    const double c = std::cos(angle), sn = std::sin(angle);
+    return form ? Tw{sn, -c / sn} : Tw{c, sn / c};
+  };
   for (int k = 0; k < n / 2; ++k) {
-    const double a = -2.0 * PI * (double)k / (double)n;
-    tw[k] = make_double2(std::cos(a), std::sin(a));
+    double v = 0.0;
+    for (int b = 0; b < logn - 1; ++b)
+      if (k & (1 << b)) v += std::ldexp(1.0, -1 - b);
+    tf[k] = entry(-PI * v, fftr::fwd_form(k));
+    ti[k] = entry(2.0 * PI * (double)k / (double)n, fftr::inv_form(k, logn));
   }
 }
 
@@ -228,14 +272,15 @@ void tables(int n, double d, double mass, double dt, std::vector<double2>& kin,
 using namespace icwf;
 
 struct icwf_exact2d_ctx {
-  int nx = 0, nR = 0, logx = 0, logR = 0, CB = 1, ns = 0;
+  int nx = 0, nR = 0, logx = 0, logR = 0, ns = 0;
   double dx = 0, dR = 0, dt = 0, t = 0;
   bool has_state = false;
   cudaStream_t stream = nullptr;
   std::vector<void*> allocs;
   double* V = nullptr;
-  double2 *half = nullptr, *psi = nullptr, *work = nullptr;
-  double2 *kinx = nullptr, *kinR = nullptr, *twx = nullptr, *twR = nullptr;
+  double2 *half = nullptr, *full = nullptr, *psi = nullptr, *work = nullptr;   // phases of V dt/2, V dt
+  double2 *kinx = nullptr, *kinR = nullptr;
+  e2d::Tw *tfx = nullptr, *tix = nullptr, *tfR = nullptr, *tiR = nullptr;
   double *Tx = nullptr, *TR = nullptr, *phi = nullptr;
   double *dens_x = nullptr, *pot = nullptr, *dens_R = nullptr, *part = nullptr;
   double2* proj = nullptr;
@@ -304,18 +349,16 @@ icwf_status icwf_exact2d_create(const icwf_params* p, const double* V, icwf_exac
   h->dx = (p->x_max - p->x_min) / p->nx;
   h->dR = (p->R_max - p->R_min) / p->nR;
   h->dt = p->dt;
-  // columns per CTA: as many as fit 96 KB of shared memory, at most 8 (a power of two <= nR)
-  h->CB = 8;
-  while (h->CB > 1 && (size_t)h->CB * h->nx * sizeof(double2) > 96 * 1024) h->CB >>= 1;
   const size_t NN = (size_t)h->nx * h->nR;
   if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess) {
     delete h;
     return fail2(nullptr, ICWF_ERR_CUDA, "icwf_exact2d_create: cudaStreamCreate failed");
   }
-  const int ncb = h->nR / h->CB;
-  if (!dalloc(h, &h->V, NN) || !dalloc(h, &h->half, NN) || !dalloc(h, &h->psi, NN) ||
+  const int ncb = h->nR / e2d::CB;
+  if (!dalloc(h, &h->V, NN) || !dalloc(h, &h->half, NN) || !dalloc(h, &h->full, NN) || !dalloc(h, &h->psi, NN) ||
       !dalloc(h, &h->work, NN) || !dalloc(h, &h->kinx, h->nx) || !dalloc(h, &h->kinR, h->nR) ||
-      !dalloc(h, &h->twx, h->nx / 2) || !dalloc(h, &h->twR, h->nR / 2) ||
+      !dalloc(h, &h->tfx, h->nx / 2) || !dalloc(h, &h->tix, h->nx / 2) ||
+      !dalloc(h, &h->tfR, h->nR / 2) || !dalloc(h, &h->tiR, h->nR / 2) ||
       !dalloc(h, &h->Tx, h->nx) || !dalloc(h, &h->TR, h->nR) || !dalloc(h, &h->dens_x, h->nx) ||
       !dalloc(h, &h->pot, h->nx) || !dalloc(h, &h->dens_R, h->nR) || !dalloc(h, &h->part, ncb) ||
       !dalloc(h, &h->proj, (size_t)e2d::MAX_STATES * h->nR)) {
@@ -323,18 +366,22 @@ icwf_status icwf_exact2d_create(const icwf_params* p, const double* V, icwf_exac
     delete h;
     return fail2(nullptr, ICWF_ERR_OOM, "icwf_exact2d_create: cudaMalloc failed");
   }
-  std::vector<double2> half(NN), kx, kR, tx, tR;
+  std::vector<double2> half(NN), full(NN), kx, kR;
+  std::vector<e2d::Tw> fx, ix, fR, iR;
   std::vector<double> Tx, TR;
-  for (size_t e = 0; e < NN; ++e)
+  for (size_t e = 0; e < NN; ++e) {
     half[e] = make_double2(std::cos(-0.5 * p->dt * V[e]), std::sin(-0.5 * p->dt * V[e]));
-  e2d::tables(h->nx, h->dx, p->mass_x, p->dt, kx, Tx, tx);
-  e2d::tables(h->nR, h->dR, p->mass_R, p->dt, kR, TR, tR);
+    full[e] = make_double2(std::cos(-p->dt * V[e]), std::sin(-p->dt * V[e]));
+  }
+  e2d::tables(h->nx, h->dx, p->mass_x, p->dt, kx, Tx, fx, ix);
+  e2d::tables(h->nR, h->dR, p->mass_R, p->dt, kR, TR, fR, iR);
   const auto H2D = cudaMemcpyHostToDevice;
   bool ok = copy(h, h->V, V, NN * 8, H2D) && copy(h, h->half, half.data(), NN * 16, H2D) &&
+            copy(h, h->full, full.data(), NN * 16, H2D) &&
             copy(h, h->kinx, kx.data(), kx.size() * 16, H2D) &&
             copy(h, h->kinR, kR.data(), kR.size() * 16, H2D) &&
-            copy(h, h->twx, tx.data(), tx.size() * 16, H2D) &&
-            copy(h, h->twR, tR.data(), tR.size() * 16, H2D) &&
+            copy(h, h->tfx, fx.data(), fx.size() * 16, H2D) && copy(h, h->tix, ix.data(), ix.size() * 16, H2D) &&
+            copy(h, h->tfR, fR.data(), fR.size() * 16, H2D) && copy(h, h->tiR, iR.data(), iR.size() * 16, H2D) &&
             copy(h, h->Tx, Tx.data(), Tx.size() * 8, H2D) &&
             copy(h, h->TR, TR.data(), TR.size() * 8, H2D);
   if (!ok) {
@@ -342,11 +389,7 @@ icwf_status icwf_exact2d_create(const icwf_params* p, const double* V, icwf_exac
     delete h;
     return fail2(nullptr, ICWF_ERR_CUDA, "icwf_exact2d_create: upload failed");
   }
-  // the largest dynamic shared memory any handle uses (nR <= 4096 rows, CB * nx <= 96 KB), so
-  // that handles of different sizes can coexist
-  cudaFuncSetAttribute(e2d::k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       4096 * (int)sizeof(double2));
-  cudaFuncSetAttribute(e2d::k_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+  e2d::attributes();
   *out = h;
   return ICWF_OK;
 }
@@ -378,16 +421,16 @@ icwf_status icwf_exact2d_step(icwf_exact2d h, int32_t n_steps) {
   if (!h) return fail2(h, ICWF_ERR_ARG, "icwf_exact2d_step: null handle");
   if (n_steps < 0) return fail2(h, ICWF_ERR_ARG, "icwf_exact2d_step: n_steps < 0");
   if (!h->has_state) return fail2(h, ICWF_ERR_STATE, "icwf_exact2d_step: no state set");
-  const int smr = h->nR * (int)sizeof(double2), smc = h->CB * h->nx * (int)sizeof(double2);
   for (int s = 0; s < n_steps; ++s) {
-    e2d::k_rows<<<h->nx, e2d::TPB, smr, h->stream>>>(h->psi, h->psi, h->half, h->twR, h->nR,
-                                                     h->logR, 0);
-    e2d::k_cols<<<h->nR / h->CB, e2d::TPB, smc, h->stream>>>(h->psi, h->kinx, h->kinR, h->twx,
-                                                             h->nx, h->logx, h->nR, h->CB, 0,
-                                                             nullptr, nullptr, nullptr);
-    e2d::k_rows<<<h->nx, e2d::TPB, smr, h->stream>>>(h->psi, h->psi, h->half, h->twR, h->nR,
-                                                     h->logR, 1);
+    if (s == 0)
+      e2d::rows<false, true>(h->nx, h->nR, h->logR, h->psi, h->psi, h->half, h->tfR, h->tiR, h->stream);
+    else
+      e2d::rows<true, true>(h->nx, h->nR, h->logR, h->psi, h->psi, h->full, h->tfR, h->tiR, h->stream);
+    e2d::cols<false>(h->nx, h->nR, h->logx, h->psi, h->kinx, h->kinR, h->tfx, h->tix, nullptr, nullptr, nullptr,
+                     h->stream);
   }
+  if (n_steps > 0)
+    e2d::rows<true, false>(h->nx, h->nR, h->logR, h->psi, h->psi, h->half, h->tfR, h->tiR, h->stream);
   const icwf_status st = sync(h, "icwf_exact2d_step");
   if (st == ICWF_OK) h->t += n_steps * h->dt;
   return st;
@@ -404,14 +447,12 @@ icwf_status icwf_exact2d_get_state(icwf_exact2d h, double* psi) {
 icwf_status icwf_exact2d_observables(icwf_exact2d h, icwf_obs* out) {
   if (!h || !out) return fail2(h, ICWF_ERR_ARG, "icwf_exact2d_observables: null pointer");
   if (!h->has_state) return fail2(h, ICWF_ERR_STATE, "icwf_exact2d_observables: no state set");
-  const int nx = h->nx, nR = h->nR, ncb = nR / h->CB;
-  const int smr = nR * (int)sizeof(double2), smc = h->CB * nx * (int)sizeof(double2);
+  const int nx = h->nx, nR = h->nR, ncb = nR / e2d::CB;
   e2d::k_dens_rows<<<nx, e2d::TPB, 0, h->stream>>>(h->psi, h->V, nR, h->dens_x, h->pot);
   e2d::k_cols_obs<<<nR, e2d::TPB, 0, h->stream>>>(h->psi, nx, nR, h->phi, h->ns, h->dens_R, h->proj);
   // kinetic energy: 2D FFT of Psi into work, then sum |F|^2 (Tx + TR) per column group
-  e2d::k_rows<<<nx, e2d::TPB, smr, h->stream>>>(h->psi, h->work, nullptr, h->twR, nR, h->logR, 0);
-  e2d::k_cols<<<ncb, e2d::TPB, smc, h->stream>>>(h->work, nullptr, nullptr, h->twx, nx, h->logx,
-                                                 nR, h->CB, 1, h->Tx, h->TR, h->part);
+  e2d::rows<false, true>(nx, nR, h->logR, h->psi, h->work, nullptr, h->tfR, h->tiR, h->stream);
+  e2d::cols<true>(nx, nR, h->logx, h->work, nullptr, nullptr, h->tfx, h->tix, h->Tx, h->TR, h->part, h->stream);
   icwf_status st = sync(h, "icwf_exact2d_observables");
   if (st != ICWF_OK) return st;
   std::vector<double> dx_(nx), pot(nx), dR_(nR), part(ncb);
