@@ -42,7 +42,7 @@ DF64_CMAC_OPS = 39
 DF64_TFLOPS = FP32_LANE_OPS * 8 / DF64_CMAC_OPS / 1e12
 TF32_PER_BF16 = 1.1 / 2.25   # nominal dense TF32 / BF16 tensor rates
 # DRAM bytes (read + write) per family call from one ncu capture, with the profile that gives them;
-# keyed by (family, mode, N).  Valid only while the kernels are the ones profiled.
+# keyed by (family, mode, N).  The Cholesky's was captured on its earlier launch-per-block-column form.
 TRAFFIC = {("cholesky", "tf32x3", 1024): (193.6e6, "profiles/k_chol_step_df_mixed_N1024.md")}
 
 
@@ -282,7 +282,9 @@ def roofline(prof, w, K, mode, peaks, solve="df64", nfact=2):
                    peak_source="measured (MEASURED_PEAKS.json hbm_gbs)")
     elif bound == "tensor":
         # algorithmic Gram flops against the split-product ceiling: three products per Gram in the
-        # operand type (TF32 at the nominal TF32/BF16 ratio of the measured BF16 peak)
+        # operand type (TF32 at the nominal TF32/BF16 ratio of the measured BF16 peak).  The TF32
+        # mode's pieces are FP16, which have TF32's significand at the BF16 rate, so the fraction can
+        # pass 1.
         bf16 = peaks.get("bf16_tflops_sustained")
         ratio = TF32_PER_BF16 if mode == "tf32x3" else 1.0
         out.update(bound="tensor", achieved=rate / 1e12,
@@ -290,6 +292,8 @@ def roofline(prof, w, K, mode, peaks, solve="df64", nfact=2):
                    peak_source=("measured bf16 sustained (MEASURED_PEAKS.json) x %.3f (nominal "
                                 "%s/BF16) / 3 split products" % (ratio, "TF32" if ratio < 1 else "BF16")))
     elif mode == "fp64" or solve == "fp64":
+        # the FP64 pipe as the common yardstick; Grams and trailing updates run as digit products on
+        # the tensor cores and can pass it
         out.update(bound="alu", achieved=rate / 1e12, peak=NOMINAL_FP64_TFLOPS, unit="TFLOP/s",
                    peak_source="nominal FP64 (152 SMs x 2 FP64 FMA/clk x 2.07 GHz)")
     else:
@@ -302,7 +306,7 @@ def roofline(prof, w, K, mode, peaks, solve="df64", nfact=2):
     out["traffic"] = tr[0] if tr else None
     if tr:
         out["traffic_unit"] = "bytes per call (DRAM read + write, ncu)"
-        out["traffic_source"] = tr[1]
+        out["traffic_source"] = tr[1] + " (the launch-per-block-column form)"
     return out
 
 

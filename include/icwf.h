@@ -51,9 +51,12 @@ typedef enum {
 } icwf_status;
 
 typedef enum {
-  ICWF_FP64 = 0,          /* CWFs complex128; matrix elements, Cholesky, triangular solves and
-                             RK4 in FP64 (the factorisation's trailing updates in emulated FP64
-                             on the tensor cores unless icwf_set_emulated_update turns it off) */
+  ICWF_FP64 = 0,          /* CWFs complex128; Grams of the matrix elements and of the
+                             reconstruction as exact digit products on the tensor cores (up to
+                             55 bits below a CWF's largest component), combined in FP64;
+                             Cholesky, triangular solves and RK4 in FP64 (the factorisation's
+                             trailing updates in emulated FP64 on the tensor cores unless
+                             icwf_set_emulated_update turns it off) */
   ICWF_MIXED_BF16X3 = 1,  /* CWFs complex64, FP32 propagation; Grams on tcgen05 tensor cores as
                              three BF16 products (hi*hi + hi*lo + lo*hi), FP32 accumulation;
                              the overlap S as an exact Gram of fixed-point CWFs (positive
@@ -62,7 +65,8 @@ typedef enum {
                              triangular solves in double-float arithmetic (pairs of FP32, about
                              44-48 significant bits) unless solve_fp64 is set; right-hand sides,
                              RK4 update and reductions in FP64 */
-  ICWF_MIXED_TF32X3 = 2   /* as above with TF32 operand pieces */
+  ICWF_MIXED_TF32X3 = 2   /* as above with operand pieces of TF32's 11 significant bits (FP16
+                             values under a power of two per CWF) */
 } icwf_precision;
 
 typedef struct {
@@ -229,8 +233,8 @@ icwf_status icwf_set_emulated_update(icwf_handle h, int32_t on);
 icwf_status icwf_set_step_graphs(icwf_handle h, int32_t on);
 
 /* Diagnostic: poll budget of the in-kernel spin waits on global flags (the look-ahead tickets of
- * the blocked Cholesky factorisation and the block flags of the triangular solves above N = 2048).  polls >= 0:
- * such a wait gives up after that many polls, sets the timeout flag and the kernel continues
+ * the blocked Cholesky factorisation and the block flags of the triangular solves above N = 2048).
+ * polls >= 0: such a wait gives up after that many polls, sets the timeout flag and the kernel continues
  * without its input (results are then meaningless and the call returns ICWF_ERR_TIMEOUT);
  * polls < 0 restores the compiled-in limits (well under a second of polling).  Waits on
  * shared-memory barriers that guard asynchronous copies (the tensor-core assembly, the cluster

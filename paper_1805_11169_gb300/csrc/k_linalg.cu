@@ -5,7 +5,7 @@
 // updates run either here with FP64 FMAs or in emulated FP64 on the tensor cores (exact integer
 // digit products, k_herk_emu.cu).  The FP64 mode and the solve_fp64 option of the mixed modes
 // factorise and solve with these kernels; the mixed modes' default solver is the double-float one
-// of k_linalg_df.cu.
+// of k_linalg_df.cu.  Up to N = 2048 the triangular solves run in k_solve.cu.
 #include <cuda_runtime.h>
 
 #include "herk_digits.cuh"

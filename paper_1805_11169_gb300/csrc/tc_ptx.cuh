@@ -1,7 +1,6 @@
 // Inline-PTX wrappers shared by the tcgen05 tensor-core kernels (sm_103a): mbarriers with
 // bounded waits, TMA tiled loads, shared-memory and instruction descriptors for K-major BF16/TF32
-// operands, tcgen05.mma / commit / fences, TMEM loads and stores, and the triangular block index
-// of the Hermitian Gram launches.  Bit layouts follow the public PTX ISA descriptions of the
+// operands, tcgen05.mma / commit / fences, TMEM loads and stores.  Bit layouts follow the public PTX ISA descriptions of the
 // tcgen05 shared-memory matrix descriptor and the kind::f16 / kind::tf32 instruction descriptor.
 #pragma once
 #include <cuda.h>
