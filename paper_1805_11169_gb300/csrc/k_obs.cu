@@ -99,7 +99,8 @@ __global__ void __launch_bounds__(256) k_obs_lines(JobView j, ObsArgs o) {
 
 // One CTA: out = {norm, ekx, ekR, epot}; pop[n]; decoh[n*ns + m].  A warp per sum (4 + ns + ns (ns + 1)
 // / 2 of them), lanes striding over the line sums, so the sums run side by side without barriers
-// (256 threads with a block reduction per sum, D_nm computed twice: 31 us; now 6 us at nR = 512).
+// (256 threads with a block reduction per sum, D_nm computed twice: 31 us at nR = 512 with cold
+// caches; now 19).
 constexpr int OF_WARPS = 32;
 __global__ void __launch_bounds__(OF_WARPS * 32) k_obs_final(JobView j, ObsArgs o, double* out, double* pop,
                                                              double* decoh) {
