@@ -65,8 +65,7 @@ typedef enum {
                              triangular solves in double-float arithmetic (pairs of FP32, about
                              44-48 significant bits) unless solve_fp64 is set; right-hand sides,
                              RK4 update and reductions in FP64 */
-  ICWF_MIXED_TF32X3 = 2   /* as above with operand pieces of TF32's 11 significant bits (FP16
-                             values under a power of two per CWF) */
+  ICWF_MIXED_TF32X3 = 2   /* as above with TF32 operand pieces */
 } icwf_precision;
 
 typedef struct {

@@ -112,8 +112,16 @@ bool add_group_nodes(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndep
                      const GroupJob* table, int njobs, int total_traj, int total_cwf, int nmax,
                      int threads, int max_ctas, cudaGraphNode_t* last);
 
+// a5 (mixed modes): Heff, and S too if not NULL, from split products on the tensor cores
+// (k_assemble_tc.cu).  heff_tc_ready: the tensor maps can be encoded.  Returns the number of kernels.
+bool heff_tc_ready();
+cudaError_t heff_tc_attributes();
+size_t heff_tc_scratch_bytes(int N, int nx, int nR, int K);
+int launch_heff_tc(const JobView& j, int precision, double2* S, double2* H, void* scratch, cudaStream_t s);
+
 // a5: S = S1 o S2 and Heff from the rank-K factors at the current positions, every mode, on the
-// tensor cores (k_sliced.cu).  A handle's plan lays out its operand slices, Grams and tables in one
+// tensor cores: sliced Grams (k_sliced.cu) for S and, in the FP64 mode, Heff; launch_heff_tc for the
+// mixed modes' Heff.  A handle's plan lays out its operand slices, Grams and tables in one
 // scratch region of its arena; the tables are uploaded once, so launch() can be captured.
 struct AsmShape {
   int N, nx, nR, K, precision, overlap_split;

@@ -1,17 +1,13 @@
-// Matrix elements (Eq. M, W, W1, W2) of every mode as Grams of sliced operands on the sm_103a tensor
-// cores, and their combination into S and Heff.
+// Matrix elements (Eq. M, W, W1, W2) as Grams of sliced operands on the sm_103a tensor cores, and their
+// combination into S and Heff: both in the FP64 mode, S in the mixed modes (their Heff is made of
+// floating-point products, k_assemble_tc.cu).
 //
 // Slicing.  A CWF column (weighted by u_g(x) for the rank-k terms) is scaled by a power of two 2^-e so
-// that its components lie in (-1, 1) and is cut into D pieces of a 16-bit type that sum to it:
-//   digits  balanced integers d_p, value = 2^e sum_p d_p 2^-(b0 + beta p), stored exactly as BF16;
-//           products of digits are integers, so the sums over the grid are exact in FP32 as long as
-//           they stay below 2^24.  b0 = 6, beta = 7 in the FP64 mode (D = 8: 55 bits below the
-//           largest component), b0 = beta = 6 with D = 4 for the mixed modes' overlap (24 bits: S
-//           is then the exact Gram of fixed-point CWFs and positive semidefinite; b0 = beta = 5 on
-//           4096-point grids);
-//   pieces  hi + lo floating-point pieces for the mixed modes' Heff: FP16 (11 significant bits each,
-//           the significand of TF32, at twice its rate and half its bytes; the power of two keeps
-//           every piece inside FP16's range) or BF16 (8 bits each).
+// that its components lie in (-1, 1) and is cut into D balanced integers d_p, value = 2^e sum_p d_p
+// 2^-(b0 + beta p), stored exactly as BF16; products of digits are integers, so the sums over the grid
+// are exact in FP32 as long as they stay below 2^24.  b0 = 6, beta = 7 in the FP64 mode (D = 8: 55 bits
+// below the largest component), b0 = beta = 6 with D = 4 for the mixed modes' overlap (24 bits: S is
+// then the exact Gram of fixed-point CWFs and positive semidefinite; b0 = beta = 5 on 4096-point grids).
 //
 // Products.  conj(a) b = sum over piece pairs (p, q); the pairs with p + q < L are kept and every level
 // l = p + q has its own FP32 accumulator in TMEM.  With the T kets' pieces stored one after the
@@ -39,14 +35,12 @@
 // TMEM (warp w: lanes 32 (w mod 4).., column half w div 4).  Ring geometry follows the unit's D.
 // Every wait is bounded (2 s): a timeout raises the status flag, drains what is in flight, returns.
 //
-// Bound: shared-memory bandwidth of the operands (reads by the MMAs plus the copies' writes take about
-// 900 cycles per D = 2 slice against 768 of tensor time); the tensor pipe is busy 73% of the time.
+// Bound: an MMA of M = 128 takes max(N / 2, operand bytes / 128) cycles (measured over N = 32..256), so
+// the wide operands of all pieces at once keep it on the tensor pipe's side; the copies' writes into
+// shared memory come on top.
 // Measured (GB300, N = 1024 on 1024 x 512; ms per assembly, before -> now): FP64 mode, 22 terms, 144
-// (FP64 FMAs) -> 3.5; TF32-significand pieces, 16 terms, 1.16 (TF32 MMAs of N = 64 on 128 x 32 tiles,
-// bound by L2 -> shared memory) -> 0.50; BF16 pieces at N = 512 on 512 x 256 0.38 -> 0.13; FP64,
-// N = 16, 64 terms on 128 x 64, 13.1 (one CTA) -> 0.26; reconstruction in the FP64 mode 4.3 -> 0.22.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
+// (FP64 FMAs) -> 3.5; FP64, N = 16, 64 terms on 128 x 64, 13.1 (one CTA) -> 0.26; reconstruction in the
+// FP64 mode 4.3 -> 0.22.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -91,11 +85,9 @@ struct Gram {
   const unsigned char* B;   // kets: T-row tiles with d pieces per plane, or NULL: rows of A
   const int* ea;            // scale exponents of the bras and kets
   const int* eb;
-  void* out;                // [tile of 128 x 128][ket][bra], double2 (digits) or float2 (pieces)
-  float scale;              // pieces: grid spacing
+  double2* out;             // [tile of 128 x 128][ket][bra]
   int ks, da, d, l, t;      // K slices; pieces stored / used; levels; kets per unit
   int drain;                // K slices per accumulation
-  int f16, digits;          // piece type; digits or floating-point pieces
   int b0, beta, fbits;      // digit weights; fraction bits of the integer accumulators
   int unit0;                // first unit
   int cols;                 // 0: upper-triangle tiles; else a rectangular product of rows x cols
@@ -104,7 +96,7 @@ struct Gram {
 
 struct GramArgs {
   const Gram* grams;
-  void* out;                // overrides the Grams' outputs if not NULL
+  double2* out;             // overrides the Grams' outputs if not NULL
   int ngrams, units, N;
   float4* herk[2];          // if set: Gram i's conj(bra) ket is subtracted from the double-floats
   int R0;                   //    herk[i][(R0 + ket) N + R0 + bra], bra <= ket, R0 + ket < N
@@ -467,7 +459,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_gram_sliced(GramArgs args) {
         const int d = g.d, t = g.t, L = g.l, ks = g.ks, dr = g.drain;
         const int bytes = stage_bytes(d, t), slots = ring_slots(d, t);
         if (bytes != geo) { geo = bytes; slot = 0; }
-        const uint32_t id0 = idesc_f16(g.f16, MT, 0);
+        const uint32_t id0 = idesc_mn(0, MT, 0);
         for (int s0 = 0; s0 < ks && ok; s0 += dr) {
           if (!(ok = mbar_wait(acc_empty, (chunk & 1u) ^ 1u, abort_flag, status))) break;
           fence_after();
@@ -540,8 +532,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_gram_sliced(GramArgs args) {
           }
           herk_store8(A, args.N, r + 8 * h, c, xb0, 8 * h, ea, -2 * HERK_B0, a, re, im);
         }
-      } else if (g.digits) {
-        double2* out = (double2*)(args.out ? args.out : g.out) + o;
+      } else {
+        double2* out = (args.out ? args.out : g.out) + o;
         const int shift = -2 * g.b0 - g.fbits;
         if (t == 32) {
           long long re[2][8], im[2][8];
@@ -578,31 +570,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_gram_sliced(GramArgs args) {
           fence_before();
           mbar_arrive(acc_empty);
         }
-      } else {
-        ok = __all_sync(0xffffffffu, mbar_wait(acc_full, chunk & 1u, abort_flag, status));
-        if (!ok) break;
-        ++chunk;
-        fence_after();
-        float2* out = (float2*)g.out + o;
-        const float scale = g.scale;
-#pragma unroll 1
-        for (int c8 = 0; c8 < t / 2; c8 += 8) {
-          float r0[8], r1[8], i0[8], i1[8];
-          tmem_ld8(col + c8, r0);
-          tmem_ld8(col + t + c8, r1);
-          tmem_ld8(col + COL_IM + c8, i0);
-          tmem_ld8(col + COL_IM + t + c8, i1);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            // the pieces carry 2^PIECE_BITS each
-            const int x = __shfl_sync(0xffffffffu, c8 < 32 ? xb0 : xb1, (c8 + e) & 31);
-            const float f = scaled(scale, ea + x - 2 * PIECE_BITS);
-            out[(size_t)(c8 + e) * MT] = make_float2((r0[e] + r1[e]) * f, (i0[e] + i1[e]) * f);
-          }
-        }
-        fence_before();
-        mbar_arrive(acc_empty);
       }
     }
   }
@@ -624,19 +591,17 @@ __global__ void __launch_bounds__(THREADS, 1) k_gram_sliced(GramArgs args) {
 
 // ---------------------------------------------------------------------------- operands
 
-enum : int { SRC_F64_DIGITS = 0, SRC_F32_DIGITS = 1, SRC_F32_F16 = 2, SRC_F32_BF16 = 3 };
-
 // Operands of up to SLICE_GROUP terms in the same format: rows = CWF columns of one side, weighted by
-// w[i] of each term if given (FP64 weights for complex128 CWFs, FP32 for complex64).
+// w[i] of each term if given (complex128 CWFs only).
 constexpr int SLICE_GROUP = 4;
 struct Slice {
   const void* src;          // complex128 or complex64, row r at src + r n
-  const void* w;            // ng weights of n points each
+  const double* w;          // ng weights of n points each
   unsigned char* out;       // term q at out + q ostride, its exponents at ex + q estride
   int* ex;                  // rpad exponents
   size_t ostride, estride;
   int ng, n, ks, rows, rpad, R;   // terms, points, K slices, rows (and padded to tiles of R rows)
-  int d, kind, b0, beta;
+  int d, b0, beta;
 };
 
 // 8 consecutive points of one row: `part` 0 or 1 of their K slice
@@ -688,30 +653,6 @@ __device__ __forceinline__ void emit_f32_digits(const Slice& s, int row, int c8,
   }
 }
 
-template <bool F16>
-__device__ __forceinline__ void emit_pieces(const Slice& s, int row, int c8, int plane, const float (&x)[8],
-                                            float f1, float f2) {
-  uint32_t hi[4], lo[4];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float v = x[k] * f1 * f2;
-    uint32_t h, l;
-    if (F16) {
-      const __half a = __float2half_rn(v);
-      h = __half_as_ushort(a);
-      l = __half_as_ushort(__float2half_rn(v - __half2float(a)));
-    } else {
-      const __nv_bfloat16 a = __float2bfloat16_rn(v);
-      h = __bfloat16_as_ushort(a);
-      l = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(a)));
-    }
-    if (k & 1) { hi[k >> 1] |= h << 16; lo[k >> 1] |= l << 16; }
-    else { hi[k >> 1] = h; lo[k >> 1] = l; }
-  }
-  *(uint4*)slice_at(s, row, c8, plane, 0) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-  *(uint4*)slice_at(s, row, c8, plane, 1) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-}
-
 // Components of 8 points of a row (zero past the row's end and in padding rows); 16-byte loads (rows
 // are 8 or more points, so every chunk starts on a 16-byte boundary).
 __device__ __forceinline__ void load8(const Slice& s, int row, int c8, float (&re)[8], float (&im)[8]) {
@@ -732,19 +673,10 @@ __device__ __forceinline__ void load8(const Slice& s, int row, int c8, double (&
     re[k] = z.x; im[k] = z.y;
   }
 }
-__device__ __forceinline__ void weight8(const Slice& s, int q, int c8, float (&re)[8], float (&im)[8]) {
-  if (!s.w || 8 * c8 >= s.n) return;
-  const float4* w = (const float4*)((const float*)s.w + (size_t)q * s.n + 8 * c8);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const float4 f = w[k];
-    re[4 * k] *= f.x; re[4 * k + 1] *= f.y; re[4 * k + 2] *= f.z; re[4 * k + 3] *= f.w;
-    im[4 * k] *= f.x; im[4 * k + 1] *= f.y; im[4 * k + 2] *= f.z; im[4 * k + 3] *= f.w;
-  }
-}
+__device__ __forceinline__ void weight8(const Slice&, int, int, float (&)[8], float (&)[8]) {}
 __device__ __forceinline__ void weight8(const Slice& s, int q, int c8, double (&re)[8], double (&im)[8]) {
   if (!s.w || 8 * c8 >= s.n) return;
-  const double2* w = (const double2*)((const double*)s.w + (size_t)q * s.n + 8 * c8);
+  const double2* w = (const double2*)(s.w + (size_t)q * s.n + 8 * c8);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const double2 f = w[k];
@@ -785,7 +717,7 @@ __device__ __forceinline__ unsigned long long row_max(unsigned long long m, int 
   return m;
 }
 
-// pieces or digits of 8 points of row `row`, term q
+// digits of 8 points of row `row`
 __device__ __forceinline__ void emit8(const Slice& s, int row, int c, int e, const double (&re)[8],
                                       const double (&im)[8]) {
   switch (s.d) {
@@ -801,25 +733,16 @@ __device__ __forceinline__ void emit8(const Slice& s, int row, int c, int e, con
 __device__ __forceinline__ void emit8(const Slice& s, int row, int c, int e, const float (&re)[8],
                                       const float (&im)[8]) {
   // 2^k in two factors, each a normal number
-  const int k2 = (s.kind == SRC_F32_DIGITS ? s.b0 : PIECE_BITS) - e;
+  const int k2 = s.b0 - e;
   const float f1 = scaled(1.f, k2 / 2), f2 = scaled(1.f, k2 - k2 / 2);
-  if (s.kind == SRC_F32_DIGITS) {
-    emit_f32_digits(s, row, c, 0, re, f1, f2);
-    emit_f32_digits(s, row, c, 1, im, f1, f2);
-  } else if (s.kind == SRC_F32_F16) {
-    emit_pieces<true>(s, row, c, 0, re, f1, f2);
-    emit_pieces<true>(s, row, c, 1, im, f1, f2);
-  } else {
-    emit_pieces<false>(s, row, c, 0, re, f1, f2);
-    emit_pieces<false>(s, row, c, 1, im, f1, f2);
-  }
+  emit_f32_digits(s, row, c, 0, re, f1, f2);
+  emit_f32_digits(s, row, c, 1, im, f1, f2);
 }
 
 // Operands in slices, grid (row groups, operand groups): a row's 8-point chunks are spread over
 // min(2 ks, 256) threads, and a thread keeps its chunk (all of its work up to 2048 points) for every
 // term of the group: what bounds this kernel is the load/store unit's passes over scattered 32-byte
-// rows.  (N = 1024, 16 terms on 1024 x 512: 153 us with one term per thread and FP64 weights converted
-// here, 76 us with four terms and FP32 weights; 226 MB written, 33 us at the copy rate.)
+// rows.
 template <typename T>
 __device__ __forceinline__ void slice_rows(Slice s, unsigned long long (&red)[2][8]) {
   constexpr bool F64 = sizeof(T) == 8;
@@ -848,15 +771,14 @@ __device__ __forceinline__ void slice_rows(Slice s, unsigned long long (&red)[2]
       if constexpr (F64) e = exponent_above_f64(m);
       else e = m ? ilogbf(__uint_as_float((unsigned)m)) + 1 : 0;
     }
-    const bool digits = F64 || s.kind == SRC_F32_DIGITS;
     if (row < s.rpad) {
-      if (t0 == 0) s.ex[row] = bad && digits ? EX_BAD : e;
+      if (t0 == 0) s.ex[row] = bad ? EX_BAD : e;
       for (int c = t0; c < c8n; c += tpr) {
         if (c != t0) {
           load8(s, row, c, re, im);
           weight8(s, q, c, re, im);
         }
-        if (bad && digits) {
+        if (bad) {
 #pragma unroll
           for (int k = 0; k < 8; ++k) re[k] = im[k] = 0;
         }
@@ -951,37 +873,50 @@ __global__ void __launch_bounds__(ST_WARPS * 32) k_slices_t(SliceT sx, SliceT sR
 
 // Heff_ab = sum_g s_g (A_g - u_g(x_b) S1)(B_g - w_g(R_b) S2) - V(x_b, R_b) S_ab over the terms
 // [g0, g1) of this launch; `first` starts the sums at zero (else they continue from H), `last`
-// subtracts the pinned potential and writes S.
+// subtracts the pinned potential and writes S.  The raw Grams of the terms carry s_g dx and dR already
+// (folded into the operands' weights), those of the overlap don't.
 struct HeffArgs {
   int N, g0, g1, first, last;
-  const void *S1, *S2;      // raw Grams of the overlap: double2 (digits) or, with split_s, float2 scaled
-  const void *A, *B;        // Grams of the terms g0.., `tiles` 128 x 128 tiles each
+  const double2 *S1, *S2;   // raw Grams of the overlap
+  const double2 *A, *B;     // Grams of the terms g0.., `tiles` 128 x 128 tiles each
   size_t tiles;
-  int split_s;
   double dx, dR;
   const double *sig, *px, *pR, *d;
   double2 *S, *H;
   int split;                // term groups (blockIdx.z); > 1: partial sums meet in `part`
-  void* part;               // [group][tile][direct, mirrored][128 x 128] of Z
+  double2* part;            // [group][tile][direct, mirrored][128 x 128]
   unsigned* done;           // [tile][patch]: groups finished (zero between launches)
 };
 
-// Threads of one 32 x 32 patch of a 128 x 128 upper-triangle tile: lane = bra, 4 kets each.  F32: the
-// mixed modes' FP32 arithmetic on float2 Grams; else FP64 on double2 Grams that carry s_g dx and dR
-// already (folded into the operands' weights): 8 FP64 instructions per term, element and side, which
-// is what bounds the FP64 version (0.39 ms at N = 1024 and 22 terms); the F32 version reads its Grams
-// once (60 us at N = 1024, 16 terms; 136 us with the factors' conversions in the loop).  With fewer
-// patches than SMs the terms are split over CTAs as well (16 trajectories, 64 terms, FP64: 202 us
-// without, 50 us with).
+// Threads of one 32 x 32 patch of a 128 x 128 upper-triangle tile: lane = bra, 4 kets each.  Bound: 8
+// FP64 instructions per term, element and side (0.39 ms at N = 1024 and 22 terms).  With fewer patches
+// than SMs the terms are split over CTAs as well (16 trajectories, 64 terms: 202 us without, 50 us
+// with).
 constexpr int HG = 16;   // terms staged at a time
-template <bool F32>
+
+// A 32 x 32 patch of S, bras from a0 and kets from b0, lane = bra, sv[e]: ket b0 + ty + 8 e.  Each pair is
+// stored once, from its a <= b side, so that S is exactly Hermitian.
+__device__ __forceinline__ void store_s(double2* S, int N, bool mirror, int a0, int b0, const double2 (&sv)[4],
+                                        double2 (&tr)[32][33]) {
+  const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5, a = a0 + lane;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int b = b0 + ty + 8 * e;
+    tr[lane][ty + 8 * e] = sv[e];
+    if (a < N && b < N && (mirror || a < b)) S[(size_t)b * N + a] = cconj(sv[e]);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {   // rows of S: lane = ket
+    const int ao = a0 + ty + 8 * e, bo = b0 + lane;
+    if (ao < N && bo < N && (mirror || ao <= bo)) S[(size_t)ao * N + bo] = tr[ty + 8 * e][lane];
+  }
+}
+
 __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
-  using Z = typename std::conditional<F32, float2, double2>::type;
-  using T = typename std::conditional<F32, float, double>::type;
   __shared__ double2 tr[32][33];
-  // the terms' factor values at the 32 bras and 32 kets, converted once per CTA (a conversion from
-  // FP64 costs an FP64 instruction)
-  __shared__ T uxs[HG][64], wRs[HG][64];
+  // the terms' factor values at the 32 bras and 32 kets
+  __shared__ double uxs[HG][64], wRs[HG][64];
   __shared__ int s_last;
   int I, J;
   tri_tile(blockIdx.y, I, J);
@@ -991,30 +926,16 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
   if (I * MT + (int)(blockIdx.x & 3) * 32 >= N || J * MT + (int)(blockIdx.x >> 2) * 32 >= N) return;
   const bool mirror = I != J, a_ok = a < N;
   const size_t at0 = ((size_t)blockIdx.y * MT + br) * MT + ar, step = (size_t)8 * MT;
-  double2 s1d[4], s2d[4];
-  Z s1[4], s2[4], h[4], ht[4];
+  double2 s1[4], s2[4], h[4], ht[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    const size_t at = at0 + e * step;
-    if (F32 && p.split_s) {
-      const float2 x = ((const float2*)p.S1)[at], y = ((const float2*)p.S2)[at];
-      s1d[e] = make_double2(x.x, x.y);
-      s2d[e] = make_double2(y.x, y.y);
-    } else {
-      s1d[e] = cscale(((const double2*)p.S1)[at], p.dx);
-      s2d[e] = cscale(((const double2*)p.S2)[at], p.dR);
-    }
-    s1[e].x = (T)s1d[e].x; s1[e].y = (T)s1d[e].y;
-    s2[e].x = (T)s2d[e].x; s2[e].y = (T)s2d[e].y;
-    h[e].x = h[e].y = ht[e].x = ht[e].y = 0;
+    s1[e] = cscale(p.S1[at0 + e * step], p.dx);
+    s2[e] = cscale(p.S2[at0 + e * step], p.dR);
+    h[e] = ht[e] = make_double2(0.0, 0.0);
     const int b = b0 + 8 * e;
     if (!p.first && blockIdx.z == 0 && a_ok && b < N) {
-      const double2 v = p.H[(size_t)a * N + b];
-      h[e].x = (T)v.x; h[e].y = (T)v.y;
-      if (mirror) {
-        const double2 w = p.H[(size_t)b * N + a];
-        ht[e].x = (T)w.x; ht[e].y = (T)w.y;
-      }
+      h[e] = p.H[(size_t)a * N + b];
+      if (mirror) ht[e] = p.H[(size_t)b * N + a];
     }
   }
   const size_t gs = p.tiles * MT * MT;
@@ -1028,44 +949,32 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
       for (int i = threadIdx.x; i < HG * 64; i += 256) {
         const int gi = g + (i >> 6), c = i & 63, t = c < 32 ? as + c : bs + c - 32;
         if (gi < z1) {
-          const double s = F32 ? 1.0 : p.sig[gi];
-          uxs[i >> 6][c] = t < N ? (T)(s * p.px[(size_t)gi * N + t]) : (T)0;
-          wRs[i >> 6][c] = t < N ? (T)p.pR[(size_t)gi * N + t] : (T)0;
+          uxs[i >> 6][c] = t < N ? p.sig[gi] * p.px[(size_t)gi * N + t] : 0.0;
+          wRs[i >> 6][c] = t < N ? p.pR[(size_t)gi * N + t] : 0.0;
         }
       }
       __syncthreads();
     }
-    const Z* A = (const Z*)p.A + (size_t)(g - p.g0) * gs + at0;
-    const Z* B = (const Z*)p.B + (size_t)(g - p.g0) * gs + at0;
-    const T sg = F32 ? (T)p.sig[g] : (T)0;
-    const T uxa = uxs[gl][lane], wRa = wRs[gl][lane];
-    Z xs[4], ys[4];
+    const double2* A = p.A + (size_t)(g - p.g0) * gs + at0;
+    const double2* B = p.B + (size_t)(g - p.g0) * gs + at0;
+    const double uxa = uxs[gl][lane], wRa = wRs[gl][lane];
+    double2 xs[4], ys[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) { xs[e] = A[e * step]; ys[e] = B[e * step]; }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const Z x = xs[e], y = ys[e];
-      const T uxb = uxs[gl][32 + ty + 8 * e], wRb = wRs[gl][32 + ty + 8 * e];
-      const T atr = x.x - uxb * s1[e].x, ati = x.y - uxb * s1[e].y;
-      const T btr = y.x - wRb * s2[e].x, bti = y.y - wRb * s2[e].y;
-      if (F32) {
-        h[e].x = fma(sg, atr * btr - ati * bti, h[e].x);
-        h[e].y = fma(sg, atr * bti + ati * btr, h[e].y);
-      } else {
-        h[e].x = fma(atr, btr, fma(-ati, bti, h[e].x));
-        h[e].y = fma(atr, bti, fma(ati, btr, h[e].y));
-      }
+      const double2 x = xs[e], y = ys[e];
+      const double uxb = uxs[gl][32 + ty + 8 * e], wRb = wRs[gl][32 + ty + 8 * e];
+      const double atr = x.x - uxb * s1[e].x, ati = x.y - uxb * s1[e].y;
+      const double btr = y.x - wRb * s2[e].x, bti = y.y - wRb * s2[e].y;
+      h[e].x = fma(atr, btr, fma(-ati, bti, h[e].x));
+      h[e].y = fma(atr, bti, fma(ati, btr, h[e].y));
       if (mirror) {
         // entry (b, a): conj(A) - u(x_a) conj(S1), conj(B) - w(R_a) conj(S2)
-        const T mtr = x.x - uxa * s1[e].x, mti = x.y - uxa * s1[e].y;
-        const T ntr = y.x - wRa * s2[e].x, nti = y.y - wRa * s2[e].y;
-        if (F32) {
-          ht[e].x = fma(sg, mtr * ntr - mti * nti, ht[e].x);
-          ht[e].y = fma(sg, -(mtr * nti + mti * ntr), ht[e].y);
-        } else {
-          ht[e].x = fma(mtr, ntr, fma(-mti, nti, ht[e].x));
-          ht[e].y = fma(-mtr, nti, fma(-mti, ntr, ht[e].y));
-        }
+        const double mtr = x.x - uxa * s1[e].x, mti = x.y - uxa * s1[e].y;
+        const double ntr = y.x - wRa * s2[e].x, nti = y.y - wRa * s2[e].y;
+        ht[e].x = fma(mtr, ntr, fma(-mti, nti, ht[e].x));
+        ht[e].y = fma(-mtr, nti, fma(-mti, ntr, ht[e].y));
       }
     }
   }
@@ -1073,7 +982,7 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
     // few tiles: the terms are spread over CTAs; the last one to finish a patch adds the groups' sums
     // in their order (so the result does not depend on timing) and goes on
     const size_t dir = (size_t)MT * MT, grp = p.tiles * 2 * dir;
-    Z* mine = (Z*)p.part + blockIdx.z * grp + (size_t)blockIdx.y * 2 * dir + (size_t)br * MT + ar;
+    double2* mine = p.part + blockIdx.z * grp + (size_t)blockIdx.y * 2 * dir + (size_t)br * MT + ar;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       mine[e * step] = h[e];
@@ -1090,13 +999,13 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) h[e].x = h[e].y = ht[e].x = ht[e].y = 0;
     for (int z = 0; z < p.split; ++z) {
-      const Z* q = (const Z*)p.part + z * grp + (size_t)blockIdx.y * 2 * dir + (size_t)br * MT + ar;
+      const double2* q = p.part + z * grp + (size_t)blockIdx.y * 2 * dir + (size_t)br * MT + ar;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const Z v = __ldcg(q + e * step);
+        const double2 v = __ldcg(q + e * step);
         h[e].x += v.x; h[e].y += v.y;
         if (mirror) {
-          const Z w = __ldcg(q + dir + e * step);
+          const double2 w = __ldcg(q + dir + e * step);
           ht[e].x += w.x; ht[e].y += w.y;
         }
       }
@@ -1108,9 +1017,9 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
   for (int e = 0; e < 4; ++e) {
     const int b = b0 + 8 * e;
     const bool in = a_ok && b < N;
-    double2 hd = make_double2(h[e].x, h[e].y), hm = make_double2(ht[e].x, ht[e].y);
+    double2 hd = h[e], hm = ht[e];
     if (p.last) {
-      sv[e] = cmul(s1d[e], s2d[e]);
+      sv[e] = cmul(s1[e], s2[e]);
       if (a == b) sv[e].y = 0.0;
       const double db = in ? p.d[b] : 0.0;
       hd = make_double2(hd.x - db * sv[e].x, hd.y - db * sv[e].y);
@@ -1127,18 +1036,27 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
     if (ao + 8 * e < N && bo < N) p.H[(size_t)(ao + 8 * e) * N + bo] = tr[ty + 8 * e][lane];
   if (!p.last) return;
   __syncthreads();
-  // S: each pair once, from its a <= b side, so that S is exactly Hermitian
+  store_s(p.S, N, mirror, I * MT + (int)(blockIdx.x & 3) * 32, J * MT + (int)(blockIdx.x >> 2) * 32, sv, tr);
+}
+
+// S = S1 o S2 alone (the mixed modes), patches as above.
+__global__ void __launch_bounds__(256) k_overlap(int N, const double2* __restrict__ S1, const double2* __restrict__ S2,
+                                                 double dx, double dR, double2* __restrict__ S) {
+  __shared__ double2 tr[32][33];
+  int I, J;
+  tri_tile(blockIdx.y, I, J);
+  const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int ac = (int)(blockIdx.x & 3) * 32, bc = (int)(blockIdx.x >> 2) * 32;
+  if (I * MT + ac >= N || J * MT + bc >= N) return;
+  const size_t at0 = ((size_t)blockIdx.y * MT + bc + ty) * MT + ac + lane;
+  double2 sv[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    const int b = b0 + 8 * e;
-    tr[lane][ty + 8 * e] = sv[e];
-    if (a_ok && b < N && (mirror || a < b)) p.S[(size_t)b * N + a] = cconj(sv[e]);
+    const size_t at = at0 + (size_t)8 * e * MT;
+    sv[e] = cmul(cscale(S1[at], dx), cscale(S2[at], dR));
+    if (I * MT + ac + lane == J * MT + bc + ty + 8 * e) sv[e].y = 0.0;
   }
-  __syncthreads();
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    if (ao + 8 * e < N && bo < N && (mirror || ao + 8 * e <= bo))
-      p.S[(size_t)(ao + 8 * e) * N + bo] = tr[ty + 8 * e][lane];
+  store_s(S, N, I != J, I * MT + ac, J * MT + bc, sv, tr);
 }
 
 // ---------------------------------------------------------------------------- plan
@@ -1286,7 +1204,6 @@ int launch_herk_df(int N, int k0, int R0, void* const* A, int nb, void* scratch,
     g.ks = g.drain = HERK_KS;
     g.da = g.d = g.l = HERK_D;
     g.t = 32;
-    g.digits = 1;
     g.b0 = HERK_B0;
     g.beta = HERK_BETA;
     g.fbits = 62 - (1 + 7 + 2 * HERK_B0);   // sums of 128 x 2 products below 2^(2 b0)
@@ -1312,8 +1229,7 @@ struct AsmPlan::Impl {
   std::vector<sl::Slice> slices;
   std::vector<sl::Gram> grams;
   std::vector<Batch> batches;
-  std::vector<double> Uw, Ww;            // FP64: weights u_g s_g dx and w_g dR
-  std::vector<float> Uf, Wf;             // mixed modes: u_g and w_g
+  std::vector<double> Uw, Ww;            // FP64 mode: weights u_g s_g dx and w_g dR
   size_t part = 0, o_done = 0;           // split term sums of k_heff
   int split = 1;
   size_t bytes = 0, o_slices = 0, o_grams = 0, o_uw = 0, o_ww = 0, o_ticket = 0;
@@ -1321,7 +1237,9 @@ struct AsmPlan::Impl {
   size_t r_xa = 0, r_xe = 0, r_Rb = 0, r_Re = 0;   // reconstruction operands (in the batch scratch)
   int rec_gram = 0, rec_units = 0, rec_d = 0;
   unsigned char* base = nullptr;
+  int precision = 0;
   bool f64 = false, split_s = false;
+  size_t heff = 0;                       // mixed modes: scratch of launch_heff_tc
   int sms = 152;
 };
 
@@ -1334,6 +1252,7 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
   impl = new Impl;
   Impl& m = *impl;
   const bool f64 = q.precision == ICWF_FP64, split_s = !f64 && q.overlap_split;
+  m.precision = q.precision;
   m.f64 = f64;
   m.split_s = split_s;
   m.base = (unsigned char*)base;
@@ -1342,33 +1261,35 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
   const int n[2] = {q.nx, q.nR}, ks[2] = {(q.nx + 15) / 16, (q.nR + 15) / 16};
   size_t off = 0;
   auto take = [&](size_t b) { const size_t o = off; off += al(b); return o; };
-  const size_t osz = f64 ? 16 : 8;
-  const size_t out_b = (size_t)tiles * MT * MT * osz;
-  const size_t s_out_b = (size_t)tiles * MT * MT * (split_s ? 8 : 16);
+  const size_t out_b = (size_t)tiles * MT * MT * sizeof(double2);
   m.o_ticket = take(256);
-  m.S1 = take(s_out_b);
-  m.S2 = take(s_out_b);
-  // bra operands: digits for S (and, in FP64, every Gram); hi/lo pieces for the mixed modes' Heff
+  m.S1 = take(out_b);
+  m.S2 = take(out_b);
+  // digits of the CWFs: the operands of S and the bras of every term
   const int dS = f64 ? 8 : 4;
-  size_t sa[2] = {0, 0}, se[2] = {0, 0}, pa[2] = {0, 0}, pe[2] = {0, 0};
+  size_t sa[2] = {0, 0}, se[2] = {0, 0};
   auto op_bytes = [&](int side, int d) { return (size_t)rp * ks[side] * 2 * d * ROW_BYTES; };
-  for (int s = 0; s < 2; ++s) {
-    if (!split_s) { sa[s] = take(op_bytes(s, dS)); se[s] = take((size_t)rp * 4); }
-    if (!f64) { pa[s] = take(op_bytes(s, 2)); pe[s] = take((size_t)rp * 4); }
+  for (int s = 0; s < 2 && !split_s; ++s) {
+    sa[s] = take(op_bytes(s, dS));
+    se[s] = take((size_t)rp * 4);
   }
-  m.o_uw = take((size_t)K * q.nx * (f64 ? 8 : 4));
-  m.o_ww = take((size_t)K * q.nR * (f64 ? 8 : 4));
-  // few tiles leave SMs idle in k_heff: spread the terms over up to 16 groups of 4 or more
-  const int patches = tiles_of(N) == 1 ? ((N + 31) / 32) * ((N + 31) / 32) : tiles * 16;
-  m.split = std::max(1, std::min({16, 304 / patches, K / 4}));
-  m.o_done = take((size_t)tiles * 16 * 4);
-  if (m.split > 1) m.part = take((size_t)m.split * tiles * 2 * MT * MT * osz);
-  std::vector<int> dg(K);
-  for (int g = 0; g < K; ++g) dg[g] = f64 ? term_digits(q.sig[0] > 0 ? q.sig[g] / q.sig[0] : 0.0) : 2;
-  // batches of terms
-  std::vector<std::pair<int, int>> ranges;
+  std::vector<int> dg(K, 0);
+  std::vector<std::pair<int, int>> ranges;   // batches of terms (FP64 mode)
   size_t batch_max = 0;
-  for (int g = 0; g < K;) {
+  if (f64) {
+    m.o_uw = take((size_t)K * q.nx * 8);
+    m.o_ww = take((size_t)K * q.nR * 8);
+    // few tiles leave SMs idle in k_heff: spread the terms over up to 16 groups of 4 or more
+    const int patches = tiles_of(N) == 1 ? ((N + 31) / 32) * ((N + 31) / 32) : tiles * 16;
+    m.split = std::max(1, std::min({16, 304 / patches, K / 4}));
+    m.o_done = take((size_t)tiles * 16 * 4);
+    if (m.split > 1) m.part = take((size_t)m.split * tiles * 2 * MT * MT * sizeof(double2));
+    for (int g = 0; g < K; ++g) dg[g] = term_digits(q.sig[0] > 0 ? q.sig[g] / q.sig[0] : 0.0);
+  } else {
+    if (!split_s) ranges.push_back({0, 0});   // the overlap alone
+    batch_max = heff_tc_scratch_bytes(N, q.nx, q.nR, K);
+  }
+  for (int g = 0; f64 && g < K;) {
     size_t b = 0;
     int e = g;
     while (e < K && 2 * (e - g) + 4 < MAX_GRAMS) {
@@ -1391,8 +1312,8 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
   m.r_Rb = m.r_xa + al(rec_op(rxp));
   m.r_xe = m.r_Rb + al(rec_op(rRp));
   m.r_Re = m.r_xe + al((size_t)rxp * 4);
+  m.heff = scratch;
   auto ptr = [&](size_t o) { return m.base + o; };
-  const int fdig = f64 ? 7 : 0;
   for (size_t r = 0; r < ranges.size(); ++r) {
     const int g0 = ranges[r].first, g1 = ranges[r].second;
     Impl::Batch b{};
@@ -1400,7 +1321,7 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     b.gram0 = (int)m.grams.size();
     b.g0 = g0;
     b.g1 = g1;
-    auto add_slice = [&](int side, const void* w, size_t out, size_t ex, int R, int d, int kind, int b0, int beta) {
+    auto add_slice = [&](int side, const double* w, size_t out, size_t ex, int R, int d, int b0, int beta) {
       Slice s{};
       s.src = j ? (side ? j->chi : j->psi) : nullptr;
       s.w = w;
@@ -1408,41 +1329,30 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
       s.out = ptr(out);
       s.ex = (int*)ptr(ex);
       s.n = n[side]; s.ks = ks[side]; s.rows = N; s.rpad = rp; s.R = R;
-      s.d = d; s.kind = kind; s.b0 = b0; s.beta = beta;
+      s.d = d; s.b0 = b0; s.beta = beta;
       m.slices.push_back(s);
     };
     auto add_gram = [&](int side, size_t A, size_t eA, int da, const unsigned char* B, const int* eB, int d, int l,
-                        int t, int drain, bool f16, bool digits, int b0, int beta, size_t out) {
+                        int t, int drain, int b0, int beta, size_t out) {
       Gram x{};
       x.A = ptr(A);
       x.B = B;
       x.ea = (int*)ptr(eA);
       x.eb = eB ? eB : (int*)ptr(eA);
-      x.out = ptr(out);
-      x.scale = (float)(side ? q.dR : q.dx);
+      x.out = (double2*)ptr(out);
       x.ks = ks[side]; x.da = da; x.d = d; x.l = l; x.t = t; x.drain = drain;
-      x.f16 = f16; x.digits = digits; x.b0 = b0; x.beta = beta;
+      x.b0 = b0; x.beta = beta;
       // |sum| <= 2 K 2^(2 b0) units of level 0
       x.fbits = 62 - (1 + ilog2_ceil(16 * ks[side]) + 2 * b0);
       m.grams.push_back(x);
     };
-    const bool f16 = q.precision == ICWF_MIXED_TF32X3;
-    const int pk = f16 ? SRC_F32_F16 : SRC_F32_BF16;
     for (int s = 0; s < 2; ++s) {
       if (r > 0) break;   // bras and the overlap once per assembly
-      const int bd = f64 ? 6 : (n[s] <= 2048 ? 6 : 5), beta = f64 ? fdig : bd;
-      if (!split_s) {
-        add_slice(s, nullptr, sa[s], se[s], MT, dS, f64 ? SRC_F64_DIGITS : SRC_F32_DIGITS, bd, beta);
-        const int L = f64 ? dS : 2 * dS - 1;
-        add_gram(s, sa[s], se[s], dS, nullptr, nullptr, dS, L, 32, f64 ? drain_slices(dS) : 1 << 20, false, true,
-                 bd, beta, s ? m.S2 : m.S1);
-      }
-      if (!f64) {
-        add_slice(s, nullptr, pa[s], pe[s], MT, 2, pk, 0, 0);
-        if (split_s)
-          add_gram(s, pa[s], pe[s], 2, nullptr, nullptr, 2, 2, kets_per_unit(N, MT), 1 << 20, f16, false, 0, 0,
-                   s ? m.S2 : m.S1);
-      }
+      const int bd = f64 ? 6 : (n[s] <= 2048 ? 6 : 5), beta = f64 ? 7 : bd;
+      add_slice(s, nullptr, sa[s], se[s], MT, dS, bd, beta);
+      const int L = f64 ? dS : 2 * dS - 1;
+      add_gram(s, sa[s], se[s], dS, nullptr, nullptr, dS, L, 32, f64 ? drain_slices(dS) : 1 << 20, bd, beta,
+               s ? m.S2 : m.S1);
     }
     size_t so = scratch;
     auto tmp = [&](size_t bytes) { const size_t o = so; so += al(bytes); return o; };
@@ -1454,12 +1364,11 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
       for (int s = 0; s < 2; ++s) {
         const int d = dg[g];
         int t = d <= 2 ? 128 : (d <= 4 ? 64 : 32);
-        const int dr = f64 ? drain_slices(d) : 1 << 20;
+        const int dr = drain_slices(d);
         if (dr < ks[s]) t = 32;
         t = kets_per_unit(N, t);
         const size_t o = tmp(op_bytes(s, d)), oe = tmp((size_t)rp * 4);
-        const void* w = f64 ? (const void*)((const double*)ptr(s ? m.o_ww : m.o_uw) + (size_t)g * n[s])
-                            : (const void*)((const float*)ptr(s ? m.o_ww : m.o_uw) + (size_t)g * n[s]);
+        const double* w = (const double*)ptr(s ? m.o_ww : m.o_uw) + (size_t)g * n[s];
         // consecutive terms in the same format share a group (their operands are evenly spaced)
         Slice* last = grp[s] >= 0 ? &m.slices[grp[s]] : nullptr;
         if (last && last->ng < SLICE_GROUP && last->d == d && last->R == t) {
@@ -1472,10 +1381,10 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
         }
         if (!last) {
           grp[s] = (int)m.slices.size();
-          add_slice(s, w, o, oe, t, d, f64 ? SRC_F64_DIGITS : pk, f64 ? 6 : 0, f64 ? fdig : 0);
+          add_slice(s, w, o, oe, t, d, 6, 7);
         }
-        add_gram(s, f64 ? sa[s] : pa[s], f64 ? se[s] : pe[s], f64 ? dS : 2, ptr(o), (int*)ptr(oe), d, d, t, dr,
-                 !f64 && f16, f64, f64 ? 6 : 0, f64 ? fdig : 0, (s ? b.B : b.A) + (size_t)(g - g0) * out_b);
+        add_gram(s, sa[s], se[s], dS, ptr(o), (int*)ptr(oe), d, d, t, dr, 6, 7,
+                 (s ? b.B : b.A) + (size_t)(g - g0) * out_b);
       }
     b.nslice = (int)m.slices.size() - b.slice0;
     b.ngram = (int)m.grams.size() - b.gram0;
@@ -1504,7 +1413,7 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     x.A = ptr(m.r_xa); x.B = ptr(m.r_Rb);
     x.ea = (int*)ptr(m.r_xe); x.eb = (int*)ptr(m.r_Re);
     x.ks = ksN; x.da = x.d = x.l = m.rec_d; x.t = 32; x.drain = drain_slices(m.rec_d);
-    x.digits = 1; x.b0 = 6; x.beta = 7;
+    x.b0 = 6; x.beta = 7;
     x.fbits = 62 - (1 + ilog2_ceil(16 * ksN) + 12);
     x.rows = q.nx; x.cols = q.nR;
     m.rec_gram = (int)m.grams.size();
@@ -1521,7 +1430,6 @@ bool AsmPlan::upload(const AsmShape& q, const double* U, const double* W, cudaSt
   using namespace sl;
   Impl& m = *impl;
   const size_t nu = (size_t)q.K * q.nx, nw = (size_t)q.K * q.nR;
-  const void *hu, *hw;
   if (m.f64) {
     m.Uw.resize(nu);
     m.Ww.resize(nw);
@@ -1529,19 +1437,13 @@ bool AsmPlan::upload(const AsmShape& q, const double* U, const double* W, cudaSt
       for (int i = 0; i < q.nx; ++i) m.Uw[(size_t)g * q.nx + i] = U[(size_t)g * q.nx + i] * (q.sig[g] * q.dx);
       for (int i = 0; i < q.nR; ++i) m.Ww[(size_t)g * q.nR + i] = W[(size_t)g * q.nR + i] * q.dR;
     }
-    hu = m.Uw.data();
-    hw = m.Ww.data();
-  } else {
-    m.Uf.assign(U, U + nu);
-    m.Wf.assign(W, W + nw);
-    hu = m.Uf.data();
-    hw = m.Wf.data();
-  }
-  const size_t ws = m.f64 ? 8 : 4;
-  if (cudaMemcpyAsync(m.base + m.o_uw, hu, nu * ws, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(m.base + m.o_ww, hw, nw * ws, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemsetAsync(m.base + m.o_done, 0, (size_t)tiles_of(q.N) * 16 * 4, s) != cudaSuccess)
+    if (cudaMemcpyAsync(m.base + m.o_uw, m.Uw.data(), nu * 8, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(m.base + m.o_ww, m.Ww.data(), nw * 8, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemsetAsync(m.base + m.o_done, 0, (size_t)tiles_of(q.N) * 16 * 4, s) != cudaSuccess)
+      return false;
+  } else if (!heff_tc_ready()) {
     return false;
+  }
   if (cudaMemcpyAsync(m.base + m.o_slices, m.slices.data(), m.slices.size() * sizeof(Slice), cudaMemcpyHostToDevice,
                       s) != cudaSuccess ||
       cudaMemcpyAsync(m.base + m.o_grams, m.grams.data(), m.grams.size() * sizeof(Gram), cudaMemcpyHostToDevice,
@@ -1555,6 +1457,7 @@ bool AsmPlan::upload(const AsmShape& q, const double* U, const double* W, cudaSt
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
     attr = cudaFuncSetAttribute(k_gram_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    if (attr == cudaSuccess) attr = heff_tc_attributes();
   });
   return attr == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess;
 }
@@ -1577,24 +1480,30 @@ int AsmPlan::launch(const JobView& j, double2* S, double2* H, cudaStream_t s) co
     ga.ticket = (unsigned*)(m.base + m.o_ticket);
     ga.status = j.status;
     k_gram_sliced<<<std::min(b.units, m.sms), THREADS, SMEM_BYTES, s>>>(ga);
+    if (!m.f64) {
+      k_overlap<<<dim3(16, tiles), 256, 0, s>>>(j.N, (const double2*)(m.base + m.S1), (const double2*)(m.base + m.S2),
+                                                j.dx, j.dR, S);
+      break;
+    }
     HeffArgs ha;
     ha.N = j.N; ha.g0 = b.g0; ha.g1 = b.g1;
     ha.first = b.g0 == 0;
     ha.last = b.g1 == j.K;
-    ha.S1 = m.base + m.S1; ha.S2 = m.base + m.S2;
-    ha.A = m.base + b.A; ha.B = m.base + b.B;
+    ha.S1 = (const double2*)(m.base + m.S1); ha.S2 = (const double2*)(m.base + m.S2);
+    ha.A = (const double2*)(m.base + b.A); ha.B = (const double2*)(m.base + b.B);
     ha.tiles = tiles;
-    ha.split_s = m.split_s;
     ha.dx = j.dx; ha.dR = j.dR;
     ha.sig = j.sig; ha.px = j.px; ha.pR = j.pR; ha.d = j.d;
     ha.S = S; ha.H = H;
     ha.split = std::max(1, std::min(m.split, (b.g1 - b.g0) / 4));
-    ha.part = m.base + m.part;
+    ha.part = (double2*)(m.base + m.part);
     ha.done = (unsigned*)(m.base + m.o_done);
-    if (m.f64) k_heff<false><<<dim3(16, tiles, ha.split), 256, 0, s>>>(ha);
-    else k_heff<true><<<dim3(16, tiles, ha.split), 256, 0, s>>>(ha);
+    k_heff<<<dim3(16, tiles, ha.split), 256, 0, s>>>(ha);
   }
-  return 3 * (int)m.batches.size();
+  int launches = 3 * (int)m.batches.size();
+  // the overlap's operands are no longer needed: the scratch is one region
+  if (!m.f64) launches += launch_heff_tc(j, m.precision, m.split_s ? S : nullptr, H, m.base + m.heff, s);
+  return launches;
 }
 
 // Psi[i nR + j] = sum_a C_a psi_a(x_i) chi_a(R_j) as a sliced product over the trajectories: 8 digits

@@ -17,7 +17,6 @@ namespace sl {
 
 constexpr int MT = 128;          // bras (and kets) per output tile
 constexpr int ROW_BYTES = 32;    // one operand row of a K slice: 16 values of 2 bytes
-constexpr int PIECE_BITS = 14;   // hi/lo pieces are scaled to |v| < 2^14
 
 // Byte offset of the 8-point half `part` of row r inside an operand tile: rows of 32 bytes, the two
 // 16-byte halves swapped in every second group of four rows (the 32-byte swizzle: address bit 4 is

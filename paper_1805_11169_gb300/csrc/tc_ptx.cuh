@@ -134,12 +134,7 @@ __host__ __device__ constexpr uint32_t idesc_mn(int kind, int M, int N_) {
          ((uint32_t)(N_ >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// The same for kind::f16 with FP16 (f16 = 1) or BF16 pieces, without its N field (idesc_n); NEG_A
-// multiplies A by -1.
-__host__ __device__ constexpr uint32_t idesc_f16(int f16, int M, int N_) {
-  return (1u << 4) | ((f16 ? 0u : 1u) << 7) | ((f16 ? 0u : 1u) << 10) | ((uint32_t)(N_ >> 3) << 17) |
-         ((uint32_t)(M >> 4) << 24);
-}
+// The N field alone; NEG_A multiplies A by -1.
 __host__ __device__ constexpr uint32_t idesc_n(int N_) { return (uint32_t)(N_ >> 3) << 17; }
 constexpr uint32_t IDESC_NEG_A = 1u << 13;
 
