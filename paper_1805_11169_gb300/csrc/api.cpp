@@ -287,28 +287,12 @@ void kinetic_tables(int n, double d, double mass, double dt, std::vector<double>
   }
 }
 
-// Complex table in FP32: of the FP32 neighbours of (re, im) the pair whose modulus is nearest to the
-// exact one.  Rounding the components one by one leaves moduli off by up to 6e-8, always to the same
-// side for a given entry: the FFTs then lose 1.2e-7 of every CWF's norm per step (measured; a
-// quarter of that with these tables, and the CWFs' error after 10 steps falls from 1.0e-6 to 6.6e-7).
-std::vector<float> cast_modulus(const std::vector<double>& v) {
-  std::vector<float> f(v.size());
-  for (size_t e = 0; e + 1 < v.size(); e += 2) {
-    const double m2 = v[e] * v[e] + v[e + 1] * v[e + 1];
-    float c[2][2];
-    for (int k = 0; k < 2; ++k) {
-      c[k][0] = (float)v[e + k];
-      c[k][1] = std::nextafter(c[k][0], (double)c[k][0] < v[e + k] ? HUGE_VALF : -HUGE_VALF);
-      if ((double)c[k][0] == v[e + k]) c[k][1] = c[k][0];   // exact: keep it
-    }
-    double best = HUGE_VAL;
-    for (float x : c[0])
-      for (float y : c[1]) {
-        const double d = std::fabs(((double)x * x + (double)y * y) - m2);
-        if (d < best) { best = d; f[e] = x; f[e + 1] = y; }
-      }
-  }
-  return f;
+// A table in FP32, every component rounded to nearest.  (Of the neighbouring pairs the one with the
+// nearest modulus loses less of the CWFs' norm per step, but its phases are off by up to a unit in the
+// last place instead of half of one, and the CWFs, and all that S + eps I amplifies, move.)
+template <typename T>
+std::vector<T> cast_vec(const std::vector<double>& v) {
+  return std::vector<T>(v.begin(), v.end());
 }
 
 icwf_status upload(icwf_ctx* h, void* dst, const void* src, size_t bytes) {
@@ -839,8 +823,8 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
   std::vector<float> Vf, kxf, kRf, twxf, twRf;
   if (h->mixed) {
     Vf.assign(Vh, Vh + nV);
-    kxf = cast_modulus(kx); kRf = cast_modulus(kR);
-    twxf = cast_modulus(twx); twRf = cast_modulus(twR);
+    kxf = cast_vec<float>(kx); kRf = cast_vec<float>(kR);
+    twxf = cast_vec<float>(twx); twRf = cast_vec<float>(twR);
     UP(h->Vt, Vf.data(), nV * 4);
     UP(h->kinx, kxf.data(), kxf.size() * 4);
     UP(h->kinR, kRf.data(), kRf.size() * 4);

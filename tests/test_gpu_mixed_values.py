@@ -1,5 +1,5 @@
 """The mixed modes' numbers stay those their users have: values recorded on a GB300 from the library as of
-commit 2029912 (tests/golden/mixed_heff.npz).
+commit 2029912 (tests/golden/mixed_heff.npz, mixed_cwf.npz).
 
 Heff's rounding is part of a mixed mode's results: (S + eps I)^-1 with eps = 1e-6 amplifies it, so
 another rounding of the products, a more exact one too, moves the densities by 2e-5 within a few steps.
@@ -47,4 +47,14 @@ def test_densities_after_ten_steps():
     obs = sim.observables()
     want = np.load(os.path.join(GOLDEN, "mixed_heff.npz"))
     assert rel(obs["rho_x"], want["rho_x"]) < 2e-5 and rel(obs["rho_R"], want["rho_R"]) < 2e-5
+    sim.close()
+
+
+def test_cwfs_after_one_step():
+    """The propagator's FP32 tables are rounded to nearest: the same CWFs to a unit of FP32, 2^-25 = 3e-8 in
+    the 2-norm (tables rounded to the nearest modulus instead: 1.9e-7)."""
+    sim = start(717, 512, g.ICWF_MIXED_TF32X3, 1e-6)
+    sim.step(1)
+    want = np.load(os.path.join(GOLDEN, "mixed_cwf.npz"))["psi"]
+    assert rel(sim.state()["psi"][:, :2], want) < 3e-8
     sim.close()
