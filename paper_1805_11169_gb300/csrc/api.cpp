@@ -744,7 +744,14 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
       (size_t)2 * nblk * 4 + 64, chol_ctl_words(N) * sizeof(unsigned), 64 * 4};
   size_t total = 0;
   for (size_t b : sizes) total += align256(b);
-  const AsmShape shape{N, nx, nR, K, p.precision, p.overlap_split, h->dx, h->dR, sk.data()};
+  std::vector<double> peak(K);
+  for (int k = 0; k < K; ++k) {
+    double u = 0.0, w = 0.0;
+    for (int i = 0; i < nx; ++i) u = std::max(u, std::fabs(Uk[(size_t)k * nx + i]));
+    for (int i = 0; i < nR; ++i) w = std::max(w, std::fabs(Wk[(size_t)k * nR + i]));
+    peak[k] = sk[k] * u * w;
+  }
+  const AsmShape shape{N, nx, nR, K, p.precision, p.overlap_split, h->dx, h->dR, sk.data(), peak.data()};
   h->plan_bytes = h->plan.layout(shape, nullptr, nullptr) + 1024;
   total += align256(h->plan_bytes);
   if (!h->df_solve) {

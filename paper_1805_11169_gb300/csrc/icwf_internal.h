@@ -127,6 +127,7 @@ struct AsmShape {
   int N, nx, nR, K, precision, overlap_split;
   double dx, dR;
   const double* sig;      // K singular values (host)
+  const double* peak;     // K largest values s_g max|u_g| max|w_g| of the terms (host)
 };
 class AsmPlan {
  public:

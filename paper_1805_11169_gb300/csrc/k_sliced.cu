@@ -17,10 +17,11 @@
 // (One MMA per pair, N = 64, measured 88-115 cycles where the tensor pipe needs 32.)
 // L = D keeps products down to the pieces' own truncation; the overlap keeps all 2D - 1 levels.
 //
-// Digits are only as many as a term needs: term g of the interaction enters Heff with weight s_g, so
-// it takes D_g = ceil((56 + log2(s_g / s_1)) / 7) digits and its truncation error equals that of the
-// first term, 2^-56 of s_1, which is FP64's own (the FP64 products these replace rounded each sum at
-// 2^-53).  At the paper's scale (22 terms) that is 22 digit pairs on average instead of 36.
+// Digits are only as many as a term needs: term g of the interaction is at most v_g = s_g max|u_g|
+// max|w_g| anywhere on the grid, so it takes D_g = ceil((56 + log2(v_g / max v)) / 7) digits, and every
+// term is cut 2^-56 below the largest one.  That is below the factors' own rounding (the SVD leaves 2^-53
+// of s_1, spread over the grid), also for a term that sits on a few grid points, where s_g alone says
+// little.  At the paper's scale (21 terms) it is 23 digit pairs on average instead of 36.
 //
 // Level sums (digits) are combined as 64-bit integers, in units of 2^-F of level 0, and converted
 // once: no FP64 instruction in the loop (FP64 runs at 1/61 of FP32 here).  The accumulators are drained
@@ -1081,7 +1082,7 @@ int drain_slices(int d) {
   return s;
 }
 
-// Digits of term g (relative weight r = s_g / s_1).
+// Digits of a term of relative size r (of its largest value on the grid, to the largest of all terms).
 int term_digits(double r) {
   if (!(r > 0)) return 2;
   const int d = (int)std::ceil((56.0 + std::log2(r)) / 7.0);
@@ -1284,7 +1285,8 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     m.split = std::max(1, std::min({16, 304 / patches, K / 4}));
     m.o_done = take((size_t)tiles * 16 * 4);
     if (m.split > 1) m.part = take((size_t)m.split * tiles * 2 * MT * MT * sizeof(double2));
-    for (int g = 0; g < K; ++g) dg[g] = term_digits(q.sig[0] > 0 ? q.sig[g] / q.sig[0] : 0.0);
+    const double top = *std::max_element(q.peak, q.peak + K);
+    for (int g = 0; g < K; ++g) dg[g] = term_digits(top > 0 ? q.peak[g] / top : 0.0);
   } else {
     if (!split_s) ranges.push_back({0, 0});   // the overlap alone
     batch_max = heff_tc_scratch_bytes(N, q.nx, q.nR, K);
