@@ -100,7 +100,9 @@ typedef struct {
   double tail_rel;          /* ||dropped part of V_c||_F / ||V_c||_F */
   double next_rel;          /* first dropped singular value / largest (0 if none dropped) */
   double sigma_max;         /* largest singular value of V_c */
-  size_t device_bytes;      /* device memory held by the handle */
+  size_t device_bytes;      /* device memory of the handle's state: CWFs, tables, matrices, factors and
+                               the mixed modes' split operands.  A pool admits the job by it.  Work
+                               space comes on top: icwf_work_bytes, and obs_bytes */
   int64_t steps_done;       /* completed time steps since init */
   double t;                 /* simulated time */
   int64_t kernel_launches;  /* CUDA kernels launched by icwf_step on this handle since create */
@@ -178,6 +180,12 @@ icwf_status icwf_get_state(icwf_handle h, double* C, double* x, double* R, doubl
 icwf_status icwf_get_matrices(icwf_handle h, double* S, double* H, double* Heff);
 
 icwf_status icwf_get_info(icwf_handle h, icwf_info* out);
+
+/* Device memory the handle holds beyond icwf_info.device_bytes: the operands and Grams of the FP64
+ * mode's matrix elements (in batches of terms of 128 MB, or of one term where that is more), the mixed
+ * modes' overlap where the split operands' space is too small for it, and the triangular solves'
+ * products with neighbouring blocks. */
+icwf_status icwf_work_bytes(icwf_handle h, size_t* bytes);
 
 /* --- checkpoint / resume ------------------------------------------------------------------- */
 
@@ -282,7 +290,7 @@ icwf_status icwf_observables_static(icwf_handle h, icwf_obs* out);
 
 /* --- serving pool: continuous batching of independent jobs -------------------------------- */
 
-/* A pool admits jobs while their summed device footprint stays within hbm_budget_bytes and at
+/* A pool admits jobs while their summed device_bytes stay within hbm_budget_bytes and at
  * most max_jobs are live; pending jobs wait in arrival order.  Every icwf_pool_tick advances
  * every live job by one step.  By default each tick is one CUDA graph, instantiated once per live
  * set and parity pattern and launched with a single cudaGraphLaunch: first the grouped kernels,

@@ -79,6 +79,7 @@ def _load():
         "icwf_get_state": [H, d, d, d, d, d],
         "icwf_get_matrices": [H, d, d, d],
         "icwf_get_info": [H, P(icwf_info)],
+        "icwf_work_bytes": [H, P(ct.c_size_t)],
         "icwf_heff_direct": [H, ct.c_int32, P(ct.c_int32), d],
         "icwf_state_bytes": [H, P(ct.c_size_t)],
         "icwf_save_state": [H, ct.c_void_p, ct.c_size_t],
@@ -264,6 +265,12 @@ def icwf_save_state(h) -> bytes:
 def icwf_load_state(h, blob: bytes):
     buf = ct.create_string_buffer(blob, len(blob))
     _check(LIB.icwf_load_state(h, buf, len(blob)), h)
+
+
+def icwf_work_bytes(h) -> int:
+    n = ct.c_size_t()
+    _check(LIB.icwf_work_bytes(h, ct.byref(n)), h)
+    return n.value
 
 
 def icwf_get_stream(h) -> int:

@@ -93,7 +93,7 @@ struct icwf_ctx {
   double *invL[2] = {nullptr, nullptr}, *invLh = nullptr;   // reciprocal Cholesky pivots
   double2 *DL[2] = {nullptr, nullptr}, *DLh = nullptr;       // inverted 32 x 32 diagonal blocks
   unsigned *flags = nullptr, *tickets = nullptr;
-  void* herk_scratch = nullptr;                              // two-level double-float factorisation
+  void* herk_scratch = nullptr;   // two-level double-float factorisation: the plan's work region
   unsigned* cctl = nullptr;                                  // blocked-factorisation tickets/flags
   int* status = nullptr;
   int cur = 0;
@@ -108,7 +108,7 @@ struct icwf_ctx {
   std::vector<void*> extra_allocs;
   size_t obs_bytes = 0;                     // observables work buffers (allocated on first use)
   AsmPlan plan;                             // assembly: operand slices, Grams and their tables
-  size_t plan_bytes = 0;
+  size_t plan_bytes = 0, work_bytes = 0;
   // FP64 factorisation: digit planes of the emulated trailing update (allocated when !df_solve)
   void* emu_scratch = nullptr;
   size_t emu_bytes = 0;
@@ -564,6 +564,8 @@ int tune_propagate(icwf_ctx* h) {
   return best;
 }
 
+size_t footprint(const icwf_ctx* h) { return h->arena.size - h->work_bytes; }
+
 icwf_status alloc_obs(icwf_ctx* h) {
   if (h->Psi) return ICWF_OK;
   void* p = nullptr;
@@ -752,15 +754,18 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
     peak[k] = sk[k] * u * w;
   }
   const AsmShape shape{N, nx, nR, K, p.precision, p.overlap_split, h->dx, h->dR, sk.data(), peak.data()};
-  h->plan_bytes = h->plan.layout(shape, nullptr, nullptr) + 1024;
-  total += align256(h->plan_bytes);
+  const size_t herk_bytes = h->df_solve ? herk_df_bytes(N) : 0;
+  h->plan_bytes = align256(h->plan.layout(shape, nullptr, nullptr, herk_bytes) + 1024);
+  total += h->plan_bytes;
+  // the handle's size, by which a pool admits it, is that of its state, factors and the mixed modes'
+  // split operands; what the plan needs beyond them and the neighbour products are work space
+  const size_t plan_state = h->mixed ? std::min(h->plan_bytes, heff_tc_scratch_bytes(N, nx, nR, K)) : 0;
+  h->work_bytes = h->plan_bytes - plan_state + 3 * (dl - (size_t)N * 512);
   if (!h->df_solve) {
     h->emu_bytes = herk_emu_scratch_bytes(N);
     total += align256(h->emu_bytes);
     herk_emu_attributes();
   }
-  const size_t herk_bytes = h->df_solve ? herk_df_bytes(N) : 0;
-  total += align256(herk_bytes);
   total += 4096;
   if (cudaMalloc(&h->arena.base, total) != cudaSuccess) {
     destroy_streams(h);
@@ -812,9 +817,8 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
   h->cctl = (unsigned*)a.take(chol_ctl_words(N) * sizeof(unsigned));
   h->status = (int*)a.take(64 * 4);
   if (!h->df_solve) h->emu_scratch = a.take(h->emu_bytes);
-  if (herk_bytes) h->herk_scratch = a.take(herk_bytes);
   char* plan_base = (char*)a.take(h->plan_bytes);
-  if (!h->status || !plan_base || (!h->df_solve && !h->emu_scratch) || (herk_bytes && !h->herk_scratch)) {
+  if (!h->status || !plan_base || (!h->df_solve && !h->emu_scratch)) {
     cudaFree(h->arena.base);
     destroy_streams(h);
     return fail(nullptr, ICWF_ERR_OOM, "icwf_create: arena layout overflow");
@@ -854,7 +858,8 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
 #undef UP
   {
     const JobView j = view(h);
-    h->plan.layout(shape, &j, (void*)(((uintptr_t)plan_base + 1023) & ~(uintptr_t)1023));
+    h->plan.layout(shape, &j, (void*)(((uintptr_t)plan_base + 1023) & ~(uintptr_t)1023), herk_bytes);
+    if (herk_bytes) h->herk_scratch = h->plan.work();
     if (!h->plan.upload(shape, Uk.data(), Wk.data(), h->stream)) {
       cudaFree(h->arena.base);
       destroy_streams(h);
@@ -1280,12 +1285,18 @@ icwf_status icwf_get_info(icwf_handle h, icwf_info* out) {
   out->tail_rel = h->tail_rel;
   out->next_rel = h->next_rel;
   out->sigma_max = h->sigma_max;
-  out->device_bytes = h->arena.size;
+  out->device_bytes = footprint(h);
   out->steps_done = h->steps;
   out->t = h->t;
   out->kernel_launches = h->launches;
   out->obs_bytes = h->obs_bytes;
   out->prop_threads = h->prop_threads;
+  return ICWF_OK;
+}
+
+icwf_status icwf_work_bytes(icwf_handle h, size_t* bytes) {
+  if (!h || !bytes) return fail(h, ICWF_ERR_ARG, "icwf_work_bytes: NULL argument");
+  *bytes = h->work_bytes;
   return ICWF_OK;
 }
 
@@ -1540,7 +1551,7 @@ icwf_status icwf_pool_get_stats(icwf_pool pool, icwf_pool_stats* out) {
 icwf_status icwf_pool_submit(icwf_pool pool, icwf_handle job, int64_t n_steps, int32_t* job_id) {
   if (!pool || !job || n_steps < 0) return fail(nullptr, ICWF_ERR_ARG, "icwf_pool_submit: invalid argument");
   if (!job->initialised) return fail(nullptr, ICWF_ERR_STATE, "icwf_pool_submit: job not initialised");
-  if (job->arena.size > pool->budget)
+  if (footprint(job) > pool->budget)
     return fail(nullptr, ICWF_ERR_OOM, "icwf_pool_submit: job footprint exceeds the pool budget");
   PoolJob pj;
   pj.h = job;
@@ -1573,7 +1584,7 @@ static void finish_job(icwf_pool pool, int id, bool ok) {
     j.state = 3;
   }
   destroy_job_graphs(j);
-  pool->live_bytes -= h->arena.size;
+  pool->live_bytes -= footprint(h);
   icwf_destroy(h);
   j.h = nullptr;
 }
@@ -1589,7 +1600,7 @@ icwf_status icwf_pool_tick(icwf_pool pool, int32_t* n_live, int32_t* n_finished)
   if (!pool) return fail(nullptr, ICWF_ERR_ARG, "icwf_pool_tick: NULL pool");
   while (!pool->pending.empty() && (int)pool->live.size() < pool->max_jobs) {
     const int id = pool->pending.front();
-    const size_t b = pool->jobs[id].h->arena.size;
+    const size_t b = footprint(pool->jobs[id].h);
     if (pool->live_bytes + b > pool->budget) break;
     pool->pending.pop_front();
     pool->live.push_back(id);

@@ -136,8 +136,10 @@ class AsmPlan {
   AsmPlan(const AsmPlan&) = delete;
   AsmPlan& operator=(const AsmPlan&) = delete;
   // Lays the plan out at `base` (1024-byte aligned; NULL to size it) and returns its bytes; j holds
-  // the device pointers the kernels read (NULL while sizing).
-  size_t layout(const AsmShape& q, const JobView* j, void* base);
+  // the device pointers the kernels read (NULL while sizing).  work(): its region of work_min bytes or
+  // more, the caller's between launch() and reconstruct() calls of the same stream.
+  size_t layout(const AsmShape& q, const JobView* j, void* base, size_t work_min);
+  void* work() const;
   // Uploads the tables (U: K x nx and W: K x nR factors on the host) and sets the kernels' attributes.
   bool upload(const AsmShape& q, const double* U, const double* W, cudaStream_t s);
   // Returns the number of kernels launched.

@@ -86,13 +86,13 @@ struct Gram {
   const unsigned char* B;   // kets: T-row tiles with d pieces per plane, or NULL: rows of A
   const int* ea;            // scale exponents of the bras and kets
   const int* eb;
-  double2* out;             // [tile of 128 x 128][ket][bra]
+  double2* out;             // tiles [ket][bra] as in Tri
   int ks, da, d, l, t;      // K slices; pieces stored / used; levels; kets per unit
   int drain;                // K slices per accumulation
   int b0, beta, fbits;      // digit weights; fraction bits of the integer accumulators
   int unit0;                // first unit
-  int cols;                 // 0: upper-triangle tiles; else a rectangular product of rows x cols
-  int rows;                 //    elements, out row-major (double2)
+  int cols;                 // 0: upper-triangle tiles of `rows` trajectories; else a rectangular product
+  int rows;                 //    of rows x cols elements, out row-major
 };
 
 struct GramArgs {
@@ -105,22 +105,27 @@ struct GramArgs {
   int* status;
 };
 
-// Where unit v of Gram g reads and writes: bra tile, ket tile (of T rows), first output element and
-// the output's strides along bras and kets.
+// Where unit v of Gram g reads and writes: bra tile, ket tile (of T rows), first output element, the
+// output's strides along bras and kets, and how many of each are stored.
 struct UnitAt {
   int I, J, bt;             // bra tile; 128-ket tile and T-ket tile
   size_t out;
-  int sr, sc;
+  int sr, sc, nr, nc;
 };
 __device__ __forceinline__ UnitAt unit_at(const Gram& g, int v) {
   UnitAt u;
   const int qn = MT / g.t;
   if (g.cols == 0) {
-    tri_tile(v / qn, u.I, u.J);
-    u.bt = u.J * qn + v % qn;
-    u.out = ((size_t)(v / qn) * MT + (v % qn) * g.t) * MT;
+    const Tri tri(g.rows);
+    int tile, part;
+    tri.unit(v, g.t, tile, part);
+    tri_tile(tile, u.I, u.J);
+    u.bt = u.J * qn + part;
+    u.out = tri.at(tile) + (size_t)part * g.t * tri.br;
     u.sr = 1;
-    u.sc = MT;
+    u.sc = tri.br;
+    u.nr = tri.br;
+    u.nc = (tile < tri.full ? MT : tri.kl) - part * g.t;
   } else {
     const int nt = (g.cols + g.t - 1) / g.t;
     u.I = v / nt;
@@ -129,6 +134,8 @@ __device__ __forceinline__ UnitAt unit_at(const Gram& g, int v) {
     u.out = (size_t)u.I * MT * g.cols + (size_t)u.bt * g.t;
     u.sr = g.cols;
     u.sc = 1;
+    u.nr = g.rows - u.I * MT;
+    u.nc = g.cols - u.bt * g.t;
   }
   return u;
 }
@@ -509,8 +516,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_gram_sliced(GramArgs args) {
       const int xb0 = lane < t / 2 ? eb[lane] : 0, xb1 = 32 + lane < t / 2 ? eb[32 + lane] : 0;
       const size_t o = at.out + (size_t)row * at.sr + (size_t)c0 * at.sc;
       const int sc = at.sc;
-      // kets this lane stores (rows and columns past the edge of a rectangular product: none)
-      const int nk = g.cols == 0 ? t : (at.I * MT + row < g.rows ? g.cols - at.bt * t - c0 : 0);
+      const int nk = row < at.nr ? at.nc - c0 : 0;      // kets this lane stores, from c0 on
       const uint32_t col = base + half * (t / 2);
       if (args.herk[0]) {
         float4* A = args.ngrams > 1 && u >= unit0[1] ? args.herk[1] : args.herk[0];
@@ -879,13 +885,12 @@ __global__ void __launch_bounds__(ST_WARPS * 32) k_slices_t(SliceT sx, SliceT sR
 struct HeffArgs {
   int N, g0, g1, first, last;
   const double2 *S1, *S2;   // raw Grams of the overlap
-  const double2 *A, *B;     // Grams of the terms g0.., `tiles` 128 x 128 tiles each
-  size_t tiles;
+  const double2 *A, *B;     // Grams of the terms g0.., one after the other
   double dx, dR;
   const double *sig, *px, *pR, *d;
   double2 *S, *H;
   int split;                // term groups (blockIdx.z); > 1: partial sums meet in `part`
-  double2* part;            // [group][tile][direct, mirrored][128 x 128]
+  double2* part;            // [group][direct, mirrored], a Gram's storage each
   unsigned* done;           // [tile][patch]: groups finished (zero between launches)
 };
 
@@ -926,7 +931,8 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
   const int a = I * MT + ar, b0 = J * MT + br;
   if (I * MT + (int)(blockIdx.x & 3) * 32 >= N || J * MT + (int)(blockIdx.x >> 2) * 32 >= N) return;
   const bool mirror = I != J, a_ok = a < N;
-  const size_t at0 = ((size_t)blockIdx.y * MT + br) * MT + ar, step = (size_t)8 * MT;
+  const Tri tri(N);
+  const size_t gs = tri.size(), at0 = tri.at(blockIdx.y) + (size_t)br * tri.br + ar, step = (size_t)8 * tri.br;
   double2 s1[4], s2[4], h[4], ht[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
@@ -939,7 +945,6 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
       if (mirror) ht[e] = p.H[(size_t)b * N + a];
     }
   }
-  const size_t gs = p.tiles * MT * MT;
   const int as = I * MT + (int)(blockIdx.x & 3) * 32, bs = J * MT + (int)(blockIdx.x >> 2) * 32;
   const int z0 = p.g0 + (int)((long long)(p.g1 - p.g0) * blockIdx.z / p.split);
   const int z1 = p.g0 + (int)((long long)(p.g1 - p.g0) * (blockIdx.z + 1) / p.split);
@@ -982,12 +987,11 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
   if (p.split > 1) {
     // few tiles: the terms are spread over CTAs; the last one to finish a patch adds the groups' sums
     // in their order (so the result does not depend on timing) and goes on
-    const size_t dir = (size_t)MT * MT, grp = p.tiles * 2 * dir;
-    double2* mine = p.part + blockIdx.z * grp + (size_t)blockIdx.y * 2 * dir + (size_t)br * MT + ar;
+    double2* mine = p.part + blockIdx.z * 2 * gs + at0;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       mine[e * step] = h[e];
-      if (mirror) mine[dir + e * step] = ht[e];
+      if (mirror) mine[gs + e * step] = ht[e];
     }
     __threadfence();
     __syncthreads();
@@ -1000,13 +1004,13 @@ __global__ void __launch_bounds__(256) k_heff(HeffArgs p) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) h[e].x = h[e].y = ht[e].x = ht[e].y = 0;
     for (int z = 0; z < p.split; ++z) {
-      const double2* q = p.part + z * grp + (size_t)blockIdx.y * 2 * dir + (size_t)br * MT + ar;
+      const double2* q = p.part + z * 2 * gs + at0;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const double2 v = __ldcg(q + e * step);
         h[e].x += v.x; h[e].y += v.y;
         if (mirror) {
-          const double2 w = __ldcg(q + dir + e * step);
+          const double2 w = __ldcg(q + gs + e * step);
           ht[e].x += w.x; ht[e].y += w.y;
         }
       }
@@ -1049,11 +1053,12 @@ __global__ void __launch_bounds__(256) k_overlap(int N, const double2* __restric
   const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int ac = (int)(blockIdx.x & 3) * 32, bc = (int)(blockIdx.x >> 2) * 32;
   if (I * MT + ac >= N || J * MT + bc >= N) return;
-  const size_t at0 = ((size_t)blockIdx.y * MT + bc + ty) * MT + ac + lane;
+  const Tri tri(N);
+  const size_t at0 = tri.at(blockIdx.y) + (size_t)(bc + ty) * tri.br + ac + lane;
   double2 sv[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    const size_t at = at0 + (size_t)8 * e * MT;
+    const size_t at = at0 + (size_t)8 * e * tri.br;
     sv[e] = cmul(cscale(S1[at], dx), cscale(S2[at], dR));
     if (I * MT + ac + lane == J * MT + bc + ty + 8 * e) sv[e].y = 0.0;
   }
@@ -1065,10 +1070,14 @@ __global__ void __launch_bounds__(256) k_overlap(int N, const double2* __restric
 size_t al(size_t b) { return (b + 1023) & ~(size_t)1023; }
 int ilog2_ceil(int n) { int l = 0; while ((1 << l) < n) ++l; return l; }
 
-// Terms of one batch: as many as fit BATCH_BYTES of operands and Grams (at least one).
-constexpr size_t BATCH_BYTES = (size_t)512 << 20;
+// Terms of one batch: as many as fit BATCH_BYTES of operands and Grams (at least one).  A batch is three
+// launches and a last wave, so more memory is faster: at 512 / 128 / 64 / 32 MB a handle of N = 1024 on
+// 1024 x 512 has 606 / 210 / 147 / 147 MB of work space and takes 6.7 / 7.3 / 7.6 / 7.6 ms for a step and
+// the observables, one of N = 256 on 512 x 256 1.97 / 2.04 / 2.15 / 2.44 ms for two.  128 MB keeps the work
+// space near the size of the handle's own state.
+constexpr size_t BATCH_BYTES = (size_t)128 << 20;
 
-int tiles_of(int N) { const int T = (N + MT - 1) / MT; return T * (T + 1) / 2; }
+int tiles_of(int N) { return Tri(N).tiles(); }
 int kets_per_unit(int N, int most) { return N <= 32 && most > 32 ? 32 : (N <= 64 && most > 64 ? 64 : most); }
 
 // K slices per accumulation of D digits (b0 = 6, beta = 7).  The leading D - 4 levels stay below 2^24
@@ -1088,8 +1097,6 @@ int term_digits(double r) {
   const int d = (int)std::ceil((56.0 + std::log2(r)) / 7.0);
   return d < 2 ? 2 : (d > 8 ? 8 : d);
 }
-
-struct Term { int d; size_t bx, bR; };   // pieces and operand bytes of both sides
 
 // ---------------------------------------------------------------------------- trailing update
 //
@@ -1202,12 +1209,12 @@ int launch_herk_df(int N, int k0, int R0, void* const* A, int nb, void* scratch,
     Gram& g = p.g[m];
     g.A = p.out[m];
     g.ea = g.eb = p.ex[m];
+    g.rows = p.rpad;
     g.ks = g.drain = HERK_KS;
     g.da = g.d = g.l = HERK_D;
     g.t = 32;
     g.b0 = HERK_B0;
     g.beta = HERK_BETA;
-    g.fbits = 62 - (1 + 7 + 2 * HERK_B0);   // sums of 128 x 2 products below 2^(2 b0)
     g.unit0 = m * units;
     ga.herk[m] = (float4*)A[k];
   }
@@ -1231,6 +1238,7 @@ struct AsmPlan::Impl {
   std::vector<sl::Gram> grams;
   std::vector<Batch> batches;
   std::vector<double> Uw, Ww;            // FP64 mode: weights u_g s_g dx and w_g dR
+  size_t work = 0;                       // start of the region below, which every stage uses for itself
   size_t part = 0, o_done = 0;           // split term sums of k_heff
   int split = 1;
   size_t bytes = 0, o_slices = 0, o_grams = 0, o_uw = 0, o_ww = 0, o_ticket = 0;
@@ -1240,14 +1248,13 @@ struct AsmPlan::Impl {
   unsigned char* base = nullptr;
   int precision = 0;
   bool f64 = false, split_s = false;
-  size_t heff = 0;                       // mixed modes: scratch of launch_heff_tc
   int sms = 152;
 };
 
 AsmPlan::AsmPlan() {}
 AsmPlan::~AsmPlan() { delete impl; }
 
-size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
+size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base, size_t work_min) {
   using namespace sl;
   delete impl;
   impl = new Impl;
@@ -1262,18 +1269,11 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
   const int n[2] = {q.nx, q.nR}, ks[2] = {(q.nx + 15) / 16, (q.nR + 15) / 16};
   size_t off = 0;
   auto take = [&](size_t b) { const size_t o = off; off += al(b); return o; };
-  const size_t out_b = (size_t)tiles * MT * MT * sizeof(double2);
+  const size_t out_b = Tri(N).size() * sizeof(double2);
   m.o_ticket = take(256);
-  m.S1 = take(out_b);
-  m.S2 = take(out_b);
-  // digits of the CWFs: the operands of S and the bras of every term
   const int dS = f64 ? 8 : 4;
-  size_t sa[2] = {0, 0}, se[2] = {0, 0};
-  auto op_bytes = [&](int side, int d) { return (size_t)rp * ks[side] * 2 * d * ROW_BYTES; };
-  for (int s = 0; s < 2 && !split_s; ++s) {
-    sa[s] = take(op_bytes(s, dS));
-    se[s] = take((size_t)rp * 4);
-  }
+  auto op_bytes = [&](int side, int rows, int d) { return (size_t)rows * ks[side] * 2 * d * ROW_BYTES; };
+  auto padded = [&](int r) { return (N + r - 1) / r * r; };   // rows of an operand in tiles of r
   std::vector<int> dg(K, 0);
   std::vector<std::pair<int, int>> ranges;   // batches of terms (FP64 mode)
   size_t batch_max = 0;
@@ -1284,18 +1284,25 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     const int patches = tiles_of(N) == 1 ? ((N + 31) / 32) * ((N + 31) / 32) : tiles * 16;
     m.split = std::max(1, std::min({16, 304 / patches, K / 4}));
     m.o_done = take((size_t)tiles * 16 * 4);
-    if (m.split > 1) m.part = take((size_t)m.split * tiles * 2 * MT * MT * sizeof(double2));
     const double top = *std::max_element(q.peak, q.peak + K);
     for (int g = 0; g < K; ++g) dg[g] = term_digits(top > 0 ? q.peak[g] / top : 0.0);
-  } else {
-    if (!split_s) ranges.push_back({0, 0});   // the overlap alone
-    batch_max = heff_tc_scratch_bytes(N, q.nx, q.nR, K);
+  } else if (!split_s) {
+    ranges.push_back({0, 0});   // the overlap alone
   }
+  // kets per unit of a term of d digits
+  auto kets = [&](int side, int d) {
+    const int t = drain_slices(d) < ks[side] ? 32 : (d <= 2 ? 128 : (d <= 4 ? 64 : 32));
+    return kets_per_unit(N, t);
+  };
   for (int g = 0; f64 && g < K;) {
     size_t b = 0;
     int e = g;
     while (e < K && 2 * (e - g) + 4 < MAX_GRAMS) {
-      const size_t add = al(op_bytes(0, dg[e])) + al(op_bytes(1, dg[e])) + 2 * al((size_t)rp * 4) + 2 * al(out_b);
+      size_t add = 2 * al(out_b);
+      for (int s = 0; s < 2; ++s) {
+        const int r = padded(kets(s, dg[e]));
+        add += al(op_bytes(s, r, dg[e])) + al((size_t)r * 4);
+      }
       if (e > g && b + add > BATCH_BYTES) break;
       b += add;
       ++e;
@@ -1304,17 +1311,31 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     ranges.push_back({g, e});
     g = e;
   }
-  // the reconstruction runs between steps in the same scratch
+  // One region for the stages that follow each other: the assembly's operands and Grams (mixed modes: of
+  // the overlap), the mixed modes' split operands, the reconstruction's operands, and what the
+  // caller runs in between (work_min bytes).
+  m.work = off;
+  m.S1 = take(out_b);
+  m.S2 = take(out_b);
+  // digits of the CWFs: the operands of S and the bras of every term
+  size_t sa[2] = {0, 0}, se[2] = {0, 0};
+  for (int s = 0; s < 2; ++s) {
+    sa[s] = take(op_bytes(s, rp, dS));
+    se[s] = take((size_t)rp * 4);
+  }
+  if (m.split > 1) m.part = take((size_t)m.split * 2 * out_b);
   const int rxp = (q.nx + MT - 1) / MT * MT, rRp = (q.nR + MT - 1) / MT * MT, ksN = (N + 15) / 16;
   m.rec_d = f64 ? 8 : 5;
   auto rec_op = [&](int rows) { return (size_t)rows * ksN * 2 * m.rec_d * ROW_BYTES; };
   const size_t rec_bytes = al(rec_op(rxp)) + al(rec_op(rRp)) + al((size_t)rxp * 4) + al((size_t)rRp * 4);
-  const size_t scratch = take(std::max(batch_max, rec_bytes) + 2 * 1024);
-  m.r_xa = scratch;
+  const size_t scratch = take(batch_max);
+  size_t work_bytes = split_s ? 0 : off - m.work;
+  if (!f64) work_bytes = std::max(work_bytes, heff_tc_scratch_bytes(N, q.nx, q.nR, K));
+  off = m.work + al(std::max({work_bytes, rec_bytes, work_min}));
+  m.r_xa = m.work;
   m.r_Rb = m.r_xa + al(rec_op(rxp));
   m.r_xe = m.r_Rb + al(rec_op(rRp));
   m.r_Re = m.r_xe + al((size_t)rxp * 4);
-  m.heff = scratch;
   auto ptr = [&](size_t o) { return m.base + o; };
   for (size_t r = 0; r < ranges.size(); ++r) {
     const int g0 = ranges[r].first, g1 = ranges[r].second;
@@ -1330,7 +1351,7 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
       s.ng = 1;
       s.out = ptr(out);
       s.ex = (int*)ptr(ex);
-      s.n = n[side]; s.ks = ks[side]; s.rows = N; s.rpad = rp; s.R = R;
+      s.n = n[side]; s.ks = ks[side]; s.rows = N; s.rpad = padded(R); s.R = R;
       s.d = d; s.b0 = b0; s.beta = beta;
       m.slices.push_back(s);
     };
@@ -1344,6 +1365,7 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
       x.out = (double2*)ptr(out);
       x.ks = ks[side]; x.da = da; x.d = d; x.l = l; x.t = t; x.drain = drain;
       x.b0 = b0; x.beta = beta;
+      x.rows = N;
       // |sum| <= 2 K 2^(2 b0) units of level 0
       x.fbits = 62 - (1 + ilog2_ceil(16 * ks[side]) + 2 * b0);
       m.grams.push_back(x);
@@ -1365,11 +1387,8 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     for (int g = g0; g < g1; ++g)
       for (int s = 0; s < 2; ++s) {
         const int d = dg[g];
-        int t = d <= 2 ? 128 : (d <= 4 ? 64 : 32);
-        const int dr = drain_slices(d);
-        if (dr < ks[s]) t = 32;
-        t = kets_per_unit(N, t);
-        const size_t o = tmp(op_bytes(s, d)), oe = tmp((size_t)rp * 4);
+        const int dr = drain_slices(d), t = kets(s, d);
+        const size_t o = tmp(op_bytes(s, padded(t), d)), oe = tmp((size_t)padded(t) * 4);
         const double* w = (const double*)ptr(s ? m.o_ww : m.o_uw) + (size_t)g * n[s];
         // consecutive terms in the same format share a group (their operands are evenly spaced)
         Slice* last = grp[s] >= 0 ? &m.slices[grp[s]] : nullptr;
@@ -1401,12 +1420,12 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
     for (int i = 0; i < b.ngram; ++i) {
       Gram& x = m.grams[b.gram0 + i];
       x.unit0 = b.units;
-      b.units += tiles * (MT / x.t);
+      b.units += Tri(N).units(x.t);
     }
     for (int i = 0; i < b.nslice; ++i) {
       const Slice& s = m.slices[b.slice0 + i];
       const int tpr = std::min(2 * s.ks, 256), rpb = 256 / tpr;
-      b.rowgroups = std::max(b.rowgroups, (rp + rpb - 1) / rpb);
+      b.rowgroups = std::max(b.rowgroups, (s.rpad + rpb - 1) / rpb);
     }
     m.batches.push_back(b);
   }
@@ -1427,6 +1446,8 @@ size_t AsmPlan::layout(const AsmShape& q, const JobView* j, void* base) {
   m.bytes = off;
   return m.bytes;
 }
+
+void* AsmPlan::work() const { return impl->base + impl->work; }
 
 bool AsmPlan::upload(const AsmShape& q, const double* U, const double* W, cudaStream_t s) {
   using namespace sl;
@@ -1493,7 +1514,6 @@ int AsmPlan::launch(const JobView& j, double2* S, double2* H, cudaStream_t s) co
     ha.last = b.g1 == j.K;
     ha.S1 = (const double2*)(m.base + m.S1); ha.S2 = (const double2*)(m.base + m.S2);
     ha.A = (const double2*)(m.base + b.A); ha.B = (const double2*)(m.base + b.B);
-    ha.tiles = tiles;
     ha.dx = j.dx; ha.dR = j.dR;
     ha.sig = j.sig; ha.px = j.px; ha.pR = j.pR; ha.d = j.d;
     ha.S = S; ha.H = H;
@@ -1503,8 +1523,8 @@ int AsmPlan::launch(const JobView& j, double2* S, double2* H, cudaStream_t s) co
     k_heff<<<dim3(16, tiles, ha.split), 256, 0, s>>>(ha);
   }
   int launches = 3 * (int)m.batches.size();
-  // the overlap's operands are no longer needed: the scratch is one region
-  if (!m.f64) launches += launch_heff_tc(j, m.precision, m.split_s ? S : nullptr, H, m.base + m.heff, s);
+  // the overlap's operands are no longer needed
+  if (!m.f64) launches += launch_heff_tc(j, m.precision, m.split_s ? S : nullptr, H, m.base + m.work, s);
   return launches;
 }
 

@@ -3,6 +3,7 @@
 // index.  Host and device code.
 #pragma once
 #include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -31,6 +32,29 @@ SL_HD void tri_tile(int t, int& I, int& J) {
   J = c;
   I = t - c * (c + 1) / 2;
 }
+
+// Storage of a Hermitian Gram of N trajectories: 128 x 128 tiles [ket][bra] of the upper triangle, column
+// by column; those of the last column hold only the kets that there are, in whole 32s, and a single tile
+// only such bras.
+struct Tri {
+  int T, full;    // row blocks; tiles before the last column
+  int kl, br;     // kets of the last column's tiles; bras of a row of a tile
+  SL_HD explicit Tri(int N)
+      : T((N + MT - 1) / MT), full(T * (T - 1) / 2), kl((N - (T - 1) * MT + 31) / 32 * 32), br(T == 1 ? kl : MT) {}
+  SL_HD int tiles() const { return full + T; }
+  SL_HD size_t at(int tile) const {
+    return tile <= full ? (size_t)tile * MT * MT : (size_t)full * MT * MT + (size_t)(tile - full) * kl * br;
+  }
+  SL_HD size_t size() const { return at(tiles()); }
+  // units of t kets: of a tile, of all tiles, and the tile and part of unit v
+  SL_HD int units_last(int t) const { return (kl + t - 1) / t; }
+  SL_HD int units(int t) const { return full * (MT / t) + T * units_last(t); }
+  SL_HD void unit(int v, int t, int& tile, int& part) const {
+    const int q = MT / t, f = full * q, l = units_last(t);
+    tile = v < f ? v / q : full + (v - f) / l;
+    part = v < f ? v % q : (v - f) % l;
+  }
+};
 
 SL_HD unsigned long long f64_bits(double x) {
 #if defined(__CUDA_ARCH__)
