@@ -764,9 +764,14 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
   if (!h->df_solve) {
     h->emu_bytes = herk_emu_scratch_bytes(N);
     total += align256(h->emu_bytes);
-    herk_emu_attributes();
   }
   total += 4096;
+  for (cudaError_t e : {step_attributes(), sliced_attributes(), heff_tc_attributes(), cholesky_df_attributes(),
+                        herk_emu_attributes(), cluster_solve_attributes()})
+    if (e != cudaSuccess) {
+      destroy_streams(h);
+      return fail(nullptr, ICWF_ERR_CUDA, std::string("icwf_create: cudaFuncSetAttribute: ") + cudaGetErrorString(e));
+    }
   if (cudaMalloc(&h->arena.base, total) != cudaSuccess) {
     destroy_streams(h);
     return fail(nullptr, ICWF_ERR_OOM, "icwf_create: cudaMalloc of " + std::to_string(total) + " bytes failed");

@@ -115,7 +115,6 @@ bool add_group_nodes(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndep
 // a5 (mixed modes): Heff, and S too if not NULL, from split products on the tensor cores
 // (k_assemble_tc.cu).  heff_tc_ready: the tensor maps can be encoded.  Returns the number of kernels.
 bool heff_tc_ready();
-cudaError_t heff_tc_attributes();
 size_t heff_tc_scratch_bytes(int N, int nx, int nR, int K);
 int launch_heff_tc(const JobView& j, int precision, double2* S, double2* H, void* scratch, cudaStream_t s);
 
@@ -184,7 +183,6 @@ struct EmuPlanes { void* planes[2]; int* ex[2]; int rpad; };   // digit planes i
 EmuPlanes herk_emu_planes(int N, void* scratch);
 bool launch_herk_emu(int N, int jb, double2* const* A, int nbatch, void* scratch, size_t bytes,
                      bool digits_done, int* status, cudaStream_t s);
-void herk_emu_attributes();
 // y = ((1-theta) H0 + theta H1) (C + c * kp)      (kp may be NULL)
 void launch_matvec(int N, const double2* H0, const double2* H1, double theta, const double2* C,
                    const double2* kp, double c, double2* y, cudaStream_t s);
@@ -243,6 +241,16 @@ void launch_init_projection(int N, int nx, int nR, double dx, double dR, const d
                             const double2* chi, const double2* Psi0, double2* b, cudaStream_t s);
 // Convert complex128 -> complex64.
 void launch_to_c64(size_t n, const double2* in, float2* out, cudaStream_t s);
+
+// Function attributes of the kernels (shared memory, cluster size).  They belong to a device's context,
+// so every handle's creation sets them, on its device: a process may use several, and no launch,
+// captured or not, changes one.
+cudaError_t step_attributes();
+cudaError_t sliced_attributes();
+cudaError_t heff_tc_attributes();
+cudaError_t cholesky_df_attributes();
+cudaError_t herk_emu_attributes();
+cudaError_t cluster_solve_attributes();
 
 // Everything the observables kernels need from a handle (filled by handle_obs_view in api.cpp).
 struct ObsView {

@@ -36,7 +36,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "df64.cuh"
 #include "herk_digits.cuh"
@@ -297,14 +296,8 @@ int rpad_for(int N) { return (N + BM - 1) / BM * BM; }
 
 }  // namespace hemu
 
-// The update kernel's shared-memory limit, set once per process by handle creation (outside any
-// stream capture, so that no captured launch changes a function attribute).
-void herk_emu_attributes() {
-  static std::once_flag once;
-  std::call_once(once, []() {
-    cudaFuncSetAttribute(hemu::k_herk_emu, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         hemu::SMEM_BYTES);
-  });
+cudaError_t herk_emu_attributes() {
+  return cudaFuncSetAttribute(hemu::k_herk_emu, cudaFuncAttributeMaxDynamicSharedMemorySize, hemu::SMEM_BYTES);
 }
 
 size_t herk_emu_scratch_bytes(int N) {

@@ -18,7 +18,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "cdf.cuh"
 #include "icwf_internal.h"
@@ -870,6 +869,10 @@ void launch_shift_mix_df(int N, const double2* S0, const double2* S1, double eps
   dfs::k_shift_mix_df<<<N, 256, 0, s>>>(N, S0, S1, eps, theta, (float4*)A);
 }
 
+cudaError_t cholesky_df_attributes() {
+  return cudaFuncSetAttribute(dfs::k_chol_df, cudaFuncAttributeMaxDynamicSharedMemorySize, dfs::CS_SMEM_LAUNCH);
+}
+
 int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, int nbatch,
                        unsigned* ctl, void* herk_scratch, int* status, cudaStream_t s) {
   using namespace dfs;
@@ -881,14 +884,9 @@ int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, 
     mb.D[q] = (float4*)D[k];
   }
   const int T = (N + NB - 1) / NB;
-  static std::once_flag once;
-  static int sms = 0;
-  std::call_once(once, [] {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(k_chol_df, cudaFuncAttributeMaxDynamicSharedMemorySize, CS_SMEM_LAUNCH);
-  });
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaMemsetAsync(ctl, 0, chol_ctl_words(N) * sizeof(unsigned), s);
   int launches = 0;
   for (int lo = 0, hi; lo < T; lo = hi) {

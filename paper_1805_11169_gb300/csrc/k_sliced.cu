@@ -46,7 +46,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <vector>
 
 #include "df64.cuh"
@@ -1182,6 +1181,10 @@ size_t herk_operand(int N) { return herk_rows(N) * HERK_COLS * 2 * HERK_D * 2; }
 
 }  // namespace sl
 
+cudaError_t sliced_attributes() {
+  return cudaFuncSetAttribute(sl::k_gram_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, sl::SMEM_BYTES);
+}
+
 size_t herk_df_bytes(int N) {
   using namespace sl;
   return chol_panel(N) == 0 ? 0 : 1024 + 2 * (herk_rows(N) * sizeof(int) + herk_operand(N));
@@ -1476,13 +1479,7 @@ bool AsmPlan::upload(const AsmShape& q, const double* U, const double* W, cudaSt
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&m.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return false;
-  static std::once_flag once;   // outside any stream capture
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(k_gram_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    if (attr == cudaSuccess) attr = heff_tc_attributes();
-  });
-  return attr == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess;
+  return cudaStreamSynchronize(s) == cudaSuccess;
 }
 
 int AsmPlan::launch(const JobView& j, double2* S, double2* H, cudaStream_t s) const {

@@ -4,8 +4,6 @@
 // Kernels: k_near_products (beside the factorisation), k_cluster_solve.
 #include <cuda_runtime.h>
 
-#include <mutex>
-
 #include "cdf.cuh"
 #include "icwf_internal.h"
 #include "k_common.cuh"
@@ -436,15 +434,17 @@ int near_products(int N, void* const* L, void* const* D, int nbatch, cudaStream_
 }
 
 template <class T, int NI>
+cudaError_t attributes() {
+  const cudaError_t e = cudaFuncSetAttribute(k_cluster_solve<T, NI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem_bytes(NI * WARPS));
+  return e != cudaSuccess ? e
+                          : cudaFuncSetAttribute(k_cluster_solve<T, NI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+template <class T, int NI>
 void launch(int N, const void* L, const void* D, const double2* y, double2* out, bool minus_i, int* status,
             cudaStream_t s) {
   using E = typename T::E;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_cluster_solve<T, NI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem_bytes(NI * WARPS));
-    cudaFuncSetAttribute(k_cluster_solve<T, NI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  });
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = CL;
@@ -470,6 +470,14 @@ void launch_by_size(int N, const void* L, const void* D, const double2* y, doubl
 }
 
 }  // namespace slv
+
+cudaError_t cluster_solve_attributes() {
+  using namespace slv;
+  for (cudaError_t e : {attributes<Df, 1>(), attributes<Df, 2>(), attributes<Df, 4>(), attributes<F64, 1>(),
+                        attributes<F64, 2>(), attributes<F64, 4>()})
+    if (e != cudaSuccess) return e;
+  return cudaSuccess;
+}
 
 // The neighbour products follow the N x 32 inverted diagonal blocks in the D buffer, whole blocks each.
 size_t diag_inv_bytes(int N) { return 5 * slv::near_offset(N) * 16; }

@@ -346,23 +346,10 @@ __global__ void __launch_bounds__(512) k_propagate(JobView j, const T* __restric
   propagate_cta<T>(j, Vt, mode, out_psi, out_chi, kfx, kfR, blockIdx.x, (c_t<T>*)smem_raw);
 }
 
-// The propagator's dynamic shared memory limit, set once (to the largest grid's need) so that no
-// launch, captured or not, changes a function attribute.
-template <typename T>
-void propagate_attr() {
-  static bool done = false;
-  if (!done) {
-    cudaFuncSetAttribute(k_propagate<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(2 * 4096 * sizeof(c_t<T>)));
-    done = true;
-  }
-}
-
 template <typename T>
 void launch_propagate(const JobView& j, int threads, cudaStream_t s) {
   const int nmax = j.nx > j.nR ? j.nx : j.nR;
   const size_t sm = 2 * (size_t)nmax * sizeof(c_t<T>);
-  propagate_attr<T>();
   k_propagate<T><<<2 * j.N, threads, sm, s>>>(j, (const T*)j.Vt, 0, nullptr, nullptr, 0.0, 0.0);
 }
 
@@ -370,7 +357,6 @@ template <typename T>
 void launch_kinetic(const JobView& j, void* out_psi, void* out_chi, cudaStream_t s) {
   const int nmax = j.nx > j.nR ? j.nx : j.nR;
   const size_t sm = 2 * (size_t)nmax * sizeof(c_t<T>);
-  propagate_attr<T>();
   const double PI = 3.14159265358979323846;
   const double gx = 2.0 * PI / (j.nx * j.dx), gR = 2.0 * PI / (j.nR * j.dR);
   const double kfx = gx * gx * 0.5 * j.inv_mx / j.nx;
@@ -420,13 +406,6 @@ template <typename T>
 bool add_group_nodes(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndeps,
                      const GroupJob* table, int njobs, int total_traj, int total_cwf, int nmax,
                      int threads, int max_ctas, cudaGraphNode_t* last) {
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_propagate_group<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(2 * 4096 * sizeof(c_t<T>))) != cudaSuccess)
-      return false;
-    attr = true;
-  }
   if (njobs < 1 || total_traj < 1 || total_cwf < 1 || nmax < 1 || nmax > 4096 || threads < 64 ||
       threads > 512)
     return false;
@@ -469,6 +448,18 @@ template bool add_group_nodes<double>(cudaGraph_t, const cudaGraphNode_t*, size_
                                       cudaGraphNode_t*);
 template bool add_group_nodes<float>(cudaGraph_t, const cudaGraphNode_t*, size_t, const GroupJob*,
                                      int, int, int, int, int, int, cudaGraphNode_t*);
+
+// The propagators' dynamic shared memory limits, at the largest grid's need.
+template <typename T>
+cudaError_t propagate_attributes() {
+  const int bytes = (int)(2 * 4096 * sizeof(c_t<T>));
+  const cudaError_t e = cudaFuncSetAttribute(k_propagate<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(k_propagate_group<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+cudaError_t step_attributes() {
+  const cudaError_t e = propagate_attributes<double>();
+  return e != cudaSuccess ? e : propagate_attributes<float>();
+}
 
 // ------------------------------------------------------------------------------ diagnostic Grams
 
