@@ -300,7 +300,8 @@ icwf_status icwf_observables_static(icwf_handle h, icwf_obs* out);
  * grids); then every job's remaining step (assembly, factorisations, RK4), captured into CUDA
  * graphs at the job's first tick (one per parity of its ping-pong matrix buffers) and added as
  * child graphs.  The jobs share no memory, so their child graphs overlap on the device.  Job
- * handles are owned by the pool after submission. */
+ * handles are owned by the pool after submission, which destroys them when their job finishes or
+ * fails; a call with such a handle returns ICWF_ERR_ARG (icwf_pool_poll tells a job's state). */
 icwf_status icwf_pool_create(size_t hbm_budget_bytes, int32_t max_jobs, icwf_pool* out);
 
 /* Counters of a pool since creation. */

@@ -18,6 +18,7 @@
 #include <memory>
 #include <mutex>
 #include <string>
+#include <unordered_set>
 #include <vector>
 
 #include "icwf_internal.h"
@@ -136,6 +137,22 @@ struct icwf_ctx {
 };
 
 namespace {
+
+// The handles that exist.  A pool destroys its jobs' handles when they finish or fail, and a caller may
+// still hold one: every call looks its handle up before it reads it.  (Never freed: handles may be
+// destroyed while the process ends.)
+struct Handles {
+  std::mutex mutex;
+  std::unordered_set<const icwf_ctx*> set;
+};
+Handles& handles() {
+  static Handles* h = new Handles;
+  return *h;
+}
+bool live(const icwf_ctx* h) {
+  std::lock_guard<std::mutex> lock(handles().mutex);
+  return handles().set.count(h) != 0;
+}
 
 icwf_status fail(icwf_ctx* h, icwf_status st, const std::string& msg) {
   if (h) h->err = msg; else g_err = msg;
@@ -594,7 +611,7 @@ icwf_status alloc_obs(icwf_ctx* h) {
 namespace icwf {
 
 bool handle_obs_view(icwf_handle h, ObsView* v) {
-  if (!h || !v) return false;
+  if (!live(h) || !v) return false;
   v->j = view(h);
   v->plan = &h->plan;
   v->C = h->C;
@@ -622,7 +639,7 @@ void handle_set_error(icwf_handle h, const char* msg) {
 
 extern "C" {
 
-const char* icwf_last_error(icwf_handle h) { return h ? h->err.c_str() : g_err.c_str(); }
+const char* icwf_last_error(icwf_handle h) { return live(h) ? h->err.c_str() : g_err.c_str(); }
 
 icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* out) {
   icwf_ctx* h = nullptr;
@@ -879,12 +896,20 @@ icwf_status icwf_create(const icwf_params* pp, const double* Vh, icwf_handle* ou
     destroy_streams(h);
     return fail(nullptr, ICWF_ERR_CUDA, "icwf_create: initial device transfer failed");
   }
+  {
+    std::lock_guard<std::mutex> lock(handles().mutex);
+    handles().set.insert(h);
+  }
   *out = hp.release();
   return ICWF_OK;
 }
 
 icwf_status icwf_destroy(icwf_handle h) {
   if (!h) return ICWF_OK;
+  {
+    std::lock_guard<std::mutex> lock(handles().mutex);
+    if (!handles().set.erase(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_destroy: not a live handle");
+  }
   if (h->stream) cudaStreamSynchronize(h->stream);
   drop_step_graphs(h);
   for (auto& pe : h->pending) {
@@ -901,7 +926,7 @@ icwf_status icwf_destroy(icwf_handle h) {
 }
 
 icwf_status icwf_set_projectors(icwf_handle h, int32_t n_states, const double* phi) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_projectors: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_projectors: not a live handle");
   if (n_states < 0 || n_states > 8 || (n_states > 0 && !phi))
     return fail(h, ICWF_ERR_ARG, "icwf_set_projectors: n_states must be in [0, 8] with phi given");
   if (h->phi) { cudaFree(h->phi); h->phi = nullptr; }
@@ -1008,7 +1033,7 @@ static icwf_status init_common(icwf_handle h, const double* psi0, const std::vec
 
 icwf_status icwf_init_from_positions(icwf_handle h, const double* psi0, const double* x,
                                      const double* R) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_init_from_positions: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_init_from_positions: not a live handle");
   if (!psi0 || !x || !R) return fail(h, ICWF_ERR_ARG, "icwf_init_from_positions: NULL array");
   std::vector<double> xs(x, x + h->N), Rs(R, R + h->N);
   return init_common(h, psi0, xs, Rs);
@@ -1016,7 +1041,7 @@ icwf_status icwf_init_from_positions(icwf_handle h, const double* psi0, const do
 
 icwf_status icwf_init_from_density(icwf_handle h, const double* psi0, uint64_t seed) {
   NvtxRange nvtx_("icwf_init_from_density");
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_init_from_density: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_init_from_density: not a live handle");
   if (!psi0) return fail(h, ICWF_ERR_ARG, "icwf_init_from_density: psi0 is NULL");
   const int nx = h->nx, nR = h->nR, N = h->N;
   const size_t n = (size_t)nx * nR;
@@ -1050,7 +1075,7 @@ icwf_status icwf_init_from_density(icwf_handle h, const double* psi0, uint64_t s
 
 icwf_status icwf_step(icwf_handle h, int32_t n_steps) {
   NvtxRange nvtx_("icwf_step");
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_step: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_step: not a live handle");
   if (!h->initialised) return fail(h, ICWF_ERR_STATE, "icwf_step: handle not initialised");
   if (n_steps < 0) return fail(h, ICWF_ERR_ARG, "icwf_step: n_steps < 0");
   if (n_steps > 0 && h->step_graphs && !h->prof_on && step_graphs_ready(h)) {
@@ -1071,7 +1096,7 @@ icwf_status icwf_step(icwf_handle h, int32_t n_steps) {
 
 icwf_status icwf_observables(icwf_handle h, icwf_obs* out) {
   NvtxRange nvtx_("icwf_observables");
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_observables: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_observables: not a live handle");
   if (!out) return fail(h, ICWF_ERR_ARG, "icwf_observables: out is NULL");
   if (!h->initialised) return fail(h, ICWF_ERR_STATE, "icwf_observables: handle not initialised");
   icwf_status st = alloc_obs(h);
@@ -1109,7 +1134,7 @@ icwf_status icwf_observables(icwf_handle h, icwf_obs* out) {
 
 icwf_status icwf_get_state(icwf_handle h, double* C, double* x, double* R, double* psi,
                            double* chi) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_get_state: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_get_state: not a live handle");
   if (!h->initialised) return fail(h, ICWF_ERR_STATE, "icwf_get_state: handle not initialised");
   CK(cudaStreamSynchronize(h->stream));
   const int N = h->N;
@@ -1132,7 +1157,7 @@ icwf_status icwf_get_state(icwf_handle h, double* C, double* x, double* R, doubl
 }
 
 icwf_status icwf_get_matrices(icwf_handle h, double* S, double* Hout, double* Heff) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_get_matrices: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_get_matrices: not a live handle");
   if (!h->initialised) return fail(h, ICWF_ERR_STATE, "icwf_get_matrices: handle not initialised");
   CK(cudaStreamSynchronize(h->stream));
   const int N = h->N, nx = h->nx, nR = h->nR;
@@ -1223,13 +1248,14 @@ size_t state_bytes(icwf_ctx* h) {
 }  // namespace
 
 icwf_status icwf_state_bytes(icwf_handle h, size_t* bytes) {
-  if (!h || !bytes) return fail(h, ICWF_ERR_ARG, "icwf_state_bytes: NULL argument");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_state_bytes: not a live handle");
+  if (!bytes) return fail(h, ICWF_ERR_ARG, "icwf_state_bytes: NULL argument");
   *bytes = state_bytes(h);
   return ICWF_OK;
 }
 
 icwf_status icwf_save_state(icwf_handle h, void* buf, size_t bytes) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_save_state: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_save_state: not a live handle");
   NvtxRange nvtx_("icwf_save_state");
   if (!h->initialised) return fail(h, ICWF_ERR_STATE, "icwf_save_state: handle not initialised");
   if (!buf || bytes < state_bytes(h))
@@ -1251,7 +1277,7 @@ icwf_status icwf_save_state(icwf_handle h, void* buf, size_t bytes) {
 }
 
 icwf_status icwf_load_state(icwf_handle h, const void* buf, size_t bytes) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_load_state: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_load_state: not a live handle");
   NvtxRange nvtx_("icwf_load_state");
   if (!buf || bytes < sizeof(StateHeader)) return fail(h, ICWF_ERR_ARG, "icwf_load_state: buffer too small");
   StateHeader hd;
@@ -1284,7 +1310,7 @@ icwf_status icwf_load_state(icwf_handle h, const void* buf, size_t bytes) {
 }
 
 icwf_status icwf_get_info(icwf_handle h, icwf_info* out) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_get_info: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_get_info: not a live handle");
   if (!out) return fail(h, ICWF_ERR_ARG, "icwf_get_info: out is NULL");
   out->rank = h->K;
   out->tail_rel = h->tail_rel;
@@ -1300,13 +1326,14 @@ icwf_status icwf_get_info(icwf_handle h, icwf_info* out) {
 }
 
 icwf_status icwf_work_bytes(icwf_handle h, size_t* bytes) {
-  if (!h || !bytes) return fail(h, ICWF_ERR_ARG, "icwf_work_bytes: NULL argument");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_work_bytes: not a live handle");
+  if (!bytes) return fail(h, ICWF_ERR_ARG, "icwf_work_bytes: NULL argument");
   *bytes = h->work_bytes;
   return ICWF_OK;
 }
 
 icwf_status icwf_set_regularisation(icwf_handle h, double eps) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_regularisation: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_regularisation: not a live handle");
   if (!std::isfinite(eps)) return fail(h, ICWF_ERR_ARG, "icwf_set_regularisation: eps is not finite");
   h->p.s_reg_eps = eps;
   h->version += 1;   // a pool re-captures this job's step graphs
@@ -1314,21 +1341,21 @@ icwf_status icwf_set_regularisation(icwf_handle h, double eps) {
 }
 
 icwf_status icwf_set_emulated_update(icwf_handle h, int32_t on) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_emulated_update: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_emulated_update: not a live handle");
   h->emu_update = on != 0;
   h->version += 1;   // the step graphs hold the previous update kernels: re-capture them
   return ICWF_OK;
 }
 
 icwf_status icwf_set_step_graphs(icwf_handle h, int32_t on) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_step_graphs: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_step_graphs: not a live handle");
   h->step_graphs = on != 0;
   if (!h->step_graphs) drop_step_graphs(h);
   return ICWF_OK;
 }
 
 icwf_status icwf_set_wait_limit(icwf_handle h, int64_t polls) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_wait_limit: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_set_wait_limit: not a live handle");
   if (polls > (int64_t)INT32_MAX - 1) return fail(h, ICWF_ERR_ARG, "icwf_set_wait_limit: polls too large");
   const int v = polls < 0 ? 0 : (int)polls + 1;
   CK(cudaStreamSynchronize(h->stream));
@@ -1337,19 +1364,20 @@ icwf_status icwf_set_wait_limit(icwf_handle h, int64_t polls) {
 }
 
 icwf_status icwf_get_stream(icwf_handle h, void** stream) {
-  if (!h || !stream) return fail(h, ICWF_ERR_ARG, "icwf_get_stream: NULL argument");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_get_stream: not a live handle");
+  if (!stream) return fail(h, ICWF_ERR_ARG, "icwf_get_stream: NULL argument");
   *stream = (void*)h->stream;
   return ICWF_OK;
 }
 
 icwf_status icwf_profile_enable(icwf_handle h, int32_t on) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_profile_enable: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_profile_enable: not a live handle");
   h->prof_on = on != 0;
   return ICWF_OK;
 }
 
 icwf_status icwf_profile_reset(icwf_handle h) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_profile_reset: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_profile_reset: not a live handle");
   CK(cudaStreamSynchronize(h->stream));
   prof_collect(h);
   for (int f = 0; f < F_COUNT; ++f) { h->prof_ms[f] = 0; h->prof_n[f] = 0; }
@@ -1358,7 +1386,7 @@ icwf_status icwf_profile_reset(icwf_handle h) {
 
 icwf_status icwf_profile_read(icwf_handle h, int32_t n, const char** names, double* ms,
                               int64_t* launches, int32_t* n_out) {
-  if (!h) return fail(nullptr, ICWF_ERR_ARG, "icwf_profile_read: NULL handle");
+  if (!live(h)) return fail(nullptr, ICWF_ERR_ARG, "icwf_profile_read: not a live handle");
   CK(cudaStreamSynchronize(h->stream));
   prof_collect(h);
   for (int f = 0; f < F_COUNT && f < n; ++f) {
@@ -1554,7 +1582,7 @@ icwf_status icwf_pool_get_stats(icwf_pool pool, icwf_pool_stats* out) {
 }
 
 icwf_status icwf_pool_submit(icwf_pool pool, icwf_handle job, int64_t n_steps, int32_t* job_id) {
-  if (!pool || !job || n_steps < 0) return fail(nullptr, ICWF_ERR_ARG, "icwf_pool_submit: invalid argument");
+  if (!pool || !live(job) || n_steps < 0) return fail(nullptr, ICWF_ERR_ARG, "icwf_pool_submit: invalid argument");
   if (!job->initialised) return fail(nullptr, ICWF_ERR_STATE, "icwf_pool_submit: job not initialised");
   if (footprint(job) > pool->budget)
     return fail(nullptr, ICWF_ERR_OOM, "icwf_pool_submit: job footprint exceeds the pool budget");

@@ -148,7 +148,7 @@ extern "C" icwf_status icwf_heff_direct(icwf_handle h, int32_t n_cols, const int
   using namespace icwf;
   ObsView v;
   if (!h || !handle_obs_view(h, &v)) {
-    handle_set_error(nullptr, "icwf_heff_direct: NULL handle");
+    handle_set_error(nullptr, "icwf_heff_direct: not a live handle");
     return ICWF_ERR_ARG;
   }
   if (!v.initialised) {

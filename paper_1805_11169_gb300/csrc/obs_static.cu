@@ -59,7 +59,7 @@ extern "C" icwf_status icwf_observables_static(icwf_handle h, icwf_obs* out) {
   using namespace icwf;
   ObsView v;
   if (!h || !handle_obs_view(h, &v)) {
-    handle_set_error(nullptr, "icwf_observables_static: NULL handle");
+    handle_set_error(nullptr, "icwf_observables_static: not a live handle");
     return ICWF_ERR_ARG;
   }
   if (!out) {
