@@ -1116,18 +1116,6 @@ struct HerkSlices {
   unsigned* ticket;
 };
 
-// round(x 2^q), |x| 2^q < 2^62, half away from zero
-__device__ __forceinline__ long long fixed_of_f32(float x, int q) {
-  const uint32_t u = __float_as_uint(x), E = (u >> 23) & 0xFFu;
-  const unsigned long long mant = (u & 0x7FFFFFu) | (E ? 0x800000u : 0u);
-  const int s = (E ? (int)E - 150 : -149) + q;
-  unsigned long long r;
-  if (s >= 0) r = mant << s;
-  else if (s <= -25) r = 0;
-  else r = (mant + (1ull << (-s - 1))) >> (-s);
-  return u >> 31 ? -(long long)r : (long long)r;
-}
-
 // Digits of the panel's rows from R0 on, 16 threads per row with 8 columns each; rows past N: zeros.
 // Also resets the Gram launch's ticket and writes its table.
 __global__ void __launch_bounds__(256) k_herk_slices(HerkSlices p) {
@@ -1158,12 +1146,11 @@ __global__ void __launch_bounds__(256) k_herk_slices(HerkSlices p) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const float h = plane ? v[k].z : v[k].x, l = plane ? v[k].w : v[k].y;
-      long long X = bad ? 0 : fixed_of_f32(h, q) + fixed_of_f32(l, q);
+      int dg[HERK_D];
+      cut_digits<HERK_D>(bad ? 0 : fixed_of_f32(h, q) + fixed_of_f32(l, q), dg);
 #pragma unroll
-      for (int d = HERK_D - 1; d >= 0; --d) {
-        const int dg = d > 0 ? (int)((X + 64) & 127) - 64 : (int)X;
-        X = (X - dg) >> 7;
-        const uint32_t b = __float_as_uint(small_int_to_float(dg)) >> 16;
+      for (int d = 0; d < HERK_D; ++d) {
+        const uint32_t b = __float_as_uint(small_int_to_float(dg[d])) >> 16;
         if (k & 1) pk[d][k >> 1] |= b << 16;
         else pk[d][k >> 1] = b;
       }

@@ -104,11 +104,28 @@ SL_HD long long fixed_of(double x, int q) {
   return (u >> 63) ? -(long long)r : (long long)r;
 }
 
-// D balanced base-2^7 digits of round(x 2^q), most significant first: the lower ones in [-64, 63], the
-// first takes what is left (|d_0| <= 64 when |x| 2^q <= 2^(6 + 7 (D - 1))).
+// The same of an FP32 number.
+SL_HD long long fixed_of_f32(float x, int q) {
+#if defined(__CUDA_ARCH__)
+  const uint32_t u = __float_as_uint(x);
+#else
+  uint32_t u;
+  memcpy(&u, &x, 4);
+#endif
+  const uint32_t E = (u >> 23) & 0xFFu;
+  const unsigned long long mant = (u & 0x7FFFFFu) | (E ? 0x800000u : 0u);
+  const int s = (E ? (int)E - 150 : -149) + q;
+  unsigned long long r;
+  if (s >= 0) r = mant << s;
+  else if (s <= -25) r = 0;
+  else r = (mant + (1ull << (-s - 1))) >> (-s);
+  return u >> 31 ? -(long long)r : (long long)r;
+}
+
+// D balanced base-2^7 digits of X, most significant first: the lower ones in [-64, 63], the first takes
+// what is left (|d_0| <= 64 when |X| <= 2^(6 + 7 (D - 1))).
 template <int D>
-SL_HD void digits_of(double x, int q, int (&dg)[D]) {
-  long long X = fixed_of(x, q);
+SL_HD void cut_digits(long long X, int (&dg)[D]) {
 #if defined(__CUDACC__)
 #pragma unroll
 #endif
@@ -118,6 +135,11 @@ SL_HD void digits_of(double x, int q, int (&dg)[D]) {
     X = (X - d) >> 7;
   }
   dg[0] = (int)X;
+}
+// digits of round(x 2^q)
+template <int D>
+SL_HD void digits_of(double x, int q, int (&dg)[D]) {
+  cut_digits<D>(fixed_of(x, q), dg);
 }
 
 // An integer of at most 22 bits as a float: added to the bits of 1.5 2^23, whose unit is 1.
