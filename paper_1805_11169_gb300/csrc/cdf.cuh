@@ -55,17 +55,6 @@ __device__ __forceinline__ void cacc_mul(cacc& a, cdf x, cdf y) {
   acc_small(a.im, DF_FMA(x.re.h, y.im.l, DF_MUL(x.re.l, y.im.h)));
   acc_small(a.im, DF_FMA(x.im.h, y.re.l, DF_MUL(x.im.l, y.re.h)));
 }
-// a += x * conj(y)
-__device__ __forceinline__ void cacc_mulc(cacc& a, cdf x, cdf y) {
-  acc_prod(a.re, x.re.h, y.re.h);
-  acc_prod(a.re, x.im.h, y.im.h);
-  acc_small(a.re, DF_FMA(x.re.h, y.re.l, DF_MUL(x.re.l, y.re.h)));
-  acc_small(a.re, DF_FMA(x.im.h, y.im.l, DF_MUL(x.im.l, y.im.h)));
-  acc_prod(a.im, x.im.h, y.re.h);
-  acc_prod(a.im, -x.re.h, y.im.h);
-  acc_small(a.im, DF_FMA(x.im.h, y.re.l, DF_MUL(x.im.l, y.re.h)));
-  acc_small(a.im, -DF_FMA(x.re.h, y.im.l, DF_MUL(x.re.l, y.im.h)));
-}
 // a += conj(x) * y
 __device__ __forceinline__ void cacc_cmul(cacc& a, cdf x, cdf y) {
   acc_prod(a.re, x.re.h, y.re.h);

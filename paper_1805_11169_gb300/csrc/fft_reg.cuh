@@ -2,7 +2,8 @@
 // element in eight), 2 to 4 radix-2 stages per pass in a thread's registers.
 //
 // FP64 instructions bound these transforms (an SM takes one warp's instruction per 19 cycles), so the
-// butterflies a +- w b take six of them instead of eight: with w = m (1 + i r), |r| <= 1,
+// butterflies a +- w b take six of them instead of eight (the fused multiply-add butterfly of Linzer
+// and Feig, with the larger part of the twiddle factored out): with w = m (1 + i r), |r| <= 1,
 //   u = p - r q, v = q + r p, (a.x +- m u, a.y +- m v),   p + i q = b or i b,
 // where the second form (w = -i m (1 + i r) i) serves the angles whose sine is the larger part.  Both
 // directions have the twiddle on the second operand: forward, natural to bit-reversed order, with one

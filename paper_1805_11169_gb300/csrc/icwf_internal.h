@@ -198,8 +198,9 @@ int launch_chol_solve(int N, const double2* L, const double2* D, const double2* 
 // double-float reciprocal pivots (8 bytes each); y and out are complex128.
 void launch_shift_mix_df(int N, const double2* S0, const double2* S1, double eps, double theta,
                          void* A, cudaStream_t s);
-// One launch per block column with look-ahead; ctl holds chol_ctl_words(N) words of ticket and
-// flag state (the launcher zeroes it).
+// One persistent launch with look-ahead, or panels of chol_panel(N) block columns with their trailing
+// updates on the tensor cores in herk_scratch (herk_df_bytes(N); NULL: one launch at every size).  ctl
+// holds chol_ctl_words(N) words of ticket and flag state (the launcher zeroes it).
 int launch_cholesky_df(int N, void* const* A, void* const* inv, void* const* D, int nbatch,
                        unsigned* ctl, void* herk_scratch, int* status, cudaStream_t s);
 size_t chol_ctl_words(int N);

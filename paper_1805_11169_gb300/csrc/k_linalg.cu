@@ -86,7 +86,6 @@ __device__ __forceinline__ bool pivot_ok(double d) {
   const long long b = __double_as_longlong(d);
   return b > 0 && b < 0x7FF0000000000000ll;
 }
-__device__ __forceinline__ double2 cmul_conj(double2 a, double2 b) { return cmul(a, cconj(b)); }
 // a -= t conj(b) in four FMAs
 __device__ __forceinline__ double2 csub_mul_conj(double2 a, double2 t, double2 b) {
   a.x = fma(-t.x, b.x, fma(-t.y, b.y, a.x));
@@ -165,7 +164,7 @@ __global__ void __launch_bounds__(PF_THREADS) k_potrf_diag(int N, MatBatch mb, i
 // Rows (warps) per panel-solve CTA: one per scheduler while that fills no more than the chip (a
 // scheduler takes a warp's FP64 instruction every 64 cycles: two warps double the substitution's time),
 // else two.  At N = 500 the last panels take 12.8 us with 4 and 14.8 with 8, the first 17.3 and 14.8.
-constexpr int TR_WARPS = 8, TR_WARPS_FEW = 4, TR_FEW_ROWS = TR_WARPS_FEW * 148;
+constexpr int TR_WARPS = 8, TR_WARPS_FEW = 4, TR_FEW_ROWS = TR_WARPS_FEW * 152;   // 152 SMs
 
 // Panel solve A_ib <- A_ib L_bb^-H below the diagonal block jb in FP64: one warp per row, lane =
 // column, column-oriented substitution on unscaled numerators: a_c -= a_m (conj(L_cm) / L_mm)

@@ -122,9 +122,6 @@ struct Grp {
 };
 
 __device__ __forceinline__ cdf ldcg4(const float4* p) { return ld4(__ldcg(p)); }
-__device__ __forceinline__ cdf cdf_sub_sloppy(cdf a, cdf b) {
-  return cdf_make(df_add_sloppy(a.re, df_neg(b.re)), df_add_sloppy(a.im, df_neg(b.im)));
-}
 // a += x y for double-float reals (Dot2 step on the high parts, cross terms in FP32)
 __device__ __forceinline__ void acc_prod_df(acc2& a, df x, df y) {
   acc_prod(a, x.h, y.h);

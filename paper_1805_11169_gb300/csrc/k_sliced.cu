@@ -1513,8 +1513,10 @@ int AsmPlan::launch(const JobView& j, double2* S, double2* H, cudaStream_t s) co
 }
 
 // Psi[i nR + j] = sum_a C_a psi_a(x_i) chi_a(R_j) as a sliced product over the trajectories: 8 digits
-// in the FP64 mode, 5 (34 bits below each grid point's largest term) in the mixed modes, whose terms
-// carry FP32 rounding.
+// in the FP64 mode, 5 in the mixed modes, whose terms carry FP32 rounding.  Digits are cut below the largest
+// component of an operand's row, so a sum is good to 2^-55 (2^-34) of max_a |C_a psi_a(x_i)| max_a
+// |chi_a(R_j)|, which is more than the largest term where different trajectories give the two maxima: far
+// out in the tails of Psi.
 int AsmPlan::reconstruct(const JobView& j, const double2* C, double2* Psi, cudaStream_t s) const {
   using namespace sl;
   const Impl& m = *impl;
