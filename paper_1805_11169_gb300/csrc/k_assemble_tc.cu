@@ -25,8 +25,8 @@
 // there the small cross products are summed first, in a pass of their own, and only the 512 leading
 // ones meet large sums: 7.7e-6.
 //
-// Bound: operands from L2 into shared memory, 80 KB per 24 MMAs (1.16 ms at N = 1024, 16 terms on
-// 1024 x 512).  Sliced FP16 pieces with an accumulator per level took 0.50 ms there and left Heff closer
+// Bound: operands from L2 into shared memory, 80 KB per 24 MMAs (0.95 ms at N = 1024, 16 terms on 1024 x
+// 512; 7.1 GB of L2 traffic, the tensor pipe busy 32%; 1.1 ms with k_prep and the overlap).  Sliced FP16 pieces with an accumulator per level took 0.50 ms there and left Heff closer
 // to its exact value (4e-8 instead of 8e-7), but moved rho_x by 2e-5 against the results users have.
 //
 // Every wait on an mbarrier is bounded (globaltimer, 2 s); a timeout sets the status flag, stops

@@ -39,9 +39,10 @@
 // Bound: an MMA of M = 128 takes max(N / 2, operand bytes / 128) cycles (measured over N = 32..256), so
 // the wide operands of all pieces at once keep it on the tensor pipe's side; the copies' writes into
 // shared memory come on top.
-// Measured (GB300, N = 1024 on 1024 x 512; ms per assembly, before -> now): FP64 mode, 22 terms, 144
-// (FP64 FMAs) -> 3.5; FP64, N = 16, 64 terms on 128 x 64, 13.1 (one CTA) -> 0.26; reconstruction in the
-// FP64 mode 4.3 -> 0.22.
+// Measured (GB300; ms per assembly, before -> now): FP64 mode, N = 1024, 22 terms on 1024 x 512, 144 (FP64
+// FMAs) -> 4.0, the tensor pipe busy 63-66% of k_gram_sliced; N = 16, 64 terms on 128 x 64, 13.1 (one CTA)
+// -> 0.11; N = 256, 21 terms on 512 x 256, 17.7 -> 0.32; reconstruction at N = 1024 in the FP64 mode
+// 4.3 -> 0.22.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -894,7 +895,7 @@ struct HeffArgs {
 };
 
 // Threads of one 32 x 32 patch of a 128 x 128 upper-triangle tile: lane = bra, 4 kets each.  Bound: 8
-// FP64 instructions per term, element and side (0.39 ms at N = 1024 and 22 terms).  With fewer patches
+// FP64 instructions per term, element and side (0.4 ms at N = 1024 and 22 terms).  With fewer patches
 // than SMs the terms are split over CTAs as well (16 trajectories, 64 terms: 202 us without, 50 us
 // with).
 constexpr int HG = 16;   // terms staged at a time
