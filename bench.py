@@ -323,6 +323,8 @@ def line_roofline(prof, w, K, mode, peaks, solve="df64", nfact=2):
     if tr:
         out["traffic_unit"] = "bytes per call (DRAM read + write, ncu)"
         out["traffic_source"] = tr[1]
+    if out["kernel"] == "cholesky" and solve == "df64" and mode != "fp64" and w.n_traj > 832:
+        out["peak_source"] += "; above N = 832 the trailing updates run on the tensor cores"
     return out
 
 
